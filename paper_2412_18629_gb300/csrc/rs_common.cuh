@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -187,6 +188,9 @@ struct ProfScope {
 int after_launch(rs_ctx* ctx, const char* name);
 #define RS_LAUNCHED(ctx, name) RS_TRY(rs::after_launch((ctx), (name)))
 
+// Whether the squared softening is a normal float32 (rsd::inv_sqrt<true> then holds).
+inline bool normal_eps2(float eps2) { return eps2 >= FLT_MIN; }
+
 inline unsigned grid_for(int64_t work, int block) {
   int64_t g = (work + block - 1) / block;
   if (g < 1) g = 1;
@@ -276,6 +280,19 @@ __device__ __forceinline__ float wrap_diff(float a, float b, float L, float hL) 
 // (dx*dx + dy*dy) + dz*dz in float32 with every operation rounded separately.
 __device__ __forceinline__ float sq3(float dx, float dy, float dz) {
   return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+}
+
+// 1 / sqrt(x) for the float32 potentials. rsqrtf of a library built without flush-to-zero scales
+// subnormal operands before and after the hardware instruction: three more instructions a pair in
+// loops that are bound by issue slots and the special-function unit. With a normal squared
+// softening every argument is at least eps^2, so kNormal takes the flush-to-zero form of the same
+// instruction, whose value for a normal or infinite argument is the same.
+template <bool kNormal>
+__device__ __forceinline__ float inv_sqrt(float x) {
+  if (!kNormal) return rsqrtf(x);
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 // Union-find over uint32 indices; roots are the smallest index of their set. Parent reads

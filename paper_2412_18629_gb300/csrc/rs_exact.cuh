@@ -34,7 +34,7 @@ __device__ __forceinline__ double kinetic(float4 v, const double* vb) {
 // (the same per-member summation as the direct-sum kernels). Including the self term, whose
 // computed value is exactly w0 = rsqrt(eps^2), removes every per-pair index test; k_flags_list
 // subtracts it and widens the certified bound accordingly.
-template <int kListR>
+template <int kListR, bool kNormal>
 __global__ void __launch_bounds__(kListThreads)
 k_potential_list(int64_t nbig, const int64_t* __restrict__ tile_off, const int64_t* __restrict__ nodes,
                  const int64_t* __restrict__ lofs, const int64_t* __restrict__ lend,
@@ -90,7 +90,7 @@ k_potential_list(int64_t nbig, const int64_t* __restrict__ tile_off, const int64
           const float2 dy = __fadd2_rn(make_float2(a.z, a.w), ny[pp]);
           const float2 dz = __fadd2_rn(zz, nz[pp]);
           const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
-          blk[pp] = __fadd2_rn(blk[pp], make_float2(rsqrtf(r2.x), rsqrtf(r2.y)));
+          blk[pp] = __fadd2_rn(blk[pp], make_float2(rsd::inv_sqrt<kNormal>(r2.x), rsd::inv_sqrt<kNormal>(r2.y)));
         }
       }
 #pragma unroll
@@ -108,6 +108,21 @@ k_potential_list(int64_t nbig, const int64_t* __restrict__ tile_off, const int64
   for (int k = 0; k < kListR; ++k) {
     const int64_t a = l0 + threadIdx.x + kListThreads * k;
     if (a < l1) Sx[list[a]] = S[k];
+  }
+}
+
+// The kernel's launch for R members per thread (2, 4 or 8).
+template <class... Args>
+void launch_potential_list(int R, float eps2, unsigned grid, cudaStream_t st, Args... args) {
+  auto launch = [&](auto kernel) { kernel<<<grid, kListThreads, 0, st>>>(args...); };
+  if (rs::normal_eps2(eps2)) {
+    if (R == 2) launch(k_potential_list<2, true>);
+    else if (R == 8) launch(k_potential_list<8, true>);
+    else launch(k_potential_list<4, true>);
+  } else {
+    if (R == 2) launch(k_potential_list<2, false>);
+    else if (R == 8) launch(k_potential_list<8, false>);
+    else launch(k_potential_list<4, false>);
   }
 }
 

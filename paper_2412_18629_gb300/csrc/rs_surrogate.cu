@@ -463,6 +463,7 @@ __global__ void k_sur_spot_mark(int64_t ns, const uint32_t* __restrict__ sur_mem
 
 // Exact float32 potential of listed members (one warp each) and the certified flag; members
 // whose energy is within the bound of zero are queued for the float64 potential.
+template <bool kNormal>
 __global__ void __launch_bounds__(kT)
 k_pot_member(const unsigned long long* __restrict__ count, const uint32_t* __restrict__ list,
              const uint32_t* __restrict__ sur_mem, const uint32_t* __restrict__ mnode,
@@ -489,7 +490,7 @@ k_pot_member(const unsigned long long* __restrict__ count, const uint32_t* __res
           const float dx = __fsub_rn(uj.x, ui.x);
           const float dy = __fsub_rn(uj.y, ui.y);
           const float dz = __fsub_rn(uj.z, ui.z);
-          const float wv = rsqrtf(__fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, eps2))));
+          const float wv = rsd::inv_sqrt<kNormal>(__fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, eps2))));
           blk = __fadd_rn(blk, j == i ? 0.f : wv);
         }
       }
@@ -516,6 +517,7 @@ k_pot_member(const unsigned long long* __restrict__ count, const uint32_t* __res
 // k_pot_member for groups of 4 consecutive list entries of the same node (the calibration
 // list: 64 per node): one warp per group shares every target load among the 4 members; each
 // member's sum has the same per-lane order as k_pot_member (bit-identical result).
+template <bool kNormal>
 __global__ void __launch_bounds__(kT)
 k_pot_member4(const unsigned long long* __restrict__ count, const uint32_t* __restrict__ list,
               const uint32_t* __restrict__ sur_mem, const uint32_t* __restrict__ mnode,
@@ -554,7 +556,7 @@ k_pot_member4(const unsigned long long* __restrict__ count, const uint32_t* __re
             const float dx = __fsub_rn(uj.x, ui[r].x);
             const float dy = __fsub_rn(uj.y, ui[r].y);
             const float dz = __fsub_rn(uj.z, ui[r].z);
-            const float wv = rsqrtf(__fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, eps2))));
+            const float wv = rsd::inv_sqrt<kNormal>(__fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, eps2))));
             blk[r] = __fadd_rn(blk[r], j == i[r] ? 0.f : wv);
           }
         }
@@ -826,7 +828,8 @@ int surrogate_unbind(rs_ctx* ctx, const double* vbulk, uint8_t* bound, unsigned 
     RS_LAUNCHED(ctx, "k_sur_calib_list");
     {
       ProfScope prof_(ctx, "k_pot_member", st);
-      k_pot_member4<<<grid, kT, 0, st>>>(counters + 9, calib_list, sur_mem, h.mnode, h.node_off,
+      auto* kernel = normal_eps2(eps * eps) ? k_pot_member4<true> : k_pot_member4<false>;
+      kernel<<<grid, kT, 0, st>>>(counters + 9, calib_list, sur_mem, h.mnode, h.node_off,
                                          h.node_size, h.U, h.V, vbulk, eps * eps, Gm, Sx, bound, ambig,
                                          counters + 2);
     }
@@ -890,15 +893,8 @@ int surrogate_unbind(rs_ctx* ctx, const double* vbulk, uint8_t* bound, unsigned 
       if (c < 3) RS_CUDA(ctx, cudaEventRecord(e0, st));
       {
         ProfScope prof_(ctx, c < 3 ? "k_potential_list_tune" : "k_potential_list", st);
-        if (R == 2)
-          k_potential_list<2><<<grid, kListThreads, 0, st>>>(nbig, ltiles, big_nodes, lofs, lend, exact_list,
-                                                             sur_mem, h.node_off, h.node_size, h.U, eps * eps, Sx);
-        else if (R == 8)
-          k_potential_list<8><<<grid, kListThreads, 0, st>>>(nbig, ltiles, big_nodes, lofs, lend, exact_list,
-                                                             sur_mem, h.node_off, h.node_size, h.U, eps * eps, Sx);
-        else
-          k_potential_list<4><<<grid, kListThreads, 0, st>>>(nbig, ltiles, big_nodes, lofs, lend, exact_list,
-                                                             sur_mem, h.node_off, h.node_size, h.U, eps * eps, Sx);
+        launch_potential_list(R, eps * eps, grid, st, nbig, ltiles, big_nodes, lofs, lend, exact_list, sur_mem,
+                              h.node_off, h.node_size, h.U, eps * eps, Sx);
       }
       RS_LAUNCHED(ctx, "k_potential_list");
       if (c < 3) {
@@ -936,7 +932,8 @@ int surrogate_unbind(rs_ctx* ctx, const double* vbulk, uint8_t* bound, unsigned 
   RS_LAUNCHED(ctx, "k_sur_spot_mark");
   {
     ProfScope prof_(ctx, "k_pot_member", st);
-    k_pot_member<<<grid, kT, 0, st>>>(counters + 1, check_list, sur_mem, h.mnode, h.node_off, h.node_size,
+    auto* kernel = normal_eps2(eps * eps) ? k_pot_member<true> : k_pot_member<false>;
+    kernel<<<grid, kT, 0, st>>>(counters + 1, check_list, sur_mem, h.mnode, h.node_off, h.node_size,
                                       h.U, h.V, vbulk, eps * eps, Gm, Sx, bound, ambig, counters + 2);
   }
   RS_LAUNCHED(ctx, "k_pot_member");

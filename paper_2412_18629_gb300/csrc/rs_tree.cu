@@ -732,15 +732,8 @@ int rs::tree_decide(rs_ctx* ctx, const int* only, const uint8_t* want, const dou
   const unsigned grid = grid_for(T / (kListThreads * R) + nt + 1, 1);
   {
     ProfScope prof_(ctx, "k_potential_list", st);
-    if (R == 2)
-      k_potential_list<2><<<grid, kListThreads, 0, st>>>(nt, ltiles, tnode, lofs, lend, ulist, tpos, h.node_off,
-                                                         h.node_size, h.U, eps2, Sx);
-    else if (R == 8)
-      k_potential_list<8><<<grid, kListThreads, 0, st>>>(nt, ltiles, tnode, lofs, lend, ulist, tpos, h.node_off,
-                                                         h.node_size, h.U, eps2, Sx);
-    else
-      k_potential_list<4><<<grid, kListThreads, 0, st>>>(nt, ltiles, tnode, lofs, lend, ulist, tpos, h.node_off,
-                                                         h.node_size, h.U, eps2, Sx);
+    launch_potential_list(R, eps2, grid, st, nt, ltiles, tnode, lofs, lend, ulist, tpos, h.node_off, h.node_size,
+                          h.U, eps2, Sx);
   }
   RS_LAUNCHED(ctx, "k_potential_list");
   const double Gm = ctx->cfg.G * ctx->cfg.particle_mass;

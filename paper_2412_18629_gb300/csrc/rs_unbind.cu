@@ -52,6 +52,7 @@ constexpr int kCounters = 24;  // the unbinding counters (see rs_unbind)
 // a warp are consecutive members, mostly of one node), the node's members read through L1 in
 // ascending order; the same 32-term blocks and Kahan steps as the blocked kernel. A node is
 // selected when its tile count (scanned) is non-zero.
+template <bool kNormal>
 __global__ void __launch_bounds__(kT)
 k_potential(int64_t m, const uint32_t* __restrict__ mnode, const int64_t* __restrict__ tile_off,
             const int64_t* __restrict__ node_off, const int64_t* __restrict__ node_size,
@@ -73,7 +74,7 @@ k_potential(int64_t m, const uint32_t* __restrict__ mnode, const int64_t* __rest
       const float dy = __fsub_rn(uj.y, ui.y);
       const float dz = __fsub_rn(uj.z, ui.z);
       const float r2 = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, eps2)));
-      const float w = rsqrtf(r2);
+      const float w = rsd::inv_sqrt<kNormal>(r2);
       blk = __fadd_rn(blk, jj == self ? 0.f : w);
     }
     const float y = __fsub_rn(blk, C);
@@ -92,7 +93,10 @@ k_potential(int64_t m, const uint32_t* __restrict__ mnode, const int64_t* __rest
 // are formed as u_j + (-u_i), which equals fl(u_j - u_i). The per-member summation is
 // unchanged (32-term sequential blocks, Kahan across blocks), so the certified bound kCertB
 // holds as is. The self pair is tested only on the diagonal j-tiles. Blocks are ordered by
-// the node's size class, largest first, so the longest blocks start first.
+// the node's size class, largest first, so the longest blocks start first. Bound by issue slots
+// and the special-function unit (one rsqrt a pair); the flush-to-zero rsqrt (rsd::inv_sqrt) took
+// this kernel from 56.3 to 41.8 ms on the nodes below 16384 members of the 2^27 snapshot and the
+// list form of rs_exact.cuh from 110 to 82 ms.
 constexpr int kBlkThreads = 128;
 // Members per thread (kBlkR) is a template parameter chosen per context by the autotuner among
 // 2, 4 and 8 (tiles of 256, 512 or 1024 members); every choice gives bit-identical sums.
@@ -137,6 +141,7 @@ __global__ void k_tiles_split(int64_t nn, const int64_t* __restrict__ node_size,
 // blocks, self term 0) is the blocked kernel's, so the sums are bit-identical to it.
 constexpr int kTileThreads = 128;
 
+template <bool kNormal>
 __global__ void __launch_bounds__(kTileThreads)
 k_potential_tiled(int64_t nn, const int64_t* __restrict__ tile_off, const int64_t* __restrict__ node_off,
                   const int64_t* __restrict__ node_size, const float4* __restrict__ U, float eps2,
@@ -162,7 +167,7 @@ k_potential_tiled(int64_t nn, const int64_t* __restrict__ tile_off, const int64_
         const float dx = __fsub_rn(uj.x, ui.x);
         const float dy = __fsub_rn(uj.y, ui.y);
         const float dz = __fsub_rn(uj.z, ui.z);
-        const float w = rsqrtf(__fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, eps2))));
+        const float w = rsd::inv_sqrt<kNormal>(__fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, eps2))));
         blk = __fadd_rn(blk, j0 + jj == i ? 0.f : w);
       }
       const float y = __fsub_rn(blk, C);
@@ -189,16 +194,17 @@ __global__ void k_perm_tiles(int64_t nn, const uint32_t* __restrict__ perm,
   if (r < nn) out[r] = big[perm[r]];
 }
 
+template <bool kNormal>
 __device__ __forceinline__ void pot_pair(float4 a, float2 zz, float2 nx, float2 ny, float2 nz,
                                          float2 e2, float2& w) {
   const float2 dx = __fadd2_rn(make_float2(a.x, a.y), nx);
   const float2 dy = __fadd2_rn(make_float2(a.z, a.w), ny);
   const float2 dz = __fadd2_rn(zz, nz);
   const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
-  w = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+  w = make_float2(rsd::inv_sqrt<kNormal>(r2.x), rsd::inv_sqrt<kNormal>(r2.y));
 }
 
-template <int kBlkR>
+template <int kBlkR, bool kNormal>
 __global__ void __launch_bounds__(kBlkThreads)
 k_potential_blocked(int64_t nn, const int64_t* __restrict__ tile_off, const uint32_t* __restrict__ perm,
                     const int64_t* __restrict__ node_off, const int64_t* __restrict__ node_size,
@@ -253,7 +259,7 @@ k_potential_blocked(int64_t nn, const int64_t* __restrict__ tile_off, const uint
 #pragma unroll
           for (int p = 0; p < kBlkR / 2; ++p) {
             float2 w;
-            pot_pair(a, zz, nx[p], ny[p], nz[p], e2, w);
+            pot_pair<kNormal>(a, zz, nx[p], ny[p], nz[p], e2, w);
             blk[p] = __fadd2_rn(blk[p], w);
           }
         }
@@ -265,7 +271,7 @@ k_potential_blocked(int64_t nn, const int64_t* __restrict__ tile_off, const uint
 #pragma unroll
           for (int p = 0; p < kBlkR / 2; ++p) {
             float2 w;
-            pot_pair(a, zz, nx[p], ny[p], nz[p], e2, w);
+            pot_pair<kNormal>(a, zz, nx[p], ny[p], nz[p], e2, w);
             if (self && jt == 2 * p) w.x = 0.f;
             if (self && jt == 2 * p + 1) w.y = 0.f;
             blk[p] = __fadd2_rn(blk[p], w);
@@ -602,12 +608,18 @@ int launch_blocked(rs_ctx* ctx, int R, const int64_t* tile_perm, const uint32_t*
   const int64_t m = ctx->n_members, nn = ctx->n_nodes;
   const float eps2 = ctx->cfg.softening * ctx->cfg.softening;
   const unsigned grid = grid_for(m / (kBlockedMin + 1) + m / (kBlkThreads * R) + 1, 1);
-  if (R == 2)
-    k_potential_blocked<2><<<grid, kBlkThreads, 0, st>>>(nn, tile_perm, perm, h.node_off, h.node_size, h.U, eps2, S);
-  else if (R == 8)
-    k_potential_blocked<8><<<grid, kBlkThreads, 0, st>>>(nn, tile_perm, perm, h.node_off, h.node_size, h.U, eps2, S);
-  else
-    k_potential_blocked<4><<<grid, kBlkThreads, 0, st>>>(nn, tile_perm, perm, h.node_off, h.node_size, h.U, eps2, S);
+  auto launch = [&](auto kernel) {
+    kernel<<<grid, kBlkThreads, 0, st>>>(nn, tile_perm, perm, h.node_off, h.node_size, h.U, eps2, S);
+  };
+  if (normal_eps2(eps2)) {
+    if (R == 2) launch(k_potential_blocked<2, true>);
+    else if (R == 8) launch(k_potential_blocked<8, true>);
+    else launch(k_potential_blocked<4, true>);
+  } else {
+    if (R == 2) launch(k_potential_blocked<2, false>);
+    else if (R == 8) launch(k_potential_blocked<8, false>);
+    else launch(k_potential_blocked<4, false>);
+  }
   RS_LAUNCHED(ctx, "k_potential_blocked");
   return RS_OK;
 }
@@ -661,8 +673,8 @@ int direct_potential(rs_ctx* ctx, int64_t sur_min, const int* only, int64_t max_
   RS_TRY(potential_tiles(ctx, sur_min, only, max_g, R, tile_small, tile_perm, &perm, st, pairs));
   {
     ProfScope prof_(ctx, "k_potential", st);
-    k_potential<<<grid_for(m, kT), kT, 0, st>>>(m, h.mnode, tile_small, h.node_off, h.node_size, h.U,
-                                               eps * eps, S);
+    auto* kernel = normal_eps2(eps * eps) ? k_potential<true> : k_potential<false>;
+    kernel<<<grid_for(m, kT), kT, 0, st>>>(m, h.mnode, tile_small, h.node_off, h.node_size, h.U, eps * eps, S);
   }
   RS_LAUNCHED(ctx, "k_potential");
   if (plain) {  // one member per thread, node order (the plain form has no size-ordered tiles)
@@ -670,7 +682,8 @@ int direct_potential(rs_ctx* ctx, int64_t sur_min, const int* only, int64_t max_
     RS_LAUNCHED(ctx, "k_tiles_plain");
     RS_TRY(exclusive_scan_i64(ctx, nn, tile_perm, tile_perm + nn, st));
     ProfScope prof_(ctx, "k_potential_tiled", st);
-    k_potential_tiled<<<grid_for(m / (kBlockedMin + 1) + m / kTileThreads + 1, 1), kTileThreads, 0, st>>>(
+    auto* kernel = normal_eps2(eps * eps) ? k_potential_tiled<true> : k_potential_tiled<false>;
+    kernel<<<grid_for(m / (kBlockedMin + 1) + m / kTileThreads + 1, 1), kTileThreads, 0, st>>>(
         nn, tile_perm, h.node_off, h.node_size, h.U, eps * eps, S);
     RS_LAUNCHED(ctx, "k_potential_tiled");
     return RS_OK;
