@@ -637,8 +637,10 @@ Hier hier_of(rs_ctx* ctx) {
 // Batched form: exactly pruned nearest-neighbour and link searches (rs_prune6d.cu).
 int prune6d_prepare(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m,
                     const double* sums, cudaStream_t st);
-int prune6d_nn(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, float* nn2,
-               cudaStream_t st);
+int prune6d_near(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, float* nn2,
+                 cudaStream_t st);
+int prune6d_far(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, float* nn2,
+                cudaStream_t st);
 int prune6d_check(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t m, float* nn2, const int** failed_out,
                   cudaStream_t st);
 int prune6d_link(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, const float* nn2,
@@ -862,9 +864,23 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
     // where the brute-force pair kernels (identical results) cost less than the bucket set-up
     const bool batched = ctx->cfg.batched != 0 && m > kPrunedMinMembers;
     const int64_t tiles_ub = nn + m / kTile6 + 1;
+    // k-th smallest nn2 of the level's nodes (of those with only[k] != 0 when `only` is given); the
+    // batched form's nn2 is in its sorted order, in which every node keeps its range
+    auto select = [&](const int* only) -> int {
+      Hier hs = hier_of(ctx);
+      ProfScope prof_(ctx, "k_select_l2", st);
+      k_select_l2_warp<<<grid_for(nn, kT / 32), kT, 0, st>>>(nb, nn, hs.node_off, hs.node_size, nn2, mb, f_num,
+                                                            f_den, hs.inv, only);
+      RS_LAUNCHED(ctx, "k_select_l2_warp");
+      k_select_l2<<<unsigned(nn), kT, 0, st>>>(nb, hs.node_off, hs.node_size, nn2, mb, f_num, f_den, hs.inv, only);
+      RS_LAUNCHED(ctx, "k_select_l2");
+      return RS_OK;
+    };
     if (batched) {
       RS_TRY(prune6d_prepare(ctx, nb, nn, mb, m, sums, st));
-      RS_TRY(prune6d_nn(ctx, nb, nn, mb, m, nn2, st));
+      RS_TRY(prune6d_near(ctx, nb, nn, mb, m, nn2, st));
+      RS_TRY(select(nullptr));  // of the near values: bounds the far searches
+      RS_TRY(prune6d_far(ctx, nb, nn, mb, m, nn2, st));
       h = hier_of(ctx);
     } else {
       k_tile_counts<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.node_size, kTile6, tile_off);
@@ -877,26 +893,12 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       }
       RS_LAUNCHED(ctx, "k_nn6d");
     }
-    {
-      ProfScope prof_(ctx, "k_select_l2", st);
-      k_select_l2_warp<<<grid_for(nn, kT / 32), kT, 0, st>>>(nb, nn, h.node_off, h.node_size, nn2, mb, f_num,
-                                                            f_den, h.inv, nullptr);
-      k_select_l2<<<unsigned(nn), kT, 0, st>>>(nb, h.node_off, h.node_size, nn2, mb, f_num, f_den, h.inv,
-                                               nullptr);
-    }
-    RS_LAUNCHED(ctx, "k_select_l2");
+    RS_TRY(select(nullptr));
     if (batched) {  // bounded searches: nodes whose l2 fell outside their bounds, exactly again
       const int* failed = nullptr;
       RS_TRY(prune6d_check(ctx, nb, nn, m, nn2, &failed, st));
-      if (failed) {  // bounded nodes can be small enough for the warp selection too
-        h = hier_of(ctx);
-        ProfScope prof_(ctx, "k_select_l2", st);
-        k_select_l2_warp<<<grid_for(nn, kT / 32), kT, 0, st>>>(nb, nn, h.node_off, h.node_size, nn2, mb, f_num,
-                                                              f_den, h.inv, failed);
-        k_select_l2<<<unsigned(nn), kT, 0, st>>>(nb, h.node_off, h.node_size, nn2, mb, f_num, f_den, h.inv,
-                                                 failed);
-        RS_LAUNCHED(ctx, "k_select_l2");
-      }
+      if (failed) RS_TRY(select(failed));
+      h = hier_of(ctx);
     }
     k_iota_u32<<<grid_for(m, kT), kT, 0, st>>>(m, uf);
     RS_LAUNCHED(ctx, "k_iota_u32");

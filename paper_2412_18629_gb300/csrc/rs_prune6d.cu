@@ -1,30 +1,50 @@
 // Pruned 6D nearest-neighbour and link searches for the batched form of rs_fof6d.
 //
 // The plain form evaluates d6 for every pair of a node. Here the members of every node of a
-// level are ordered by a 3D Hilbert key of their scaled position offsets (every candidate of a
-// 6D search lies within sqrt(bound / inv_sx2) in position) and cut into buckets of 32
-// consecutive members; each bucket has a 6D bounding box, four 8-member sub-boxes, and every
-// 32 consecutive buckets of a node form a superbucket with its own box. Persistent warps pull
-// query buckets from a queue ordered by node size (largest first) and, lane = member, visit
-// the node's superbuckets, buckets and sub-buckets, skipping any whose lower bound exceeds the
-// lane's current best (nearest neighbour) or l2 (link, upper triangle of bucket pairs). The
-// link pass runs on the members with a friend only (nn2 <= l2: no other member can be linked),
-// compacted in the same order and bucketed again, so its boxes are tighter and no lane idles.
-// Nodes of 4096 members or more search their nearest neighbours within bounds of l2 taken
-// from an exactly searched sample (see k_sample_bounds; a device check re-searches any node
-// whose l2 falls outside them). Distances and bounds use packed float32x2 arithmetic with each
-// half rounded like the scalar operation. Lower bounds are computed with the same
-// round-to-nearest float32 operations as d6 on the per-axis gaps to the box: every step is
-// monotone, so the bound never exceeds the computed d6 of any member inside the box, and
-// pruning cannot change the minimum or the set of links. Results are therefore bit-identical
-// to the brute-force kernels (and to the definition).
+// level are ordered by a 6D Hilbert key of their scaled position and velocity offsets and cut
+// into buckets of 32 consecutive members; each bucket has a 6D bounding box, and every 32
+// consecutive buckets of a node form a superbucket (1024 members) with its own box. Ordering by
+// all six coordinates keeps a bucket small in velocity too: in a node of 7e5 members a search
+// evaluates about a sixth of the pairs that buckets of a 3D position curve need.
+//
+// Persistent warps pull query buckets from a queue ordered by node size (largest first). A
+// search tests 32 boxes at a time against the box of the warp's open queries (lane = box), then
+// each surviving bucket box against every query (lane = query); a bucket that some queries need
+// is loaded with lane = target, and the warp loops over those queries (about 3 of 32 lanes need a
+// given bucket, so lane = query would idle most of the warp). Distances and bounds use packed
+// float32x2 arithmetic over (position, velocity) pairs, each half rounded like the scalar
+// operation. Lower bounds are computed with the same round-to-nearest float32 operations as d6
+// on the per-axis gaps to the box: every step is monotone, so the bound never exceeds the
+// computed d6 of any member inside the box, and pruning cannot change the minimum or the set of
+// links. Results are therefore bit-identical to the brute-force kernels (and to the definition).
+//
+// Nearest neighbours: every member inside its own superbucket first (k_nn_near; complete for
+// nodes of one superbucket). The k-th smallest of those values bounds l2 from above, so the rest
+// of the search (k_nn_far) goes no further than that; nodes of 4096 members or more also get a
+// lower bound from an exactly searched sample of their buckets and search only their members at
+// or above it (a device check after the selection re-searches any node whose l2 falls outside).
+//
+// Links: only members with a friend (nn2 <= l2) can be linked; they are compacted in the same
+// order and bucketed again, and each is first united with its nearest neighbour. k_link_near
+// unites inside each superbucket, skipping targets that already share the query's root;
+// k_link_far then searches the rest of the node for the members outside the node's largest
+// component only (every remaining link has such an end), skipping buckets and targets that
+// already share the query's root. Few distances are left to evaluate and few unions are made
+// (about 0.3 a member instead of 17).
+//
+// Measured on the 2^27-particle snapshot (12 levels, 1.2e8 members), before and after this form:
+// nearest-neighbour kernels 382 -> 99 ms, link kernels 266 -> 100 ms (3D Hilbert buckets with
+// sub-boxes, lane = query). Both are bound by issue slots (box tests and distance evaluations from
+// L1 and L2).
 #include "rs_cro.cuh"
 
 namespace rs {
 int prune6d_prepare(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m,
                     const double* sums, cudaStream_t st);
-int prune6d_nn(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, float* nn2,
-               cudaStream_t st);
+int prune6d_near(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, float* nn2,
+                 cudaStream_t st);
+int prune6d_far(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, float* nn2,
+                cudaStream_t st);
 int prune6d_check(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t m, float* nn2, const int** failed_out,
                   cudaStream_t st);
 int prune6d_link(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, const float* nn2,
@@ -37,6 +57,7 @@ namespace {
 
 constexpr int kT = 256;
 constexpr int kWarpsPerBlock = 8;
+constexpr unsigned kFull = 0xffffffffu;
 
 struct Bucket {
   uint32_t start;    // level-local sorted position of the first member
@@ -51,56 +72,98 @@ struct Bucket {
 
 // 6D box, stored for the packed float32x2 bounds: (position, velocity) pairs per axis, the
 // lower corner and the NEGATED upper corner (so both gaps are additions).
-struct Box {
+struct __align__(16) Box {
   float4 lo01;   // (x, vx, y, vy)
   float4 nhi01;  // -(x, vx, y, vy) of the upper corner
   float2 lo2;    // (z, vz)
   float2 nhi2;
 };
 
-__device__ __forceinline__ uint32_t quant8(float c) {
-  // scaled offset (in units of the node's total position sigma) in [-4, 4) -> 0..255
-  float t = (c + 4.0f) * 32.0f;
-  t = fminf(fmaxf(t, 0.0f), 255.0f);
-  return uint32_t(t);
+// 4 bits an axis: 24 key bits (three sort passes below the node index); in a CPU model of a
+// 7e5-member node a fifth bit saves 1% of the searches' work.
+constexpr int kAxisBits = 4;
+constexpr int kKeyBits = 6 * kAxisBits;
+
+// Scaled offset c (units of the node's total sigma) to 0 .. 2^kAxisBits - 1 through c / (0.5 + |c|),
+// which spends most cells on the node's dense middle (12% fewer box tests than a linear map).
+__device__ __forceinline__ uint32_t quant_axis(float c) {
+  constexpr float half = float(1 << (kAxisBits - 1));
+  const float t = half + half * (c / (0.5f + fabsf(c)));
+  return uint32_t(fminf(fmaxf(t, 0.0f), 2.0f * half - 1.0f));
 }
 
-// 3D Hilbert key of each member's position offset from the node mean (scaled by the node's
-// sigma_x), prefixed by the node index.
-__global__ void k_hilbert3(int64_t mb, int64_t m, int64_t nb, const uint32_t* __restrict__ mnode,
-                          const float4* __restrict__ U, const float4* __restrict__ inv,
-                          const float4* __restrict__ mean_u, uint64_t* __restrict__ keys,
-                          uint32_t* __restrict__ vals) {
+// 6D Hilbert index of quantised coordinates by Skilling's transform (J. Skilling, "Programming
+// the Hilbert curve", AIP Conf. Proc. 707, 2004), axis 0 leading.
+__device__ __forceinline__ uint32_t hilbert6(uint32_t (&X)[6]) {
+#pragma unroll
+  for (uint32_t q = 1u << (kAxisBits - 1); q > 1; q >>= 1) {
+    const uint32_t p = q - 1;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      if (X[i] & q) {
+        X[0] ^= p;
+      } else {
+        const uint32_t t = (X[0] ^ X[i]) & p;
+        X[0] ^= t;
+        X[i] ^= t;
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 1; i < 6; ++i) X[i] ^= X[i - 1];
+  uint32_t t = 0;
+#pragma unroll
+  for (uint32_t q = 1u << (kAxisBits - 1); q > 1; q >>= 1)
+    if (X[5] & q) t ^= q - 1;
+  uint32_t key = 0;
+#pragma unroll
+  for (int b = kAxisBits - 1; b >= 0; --b)
+#pragma unroll
+    for (int i = 0; i < 6; ++i) key = (key << 1) | (((X[i] ^ t) >> b) & 1u);
+  return key;
+}
+
+// 6D Hilbert key of each member's offset from the node mean (scaled by the node's sigmas),
+// prefixed by the node index.
+__global__ void k_hilbert6(int64_t mb, int64_t m, int64_t nb, const uint32_t* __restrict__ mnode,
+                           const float4* __restrict__ U, const float4* __restrict__ V,
+                           const float4* __restrict__ inv, const float4* __restrict__ mean_u,
+                           const float4* __restrict__ mean_v, uint64_t* __restrict__ keys,
+                           uint32_t* __restrict__ vals) {
   const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (p >= m) return;
   const uint32_t q = mnode[mb + p];
-  const float sx = sqrtf(inv[q].x);
-  const float4 u = U[mb + p], mu = mean_u[q];
-  const uint32_t code = rsd::hilbert3<8>(quant8((u.x - mu.x) * sx), quant8((u.y - mu.y) * sx),
-                                   quant8((u.z - mu.z) * sx));
-  keys[p] = (uint64_t(q - nb) << 24) | uint64_t(code);
+  const float4 iv = inv[q];
+  const float sx = sqrtf(iv.x), sv = sqrtf(iv.y);
+  const float4 u = U[mb + p], mu = mean_u[q], v = V[mb + p], mv = mean_v[q];
+  uint32_t X[6] = {quant_axis((u.x - mu.x) * sx), quant_axis((u.y - mu.y) * sx), quant_axis((u.z - mu.z) * sx),
+                   quant_axis((v.x - mv.x) * sv), quant_axis((v.y - mv.y) * sv), quant_axis((v.z - mv.z) * sv)};
+  keys[p] = (uint64_t(q - nb) << kKeyBits) | uint64_t(hilbert6(X));
   vals[p] = uint32_t(p);
 }
 
-// Node mean positions (float) from the canonical-order moment sums, for the quantisation only.
+// Node means (float) from the canonical-order moment sums, for the quantisation only.
 __global__ void k_node_means(int64_t nb, int64_t nn, const int64_t* __restrict__ node_size,
-                             const double* __restrict__ sums, float4* __restrict__ mean_u) {
+                             const double* __restrict__ sums, float4* __restrict__ mean_u,
+                             float4* __restrict__ mean_v) {
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (k >= nn) return;
   const double g = double(node_size[nb + k]);
   const double* S = sums + 12 * k;
   mean_u[nb + k] = make_float4(float(S[0] / g), float(S[1] / g), float(S[2] / g), 0.f);
+  mean_v[nb + k] = make_float4(float(S[6] / g), float(S[7] / g), float(S[8] / g), 0.f);
 }
 
+// Members in sorted order as (position, velocity) pairs: XY = (x, vx, y, vy), Z = (z, vz).
 __global__ void k_gather_sorted(int64_t mb, int64_t m, const uint32_t* __restrict__ order,
                                 const float4* __restrict__ U, const float4* __restrict__ V,
-                                float4* __restrict__ Us, float4* __restrict__ Vs,
-                                uint32_t* __restrict__ sp) {
+                                float4* __restrict__ XY, float2* __restrict__ Z, uint32_t* __restrict__ sp) {
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (s >= m) return;
   const uint32_t p = order[s];
-  Us[s] = U[mb + p];
-  Vs[s] = V[mb + p];
+  const float4 u = U[mb + p], v = V[mb + p];
+  XY[s] = make_float4(u.x, v.x, u.y, v.y);
+  Z[s] = make_float2(u.z, v.z);
   sp[s] = p;
 }
 
@@ -130,20 +193,30 @@ __global__ void k_active_flags(int64_t m, int64_t mb, const uint32_t* __restrict
                                const float* __restrict__ nn2, int64_t* __restrict__ flag) {
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (s >= m) return;
-  const uint32_t p = sp[s];
-  flag[s] = nn2[p] <= inv[mnode[mb + p]].z ? 1 : 0;
+  flag[s] = nn2[s] <= inv[mnode[mb + sp[s]]].z ? 1 : 0;
 }
 
-__global__ void k_compact_active(int64_t m, const int64_t* __restrict__ pos, const float4* __restrict__ Us,
-                                 const float4* __restrict__ Vs, const uint32_t* __restrict__ sp,
-                                 float4* __restrict__ UsA, float4* __restrict__ VsA,
-                                 uint32_t* __restrict__ spA) {
+__global__ void k_compact_active(int64_t m, const int64_t* __restrict__ pos, const float4* __restrict__ XY,
+                                 const float2* __restrict__ Z, const uint32_t* __restrict__ sp,
+                                 float4* __restrict__ XYA, float2* __restrict__ ZA,
+                                 uint32_t* __restrict__ spA, uint32_t* __restrict__ ufA) {
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (s >= m || pos[s + 1] == pos[s]) return;
   const int64_t a = pos[s];
-  UsA[a] = Us[s];
-  VsA[a] = Vs[s];
+  XYA[a] = XY[s];
+  ZA[a] = Z[s];
   spA[a] = sp[s];
+  ufA[a] = uint32_t(a);
+}
+
+// Each compacted member united with the neighbour that gave its nn2: their d6 is at most l2, so
+// that neighbour has a friend too.
+__global__ void k_link_friends(int64_t m, const int64_t* __restrict__ pos, const uint32_t* __restrict__ friend_of,
+                               uint32_t* __restrict__ ufA) {
+  const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (s >= m || pos[s + 1] == pos[s]) return;
+  const uint32_t f = friend_of[s];
+  if (int64_t(f) != s && pos[f + 1] != pos[f]) rsd::uf_unite(ufA, uint32_t(pos[s]), uint32_t(pos[f]));
 }
 
 __global__ void k_active_ranges(int64_t nb, int64_t nn, int64_t mb, const int64_t* __restrict__ node_off,
@@ -156,19 +229,17 @@ __global__ void k_active_ranges(int64_t nb, int64_t nn, int64_t mb, const int64_
   cnt[k] = pos[s0 + node_size[nb + k]] - pos[s0];
 }
 
-__device__ __forceinline__ void warp_box(const float (&a)[6], bool valid, int lo_off, int hi_off,
-                                         float (&lo)[6], float (&hi)[6]) {
+// Box of the warp's valid lanes' points (lane = point; a = x, y, z, vx, vy, vz); every lane gets it.
+__device__ __forceinline__ void warp_box(const float (&a)[6], bool valid, float (&lo)[6], float (&hi)[6]) {
   const float inf = __int_as_float(0x7f800000);
 #pragma unroll
   for (int d = 0; d < 6; ++d) {
-    if (lo_off == 1) {
-      lo[d] = valid ? a[d] : inf;
-      hi[d] = valid ? a[d] : -inf;
-    }
+    lo[d] = valid ? a[d] : inf;
+    hi[d] = valid ? a[d] : -inf;
 #pragma unroll
-    for (int off = lo_off; off <= hi_off; off <<= 1) {
-      lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], off));
-      hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], off));
+    for (int off = 1; off <= 16; off <<= 1) {
+      lo[d] = fminf(lo[d], __shfl_xor_sync(kFull, lo[d], off));
+      hi[d] = fmaxf(hi[d], __shfl_xor_sync(kFull, hi[d], off));
     }
   }
 }
@@ -179,15 +250,14 @@ __device__ __forceinline__ Box make_box(const float (&lo)[6], const float (&hi)[
              make_float2(lo[2], lo[5]), make_float2(-hi[2], -hi[5])};
 }
 
-// One warp per bucket (padding warps write a queue key that sorts last): bucket table entry,
-// box, four 8-member sub-boxes (an empty sub-bucket gets lo = +inf, hi = -inf, so every gap to
-// it is +inf), and the work-queue key (largest node first).
+// One warp per bucket (padding warps write a queue key that sorts last): bucket table entry, box,
+// and the work-queue key (largest node first).
 __global__ void __launch_bounds__(kT)
 k_buckets(int64_t nb, int64_t nn, int64_t nbk_ub, const int64_t* __restrict__ bucket_off,
           const int64_t* __restrict__ sb_off, const int64_t* __restrict__ nstart,
-          const int64_t* __restrict__ ncnt, const float4* __restrict__ Us,
-          const float4* __restrict__ Vs, Bucket* __restrict__ bk, Box* __restrict__ box,
-          Box* __restrict__ sub, uint64_t* __restrict__ qkey, uint32_t* __restrict__ qval) {
+          const int64_t* __restrict__ ncnt, const float4* __restrict__ XY,
+          const float2* __restrict__ Z, Bucket* __restrict__ bk, Box* __restrict__ box,
+          uint64_t* __restrict__ qkey, uint32_t* __restrict__ qval) {
   const int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= nbk_ub) return;
@@ -204,12 +274,11 @@ k_buckets(int64_t nb, int64_t nn, int64_t nbk_ub, const int64_t* __restrict__ bu
   const int64_t start = nstart[k] + 32 * kb;
   const int cnt = int(rsd::min64(32, ncnt[k] - 32 * kb));
   const bool valid = lane < cnt;
-  const float4 u = Us[start + (valid ? lane : 0)], v = Vs[start + (valid ? lane : 0)];
-  const float a[6] = {u.x, u.y, u.z, v.x, v.y, v.z};
+  const float4 xy = XY[start + (valid ? lane : 0)];
+  const float2 z = Z[start + (valid ? lane : 0)];
+  const float a[6] = {xy.x, xy.z, z.x, xy.y, xy.w, z.y};
   float lo[6], hi[6];
-  warp_box(a, valid, 1, 4, lo, hi);
-  if ((lane & 7) == 0) sub[4 * w + (lane >> 3)] = make_box(lo, hi);
-  warp_box(a, valid, 8, 16, lo, hi);
+  warp_box(a, valid, lo, hi);
   if (lane == 0) {
     Bucket b;
     b.start = uint32_t(start);
@@ -278,36 +347,6 @@ __device__ __forceinline__ float2 pmul(float2 a, float2 b) {
   return d;
 }
 
-// A query lane's coordinates, packed for the float32x2 arithmetic: (position, velocity)
-// pairs per axis and their negations for the box bounds; each coordinate negated and
-// duplicated for the distances to two targets at once; the metric scales.
-struct Query {
-  float2 qa, qb, qc, na, nb, nc;
-  float2 nux, nuy, nuz, nvx, nvy, nvz;
-  float2 s;         // (inv_sx2, inv_sv2)
-  float2 sx2, sv2;  // (inv_sx2, inv_sx2), (inv_sv2, inv_sv2)
-};
-
-__device__ __forceinline__ Query make_query(float4 u, float4 v, float isx, float isv) {
-  Query Q;
-  Q.qa = make_float2(u.x, v.x);
-  Q.qb = make_float2(u.y, v.y);
-  Q.qc = make_float2(u.z, v.z);
-  Q.na = make_float2(-u.x, -v.x);
-  Q.nb = make_float2(-u.y, -v.y);
-  Q.nc = make_float2(-u.z, -v.z);
-  Q.nux = make_float2(-u.x, -u.x);
-  Q.nuy = make_float2(-u.y, -u.y);
-  Q.nuz = make_float2(-u.z, -u.z);
-  Q.nvx = make_float2(-v.x, -v.x);
-  Q.nvy = make_float2(-v.y, -v.y);
-  Q.nvz = make_float2(-v.z, -v.z);
-  Q.s = make_float2(isx, isv);
-  Q.sx2 = make_float2(isx, isx);
-  Q.sv2 = make_float2(isv, isv);
-  return Q;
-}
-
 __device__ __forceinline__ float2 max0(float2 a, float2 b) {
   return make_float2(fmaxf(fmaxf(a.x, b.x), 0.f), fmaxf(fmaxf(a.y, b.y), 0.f));
 }
@@ -332,12 +371,6 @@ __device__ __forceinline__ float metric(float2 ga, float2 gb, float2 gc, float2 
   return __fadd_rn(t.x, t.y);
 }
 
-__device__ __forceinline__ float lb_point_box(const Query& Q, const Box& b) {
-  return metric(gap_pt(make_float2(b.lo01.x, b.lo01.y), make_float2(b.nhi01.x, b.nhi01.y), Q.qa, Q.na),
-                gap_pt(make_float2(b.lo01.z, b.lo01.w), make_float2(b.nhi01.z, b.nhi01.w), Q.qb, Q.nb),
-                gap_pt(b.lo2, b.nhi2, Q.qc, Q.nc), Q.s);
-}
-
 __device__ __forceinline__ float lb_box_box(const Box& a, const Box& b, float2 s) {
   return metric(gap_bb(make_float2(a.lo01.x, a.lo01.y), make_float2(a.nhi01.x, a.nhi01.y),
                        make_float2(b.lo01.x, b.lo01.y), make_float2(b.nhi01.x, b.nhi01.y)),
@@ -346,124 +379,82 @@ __device__ __forceinline__ float lb_box_box(const Box& a, const Box& b, float2 s
                 gap_bb(a.lo2, a.nhi2, b.lo2, b.nhi2), s);
 }
 
-// Staged targets of one warp, structure of arrays (x, y, z, vx, vy, vz); slots past the
-// bucket's count hold NaN, whose distance is NaN: it lowers no minimum and passes no test.
-struct __align__(16) Stage {  // 16-byte aligned: pairs of slots load as float2
-  float c[6][32];
+// A query lane's own coordinates as (position, velocity) pairs per axis, with their negations.
+struct Query {
+  float2 a, b, c, na, nb, nc;
 };
 
-// d6 of the query to targets j and j + 1 (j even): fl(fl(rx * isx) + fl(rv * isv)) with
-// rx = (dx^2 + dy^2) + dz^2, d = fl(u_j - u_i) formed as u_j + (-u_i), every operation rounded
-// separately; each half equals the scalar d6.
-__device__ __forceinline__ float2 d6_pair(const Query& Q, const Stage& S, int j) {
-  const float2 dx = padd(*reinterpret_cast<const float2*>(&S.c[0][j]), Q.nux);
-  const float2 dy = padd(*reinterpret_cast<const float2*>(&S.c[1][j]), Q.nuy);
-  const float2 dz = padd(*reinterpret_cast<const float2*>(&S.c[2][j]), Q.nuz);
-  const float2 ex = padd(*reinterpret_cast<const float2*>(&S.c[3][j]), Q.nvx);
-  const float2 ey = padd(*reinterpret_cast<const float2*>(&S.c[4][j]), Q.nvy);
-  const float2 ez = padd(*reinterpret_cast<const float2*>(&S.c[5][j]), Q.nvz);
-  const float2 rx = padd(padd(pmul(dx, dx), pmul(dy, dy)), pmul(dz, dz));
-  const float2 rv = padd(padd(pmul(ex, ex), pmul(ey, ey)), pmul(ez, ez));
-  return padd(pmul(rx, Q.sx2), pmul(rv, Q.sv2));
+__device__ __forceinline__ Query make_query(float4 xy, float2 z) {
+  Query Q;
+  Q.a = make_float2(xy.x, xy.y);
+  Q.b = make_float2(xy.z, xy.w);
+  Q.c = z;
+  Q.na = make_float2(-xy.x, -xy.y);
+  Q.nb = make_float2(-xy.z, -xy.w);
+  Q.nc = make_float2(-z.x, -z.y);
+  return Q;
 }
 
-__device__ __forceinline__ void stage(Stage& S, const float4* __restrict__ Us, const float4* __restrict__ Vs,
-                                      uint32_t start, int cnt, int lane) {
+__device__ __forceinline__ float lb_point_box(const Query& Q, const Box& b, float2 s) {
+  return metric(gap_pt(make_float2(b.lo01.x, b.lo01.y), make_float2(b.nhi01.x, b.nhi01.y), Q.a, Q.na),
+                gap_pt(make_float2(b.lo01.z, b.lo01.w), make_float2(b.nhi01.z, b.nhi01.w), Q.b, Q.nb),
+                gap_pt(b.lo2, b.nhi2, Q.c, Q.nc), s);
+}
+
+// d6 of target (xy, z) to the query with negated coordinates (nxy, nz): the differences formed as
+// u_j + (-u_i) = fl(u_j - u_i), then d6's order of operations.
+__device__ __forceinline__ float d6_pair(float4 xy, float2 z, float4 nxy, float2 nz, float2 s) {
+  return metric(padd(make_float2(xy.x, xy.y), make_float2(nxy.x, nxy.y)),
+                padd(make_float2(xy.z, xy.w), make_float2(nxy.z, nxy.w)), padd(z, nz), s);
+}
+
+// Shared memory of one warp: its queries' negated coordinates and roots, and 32 staged boxes.
+struct __align__(16) WarpShared {
+  Box box[32];
+  float4 nxy[32];
+  float2 nz[32];
+  uint32_t root[32];   // link: root of each query
+  uint32_t uni[32];    // link, far: root shared by all members of the staged box's bucket
+};
+
+// Target coordinates of a bucket, lane = member; lanes past its count hold NaN, whose distance is
+// NaN: as an unsigned value above every distance, and it passes no <= test.
+__device__ __forceinline__ void load_targets(const float4* __restrict__ XY, const float2* __restrict__ Z,
+                                             uint32_t start, int cnt, int lane, float4& xy, float2& z) {
   const float nan = __int_as_float(0x7fc00000);
-  float4 u = make_float4(nan, nan, nan, nan), v = u;
+  xy = make_float4(nan, nan, nan, nan);
+  z = make_float2(nan, nan);
   if (lane < cnt) {
-    u = Us[start + lane];
-    v = Vs[start + lane];
+    xy = XY[start + lane];
+    z = Z[start + lane];
   }
-  S.c[0][lane] = u.x;
-  S.c[1][lane] = u.y;
-  S.c[2][lane] = u.z;
-  S.c[3][lane] = v.x;
-  S.c[4][lane] = v.y;
-  S.c[5][lane] = v.z;
-}
-
-// Index visited at step t of the outward walk from a: a, a+1, a-1, a+2, a-2, ...
-__device__ __forceinline__ int64_t outward(int64_t a, int64_t t) {
-  const int64_t h = (t + 1) >> 1;
-  return (t & 1) ? a + h : a - h;
 }
 
 // Next query bucket from the size-ordered queue (one atomic per warp).
 __device__ __forceinline__ int64_t next_work(unsigned long long* counter, int lane) {
   unsigned long long w = 0;
   if (lane == 0) w = atomicAdd(counter, 1ull);
-  return int64_t(__shfl_sync(0xffffffffu, w, 0));
+  return int64_t(__shfl_sync(kFull, w, 0));
 }
 
-struct NNArgs {
+struct SearchArgs {
   const int64_t* nbuckets;
   const Bucket* bk;
   const Box* box;
-  const Box* sub;
   const Box* sbox;
   const uint32_t* order;
-  const float4* Us;
-  const float4* Vs;
-  const uint32_t* sp;
+  const float4* XY;
+  const float2* Z;
   const float4* inv;
   unsigned long long* counter;
   unsigned long long* work;  // [4]: NN d6, NN box tests, link d6, link box tests (counting variant)
-  const float2* bounds;      // NN only: per node of the level (node - nb): (lo, hi), or nullptr
   int64_t nb;
 };
-
-// Search limit of a nearest-neighbour lane with current minimum `best` and node bounds
-// [lo, hi]: boxes whose lower bound exceeds it are skipped. A lane below lo is done (-1: no
-// bound is negative); otherwise min(best, hi): a minimum above hi only needs to be known above
-// hi. With (lo, hi) = (-inf, +inf) this is best itself: the exact search.
-__device__ __forceinline__ float nn_limit(float best, float lo, float hi) {
-  return best < lo ? -1.f : fminf(best, hi);
-}
 
 // Per-lane tallies of the counting variant (evaluated d6 and box tests).
 struct Tally {
   unsigned long long d6 = 0, box = 0;
 };
-
-// Evaluate target bucket b for the warp's query lanes (nearest-neighbour search).
-template <bool kCount>
-__device__ __forceinline__ void nn_bucket(const NNArgs& A, int64_t a, int64_t b, bool valid, const Query& Q,
-                                          float& best, float lo, float hi, int lane, Stage& S, Tally& T) {
-  const Box B = A.box[b];
-  const bool need = valid && lb_point_box(Q, B) <= nn_limit(best, lo, hi);
-  if (kCount) T.box += valid;
-  if (!__any_sync(0xffffffffu, need)) return;
-  const Bucket Bb = A.bk[b];
-  __syncwarp();
-  stage(S, A.Us, A.Vs, Bb.start, int(Bb.count), lane);
-  __syncwarp();
-  for (uint32_t s0 = 0; s0 < Bb.count; s0 += 8) {
-    const Box Sb = A.sub[4 * b + (s0 >> 3)];
-    const bool sneed = need && lb_point_box(Q, Sb) <= nn_limit(best, lo, hi);
-    if (kCount) T.box += need;
-    if (!__any_sync(0xffffffffu, sneed)) continue;
-    if (sneed) {
-      const int s1 = int(min(s0 + 8, Bb.count));
-      if (kCount) T.d6 += uint32_t(s1) - s0;
-      if (b == a) {
-        for (int j = int(s0); j < s1; j += 2) {
-          const float2 d = d6_pair(Q, S, j);
-          best = fminf(best, j == lane ? best : d.x);
-          best = fminf(best, j + 1 == lane ? best : d.y);
-        }
-      } else {
-#pragma unroll
-        for (int j = int(s0); j < int(s0) + 8; j += 2) {
-          if (j < s1) {
-            const float2 d = d6_pair(Q, S, j);
-            best = fminf(fminf(best, d.x), d.y);
-          }
-        }
-      }
-    }
-  }
-}
 
 template <bool kCount>
 __device__ __forceinline__ void flush_tally(const Tally& T, unsigned long long* work, int lane) {
@@ -471,8 +462,8 @@ __device__ __forceinline__ void flush_tally(const Tally& T, unsigned long long* 
   unsigned long long d = T.d6, b = T.box;
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) {
-    d += __shfl_xor_sync(0xffffffffu, d, off);
-    b += __shfl_xor_sync(0xffffffffu, b, off);
+    d += __shfl_xor_sync(kFull, d, off);
+    b += __shfl_xor_sync(kFull, b, off);
   }
   if (lane == 0) {
     atomicAdd(work, d);
@@ -480,10 +471,67 @@ __device__ __forceinline__ void flush_tally(const Tally& T, unsigned long long* 
   }
 }
 
+// ---- Nearest neighbours -----------------------------------------------------------------------
+
+// Minimum over bucket b's members for every query in the mask `need`: the lane of each such query
+// lowers its best (float bits) and neighbour. kSelf: b is the query bucket itself.
+template <bool kCount, bool kSelf>
+__device__ __forceinline__ void nn_eval(const SearchArgs& A, uint32_t start, int cnt, unsigned need, float2 s,
+                                        uint32_t& best, uint32_t& nbr, int lane, const WarpShared& W, Tally& T) {
+  float4 xy;
+  float2 z;
+  load_targets(A.XY, A.Z, start, cnt, lane, xy, z);
+  if (kCount && lane < cnt) T.d6 += __popc(need) - ((kSelf && ((need >> lane) & 1u)) ? 1 : 0);
+  while (need) {
+    const int l0 = __ffs(need) - 1;
+    need &= need - 1u;
+    const int l1 = need ? __ffs(need) - 1 : l0;  // two queries side by side
+    need &= need - 1u;
+    uint32_t d0 = __float_as_uint(d6_pair(xy, z, W.nxy[l0], W.nz[l0], s));
+    uint32_t d1 = __float_as_uint(d6_pair(xy, z, W.nxy[l1], W.nz[l1], s));
+    if (kSelf) {
+      d0 = lane == l0 ? 0xffffffffu : d0;
+      d1 = lane == l1 ? 0xffffffffu : d1;
+    }
+    const uint32_t m0 = __reduce_min_sync(kFull, d0), m1 = __reduce_min_sync(kFull, d1);
+    const int j0 = __ffs(__ballot_sync(kFull, d0 == m0)) - 1, j1 = __ffs(__ballot_sync(kFull, d1 == m1)) - 1;
+    if (lane == l0 && m0 < best) {
+      best = m0;
+      nbr = start + j0;
+    }
+    if (lane == l1 && m1 < best) {
+      best = m1;
+      nbr = start + j1;
+    }
+  }
+}
+
+// Candidate buckets of one superbucket, [b_lo, b_hi) (at most 32): boxes staged in shared memory
+// by lane = box, those within `limit` (float bits) of the query box returned as a mask.
 template <bool kCount>
-__global__ void __launch_bounds__(kT, 4) k_nn6d_pruned(NNArgs A, float* __restrict__ nn2) {
-  __shared__ Stage stg[kWarpsPerBlock];
-  const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
+__device__ __forceinline__ unsigned stage_boxes(const SearchArgs& A, int64_t b_lo, int64_t b_hi, const Box& Q,
+                                                float limit, float2 s, int lane, WarpShared& W, Tally& T) {
+  const bool in = b_lo + lane < b_hi;
+  bool near = false;
+  __syncwarp();
+  if (in) {
+    const Box B = A.box[b_lo + lane];
+    W.box[lane] = B;
+    near = lb_box_box(Q, B, s) <= limit;
+    if (kCount) T.box += 1;
+  }
+  __syncwarp();
+  return __ballot_sync(kFull, near);
+}
+
+// Exact nearest neighbour of every member inside its own superbucket -> nn2 (sorted order) and
+// neighbour (sorted position).
+template <bool kCount>
+__global__ void __launch_bounds__(kT, 4)
+k_nn_near(SearchArgs A, float* __restrict__ nn2, uint32_t* __restrict__ friend_of) {
+  __shared__ WarpShared sh[kWarpsPerBlock];
+  const int lane = threadIdx.x & 31;
+  WarpShared& W = sh[threadIdx.x >> 5];
   const int64_t nbk = *A.nbuckets;
   Tally T;
   while (true) {
@@ -492,149 +540,352 @@ __global__ void __launch_bounds__(kT, 4) k_nn6d_pruned(NNArgs A, float* __restri
     const int64_t a = A.order[w];
     const Bucket Aq = A.bk[a];
     const float4 iv = A.inv[Aq.node];
+    const float2 s = make_float2(iv.x, iv.y);
     const bool valid = lane < int(Aq.count);
     const uint32_t si = Aq.start + (valid ? lane : 0);
-    const Query Q = make_query(A.Us[si], A.Vs[si], iv.x, iv.y);
-    float best = __int_as_float(0x7f800000);
-    float lo = -best, hi = best;
-    if (A.bounds) {
-      const float2 bd = A.bounds[int64_t(Aq.node) - A.nb];
-      lo = bd.x;
-      hi = bd.y;
-    }
-    const int64_t own = (a - int64_t(Aq.first)) >> 5, nsb = Aq.sbcount;
-    for (int64_t t = 0; t <= 2 * nsb; ++t) {
-      if (__all_sync(0xffffffffu, !valid || best < lo)) break;  // every lane known below lo
-      const int64_t s = outward(own, t);
-      if (s < 0 || s >= nsb) continue;
-      const Box SB = A.sbox[Aq.sbfirst + s];
-      const bool need = valid && lb_point_box(Q, SB) <= nn_limit(best, lo, hi);
-      if (kCount) T.box += valid;
-      if (!__any_sync(0xffffffffu, need)) continue;
-      const int64_t b_lo = int64_t(Aq.first) + 32 * s;
-      const int64_t b_hi = rsd::min64(b_lo + 32, int64_t(Aq.last) + 1);
-      if (s == own) {
-        for (int64_t t2 = 0; t2 <= 2 * 32; ++t2) {
-          const int64_t b = outward(a, t2);
-          if (b < b_lo || b >= b_hi) continue;
-          nn_bucket<kCount>(A, a, b, valid, Q, best, lo, hi, lane, stg[wb], T);
-        }
-      } else if (s > own) {
-        for (int64_t b = b_lo; b < b_hi; ++b)
-          nn_bucket<kCount>(A, a, b, valid, Q, best, lo, hi, lane, stg[wb], T);
-      } else {
-        for (int64_t b = b_hi - 1; b >= b_lo; --b)
-          nn_bucket<kCount>(A, a, b, valid, Q, best, lo, hi, lane, stg[wb], T);
+    const Query Q = make_query(A.XY[si], A.Z[si]);
+    __syncwarp();
+    W.nxy[lane] = make_float4(Q.na.x, Q.na.y, Q.nb.x, Q.nb.y);
+    W.nz[lane] = Q.nc;
+    __syncwarp();
+    uint32_t best = 0x7f800000u, nbr = si;
+    nn_eval<kCount, true>(A, Aq.start, int(Aq.count), Aq.count == 32 ? kFull : (1u << Aq.count) - 1u, s, best,
+                          nbr, lane, W, T);
+    const int64_t b_lo = int64_t(Aq.first) + ((a - int64_t(Aq.first)) & ~int64_t(31));
+    const int64_t b_hi = rsd::min64(b_lo + 32, int64_t(Aq.last) + 1);
+    if (b_hi - b_lo > 1) {
+      const float lim = __uint_as_float(__reduce_max_sync(kFull, valid ? best : 0u));
+      unsigned mask = stage_boxes<kCount>(A, b_lo, b_hi, A.box[a], lim, s, lane, W, T);
+      const int own = int(a - b_lo);
+      unsigned up = mask & ~((2u << own) - 1u), dn = mask & ((1u << own) - 1u);
+      while (up | dn) {  // outward from the query bucket: near buckets lower the limit first
+        const int iu = up ? __ffs(up) - 1 : 64, id = dn ? 31 - __clz(dn) : -64;
+        const int i = iu - own <= own - id ? iu : id;
+        if (i > own) up &= up - 1u; else dn &= ~(1u << i);
+        const bool need = valid && lb_point_box(Q, W.box[i], s) <= __uint_as_float(best);
+        if (kCount) T.box += valid;
+        const unsigned nm = __ballot_sync(kFull, need);
+        if (!nm) continue;
+        const int64_t b = b_lo + i;
+        const int cnt = b == int64_t(Aq.last) ? int(A.bk[b].count) : 32;
+        nn_eval<kCount, false>(A, uint32_t(int64_t(Aq.start) + 32 * (b - a)), cnt, nm, s, best, nbr, lane, W, T);
       }
     }
-    if (valid) nn2[A.sp[si]] = best;
+    if (valid) {
+      nn2[si] = __uint_as_float(best);
+      friend_of[si] = nbr;
+    }
   }
   flush_tally<kCount>(T, A.work, lane);
 }
 
-// Pending unions of each lane of a warp: member indices of its friends, lane-major columns.
-struct LinkQueue {
-  uint32_t j[32][32];
+// Which query buckets a k_nn_far launch takes. The first launch: the sampled buckets of the nodes
+// searched with bounds and every bucket of the other nodes; the second: the remaining buckets of the
+// bounded nodes; the third: every bucket of the nodes that failed the check.
+enum FarPass : int { kFarFirst, kFarRest, kFarFailed };
+
+struct FarArgs {
+  const float2* bounds;       // per node of the level: (lo, hi)
+  const int64_t* node_size;
+  const int* failed;          // third launch only
+  int64_t min_members;        // smallest node searched with sampled bounds
+  int pass;
 };
 
-// Union the warp's pending friends with their lanes' members, the lanes side by side (the
-// union order does not change the resulting components).
-__device__ __forceinline__ void flush_links(uint32_t* uf, uint32_t pi, const LinkQueue& LQ, int& qn,
-                                            int lane) {
-  const int mx = int(__reduce_max_sync(0xffffffffu, uint32_t(qn)));
-  for (int k = 0; k < mx; ++k)
-    if (k < qn) rsd::uf_unite(uf, pi, LQ.j[k][lane]);
-  qn = 0;
+constexpr int64_t kSampleBuckets = 48;
+
+__device__ __forceinline__ int64_t sample_stride(int64_t nbk) {
+  return nbk / kSampleBuckets > 1 ? nbk / kSampleBuckets : 1;
 }
 
-// Link pairs of query bucket a (box Abox) with target bucket b >= a.
+// The rest of the node for the members whose value is not yet known to be below lo: no further
+// than min(best, hi) (a minimum above hi only needs to be known above hi). Members of nodes with
+// one superbucket are complete.
 template <bool kCount>
-__device__ __forceinline__ void link_bucket(const NNArgs& A, int64_t a, int64_t b, const Box& Abox,
-                                            bool active, const Query& Q, uint32_t pi, float l2,
-                                            uint32_t* uf, int lane, Stage& S, uint32_t (&sj)[32],
-                                            LinkQueue& LQ, int& qn, Tally& T) {
-  const Box B = A.box[b];
-  if (kCount) T.box += (lane == 0);
-  if (lb_box_box(Abox, B, Q.s) > l2) return;
-  const bool need = active && lb_point_box(Q, B) <= l2;
-  if (kCount) T.box += active;
-  if (!__any_sync(0xffffffffu, need)) return;
-  const Bucket Bb = A.bk[b];
-  __syncwarp();
-  stage(S, A.Us, A.Vs, Bb.start, int(Bb.count), lane);
-  if (lane < int(Bb.count)) sj[lane] = A.sp[Bb.start + lane];
-  __syncwarp();
-  const int j0 = (b == a) ? lane + 1 : 0;
-  uint32_t pending = 0;  // targets of this bucket the lane links to (unions after the scan)
-  for (uint32_t s0 = 0; s0 < Bb.count; s0 += 8) {
-    const Box Sb = A.sub[4 * b + (s0 >> 3)];
-    if (kCount) T.box += (lane == 0);
-    if (lb_box_box(Abox, Sb, Q.s) > l2) continue;
-    const bool sneed = need && lb_point_box(Q, Sb) <= l2;
-    if (kCount) T.box += need;
-    if (!__any_sync(0xffffffffu, sneed)) continue;
-    if (sneed) {
-      const int s1 = int(min(s0 + 8, Bb.count));
-      if (kCount) T.d6 += s1 > max(int(s0), j0) ? uint32_t(s1 - max(int(s0), j0)) : 0u;
-      for (int j = int(s0); j < s1; j += 2) {
-        if (j + 1 < j0) continue;
-        const float2 d = d6_pair(Q, S, j);
-        if (j >= j0 && d.x <= l2) pending |= 1u << j;
-        if (j + 1 >= j0 && j + 1 < s1 && d.y <= l2) pending |= 2u << j;
+__global__ void __launch_bounds__(kT, 4)
+k_nn_far(SearchArgs A, FarArgs F, float* __restrict__ nn2, uint32_t* __restrict__ friend_of) {
+  __shared__ WarpShared sh[kWarpsPerBlock];
+  const int lane = threadIdx.x & 31;
+  WarpShared& W = sh[threadIdx.x >> 5];
+  const int64_t nbk = *A.nbuckets;
+  Tally T;
+  while (true) {
+    const int64_t w = next_work(A.counter, lane);
+    if (w >= nbk) break;
+    const int64_t a = A.order[w];
+    const Bucket Aq = A.bk[a];
+    const int64_t g = F.node_size[Aq.node];
+    if (g < 1024) break;  // size-class order: only nodes of one superbucket follow
+    if (Aq.sbcount == 1) continue;
+    const int64_t k = int64_t(Aq.node) - A.nb;
+    const int64_t own_rel = a - int64_t(Aq.first);
+    if (F.pass == kFarFailed) {
+      if (!F.failed[k]) continue;
+    } else {
+      const bool first = g < F.min_members ||
+                         own_rel % sample_stride(int64_t(Aq.last) - int64_t(Aq.first) + 1) == 0;
+      if (first != (F.pass == kFarFirst)) continue;
+    }
+    const float4 iv = A.inv[Aq.node];
+    const float2 s = make_float2(iv.x, iv.y);
+    const float2 bd = F.bounds[k];
+    const bool valid = lane < int(Aq.count);
+    const uint32_t si = Aq.start + (valid ? lane : 0);
+    uint32_t best = __float_as_uint(nn2[si]), nbr = friend_of[si];
+    bool open = valid && __uint_as_float(best) >= bd.x;
+    if (!__any_sync(kFull, open)) continue;
+    const float4 xy = A.XY[si];
+    const float2 z = A.Z[si];
+    const Query Q = make_query(xy, z);
+    __syncwarp();
+    W.nxy[lane] = make_float4(Q.na.x, Q.na.y, Q.nb.x, Q.nb.y);
+    W.nz[lane] = Q.nc;
+    __syncwarp();
+    const float c[6] = {xy.x, xy.z, z.x, xy.y, xy.w, z.y};
+    float lo[6], hi[6];
+    warp_box(c, open, lo, hi);
+    const Box QB = make_box(lo, hi);
+    float lim = open ? fminf(__uint_as_float(best), bd.y) : -1.f;
+    int wl = __reduce_max_sync(kFull, __float_as_int(lim));  // signed: a closed lane's -1 is below all
+    const int64_t own = own_rel >> 5, nsb = Aq.sbcount;
+    for (int64_t s0 = 0; s0 < nsb && wl >= 0; s0 += 32) {
+      bool near = false;
+      if (s0 + lane < nsb && s0 + lane != own) {
+        near = lb_box_box(QB, A.sbox[Aq.sbfirst + s0 + lane], s) <= __int_as_float(wl);
+        if (kCount) T.box += 1;
+      }
+      unsigned sm = __ballot_sync(kFull, near);
+      while (sm && wl >= 0) {
+        const int64_t sb = s0 + __ffs(sm) - 1;
+        sm &= sm - 1u;
+        const int64_t b_lo = int64_t(Aq.first) + 32 * sb;
+        const int64_t b_hi = rsd::min64(b_lo + 32, int64_t(Aq.last) + 1);
+        unsigned mask = stage_boxes<kCount>(A, b_lo, b_hi, QB, __int_as_float(wl), s, lane, W, T);
+        while (mask) {
+          const int i = __ffs(mask) - 1;
+          mask &= mask - 1u;
+          const bool need = open && lb_point_box(Q, W.box[i], s) <= lim;
+          if (kCount) T.box += open;
+          const unsigned nm = __ballot_sync(kFull, need);
+          if (!nm) continue;
+          const int64_t b = b_lo + i;
+          const int cnt = b == int64_t(Aq.last) ? int(A.bk[b].count) : 32;
+          nn_eval<kCount, false>(A, uint32_t(int64_t(Aq.start) + 32 * (b - a)), cnt, nm, s, best, nbr, lane, W, T);
+          if (need) {
+            open = __uint_as_float(best) >= bd.x;
+            lim = open ? fminf(__uint_as_float(best), bd.y) : -1.f;
+          }
+        }
+        wl = __reduce_max_sync(kFull, __float_as_int(lim));
       }
     }
+    if (valid) {
+      nn2[si] = __uint_as_float(best);
+      friend_of[si] = nbr;
+    }
   }
-  // Friends go to the lane's queue; the queues are flushed (union-find calls of all lanes side
-  // by side) when one would overflow and at the end of the query bucket, instead of one
-  // diverging lane at a time inside the distance loop.
-  if (__any_sync(0xffffffffu, qn + __popc(pending) > 32)) flush_links(uf, pi, LQ, qn, lane);
-  while (pending) {
-    const int j = __ffs(pending) - 1;
-    pending &= pending - 1u;
-    LQ.j[qn++][lane] = sj[j];
+  flush_tally<kCount>(T, A.work, lane);
+}
+
+// ---- Links ------------------------------------------------------------------------------------
+
+// Unite the queries in `need` with the members of one bucket that lie within l2 and do not share
+// their root yet. rj: this lane's target's root. kSelf: the bucket is the query bucket itself
+// (pairs j > l only).
+template <bool kCount, bool kSelf>
+__device__ __forceinline__ void link_eval(const SearchArgs& A, uint32_t* uf, uint32_t start, int cnt, unsigned need,
+                                          float2 s, float l2, uint32_t rj, int lane, WarpShared& W, Tally& T) {
+  float4 xy;
+  float2 z;
+  load_targets(A.XY, A.Z, start, cnt, lane, xy, z);
+  while (need) {
+    const int l = __ffs(need) - 1;
+    need &= need - 1u;
+    const uint32_t rq = W.root[l];
+    const bool cand = lane < cnt && rj != rq && (!kSelf || lane > l);
+    if (!__any_sync(kFull, cand)) continue;
+    if (kCount) T.d6 += cand;
+    const bool hit = cand && d6_pair(xy, z, W.nxy[l], W.nz[l], s) <= l2;
+    if (!__any_sync(kFull, hit)) continue;
+    if (hit) rsd::uf_unite(uf, rq, rj);
+    __syncwarp();
+    const uint32_t r = rsd::uf_find(uf, rq);
+    if (hit) rj = r;
+    if (lane == 0) W.root[l] = r;
+    if (kSelf && hit) W.root[lane] = r;
+    __syncwarp();
   }
 }
 
-// Over the buckets of the members with a friend: every valid lane is active.
+// Links inside every superbucket (bucket pairs b >= a).
 template <bool kCount>
-__global__ void __launch_bounds__(kT)
-k_link6d_pruned(NNArgs A, uint32_t* __restrict__ uf) {
-  Tally T;
-  __shared__ Stage stg[kWarpsPerBlock];
-  __shared__ uint32_t sj[kWarpsPerBlock][32];
-  __shared__ LinkQueue lq[kWarpsPerBlock];
-  const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
+__global__ void __launch_bounds__(kT, 4) k_link_near(SearchArgs A, uint32_t* __restrict__ uf) {
+  __shared__ WarpShared sh[kWarpsPerBlock];
+  const int lane = threadIdx.x & 31;
+  WarpShared& W = sh[threadIdx.x >> 5];
   const int64_t nbk = *A.nbuckets;
+  Tally T;
   while (true) {
     const int64_t w = next_work(A.counter, lane);
     if (w >= nbk) break;
     const int64_t a = A.order[w];
     const Bucket Aq = A.bk[a];
     const float4 iv = A.inv[Aq.node];
+    const float2 s = make_float2(iv.x, iv.y);
     const float l2 = iv.z;
     const bool valid = lane < int(Aq.count);
     const uint32_t si = Aq.start + (valid ? lane : 0);
-    const Query Q = make_query(A.Us[si], A.Vs[si], iv.x, iv.y);
-    const uint32_t pi = A.sp[si];
-    const bool active = valid;
-    const Box Abox = A.box[a];
-    int qn = 0;  // this lane's pending unions in lq[wb]
-    const int64_t own = (a - int64_t(Aq.first)) >> 5, nsb = Aq.sbcount;
-    for (int64_t s = own; s < nsb; ++s) {
-      const Box SB = A.sbox[Aq.sbfirst + s];
-      if (kCount) T.box += (lane == 0);
-      if (lb_box_box(Abox, SB, Q.s) > l2) continue;
-      const bool need = active && lb_point_box(Q, SB) <= l2;
-      if (kCount) T.box += active;
-      if (!__any_sync(0xffffffffu, need)) continue;
-      const int64_t b_lo = rsd::min64(int64_t(Aq.first) + 32 * s, int64_t(Aq.last) + 1);
-      const int64_t b_hi = rsd::min64(int64_t(Aq.first) + 32 * s + 32, int64_t(Aq.last) + 1);
-      for (int64_t b = (s == own ? a : b_lo); b < b_hi; ++b)
-        link_bucket<kCount>(A, a, b, Abox, active, Q, pi, l2, uf, lane, stg[wb], sj[wb], lq[wb], qn, T);
+    const Query Q = make_query(A.XY[si], A.Z[si]);
+    const uint32_t rl = rsd::uf_find(uf, si);
+    __syncwarp();
+    W.nxy[lane] = make_float4(Q.na.x, Q.na.y, Q.nb.x, Q.nb.y);
+    W.nz[lane] = Q.nc;
+    W.root[lane] = rl;
+    __syncwarp();
+    const unsigned all = Aq.count == 32 ? kFull : (1u << Aq.count) - 1u;
+    link_eval<kCount, true>(A, uf, Aq.start, int(Aq.count), all, s, l2, rl, lane, W, T);
+    const int64_t b_lo = int64_t(Aq.first) + ((a - int64_t(Aq.first)) & ~int64_t(31));
+    const int64_t b_hi = rsd::min64(b_lo + 32, int64_t(Aq.last) + 1);
+    if (a + 1 >= b_hi) continue;
+    unsigned mask = stage_boxes<kCount>(A, b_lo, b_hi, A.box[a], l2, s, lane, W, T);
+    mask &= ~((2u << int(a - b_lo)) - 1u);
+    while (mask) {
+      const int i = __ffs(mask) - 1;
+      mask &= mask - 1u;
+      const unsigned nm = __ballot_sync(kFull, valid && lb_point_box(Q, W.box[i], s) <= l2);
+      if (kCount) T.box += valid;
+      if (!nm) continue;
+      const int64_t b = b_lo + i;
+      const int cnt = b == int64_t(Aq.last) ? int(A.bk[b].count) : 32;
+      const uint32_t start = uint32_t(int64_t(Aq.start) + 32 * (b - a));
+      const uint32_t rj = lane < cnt ? rsd::uf_find(uf, start + lane) : 0u;
+      link_eval<kCount, false>(A, uf, start, cnt, nm, s, l2, rj, lane, W, T);
     }
-    flush_links(uf, pi, lq[wb], qn, lane);
   }
   flush_tally<kCount>(T, A.work + 2, lane);
+}
+
+// Full compression, component sizes by root.
+__global__ void k_link_compress(const int64_t* __restrict__ na, uint32_t* __restrict__ uf,
+                                uint32_t* __restrict__ cnt) {
+  const int64_t a = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const bool valid = a < *na;  // every lane stays: lanes with the same root add once
+  const uint32_t r = valid ? rsd::uf_find_ro(uf, uint32_t(a)) : 0xffffffffu;
+  if (valid) uf[a] = r;
+  const unsigned peers = __match_any_sync(kFull, r);
+  if (valid && int(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(cnt + r, uint32_t(__popc(peers)));
+}
+
+// One warp per bucket: the root all its members share (0xffffffff: several), and the node's
+// largest component, as (size << 32 | root), from the roots among its members.
+__global__ void __launch_bounds__(kT)
+k_link_uniform(int64_t nb, const int64_t* __restrict__ nbk, const Bucket* __restrict__ bk,
+               const uint32_t* __restrict__ uf, const uint32_t* __restrict__ cnt, uint32_t* __restrict__ uni,
+               unsigned long long* __restrict__ big) {
+  const int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (w >= *nbk) return;
+  const Bucket B = bk[w];
+  if (B.sbcount == 1) return;  // such nodes have no far search
+  const uint32_t r = uf[B.start + (lane < int(B.count) ? lane : 0)];
+  int same;
+  __match_all_sync(kFull, r, &same);
+  if (lane == 0) uni[w] = same ? r : 0xffffffffu;
+  if (lane < int(B.count) && r == B.start + lane)
+    atomicMax(big + (int64_t(B.node) - nb), ((unsigned long long)cnt[r] << 32) | r);
+}
+
+// Links between superbuckets, for the members outside their node's largest component.
+template <bool kCount>
+__global__ void __launch_bounds__(kT, 4)
+k_link_far(SearchArgs A, const uint32_t* __restrict__ uni, const unsigned long long* __restrict__ big,
+           const int64_t* __restrict__ active, uint32_t* __restrict__ uf) {
+  __shared__ WarpShared sh[kWarpsPerBlock];
+  const int lane = threadIdx.x & 31;
+  WarpShared& W = sh[threadIdx.x >> 5];
+  const int64_t nbk = *A.nbuckets;
+  Tally T;
+  while (true) {
+    const int64_t w = next_work(A.counter, lane);
+    if (w >= nbk) break;
+    const int64_t a = A.order[w];
+    const Bucket Aq = A.bk[a];
+    if (active[int64_t(Aq.node) - A.nb] < 1024) break;  // size-class order: one superbucket from here on
+    if (Aq.sbcount == 1) continue;
+    const float4 iv = A.inv[Aq.node];
+    const float2 s = make_float2(iv.x, iv.y);
+    const float l2 = iv.z;
+    const bool valid = lane < int(Aq.count);
+    const uint32_t si = Aq.start + (valid ? lane : 0);
+    const uint32_t rl = rsd::uf_find(uf, si);
+    const bool open = valid && rl != uint32_t(big[int64_t(Aq.node) - A.nb]);
+    if (!__any_sync(kFull, open)) continue;
+    const float4 xy = A.XY[si];
+    const float2 z = A.Z[si];
+    const Query Q = make_query(xy, z);
+    __syncwarp();
+    W.nxy[lane] = make_float4(Q.na.x, Q.na.y, Q.nb.x, Q.nb.y);
+    W.nz[lane] = Q.nc;
+    W.root[lane] = rl;
+    __syncwarp();
+    const float c[6] = {xy.x, xy.z, z.x, xy.y, xy.w, z.y};
+    float lo[6], hi[6];
+    warp_box(c, open, lo, hi);
+    const Box QB = make_box(lo, hi);
+    const int64_t own = (a - int64_t(Aq.first)) >> 5, nsb = Aq.sbcount;
+    for (int64_t s0 = 0; s0 < nsb; s0 += 32) {
+      bool near = false;
+      if (s0 + lane < nsb && s0 + lane != own) {
+        near = lb_box_box(QB, A.sbox[Aq.sbfirst + s0 + lane], s) <= l2;
+        if (kCount) T.box += 1;
+      }
+      unsigned sm = __ballot_sync(kFull, near);
+      while (sm) {
+        const int64_t sb = s0 + __ffs(sm) - 1;
+        sm &= sm - 1u;
+        const int64_t b_lo = int64_t(Aq.first) + 32 * sb;
+        const int64_t b_hi = rsd::min64(b_lo + 32, int64_t(Aq.last) + 1);
+        unsigned mask = stage_boxes<kCount>(A, b_lo, b_hi, QB, l2, s, lane, W, T);
+        if (b_lo + lane < b_hi) W.uni[lane] = uni[b_lo + lane];
+        __syncwarp();
+        while (mask) {
+          const int i = __ffs(mask) - 1;
+          mask &= mask - 1u;
+          const bool need = open && W.uni[i] != W.root[lane] && lb_point_box(Q, W.box[i], s) <= l2;
+          if (kCount) T.box += open;
+          const unsigned nm = __ballot_sync(kFull, need);
+          if (!nm) continue;
+          const int64_t b = b_lo + i;
+          const int cnt = b == int64_t(Aq.last) ? int(A.bk[b].count) : 32;
+          const uint32_t start = uint32_t(int64_t(Aq.start) + 32 * (b - a));
+          const uint32_t rj = lane < cnt ? rsd::uf_find(uf, start + lane) : 0u;
+          link_eval<kCount, false>(A, uf, start, cnt, nm, s, l2, rj, lane, W, T);
+        }
+      }
+    }
+  }
+  flush_tally<kCount>(T, A.work + 2, lane);
+}
+
+// Components over the compacted members -> level-local member positions: the smallest position of
+// each component (the root of the definition), then every member's root.
+__global__ void k_link_min(const int64_t* __restrict__ na, const uint32_t* __restrict__ uf,
+                           const uint32_t* __restrict__ spA, uint32_t* __restrict__ root,
+                           uint32_t* __restrict__ minp) {
+  const int64_t a = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const bool valid = a < *na;
+  const uint32_t r = valid ? rsd::uf_find_ro(uf, uint32_t(a)) : 0xffffffffu;
+  if (valid) root[a] = r;
+  const unsigned peers = __match_any_sync(kFull, r);
+  const uint32_t least = __reduce_min_sync(peers, valid ? spA[a] : 0xffffffffu);
+  if (valid && int(threadIdx.x & 31) == __ffs(peers) - 1) atomicMin(minp + r, least);
+}
+
+__global__ void k_link_roots(const int64_t* __restrict__ na, const uint32_t* __restrict__ root,
+                             const uint32_t* __restrict__ spA, const uint32_t* __restrict__ minp,
+                             uint32_t* __restrict__ uf) {
+  const int64_t a = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (a < *na) uf[spA[a]] = minp[root[a]];
 }
 
 int bits_for(uint64_t v) {
@@ -643,56 +894,47 @@ int bits_for(uint64_t v) {
   return b;
 }
 
-NNArgs nn_args(rs_ctx* ctx, int64_t nn) {
+SearchArgs search_args(rs_ctx* ctx, int64_t nb, int64_t nn) {
   Hier h = hier_of(ctx);
-  NNArgs A;
+  SearchArgs A;
   A.nbuckets = static_cast<const int64_t*>(ctx->buf[S_P_BOFF].ptr) + nn;
   A.bk = static_cast<const Bucket*>(ctx->buf[S_P_BUCKET].ptr);
   A.box = static_cast<const Box*>(ctx->buf[S_P_BOX].ptr);
-  A.sub = static_cast<const Box*>(ctx->buf[S_P_SUB].ptr);
   A.sbox = static_cast<const Box*>(ctx->buf[S_P_SBOX].ptr);
   A.order = static_cast<const uint32_t*>(ctx->buf[S_P_ORDER].ptr);
-  A.Us = static_cast<const float4*>(ctx->buf[S_P_US].ptr);
-  A.Vs = static_cast<const float4*>(ctx->buf[S_P_VS].ptr);
-  A.sp = static_cast<const uint32_t*>(ctx->buf[S_P_SP].ptr);
+  A.XY = static_cast<const float4*>(ctx->buf[S_P_XY].ptr);
+  A.Z = static_cast<const float2*>(ctx->buf[S_P_Z].ptr);
   A.inv = h.inv;
   A.counter = static_cast<unsigned long long*>(ctx->buf[S_P_QCTR].ptr);
   A.work = static_cast<unsigned long long*>(ctx->buf[S_P_WORK].ptr);
-  A.bounds = nullptr;
-  A.nb = 0;
+  A.nb = nb;
   return A;
 }
 
-}  // namespace
-
-namespace {
-
 // Bucket tables of the level over the members [start[k], start[k] + cnt[k]) of each node k in
-// the arrays Us, Vs (m entries at most): buckets of 32, boxes, sub-boxes, superboxes and the
-// work queue ordered by node size class.
+// the arrays XY, Z (m entries at most): buckets of 32, boxes, superboxes and the work queue
+// ordered by node size class.
 int build_buckets(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t m, const int64_t* start, const int64_t* cnt,
-                  const float4* Us, const float4* Vs, cudaStream_t st) {
+                  const float4* XY, const float2* Z, cudaStream_t st) {
   int64_t* boff = scratch_t<int64_t>(ctx, S_P_BOFF, size_t(nn) + 1);
   int64_t* sboff = scratch_t<int64_t>(ctx, S_P_SBOFF, size_t(nn) + 1);
   const int64_t nbk_ub = nn + m / 32 + 1;
   const int64_t nsb_ub = nn + nbk_ub / 32 + 1;
   Bucket* bk = scratch_t<Bucket>(ctx, S_P_BUCKET, size_t(nbk_ub));
   Box* box = scratch_t<Box>(ctx, S_P_BOX, size_t(nbk_ub));
-  Box* sub = scratch_t<Box>(ctx, S_P_SUB, size_t(nbk_ub) * 4);
   Box* sbox = scratch_t<Box>(ctx, S_P_SBOX, size_t(nsb_ub));
   uint64_t* qk = scratch_t<uint64_t>(ctx, S_P_QKEY_A, size_t(nbk_ub));
   uint64_t* qk2 = scratch_t<uint64_t>(ctx, S_P_QKEY_B, size_t(nbk_ub));
   uint32_t* qv = scratch_t<uint32_t>(ctx, S_P_QVAL_A, size_t(nbk_ub));
   uint32_t* qv2 = scratch_t<uint32_t>(ctx, S_P_QVAL_B, size_t(nbk_ub));
   uint32_t* qorder = scratch_t<uint32_t>(ctx, S_P_ORDER, size_t(nbk_ub));
-  if (!boff || !sboff || !bk || !box || !sub || !sbox || !qk || !qk2 || !qv || !qv2 || !qorder)
-    return RS_ERR_OOM;
+  if (!boff || !sboff || !bk || !box || !sbox || !qk || !qk2 || !qv || !qv2 || !qorder) return RS_ERR_OOM;
   k_bucket_counts<<<grid_for(nn, kT), kT, 0, st>>>(nn, cnt, boff, sboff);
   RS_LAUNCHED(ctx, "k_bucket_counts");
   RS_TRY(exclusive_scan_i64(ctx, nn, boff, boff + nn, st));
   RS_TRY(exclusive_scan_i64(ctx, nn, sboff, sboff + nn, st));
-  k_buckets<<<grid_for(nbk_ub * 32, kT), kT, 0, st>>>(nb, nn, nbk_ub, boff, sboff, start, cnt, Us, Vs, bk, box,
-                                                     sub, qk, qv);
+  k_buckets<<<grid_for(nbk_ub * 32, kT), kT, 0, st>>>(nb, nn, nbk_ub, boff, sboff, start, cnt, XY, Z, bk, box, qk,
+                                                     qv);
   RS_LAUNCHED(ctx, "k_buckets");
   k_superboxes<<<grid_for(nsb_ub * 32, kT), kT, 0, st>>>(nn, boff, sboff, box, sbox);
   RS_LAUNCHED(ctx, "k_superboxes");
@@ -703,58 +945,18 @@ int build_buckets(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t m, const int64_t*
   return RS_OK;
 }
 
-// ---- Bounded nearest-neighbour searches for large nodes ---------------------------------------
+// ---- Bounds of l2 for the far searches ----------------------------------------------------------
 // The split needs each member's nn2 exactly only near the k-th smallest value (the adaptive l2)
-// and, elsewhere, only whether it lies below or above it (k_select_l2 and the link pass's
-// member filter). For nodes of at least min_members (4096 by default) members a sample of
-// buckets (every S-th of the node, about kSampleBuckets of them) is searched exactly first;
-// the sample's order statistics around rank p s (p = (k + 1/2) / g) give bounds lo <= hi; the
-// other members are searched with the limit of nn_limit: a lane stops once its minimum is below lo (its nn2 is
-// then some value below lo) and prunes with hi (a minimum above hi is kept as some value above
-// hi). Members whose nn2 lies in [lo, hi] are found exactly, so the k-th smallest of the stored
-// values equals the exact one whenever it lies in [lo, hi]; k_bounds_check verifies that per
-// node after the selection and sends every node that fails through the exact search again.
+// and, elsewhere, only whether it lies below or above it (the selection and the link pass's member
+// filter). hi: the k-th smallest of the near values, each at or above its member's nn2, so hi >= l2
+// always. lo: for nodes of at least min_members (4096 by default) members a sample of buckets
+// (every S-th of the node, about kSampleBuckets of them) is searched up to hi first, and the
+// sample's order statistics below and above rank p s (p = (k + 1/2) / g) give lo and a lower hi;
+// smaller nodes keep lo = -inf. A member below lo keeps some value below lo, one in [lo, hi] its
+// exact nn2, one above hi some value above hi, so the k-th smallest stored value is the exact l2
+// whenever it lies in [lo, hi]; k_bounds_check verifies that per node after the selection and sends
+// every node that fails through the search without bounds.
 constexpr int64_t kBoundMinDefault = 4096;
-constexpr int64_t kSampleBuckets = 48;
-
-__device__ __forceinline__ int64_t sample_stride(int64_t nbk) {
-  return nbk / kSampleBuckets > 1 ? nbk / kSampleBuckets : 1;
-}
-
-// Queue entry w (bucket order[w]) goes to the first, exact queue (flag s: the samples of the
-// nodes searched with bounds, and every bucket of the smaller nodes, so that the first launch
-// fills the GPU) or to the second (flag r: the other buckets of the bounded nodes).
-__global__ void k_queue_flags(int64_t nbk_ub, const int64_t* __restrict__ nbk, const uint32_t* __restrict__ order,
-                              const Bucket* __restrict__ bk, const int64_t* __restrict__ node_size,
-                              int64_t min_members, int64_t* __restrict__ fs, int64_t* __restrict__ fr) {
-  const int64_t w = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (w >= nbk_ub) return;
-  int64_t smp = 0, rest = 0;
-  if (w < *nbk) {
-    const Bucket B = bk[order[w]];
-    const int64_t nb_node = int64_t(B.last) - int64_t(B.first) + 1;
-    const bool bounded = node_size[B.node] >= min_members;
-    smp = !bounded || ((int64_t(order[w]) - int64_t(B.first)) % sample_stride(nb_node)) == 0;
-    rest = !smp;
-  }
-  fs[w] = smp;
-  fr[w] = rest;
-}
-
-// Stable scatter of the two queues (order preserved: largest nodes first in both); counts at
-// qcount[0] (sample) and qcount[1] (others).
-__global__ void k_queue_scatter(int64_t nbk_ub, const uint32_t* __restrict__ order, const int64_t* __restrict__ fs,
-                                const int64_t* __restrict__ fr, uint32_t* __restrict__ qs,
-                                uint32_t* __restrict__ qr, int64_t* __restrict__ qcount) {
-  const int64_t w = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (w == 0) {
-    qcount[0] = fs[nbk_ub];
-    qcount[1] = fr[nbk_ub];
-  }
-  if (w >= nbk_ub) return;
-  if (fs[w + 1] != fs[w]) qs[fs[w]] = order[w];
-  if (fr[w + 1] != fr[w]) qr[fr[w]] = order[w];
-}
 
 // Radix select (4 passes of 8 bits over non-negative float bit patterns) of rank k among the
 // sample values of one node, read through `val(t)` for t < n (invalid entries return false).
@@ -794,25 +996,29 @@ __device__ float block_select(Val val, int64_t n, uint32_t k, uint32_t* hist, ui
   return __uint_as_float(*s_prefix);
 }
 
+// First bounds of every node of the level: (-inf, k-th smallest near value), which the selection
+// left in inv.z.
+__global__ void k_first_bounds(int64_t nb, int64_t nn, const float4* __restrict__ inv, float2* __restrict__ bounds) {
+  const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (k < nn) bounds[k] = make_float2(-__int_as_float(0x7f800000), inv[nb + k].z);
+}
+
 // One block per node of the level: bounds (lo, hi) from the sample of a node of at least
-// min_members members, (-inf, +inf) (exact search) otherwise. The sample of a node is every
-// S-th of its buckets; its size s and the target rank r = p s with p = (k + 1/2) / g; the
-// bounds are the sample's order statistics at r -+ d, d = 6 sqrt(s p (1 - p)) + 8 (twice
-// three binomial standard deviations: the sampled buckets are clusters of neighbours).
+// min_members members, unchanged otherwise. The sample of a node is every S-th of its buckets;
+// its size s and the target rank r = p s with p = (k + 1/2) / g; the bounds are the sample's order
+// statistics at r -+ d, d = 6 sqrt(s p (1 - p)) + 8 (twice three binomial standard deviations:
+// the sampled buckets are clusters of neighbours).
 __global__ void __launch_bounds__(256)
 k_sample_bounds(int64_t nb, int64_t nn, const int64_t* __restrict__ node_size, const int64_t* __restrict__ boff,
-                const Bucket* __restrict__ bk, const uint32_t* __restrict__ sp, const float* __restrict__ nn2,
+                const Bucket* __restrict__ bk, const float* __restrict__ nn2,
                 int f_num, int f_den, float margin, int64_t min_members, float2* __restrict__ bounds) {
   __shared__ uint32_t hist[256];
   __shared__ uint32_t s_prefix, s_k;
   const int64_t k = blockIdx.x;
   if (k >= nn) return;
   const int64_t g = node_size[nb + k];
+  if (g < min_members) return;
   const float inf = __int_as_float(0x7f800000);
-  if (g < min_members) {
-    if (threadIdx.x == 0) bounds[k] = make_float2(-inf, inf);
-    return;
-  }
   const int64_t b0 = boff[k], nbk = boff[k + 1] - b0;
   const int64_t S = sample_stride(nbk), ns = (nbk + S - 1) / S;
   // sample members: 32 per sampled bucket except possibly the node's last bucket
@@ -832,46 +1038,64 @@ k_sample_bounds(int64_t nb, int64_t nn, const int64_t* __restrict__ node_size, c
     const Bucket B = bk[b0 + (t >> 5) * S];
     const uint32_t l = uint32_t(t & 31);
     if (l >= B.count) return false;
-    v = nn2[sp[B.start + l]];
+    v = nn2[B.start + l];
     return true;
   };
   const float lo = r_lo <= 0 ? -inf : block_select(val, ns * 32, uint32_t(r_lo), hist, &s_prefix, &s_k);
   __syncthreads();
   const float hi = r_hi >= s - 1 ? inf : block_select(val, ns * 32, uint32_t(r_hi), hist, &s_prefix, &s_k);
-  if (threadIdx.x == 0) bounds[k] = make_float2(lo, hi);
+  if (threadIdx.x == 0) bounds[k] = make_float2(lo, fminf(hi, bounds[k].y));
 }
 
 // After the selection: a bounded node whose l2 lies outside its [lo, hi] failed (its stored
-// values are not exact there): mark it, reset its bounds to the exact search and queue all its
-// buckets again (qcount[2]; order of the queue does not matter for exact results).
-// tally (counting variant, may be null): [0] nodes searched with bounds, [1] nodes that failed.
-__global__ void k_bounds_check(int64_t nb, int64_t nn, const float4* __restrict__ inv, float2* __restrict__ bounds,
-                               int* __restrict__ failed, unsigned long long* __restrict__ tally) {
+// values are not exact there): mark it and open its bounds for the search again.
+// tally (counting variant, may be null): [0] nodes searched with sampled bounds, [1] failed.
+__global__ void k_bounds_check(int64_t nb, int64_t nn, const float4* __restrict__ inv,
+                               const int64_t* __restrict__ node_size, int64_t min_members,
+                               float2* __restrict__ bounds, int* __restrict__ failed,
+                               unsigned long long* __restrict__ tally) {
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (k >= nn) return;
   const float inf = __int_as_float(0x7f800000);
+  const bool sampled = node_size[nb + k] >= min_members;
   const float2 bd = bounds[k];
   const float l2 = inv[nb + k].z;
-  const bool bad = !(bd.x <= l2 && l2 <= bd.y);
+  const bool bad = sampled && !(bd.x <= l2 && l2 <= bd.y);
   failed[k] = bad ? 1 : 0;
   if (bad) bounds[k] = make_float2(-inf, inf);
-  if (tally && (bd.x > -inf || bd.y < inf)) {
+  if (tally && sampled) {
     atomicAdd(tally, 1ull);
     if (bad) atomicAdd(tally + 1, 1ull);
   }
 }
 
-__global__ void k_fail_queue(int64_t nbk_ub, const int64_t* __restrict__ nbk, const uint32_t* __restrict__ order,
-                             const Bucket* __restrict__ bk, int64_t nb, const int* __restrict__ failed,
-                             uint32_t* __restrict__ qf, unsigned long long* __restrict__ qcount) {
-  const int64_t w = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (w >= nbk_ub || w >= *nbk) return;
-  const uint32_t a = order[w];
-  if (failed[int64_t(bk[a].node) - nb]) qf[atomicAdd(qcount, 1ull)] = a;
+unsigned persistent_grid(int64_t nbk_ub) {
+  return unsigned(std::min<int64_t>((nbk_ub + kWarpsPerBlock - 1) / kWarpsPerBlock, 152 * 4));
 }
 
-unsigned persistent_grid(int64_t nbk_ub) {
-  return unsigned(std::min<int64_t>((nbk_ub + kWarpsPerBlock - 1) / kWarpsPerBlock, 152 * 8));
+// One persistent launch of a search kernel over the level's queue.
+template <class K, class... Args>
+int run_search(rs_ctx* ctx, const char* name, K counting, K plain, SearchArgs A, int64_t nbk_ub, cudaStream_t st,
+               Args... args) {
+  RS_CUDA(ctx, cudaMemsetAsync(A.counter, 0, sizeof(unsigned long long), st));
+  const unsigned grid = persistent_grid(nbk_ub);
+  {
+    ProfScope prof_(ctx, name, st);
+    (ctx->count_work ? counting : plain)<<<grid, kT, 0, st>>>(A, args...);
+  }
+  RS_LAUNCHED(ctx, name);
+  return RS_OK;
+}
+
+// Smallest node of the level's searches with sampled bounds.
+int64_t bound_min(rs_ctx* ctx) { return ctx->nn_bound_min > 0 ? ctx->nn_bound_min : kBoundMinDefault; }
+
+int run_far(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t m, FarPass pass, const int* failed, float* nn2,
+            cudaStream_t st) {
+  const FarArgs F{static_cast<const float2*>(ctx->buf[S_P_BOUNDS].ptr), hier_of(ctx).node_size, failed,
+                  bound_min(ctx), pass};
+  return run_search(ctx, "k_nn6d_pruned", k_nn_far<true>, k_nn_far<false>, search_args(ctx, nb, nn),
+                    nn + m / 32 + 1, st, F, nn2, static_cast<uint32_t*>(ctx->buf[S_P_FRIEND].ptr));
 }
 
 }  // namespace
@@ -880,150 +1104,137 @@ int rs::prune6d_prepare(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t
                         const double* sums, cudaStream_t st) {
   Hier h = hier_of(ctx);
   float4* mean_u = scratch_t<float4>(ctx, S_P_MEANU, size_t(nb + nn));
+  float4* mean_v = scratch_t<float4>(ctx, S_P_MEANV, size_t(nb + nn));
   uint64_t* ka = scratch_t<uint64_t>(ctx, S_KEY_A, size_t(m));
   uint64_t* kb = scratch_t<uint64_t>(ctx, S_KEY_B, size_t(m));
   uint32_t* va = scratch_t<uint32_t>(ctx, S_VAL_A, size_t(m));
   uint32_t* vb = scratch_t<uint32_t>(ctx, S_VAL_B, size_t(m));
-  float4* Us = scratch_t<float4>(ctx, S_P_US, size_t(m));
-  float4* Vs = scratch_t<float4>(ctx, S_P_VS, size_t(m));
+  float4* XY = scratch_t<float4>(ctx, S_P_XY, size_t(m));
+  float2* Z = scratch_t<float2>(ctx, S_P_Z, size_t(m));
   uint32_t* sp = scratch_t<uint32_t>(ctx, S_P_SP, size_t(m));
   int64_t* nstart = scratch_t<int64_t>(ctx, S_P_NSTART, size_t(nn));
   int64_t* ncnt = scratch_t<int64_t>(ctx, S_P_NCNT, size_t(nn));
   unsigned long long* qctr = scratch_t<unsigned long long>(ctx, S_P_QCTR, 2);
   if (!scratch_t<unsigned long long>(ctx, S_P_WORK, 6)) return RS_ERR_OOM;
-  if (!mean_u || !ka || !kb || !va || !vb || !Us || !Vs || !sp || !nstart || !ncnt || !qctr) return RS_ERR_OOM;
-  k_node_means<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.node_size, sums, mean_u);
+  if (!mean_u || !mean_v || !ka || !kb || !va || !vb || !XY || !Z || !sp || !nstart || !ncnt || !qctr)
+    return RS_ERR_OOM;
+  k_node_means<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.node_size, sums, mean_u, mean_v);
   RS_LAUNCHED(ctx, "k_node_means");
-  k_hilbert3<<<grid_for(m, kT), kT, 0, st>>>(mb, m, nb, h.mnode, h.U, h.inv, mean_u, ka, va);
-  RS_LAUNCHED(ctx, "k_hilbert3");
+  k_hilbert6<<<grid_for(m, kT), kT, 0, st>>>(mb, m, nb, h.mnode, h.U, h.V, h.inv, mean_u, mean_v, ka, va);
+  RS_LAUNCHED(ctx, "k_hilbert6");
   uint64_t* keys;
   uint32_t* order;
-  RS_TRY(radix_sort_u64(ctx, m, 24 + bits_for(uint64_t(nn)), ka, va, kb, vb, &keys, &order, st));
-  k_gather_sorted<<<grid_for(m, kT), kT, 0, st>>>(mb, m, order, h.U, h.V, Us, Vs, sp);
+  RS_TRY(radix_sort_u64(ctx, m, kKeyBits + bits_for(uint64_t(nn)), ka, va, kb, vb, &keys, &order, st));
+  k_gather_sorted<<<grid_for(m, kT), kT, 0, st>>>(mb, m, order, h.U, h.V, XY, Z, sp);
   RS_LAUNCHED(ctx, "k_gather_sorted");
   k_node_ranges<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, mb, h.node_off, h.node_size, nstart, ncnt);
   RS_LAUNCHED(ctx, "k_node_ranges");
-  return build_buckets(ctx, nb, nn, m, nstart, ncnt, Us, Vs, st);
+  return build_buckets(ctx, nb, nn, m, nstart, ncnt, XY, Z, st);
 }
 
-// One persistent launch of the nearest-neighbour kernel over the queue (order, count).
-static int run_nn(rs_ctx* ctx, NNArgs A, const uint32_t* order, const int64_t* count, int64_t nbk_ub,
-                  float* nn2, cudaStream_t st) {
-  A.order = order;
-  A.nbuckets = count;
-  const unsigned grid = persistent_grid(nbk_ub);
-  RS_CUDA(ctx, cudaMemsetAsync(A.counter, 0, sizeof(unsigned long long), st));
-  if (ctx->count_work) {
-    k_nn6d_pruned<true><<<grid, kT, 0, st>>>(A, nn2);
-  } else {
-    ProfScope prof_(ctx, "k_nn6d_pruned", st);
-    k_nn6d_pruned<false><<<grid, kT, 0, st>>>(A, nn2);
-  }
-  RS_LAUNCHED(ctx, "k_nn6d_pruned");
-  return RS_OK;
+// Nearest neighbours inside the superbuckets -> nn2 [m] in sorted order (each node's members keep
+// their range), upper bounds of the exact values.
+int rs::prune6d_near(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, float* nn2,
+                     cudaStream_t st) {
+  (void)mb;
+  uint32_t* friend_of = scratch_t<uint32_t>(ctx, S_P_FRIEND, size_t(m));
+  if (!friend_of) return RS_ERR_OOM;
+  return run_search(ctx, "k_nn6d_pruned", k_nn_near<true>, k_nn_near<false>, search_args(ctx, nb, nn),
+                    nn + m / 32 + 1, st, nn2, friend_of);
 }
 
-// Nearest neighbours of the level: the smaller nodes and the sample of every large node
-// exactly, the large nodes' bounds, then their other buckets with those bounds. No host round
-// trip: the queues and their counts stay on the device.
-int rs::prune6d_nn(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, float* nn2,
-                   cudaStream_t st) {
+// The far searches, after a selection over the near values (left in inv.z). No host round trip.
+int rs::prune6d_far(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, float* nn2,
+                    cudaStream_t st) {
   (void)mb;
   Hier h = hier_of(ctx);
-  NNArgs A = nn_args(ctx, nn);
-  const int64_t nbk_ub = nn + m / 32 + 1;
-  const int64_t bmin = ctx->nn_bound_min > 0 ? ctx->nn_bound_min : kBoundMinDefault;
-  ctx->nn_bounded_level = m >= bmin;  // a node of bmin members needs that many at the level
-  if (!ctx->nn_bounded_level) return run_nn(ctx, A, A.order, A.nbuckets, nbk_ub, nn2, st);
-  int64_t* fs = scratch_t<int64_t>(ctx, S_P_QFS, size_t(nbk_ub) + 1);
-  int64_t* fr = scratch_t<int64_t>(ctx, S_P_QFR, size_t(nbk_ub) + 1);
-  uint32_t* qs = scratch_t<uint32_t>(ctx, S_P_QS, size_t(nbk_ub));
-  uint32_t* qr = scratch_t<uint32_t>(ctx, S_P_QR, size_t(nbk_ub));
-  int64_t* qcount = scratch_t<int64_t>(ctx, S_P_QCOUNT, 4);
   float2* bounds = scratch_t<float2>(ctx, S_P_BOUNDS, size_t(std::max<int64_t>(nn, 1)));
-  if (!fs || !fr || !qs || !qr || !qcount || !bounds) return RS_ERR_OOM;
-  k_queue_flags<<<grid_for(nbk_ub, kT), kT, 0, st>>>(nbk_ub, A.nbuckets, A.order, A.bk, h.node_size, bmin, fs,
-                                                     fr);
-  RS_LAUNCHED(ctx, "k_queue_flags");
-  RS_TRY(exclusive_scan_i64(ctx, nbk_ub, fs, fs + nbk_ub, st));
-  RS_TRY(exclusive_scan_i64(ctx, nbk_ub, fr, fr + nbk_ub, st));
-  k_queue_scatter<<<grid_for(nbk_ub, kT), kT, 0, st>>>(nbk_ub, A.order, fs, fr, qs, qr, qcount);
-  RS_LAUNCHED(ctx, "k_queue_scatter");
-  RS_TRY(run_nn(ctx, A, qs, qcount + 0, nbk_ub, nn2, st));  // exactly
+  if (!bounds) return RS_ERR_OOM;
+  k_first_bounds<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.inv, bounds);
+  RS_LAUNCHED(ctx, "k_first_bounds");
+  RS_TRY(run_far(ctx, nb, nn, m, kFarFirst, nullptr, nn2, st));
+  const int64_t bmin = bound_min(ctx);
+  ctx->nn_bounded_level = m >= bmin;  // a node of bmin members needs that many at the level
+  if (!ctx->nn_bounded_level) return RS_OK;
   const int64_t* boff = static_cast<const int64_t*>(ctx->buf[S_P_BOFF].ptr);
-  k_sample_bounds<<<unsigned(std::max<int64_t>(nn, 1)), 256, 0, st>>>(nb, nn, h.node_size, boff, A.bk, A.sp, nn2,
-                                                                   ctx->cfg.f_num, ctx->cfg.f_den,
-                                                                   ctx->nn_bound_margin, bmin, bounds);
+  k_sample_bounds<<<unsigned(std::max<int64_t>(nn, 1)), 256, 0, st>>>(
+      nb, nn, h.node_size, boff, static_cast<const Bucket*>(ctx->buf[S_P_BUCKET].ptr), nn2, ctx->cfg.f_num,
+      ctx->cfg.f_den, ctx->nn_bound_margin, bmin, bounds);
   RS_LAUNCHED(ctx, "k_sample_bounds");
-  A.bounds = bounds;
-  A.nb = nb;
-  return run_nn(ctx, A, qr, qcount + 1, nbk_ub, nn2, st);
+  return run_far(ctx, nb, nn, m, kFarRest, nullptr, nn2, st);
 }
 
-// After the selection of l2: nodes whose l2 fell outside their bounds are searched again
-// exactly (*failed_out: int [nn], 1 for those nodes, for the selection to be repeated there).
+// After the selection of l2: nodes whose l2 fell outside their bounds are searched again without
+// (*failed_out: int [nn], 1 for those nodes, for the selection to be repeated there).
 int rs::prune6d_check(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t m, float* nn2, const int** failed_out,
                       cudaStream_t st) {
   *failed_out = nullptr;
-  if (!ctx->nn_bounded_level) return RS_OK;  // every search of the level was exact
+  if (!ctx->nn_bounded_level) return RS_OK;  // no node of the level was sampled
   Hier h = hier_of(ctx);
-  NNArgs A = nn_args(ctx, nn);
-  const int64_t nbk_ub = nn + m / 32 + 1;
   float2* bounds = static_cast<float2*>(ctx->buf[S_P_BOUNDS].ptr);
   int* failed = scratch_t<int>(ctx, S_P_FAILED, size_t(std::max<int64_t>(nn, 1)));
-  uint32_t* qf = scratch_t<uint32_t>(ctx, S_P_QS, size_t(nbk_ub));  // the sample queue is done
-  unsigned long long* fcount = reinterpret_cast<unsigned long long*>(
-      static_cast<int64_t*>(ctx->buf[S_P_QCOUNT].ptr) + 2);
-  if (!failed || !qf) return RS_ERR_OOM;
-  k_bounds_check<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.inv, bounds, failed,
-                                                  ctx->count_work ? A.work + 4 : nullptr);
+  if (!failed) return RS_ERR_OOM;
+  unsigned long long* work = static_cast<unsigned long long*>(ctx->buf[S_P_WORK].ptr);
+  k_bounds_check<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.inv, h.node_size, bound_min(ctx), bounds, failed,
+                                                  ctx->count_work ? work + 4 : nullptr);
   RS_LAUNCHED(ctx, "k_bounds_check");
-  RS_CUDA(ctx, cudaMemsetAsync(fcount, 0, sizeof(unsigned long long), st));
-  k_fail_queue<<<grid_for(nbk_ub, kT), kT, 0, st>>>(nbk_ub, A.nbuckets, A.order, A.bk, nb, failed, qf, fcount);
-  RS_LAUNCHED(ctx, "k_fail_queue");
-  A.bounds = bounds;
-  A.nb = nb;
-  RS_TRY(run_nn(ctx, A, qf, reinterpret_cast<const int64_t*>(fcount), nbk_ub, nn2, st));
+  RS_TRY(run_far(ctx, nb, nn, m, kFarFailed, failed, nn2, st));
   *failed_out = failed;
   return RS_OK;
 }
 
-// The link pass runs over the members with a friend only (the others can join no link): they
-// are compacted in the sorted order and get their own, tighter buckets.
+// Components of the level's links -> uf [m] (level-local positions; a member without friends stays
+// its own root).
 int rs::prune6d_link(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t mb, int64_t m, const float* nn2,
                      uint32_t* uf, cudaStream_t st) {
   Hier h = hier_of(ctx);
-  const float4* Us = static_cast<const float4*>(ctx->buf[S_P_US].ptr);
-  const float4* Vs = static_cast<const float4*>(ctx->buf[S_P_VS].ptr);
+  const float4* XY = static_cast<const float4*>(ctx->buf[S_P_XY].ptr);
+  const float2* Z = static_cast<const float2*>(ctx->buf[S_P_Z].ptr);
   const uint32_t* sp = static_cast<const uint32_t*>(ctx->buf[S_P_SP].ptr);
+  const uint32_t* friend_of = static_cast<const uint32_t*>(ctx->buf[S_P_FRIEND].ptr);
+  const int64_t nbk_ub = nn + m / 32 + 1;
   int64_t* pos = scratch_t<int64_t>(ctx, S_P_APOS, size_t(m) + 1);
-  float4* UsA = scratch_t<float4>(ctx, S_P_USA, size_t(std::max<int64_t>(m, 1)));
-  float4* VsA = scratch_t<float4>(ctx, S_P_VSA, size_t(std::max<int64_t>(m, 1)));
-  uint32_t* spA = scratch_t<uint32_t>(ctx, S_P_SPA, size_t(std::max<int64_t>(m, 1)));
+  float4* XYA = scratch_t<float4>(ctx, S_P_XYA, size_t(m));
+  float2* ZA = scratch_t<float2>(ctx, S_P_ZA, size_t(m));
+  uint32_t* spA = scratch_t<uint32_t>(ctx, S_P_SPA, size_t(m));
+  uint32_t* ufA = scratch_t<uint32_t>(ctx, S_P_UFA, size_t(m));
+  uint32_t* cnt = scratch_t<uint32_t>(ctx, S_P_CNT, size_t(m));
+  uint32_t* uni = scratch_t<uint32_t>(ctx, S_P_UNI, size_t(nbk_ub));
+  unsigned long long* big = scratch_t<unsigned long long>(ctx, S_P_BIG, size_t(nn));
   int64_t* nstart = scratch_t<int64_t>(ctx, S_P_NSTART, size_t(nn));
   int64_t* ncnt = scratch_t<int64_t>(ctx, S_P_NCNT, size_t(nn));
-  if (!pos || !UsA || !VsA || !spA || !nstart || !ncnt) return RS_ERR_OOM;
-  k_active_flags<<<grid_for(m, kT), kT, 0, st>>>(m, mb, sp, h.mnode, h.inv, nn2, pos);
+  if (!pos || !XYA || !ZA || !spA || !ufA || !cnt || !uni || !big || !nstart || !ncnt) return RS_ERR_OOM;
+  const unsigned grid = grid_for(m, kT);
+  k_active_flags<<<grid, kT, 0, st>>>(m, mb, sp, h.mnode, h.inv, nn2, pos);
   RS_LAUNCHED(ctx, "k_active_flags");
   RS_TRY(exclusive_scan_i64(ctx, m, pos, pos + m, st));
-  k_compact_active<<<grid_for(m, kT), kT, 0, st>>>(m, pos, Us, Vs, sp, UsA, VsA, spA);
+  const int64_t* na = pos + m;
+  k_compact_active<<<grid, kT, 0, st>>>(m, pos, XY, Z, sp, XYA, ZA, spA, ufA);
   RS_LAUNCHED(ctx, "k_compact_active");
+  k_link_friends<<<grid, kT, 0, st>>>(m, pos, friend_of, ufA);
+  RS_LAUNCHED(ctx, "k_link_friends");
   k_active_ranges<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, mb, h.node_off, h.node_size, pos, nstart, ncnt);
   RS_LAUNCHED(ctx, "k_active_ranges");
-  RS_TRY(build_buckets(ctx, nb, nn, m, nstart, ncnt, UsA, VsA, st));
-  NNArgs A = nn_args(ctx, nn);
-  A.Us = UsA;
-  A.Vs = VsA;
-  A.sp = spA;
-  A.counter += 1;
-  const unsigned grid = persistent_grid(nn + m / 32 + 1);
-  RS_CUDA(ctx, cudaMemsetAsync(A.counter, 0, sizeof(unsigned long long), st));
-  if (ctx->count_work) {
-    k_link6d_pruned<true><<<grid, kT, 0, st>>>(A, uf);
-  } else {
-    ProfScope prof_(ctx, "k_link6d_pruned", st);
-    k_link6d_pruned<false><<<grid, kT, 0, st>>>(A, uf);
-  }
-  RS_LAUNCHED(ctx, "k_link6d_pruned");
+  RS_TRY(build_buckets(ctx, nb, nn, m, nstart, ncnt, XYA, ZA, st));
+  SearchArgs A = search_args(ctx, nb, nn);
+  A.XY = XYA;
+  A.Z = ZA;
+  RS_TRY(run_search(ctx, "k_link6d_pruned", k_link_near<true>, k_link_near<false>, A, nbk_ub, st, ufA));
+  RS_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * m, st));
+  RS_CUDA(ctx, cudaMemsetAsync(big, 0, sizeof(unsigned long long) * nn, st));
+  k_link_compress<<<grid, kT, 0, st>>>(na, ufA, cnt);
+  RS_LAUNCHED(ctx, "k_link_compress");
+  k_link_uniform<<<grid_for(nbk_ub * 32, kT), kT, 0, st>>>(nb, A.nbuckets, A.bk, ufA, cnt, uni, big);
+  RS_LAUNCHED(ctx, "k_link_uniform");
+  RS_TRY(run_search(ctx, "k_link6d_pruned", k_link_far<true>, k_link_far<false>, A, nbk_ub, st,
+                    static_cast<const uint32_t*>(uni), static_cast<const unsigned long long*>(big),
+                    static_cast<const int64_t*>(ncnt), ufA));
+  // back to member positions: cnt becomes each component's smallest position
+  RS_CUDA(ctx, cudaMemsetAsync(cnt, 0xff, sizeof(uint32_t) * m, st));
+  uint32_t* root = static_cast<uint32_t*>(ctx->buf[S_P_FRIEND].ptr);  // the neighbours are done with
+  k_link_min<<<grid, kT, 0, st>>>(na, ufA, spA, root, cnt);
+  RS_LAUNCHED(ctx, "k_link_min");
+  k_link_roots<<<grid, kT, 0, st>>>(na, root, spA, cnt, uf);
+  RS_LAUNCHED(ctx, "k_link_roots");
   return RS_OK;
 }
