@@ -69,7 +69,7 @@ typedef struct rs_config {
   int32_t tree_min_members;   /* batched forms: nodes with at least this many members get their
                                  flags from the certified tree bound (see rs_tree_stats) when
                                  rs_unbind is asked for no potential; 0 = 16384, < 0 = never */
-  float tree_theta;           /* opening angle of that bound (0 = 0.45; at most 0.9) */
+  float tree_theta;           /* opening angle of that bound (0 = 0.7; at most 0.9) */
   int32_t surrogate_gate;     /* 0: the error in the gate is the held-out maximum error of the
                                  training (rs_mlp_set_err_max); 1: per node, calibrated on 64
                                  members evaluated exactly, floored at err_max / 8 */
@@ -297,10 +297,11 @@ int rs_run_batched(rs_ctx* ctx, int32_t n_snap, const rs_snapshot* snaps, int32_
  * S_i = sum_{j != i} (|u_j - u_i|^2 + eps^2)^(-1/2) instead of the O(g) direct sum: a
  * Barnes-Hut walk over a Hilbert-ordered tree of the node (leaves of 32 members, 8 children per
  * cell) takes a cell as its quadrupole expansion when its radius bound a is at most tree_theta
- * times the softened distance R', and adds the rigorous truncation bound (n/R') h^3 / (1 - h),
- * h = a / R' (Legendre expansion of the softened kernel, |P_l| <= 1); float32 rounding is
- * covered by a 1e-5 relative slack. A member is decided when the whole interval of
- * E = KE - G m S lies on one side of zero; the others take the exact path (blocked float32 sum
+ * times the softened distance R', and adds the rigorous truncation bound (b/R'^4) / (1 - h),
+ * h = a / R', b >= the cell's sum of |x_j - c|^3 (Legendre expansion of the softened kernel,
+ * |P_l| <= 1); float32 rounding is covered by a 1e-5 relative slack. A member is decided when the
+ * whole interval of E = KE - G m S lies on one side of zero; the others are walked again at 0.45
+ * times the angle, and those still open take the exact path (blocked float32 sum
  * with its certified bound, then the float64 canonical-order potential). Flags are therefore
  * identical to the direct sum's. The paper computes the exact potential; this is the build's
  * O(g log g) potential for nodes of 10^5 - 10^6 members (the next step after the exact kernel).

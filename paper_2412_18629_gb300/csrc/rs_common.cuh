@@ -51,7 +51,7 @@ enum Slot : int {
   // certified tree bound of the potential (rs_tree.cu)
   S_T_OFF, S_T_RANK, S_T_COFF, S_T_NODES, S_T_BOX, S_T_KA, S_T_KB, S_T_VA, S_T_VB, S_T_X, S_T_POS,
   S_T_CELL, S_T_ORDER, S_T_WF, S_T_WL, S_T_WR, S_T_UF, S_T_LIST, S_T_LR, S_T_SX, S_T_REC,
-  S_T_WANT,
+  S_T_WANT, S_SUR_SD,
   // seed halos (rs_seeds.cu)
   S_SEED_KIDS, S_SEED_ROOT, S_SEED_UCNT, S_SEED_UOFF, S_SEED_CEN, S_SEED_SUMS, S_SEED_SEG,
   S_SEED_COUNT, S_SEED_LIST,
@@ -70,7 +70,7 @@ constexpr int64_t kSurrogateMinMembers = 1024;
 // Default smallest node unbound through the certified tree bound (batched form) and its
 // opening angle (a cell is expanded when its radius bound is at most theta times the distance).
 constexpr int64_t kTreeMinDefault = 16384;
-constexpr float kTreeThetaDefault = 0.45f;
+constexpr float kTreeThetaDefault = 0.7f;
 
 struct Buffer {
   void* ptr = nullptr;

@@ -357,7 +357,7 @@ __global__ void k_sur_exact_flags(int64_t ns, const uint32_t* __restrict__ sur_m
 }
 
 // Exact-path list in surrogate-member order (so grouped by node), per-node list offsets and
-// the blocked kernel's tile counts per big node.
+// the blocked kernel's item counts per big node.
 __global__ void k_sur_exact_list(int64_t ns, const int64_t* __restrict__ lf, uint32_t* __restrict__ list,
                                  unsigned long long* __restrict__ counters) {
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -375,7 +375,7 @@ __global__ void k_sur_list_tiles(int64_t nbig, const int64_t* __restrict__ big_n
   const int64_t q = big_nodes[b];
   const int64_t a = lf[sur_off[q]], e = lf[sur_off[q] + node_size[q]];
   lofs[b] = a;
-  tiles[b] = (e - a + list_tile - 1) / list_tile;
+  tiles[b] = list_items(e - a, node_size[q], list_tile);
   if (list_pairs && e > a) atomicAdd(list_pairs, (unsigned long long)((e - a) * node_size[q]));
 }
 
@@ -788,6 +788,7 @@ int surrogate_unbind(rs_ctx* ctx, const double* vbulk, uint8_t* bound, unsigned 
   uint8_t* sflag = scratch_t<uint8_t>(ctx, S_SUR_SFLAG, size_t(ns));
   uint8_t* checked = scratch_t<uint8_t>(ctx, S_SUR_CHECKED, size_t(ns));
   float* Sx = scratch_t<float>(ctx, S_SUR_SX, size_t(ns));
+  double* Sd = scratch_t<double>(ctx, S_SUR_SD, size_t(ns));
   uint32_t* exact_list = scratch_t<uint32_t>(ctx, S_SUR_LIST_A, size_t(ns));
   uint32_t* check_list = scratch_t<uint32_t>(ctx, S_SUR_LIST_B, size_t(ns));
   uint32_t* ambig = scratch_t<uint32_t>(ctx, S_U_AMBIG, size_t(ctx->n_members) + 1);
@@ -796,7 +797,7 @@ int surrogate_unbind(rs_ctx* ctx, const double* vbulk, uint8_t* bound, unsigned 
   int* fail = scratch_t<int>(ctx, S_SUR_FAIL, size_t(nn));
   unsigned int* ecount = scratch_t<unsigned int>(ctx, S_SUR_ECOUNT, size_t(nn));
   int* full = scratch_t<int>(ctx, S_SUR_FULL, size_t(nn));
-  if (!psi_hat || !margin || !sflag || !checked || !Sx || !exact_list || !check_list || !ambig ||
+  if (!psi_hat || !margin || !sflag || !checked || !Sx || !Sd || !exact_list || !check_list || !ambig ||
       !gcount || !tau || !fail || !ecount || !full)
     return RS_ERR_OOM;
   const int64_t nbig = ctx->sur_nbig;
@@ -889,14 +890,12 @@ int surrogate_unbind(rs_ctx* ctx, const double* vbulk, uint8_t* bound, unsigned 
                                                           c == 3 ? counters + 18 : nullptr);
       RS_LAUNCHED(ctx, "k_sur_list_tiles");
       RS_TRY(exclusive_scan_i64(ctx, nbig, ltiles, ltiles + nbig, st));
-      const unsigned grid = grid_for(ns / (kListThreads * R) + nbig + 1, 1);
       if (c < 3) RS_CUDA(ctx, cudaEventRecord(e0, st));
       {
         ProfScope prof_(ctx, c < 3 ? "k_potential_list_tune" : "k_potential_list", st);
-        launch_potential_list(R, eps * eps, grid, st, nbig, ltiles, big_nodes, lofs, lend, exact_list, sur_mem,
-                              h.node_off, h.node_size, h.U, eps * eps, Sx);
+        RS_TRY(launch_potential_list(ctx, R, eps * eps, int64_t(1) << 30, ns, Sd, st, nbig, ltiles, big_nodes, lofs,
+                                     lend, exact_list, sur_mem, h.node_off, h.node_size, h.U));
       }
-      RS_LAUNCHED(ctx, "k_potential_list");
       if (c < 3) {
         RS_CUDA(ctx, cudaEventRecord(e1, st));
         RS_CUDA(ctx, cudaEventSynchronize(e1));
@@ -916,7 +915,7 @@ int surrogate_unbind(rs_ctx* ctx, const double* vbulk, uint8_t* bound, unsigned 
     }
   }
   k_flags_list<<<grid_for(ns, kT), kT, 0, st>>>(counters + 0, exact_list, sur_mem, h.mnode, h.V, vbulk,
-                                               eps * eps, Gm, Sx, bound, ambig, counters + 2);
+                                               eps * eps, Gm, Sd, bound, ambig, counters + 2);
   RS_LAUNCHED(ctx, "k_flags_list");
   RS_TRY(unbind_fallback(ctx, counters + 2, ambig, vbulk, bound, st));
   k_acc_counter<<<1, 1, 0, st>>>(counters, 2, 6);

@@ -12,27 +12,30 @@
 //           node's bounding box; leaf cells are runs of 32 consecutive members, every level up
 //           groups 8 consecutive cells; per cell: centre c (the member mean, rounded to float32),
 //           count n, dipole p = sum (x_j - c) (small: c is rounded), second moments
-//           Q = sum (x_j - c)(x_j - c)^T, and a >= max |x_j - c| (all from float64 sums);
+//           Q = sum (x_j - c)(x_j - c)^T (all from float64 sums), a >= max |x_j - c| and
+//           b >= sum |x_j - c|^3 (over the cell's members, rounded up);
 //   expand  with D = t - c, R'^2 = |D|^2 + eps^2, h_j = |x_j - c| / R' and
 //           x = (D.(x_j - c)) / (R' |x_j - c|), the softened kernel is
 //           (1/R') (1 - 2 h_j x + h_j^2)^(-1/2) = (1/R') sum_l h_j^l P_l(x)
 //           (the Legendre generating function; |x| <= |D| / R' <= 1), so summing l <= 2 over
 //           the cell gives n/R' + p.D/R'^3 + (3 D^T Q D - tr(Q) R'^2) / (2 R'^5), and since
-//           |P_l| <= 1 on [-1, 1] the rest is at most (n/R') h^3 / (1 - h), h = a / R';
+//           |P_l| <= 1 on [-1, 1] the rest is at most (1/R') sum_j h_j^3 / (1 - h_j)
+//           <= (b / R'^4) / (1 - h), h = a / R' <= theta, with 1 / (1 - h) <= 1 + h / (1 - theta)
+//           (the chord of a convex function);
 //   walk    one warp per 32 consecutive target members (in tree order); a cell is taken as its
-//           expansion when a <= theta R' for every lane and it holds none of the warp's
-//           targets, a leaf is summed directly (self excluded), otherwise its children are
-//           visited;
+//           expansion when a <= theta R' for the distance to the warp's target box and it holds none
+//           of the warp's targets, a leaf is summed directly (self excluded), otherwise its children
+//           are visited;
 //   slack   float32 evaluation and summation (per direct term <= ~8u, 32-term leaf blocks
 //           summed as two packed halves <= 31u, the target's own term rsqrt(eps^2) taken out of
-//           its leaf once <= u of the leaf sum, expansions with FMAs <= ~20u of n/R', Kahan across
-//           visits <= 2u) stay below 1e-5 relative; the truncation terms (fast division, <= 2
-//           ulp) are summed in float32 and widened by 0.1%:
+//           its leaf once <= u of the leaf sum, expansions with FMAs <= ~20u of n/R' in 32-cell
+//           blocks <= 31u, Kahan across blocks <= 2u) stay below 1e-5 relative; the truncation
+//           terms are summed in float32 and widened by 0.1%:
 //           S_lo = S~ (1 - 1e-5) - 1.001 B, S_hi = S~ (1 + 1e-5) + 1.001 B;
 //           the float64 sum differs from the exact one by < g 2^-53 relative.
 //   decide  bound iff KE - G m S_lo < -tol, unbound iff KE - G m S_hi > tol (tol = 1e-12 G m
-//           S_hi covers the rounding of E itself); otherwise the member is listed for the exact
-//           path.
+//           S_hi covers the rounding of E itself); otherwise the member is walked again with a
+//           smaller angle, and if that leaves it open too, listed for the exact path.
 // The paper's implementation computes the exact potential (Rockstar's unbinding); this bound is
 // the O(g log g) potential the build adds for nodes of 10^5 - 10^6 members, compared against the
 // exact flags in the tests.
@@ -54,15 +57,24 @@ constexpr int kT = 256;
 constexpr int kLeafBits = 5;   // 32 members per leaf cell
 constexpr int kBrBits = 3;     // 8 children per cell
 constexpr int kMaxLevels = 10;  // enough for g < 2^32
-constexpr int kStack = 64;      // (kMaxLevels - 1) * 7 + 1 pending cells at most
+// Pending cells of a walk: entries lie by level, highest first, four are opened a step, and their up
+// to 32 children are all the entries of their level then: at most 35 a level (rounded up).
+constexpr int kStack = 35 * kMaxLevels;
+// Angle of the second walk, over the members the first leaves undecided (about 0.7% at theta = 0.7
+// against 0.1% after it; the exact sums it saves cost 1e5 - 1e6 pairs a member).
+constexpr float kRefine = 0.45f;
+// Its warps take 8 members each, their lanes 4 slices of the interactions: the undecided members are
+// few and scattered, so 32 a warp make few warps with long walks (12 nodes of up to 1e5 members:
+// 1.3 -> 0.6 ms; 9 ms either way on the 2^27 snapshot).
+constexpr int kRefineSlices = 4;
 constexpr double kSlack = 1e-5;
 constexpr double kBoundWiden = 1.001;
 
 struct Cell {
-  float4 ca;  // centre (x, y, z) and radius bound a
+  float4 ca;  // centre (x, y, z) and radius bound a (negative: no member left in the cell)
   float4 np;  // count n, dipole (px, py, pz)
   float4 q0;  // Qxx, Qyy, Qzz, Qxy
-  float4 q1;  // Qxz, Qyz, tr Q, 0
+  float4 q1;  // Qxz, Qyz, tr Q, b (third-moment bound)
 };
 
 __host__ __device__ __forceinline__ int64_t cells_at(int64_t g, int lev) {
@@ -190,68 +202,94 @@ __device__ __forceinline__ void cell_decode(int64_t c, int64_t nt, const int64_t
   j = i;
 }
 
-__device__ __forceinline__ float round_up_f(double v) {
-  // float >= v (v >= 0), with a relative margin for the float64 rounding of v itself
-  return __double2float_ru(v * (1.0 + 1e-12));
+// An upper bound of |(x, y, z)| for offsets with at most a float32 rounding each.
+__device__ __forceinline__ float radius_up(float x, float y, float z) {
+  return sqrtf(x * x + y * y + z * z) * (1.0f + 1e-6f);
 }
 
-// Leaf cells (level 0): one warp per cell of the cell array (warps of other levels exit).
+__device__ __forceinline__ Cell empty_cell() {
+  return Cell{make_float4(0, 0, 0, -1.f), make_float4(0, 0, 0, 0), make_float4(0, 0, 0, 0), make_float4(0, 0, 0, 0)};
+}
+
+// Leaf cells (level 0): a block takes kLeafCells consecutive cells of the cell array, one warp each
+// (cells of other levels are skipped). The float64 pipe runs two lanes a clock, so the lane sums go
+// through shared memory, one thread per (cell, quantity) adding 32 values: 25 float64 warp
+// instructions a leaf instead of about 90 with butterflies (12.1 -> 5.6 ms for 4.9e7 members,
+// the third-moment bound included).
+constexpr int kLeafCells = kT / 32;
+constexpr int kLeafSums = 9;  // dx, dy, dz, then xx, yy, zz, xy, xz, yz
+
 __global__ void __launch_bounds__(kT)
 k_tree_leaves(int64_t C, int64_t nt, const int64_t* __restrict__ tcoff, const int64_t* __restrict__ tg,
               const int64_t* __restrict__ ttoff, const float4* __restrict__ TX, Cell* __restrict__ cells) {
-  const int64_t c = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (c >= C) return;
-  int64_t b, j;
-  int lev;
-  cell_decode(c, nt, tcoff, tg, b, lev, j);
-  if (lev != 0) return;
-  const int64_t s0 = ttoff[b] + (j << kLeafBits);
-  const int cnt = int(rsd::min64(32, tg[b] - (j << kLeafBits)));
+  __shared__ double val[kLeafCells][kLeafSums][33];
+  __shared__ double sum[kLeafCells][kLeafSums];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t c = int64_t(blockIdx.x) * kLeafCells + w;
+  int64_t b = 0, j = 0;
+  int lev = -1;
+  if (c < C) cell_decode(c, nt, tcoff, tg, b, lev, j);
+  const bool leaf = lev == 0;
+  const int64_t s0 = leaf ? ttoff[b] + (j << kLeafBits) : 0;
+  const int cnt = leaf ? int(rsd::min64(32, tg[b] - (j << kLeafBits))) : 0;
   const float4 xr = lane < cnt ? TX[s0 + lane] : make_float4(0, 0, 0, 0);
   // members moved to +inf (removed by an earlier unbinding pass) are left out of the moments
   const bool valid = lane < cnt && isfinite(xr.x);
   const int nv = __popc(__ballot_sync(0xffffffffu, valid));
-  if (nv == 0) {  // an empty cell: contributes nothing
-    if (lane == 0) {
-      const float4 z = make_float4(0, 0, 0, 0);
-      cells[c] = Cell{z, z, z, z};
+  const double x = valid ? rsd::f2d(xr.x) : 0.0, y = valid ? rsd::f2d(xr.y) : 0.0, z = valid ? rsd::f2d(xr.z) : 0.0;
+  auto block_sums = [&](int per) {  // sum[cell][t] of val[cell][t][0..32) for t < per
+    __syncthreads();
+    if (int(threadIdx.x) < kLeafCells * per) {
+      const double* v = val[threadIdx.x / per][threadIdx.x % per];
+      double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+      for (int k = 0; k < 32; k += 2) {
+        a0 += v[k];
+        a1 += v[k + 1];
+      }
+      sum[threadIdx.x / per][threadIdx.x % per] = a0 + a1;
     }
-    return;
-  }
-  const float4 x = valid ? xr : make_float4(0, 0, 0, 0);
-  double sx = x.x, sy = x.y, sz = x.z;
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    sx += __shfl_xor_sync(0xffffffffu, sx, off);
-    sy += __shfl_xor_sync(0xffffffffu, sy, off);
-    sz += __shfl_xor_sync(0xffffffffu, sz, off);
-  }
-  const float cx = float(sx / nv), cy = float(sy / nv), cz = float(sz / nv);
+    __syncthreads();
+  };
+  val[w][0][lane] = x;
+  val[w][1][lane] = y;
+  val[w][2][lane] = z;
+  block_sums(3);
+  const double inv = nv ? 1.0 / double(nv) : 0.0;
+  const float cx = float(sum[w][0] * inv), cy = float(sum[w][1] * inv), cz = float(sum[w][2] * inv);
   // offsets from the float32 centre are exact in float64
-  const double dx = valid ? double(x.x) - double(cx) : 0.0;
-  const double dy = valid ? double(x.y) - double(cy) : 0.0;
-  const double dz = valid ? double(x.z) - double(cz) : 0.0;
-  double v[10] = {dx, dy, dz, dx * dx, dy * dy, dz * dz, dx * dy, dx * dz, dy * dz,
-                  sqrt(dx * dx + dy * dy + dz * dz)};
+  const double dx = valid ? x - rsd::f2d(cx) : 0.0, dy = valid ? y - rsd::f2d(cy) : 0.0,
+               dz = valid ? z - rsd::f2d(cz) : 0.0;
+  __syncthreads();  // the means are read
+  const double v[kLeafSums] = {dx, dy, dz, dx * dx, dy * dy, dz * dz, dx * dy, dx * dz, dy * dz};
+#pragma unroll
+  for (int t = 0; t < kLeafSums; ++t) val[w][t][lane] = v[t];
+  block_sums(kLeafSums);
+  const float fx = float(dx), fy = float(dy), fz = float(dz);
+  const float r = valid ? radius_up(fx, fy, fz) : 0.f;
+  float a = r, r3 = r * r * r;
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) {
-#pragma unroll
-    for (int t = 0; t < 9; ++t) v[t] += __shfl_xor_sync(0xffffffffu, v[t], off);
-    v[9] = fmax(v[9], __shfl_xor_sync(0xffffffffu, v[9], off));
+    a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, off));
+    r3 += __shfl_xor_sync(0xffffffffu, r3, off);
   }
-  if (lane == 0) {
+  if (leaf && lane == 0) {
+    if (nv == 0) {
+      cells[c] = empty_cell();
+      return;
+    }
+    const double* S = sum[w];
     Cell cl;
-    cl.ca = make_float4(cx, cy, cz, round_up_f(v[9]));
-    cl.np = make_float4(float(nv), float(v[0]), float(v[1]), float(v[2]));
-    cl.q0 = make_float4(float(v[3]), float(v[4]), float(v[5]), float(v[6]));
-    cl.q1 = make_float4(float(v[7]), float(v[8]), float(v[3] + v[4] + v[5]), 0.f);
+    cl.ca = make_float4(cx, cy, cz, a);
+    cl.np = make_float4(float(nv), float(S[0]), float(S[1]), float(S[2]));
+    cl.q0 = make_float4(float(S[3]), float(S[4]), float(S[5]), float(S[6]));
+    cl.q1 = make_float4(float(S[7]), float(S[8]), float(S[3] + S[4] + S[5]), r3 * (1.0f + 4e-6f));
     cells[c] = cl;
   }
 }
 
 // Cells of level `lev` >= 1 from their (up to 8) children, moments shifted to the parent's
-// float32 centre in float64; the radius bound is max(child a + |child c - c|), rounded up.
+// float32 centre in float64 (a and b are left to k_tree_radius).
 __global__ void k_tree_up(int64_t C, int lev, int64_t nt, const int64_t* __restrict__ tcoff,
                           const int64_t* __restrict__ tg, Cell* __restrict__ cells) {
   const int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -273,12 +311,11 @@ __global__ void k_tree_up(int64_t C, int lev, int64_t nt, const int64_t* __restr
     mz += double(ch.np.x) * ch.ca.z + ch.np.w;
   }
   if (n == 0.0) {
-    const float4 z = make_float4(0, 0, 0, 0);
-    cells[c] = Cell{z, z, z, z};
+    cells[c] = empty_cell();
     return;
   }
   const float cx = float(mx / n), cy = float(my / n), cz = float(mz / n);
-  double P[3] = {0.0, 0.0, 0.0}, Q[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, a = 0.0;
+  double P[3] = {0.0, 0.0, 0.0}, Q[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   for (int k = 0; k < nch; ++k) {
     const Cell ch = cells[c0 + k];
     if (ch.np.x == 0.f) continue;
@@ -291,15 +328,70 @@ __global__ void k_tree_up(int64_t C, int lev, int64_t nt, const int64_t* __restr
     const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
     for (int t = 0; t < 6; ++t)
       Q[t] += qc[t] + pc[ia[t]] * d[ib[t]] + d[ia[t]] * pc[ib[t]] + nc * d[ia[t]] * d[ib[t]];
-    const double dist = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) * (1.0 + 1e-12);
-    a = fmax(a, double(ch.ca.w) + dist);
   }
+  const float inf = __int_as_float(0x7f800000);
   Cell cl;
-  cl.ca = make_float4(cx, cy, cz, round_up_f(a));
+  cl.ca = make_float4(cx, cy, cz, inf);
   cl.np = make_float4(float(n), float(P[0]), float(P[1]), float(P[2]));
   cl.q0 = make_float4(float(Q[0]), float(Q[1]), float(Q[2]), float(Q[3]));
-  cl.q1 = make_float4(float(Q[4]), float(Q[5]), float(Q[0] + Q[1] + Q[2]), 0.f);
+  cl.q1 = make_float4(float(Q[4]), float(Q[5]), float(Q[0] + Q[1] + Q[2]), inf);
   cells[c] = cl;
+}
+
+// a and b of the cells of level >= 1 over their members (a node's root keeps a = inf: it holds every
+// target). Bounds through the children (a_child + |c_child - c|, and the same for b by the triangle
+// inequality of the 3-norm) lose 10-20% a level in a, which costs 1.5 times the expansions and twice
+// the undecided members at theta = 0.7. A block takes 32 consecutive cells of the cell array, the
+// upper ones among them one by one.
+__global__ void __launch_bounds__(kT)
+k_tree_radius(int64_t C, int64_t nt, const int64_t* __restrict__ tcoff, const int64_t* __restrict__ tg,
+              const int64_t* __restrict__ ttoff, const float4* __restrict__ TX, Cell* __restrict__ cells) {
+  __shared__ float wa[kT / 32];
+  __shared__ double wb[kT / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t cb = int64_t(blockIdx.x) * 32;
+  int64_t b = 0, j = 0;
+  int lev = 0;
+  if (cb + lane < C) cell_decode(cb + lane, nt, tcoff, tg, b, lev, j);
+  unsigned upper = __ballot_sync(0xffffffffu, lev > 0 && cells_at(tg[b], lev) > 1);  // every warp alike
+  const int64_t first = ttoff[b] + (j << (kLeafBits + kBrBits * lev));
+  const int64_t count = rsd::min64(int64_t(1) << (kLeafBits + kBrBits * lev),
+                                   tg[b] - (j << (kLeafBits + kBrBits * lev)));
+  while (upper) {
+    const int l = __ffs(upper) - 1;
+    upper &= upper - 1u;
+    const int64_t f = __shfl_sync(0xffffffffu, first, l), n = __shfl_sync(0xffffffffu, count, l);
+    const float4 ca = cells[cb + l].ca;
+    float a = 0.f;
+    double r3 = 0.0;
+    if (ca.w >= 0.f)
+      for (int64_t i = threadIdx.x; i < n; i += kT) {
+        const float4 x = TX[f + i];
+        if (!isfinite(x.x)) continue;
+        const float r = radius_up(x.x - ca.x, x.y - ca.y, x.z - ca.z);
+        a = fmaxf(a, r);
+        r3 += rsd::f2d(r * r * r);
+      }
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+      a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, off));
+      r3 += __shfl_xor_sync(0xffffffffu, r3, off);
+    }
+    if (lane == 0) {
+      wa[w] = a;
+      wb[w] = r3;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && ca.w >= 0.f) {
+      for (int k = 1; k < kT / 32; ++k) {
+        a = fmaxf(a, wa[k]);
+        r3 += wb[k];
+      }
+      cells[cb + l].ca.w = a;
+      cells[cb + l].q1.w = __double2float_ru(r3 * (1.0 + 1e-6));
+    }
+    __syncthreads();
+  }
 }
 
 // Walk order of the tree nodes: largest size class first (stable within a class).
@@ -328,9 +420,10 @@ __global__ void k_tree_wlist(int64_t T, const int64_t* __restrict__ wf, uint32_t
   if (wf[s + 1] != wf[s]) wl[wf[s]] = uint32_t(s);
 }
 
-// Per node (walk order r): wanted range [wlo, wlo + wcnt) of the wanted list and its warp count.
+// Per node (walk order r): wanted range [wlo, wlo + wcnt) of the wanted list and its warp count at
+// `targets` members a warp.
 __global__ void k_tree_items(int64_t nt, const uint32_t* __restrict__ worder, const int64_t* __restrict__ ttoff,
-                             const int64_t* __restrict__ tg, const int64_t* __restrict__ wf,
+                             const int64_t* __restrict__ tg, const int64_t* __restrict__ wf, int targets,
                              int64_t* __restrict__ wlo, int64_t* __restrict__ wcnt,
                              int64_t* __restrict__ items) {
   const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -339,7 +432,7 @@ __global__ void k_tree_items(int64_t nt, const uint32_t* __restrict__ worder, co
   const int64_t a = wf[ttoff[b]], e = wf[ttoff[b] + tg[b]];
   wlo[r] = a;
   wcnt[r] = e - a;
-  items[r] = (e - a + 31) / 32;
+  items[r] = (e - a + targets - 1) / targets;
 }
 
 struct WalkArgs {
@@ -358,7 +451,8 @@ struct WalkArgs {
   const Cell* cells;
   const float4* V;
   const double* vbulk;
-  float eps2, theta2;
+  float eps2, theta2, chord;  // chord = 1 / (1 - theta)
+  bool last;                  // the last walk: its undecided members go to the exact path
   double Gm;
   uint8_t* bound;
   int64_t* und;             // per sorted position: 1 = undecided
@@ -367,170 +461,272 @@ struct WalkArgs {
   unsigned long long* counters;  // [0] decided, [1] undecided, [2] expansions, [3] direct pairs
 };
 
-// One warp per 32 wanted targets of one node: the certified walk, then the decision. Indices
-// inside the walk are 32-bit and relative to the node (its members are [tb, tb + g) of the
-// sorted arrays, its cells [cb, cb + cells) of the cell array); a stack entry carries the
-// cell's level, its index j within the level and its index within the node's cells.
-__global__ void __launch_bounds__(kT)
-k_tree_walk(WalkArgs A) {
-  __shared__ uint64_t s_stack[kT / 32][kStack];
-  __shared__ __align__(16) float s_leaf[kT / 32][3][32];  // a leaf's members in x / y / z rows
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  if (w >= A.item_off[A.nt]) return;
-  const int64_t r = rsd::upper_bound_i64(A.item_off, A.nt, w) - 1;
-  const int64_t b = A.worder[r];
-  const int64_t it = w - A.item_off[r];
-  const int64_t wi = A.wlo[r] + 32 * it + lane;
-  const bool valid = 32 * it + lane < A.wcnt[r];
-  const int64_t wi0 = A.wlo[r] + 32 * it;  // lane 0's entry: always valid
-  const uint32_t s_self = A.wl[valid ? wi : wi0];
-  const float4 t = A.TX[s_self];
-  const int64_t g = A.tg[b], tb = A.ttoff[b], cb = A.tcoff[b];
-  const int nlev = levels_of(g);
-  // per-level cell offsets inside the node, lane l holds level l's
-  const uint32_t my_lvoff = lane < nlev ? uint32_t(level_off(g, lane)) : 0u;
-  const uint32_t g32 = uint32_t(g), self_rel = s_self - uint32_t(tb);
-  // the warp's targets as a range of node-relative positions: a cell holds one of them iff
-  // its index at its level lies in [lo_rel >> sh, hi_rel >> sh]
-  uint32_t lo_rel = self_rel, hi_rel = self_rel;
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    lo_rel = min(lo_rel, __shfl_xor_sync(0xffffffffu, lo_rel, off));
-    hi_rel = max(hi_rel, __shfl_xor_sync(0xffffffffu, hi_rel, off));
+// Shared memory of one walking warp: pending cells to open (level << 28 | index in the level), lists
+// of accepted cells and of leaves to sum (node-relative indices), 32 staged cells as 16 pairs for the
+// packed arithmetic, and a leaf's members in x / y / z rows.
+struct __align__(16) WalkShared {
+  float4 st[8][16];
+  float leaf[3][32];
+  uint32_t stack[kStack];
+  uint32_t acc[64];
+  uint32_t dir[64];
+};
+
+// Sum and truncation bound of one target over the tree, for the warp's lanes.
+struct WalkSum {
+  float S = 0.f, C = 0.f;  // Kahan sum over blocks
+  float2 B = {0.f, 0.f};   // truncation bound (two halves)
+  __device__ __forceinline__ void add(float blk) {
+    const float y = __fsub_rn(blk, C);
+    const float t = __fadd_rn(S, y);
+    C = __fsub_rn(__fsub_rn(t, S), y);
+    S = t;
   }
-  const Cell* __restrict__ ncell = A.cells + cb;
-  const float4* __restrict__ nx = A.TX + tb;
-  uint64_t* stk = s_stack[wid];
-  float (*leaf)[32] = s_leaf[wid];
-  float S = 0.f, Cc = 0.f, Bt = 0.f;
-  uint32_t n_exp = 0, n_dir = 0;
-  const uint32_t root_off = __shfl_sync(0xffffffffu, my_lvoff, nlev - 1);
-  if (lane == 0) stk[0] = (uint64_t(nlev - 1) << 60) | uint64_t(root_off);
-  int sp = 1;
+};
+
+// Quadrupole expansions of `cnt` (1..32) accepted cells: lane = cell while they are staged (as pairs,
+// with the factors 3/2, 2 and -1/2 folded in and the centre negated), then lane = target, two cells a
+// packed step. Explicit FMAs: the evaluation only has to stay inside the slack, and the library is
+// compiled without contraction. A missing cell of the last pair has no members and lies far away.
+template <bool kNormal, int kSlices>
+__device__ __forceinline__ void walk_cells(const Cell* __restrict__ ncell, const uint32_t* idx, int cnt, float4 t,
+                                           float eps2, float chord, int lane, WalkShared& W, WalkSum& R) {
+  Cell cl{make_float4(1e18f, 1e18f, 1e18f, 0.f), make_float4(0, 0, 0, 0), make_float4(0, 0, 0, 0),
+          make_float4(0, 0, 0, 0)};
+  if (lane < cnt) cl = ncell[idx[lane]];
+  const float v[16] = {-cl.ca.x, -cl.ca.y, -cl.ca.z, cl.ca.w, cl.np.x, cl.np.y, cl.np.z, cl.np.w,
+                       1.5f * cl.q0.x, 1.5f * cl.q0.y, 1.5f * cl.q0.z, 3.0f * cl.q0.w,
+                       3.0f * cl.q1.x, 3.0f * cl.q1.y, -0.5f * cl.q1.z, cl.q1.w};
   __syncwarp();
-  while (sp > 0) {
-    --sp;
-    const uint64_t e = stk[sp];
-    __syncwarp();
-    const int lev = int(e >> 60);
-    const uint32_t j = uint32_t(e >> 32) & 0x0fffffffu;
-    const int sh = kLeafBits + kBrBits * lev;
-    const bool overlap = j >= (lo_rel >> sh) && j <= (hi_rel >> sh);
-    const Cell cl = ncell[uint32_t(e)];
-    if (cl.np.x == 0.f) continue;  // no member left in the cell (iterative unbinding)
-    const float dx = t.x - cl.ca.x, dy = t.y - cl.ca.y, dz = t.z - cl.ca.z;
-    const float R2 = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, A.eps2)));
-    const bool acc = cl.ca.w * cl.ca.w <= A.theta2 * R2;
-    if (!overlap && __all_sync(0xffffffffu, acc)) {
-      // quadrupole expansion and its truncation bound; explicit FMAs (the evaluation only has
-      // to stay inside the 1e-5 slack, and the library is compiled without contraction)
-      const float ri = rsqrtf(R2);
-      const float ri2 = ri * ri, ri3 = ri2 * ri;
-      const float ax = __fmaf_rn(cl.q1.x + cl.q1.x, dz, __fmaf_rn(cl.q0.w + cl.q0.w, dy, cl.q0.x * dx));
-      const float ay = __fmaf_rn(cl.q1.y + cl.q1.y, dz, cl.q0.y * dy);
-      const float dqd = __fmaf_rn(ax, dx, __fmaf_rn(ay, dy, cl.q0.z * dz * dz));
-      const float pd = __fmaf_rn(cl.np.y, dx, __fmaf_rn(cl.np.z, dy, cl.np.w * dz));
-      const float quad = __fmaf_rn(1.5f * dqd, ri2, -0.5f * cl.q1.z);
-      const float val = __fmaf_rn(cl.np.x, ri, ri3 * (pd + quad));
-      const float h = cl.ca.w * ri;
-      const float bnd = __fdividef(cl.np.x * ri * (h * h * h), 1.f - h);
-      const float y = __fsub_rn(val, Cc);
-      const float tt = __fadd_rn(S, y);
-      Cc = __fsub_rn(__fsub_rn(tt, S), y);
-      S = tt;
-      Bt += bnd;
-      ++n_exp;
-    } else if (lev == 0) {
-      // direct sum over the leaf's members, two per packed float32x2 step; slots past the leaf's
-      // count hold +inf, whose term is exactly 0; the target's own term rsqrt(eps^2) is taken
-      // out once (or, without softening, skipped per pair)
-      const uint32_t c0 = j << kLeafBits;
-      const int cnt = int(min(32u, g32 - c0));
-      const float inf = __int_as_float(0x7f800000);
-      const float4 xm = lane < cnt ? nx[c0 + lane] : make_float4(inf, inf, inf, 0.f);
-      leaf[0][lane] = xm.x;
-      leaf[1][lane] = xm.y;
-      leaf[2][lane] = xm.z;
-      __syncwarp();
-      float blk;
-      if (A.eps2 > 0.f) {
-        const float2 ntx = make_float2(-t.x, -t.x), nty = make_float2(-t.y, -t.y),
-                     ntz = make_float2(-t.z, -t.z), e2 = make_float2(A.eps2, A.eps2);
-        float2 acc2 = make_float2(0.f, 0.f);
-#pragma unroll 4
-        for (int k = 0; k < 32; k += 2) {
-          const float2 ex = __fadd2_rn(*reinterpret_cast<const float2*>(&leaf[0][k]), ntx);
-          const float2 ey = __fadd2_rn(*reinterpret_cast<const float2*>(&leaf[1][k]), nty);
-          const float2 ez = __fadd2_rn(*reinterpret_cast<const float2*>(&leaf[2][k]), ntz);
-          const float2 r2 = __ffma2_rn(ex, ex, __ffma2_rn(ey, ey, __ffma2_rn(ez, ez, e2)));
-          acc2 = __fadd2_rn(acc2, make_float2(rsqrtf(r2.x), rsqrtf(r2.y)));
-        }
-        blk = __fadd_rn(acc2.x, acc2.y);
-        if ((self_rel >> kLeafBits) == j) blk = __fsub_rn(blk, rsqrtf(A.eps2));
-      } else {
-        blk = 0.f;
-        for (int k = 0; k < cnt; ++k) {
-          const float ex = __fsub_rn(leaf[0][k], t.x), ey = __fsub_rn(leaf[1][k], t.y),
-                      ez = __fsub_rn(leaf[2][k], t.z);
-          const float wv = rsqrtf(__fmaf_rn(ex, ex, __fmaf_rn(ey, ey, __fmaf_rn(ez, ez, A.eps2))));
-          blk = __fadd_rn(blk, c0 + uint32_t(k) == self_rel ? 0.f : wv);
-        }
-      }
-      __syncwarp();
-      const float y = __fsub_rn(blk, Cc);
-      const float tt = __fadd_rn(S, y);
-      Cc = __fsub_rn(__fsub_rn(tt, S), y);
-      S = tt;
-      n_dir += uint32_t(cnt);
-    } else {
-      const int shc = sh - kBrBits;  // the children's level
-      const uint32_t nchild = uint32_t((uint64_t(g32) + (1ull << shc) - 1) >> shc);
-      const uint32_t j0 = j << kBrBits;
-      const int nch = int(min(1u << kBrBits, nchild - j0));
-      const uint32_t lvc = __shfl_sync(0xffffffffu, my_lvoff, lev - 1);
-      if (lane < nch)
-        stk[sp + lane] = (uint64_t(lev - 1) << 60) | (uint64_t(j0 + lane) << 32) | uint64_t(lvc + j0 + lane);
-      sp += nch;
-      __syncwarp();
-    }
-  }
-  bool decided = false;
-  if (valid) {
-    const uint32_t p = A.tpos[s_self];
-    const int64_t q = A.tnode[b];
-    const double Sd = double(S), Bd = kBoundWiden * double(Bt);
-    const double slo = Sd * (1.0 - kSlack) - Bd, shi = Sd * (1.0 + kSlack) + Bd;
-    const double ke = kinetic(A.V[p], A.vbulk + 3 * q);
-    const double tol = 1e-12 * A.Gm * fabs(shi);
-    const double e_hi = ke - A.Gm * slo, e_lo = ke - A.Gm * shi;
-    if (slo > 0.0 && e_hi < -tol) {
-      A.bound[p] = 1;
-      decided = true;
-    } else if (e_lo > tol) {
-      A.bound[p] = 0;
-      decided = true;
-    } else {
-      A.und[s_self] = 1;
-    }
-    if (A.rec_lo) {
-      A.rec_lo[p] = slo;
-      A.rec_hi[p] = shi;
-    }
-  }
-  const unsigned dec = __ballot_sync(0xffffffffu, valid && decided);
-  const unsigned und = __ballot_sync(0xffffffffu, valid && !decided);
-  unsigned long long n_exp64 = n_exp, n_dir64 = n_dir;
 #pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    n_exp64 += __shfl_xor_sync(0xffffffffu, n_exp64, off);
-    n_dir64 += __shfl_xor_sync(0xffffffffu, n_dir64, off);
+  for (int k = 0; k < 8; ++k) {
+    float* p = reinterpret_cast<float*>(&W.st[k][lane >> 1]) + (lane & 1);
+    p[0] = v[2 * k];
+    p[2] = v[2 * k + 1];
   }
-  if (lane == 0) {
-    if (dec) atomicAdd(A.counters + 0, (unsigned long long)__popc(dec));
-    if (und) atomicAdd(A.counters + 1, (unsigned long long)__popc(und));
-    atomicAdd(A.counters + 2, n_exp64);
-    atomicAdd(A.counters + 3, n_dir64);
+  __syncwarp();
+  const float2 tx = make_float2(t.x, t.x), ty = make_float2(t.y, t.y), tz = make_float2(t.z, t.z);
+  const float2 e2 = make_float2(eps2, eps2), kc = make_float2(chord, chord), one = make_float2(1.f, 1.f);
+  float2 blk = make_float2(0.f, 0.f);
+  auto lo = [](float4 a) { return make_float2(a.x, a.y); };
+  auto hi = [](float4 a) { return make_float2(a.z, a.w); };
+  for (int k = lane / (32 / kSlices); 2 * k < cnt; k += kSlices) {
+    const float4 a0 = W.st[0][k], a1 = W.st[1][k], a2 = W.st[2][k], a3 = W.st[3][k];
+    const float2 dx = __fadd2_rn(tx, lo(a0)), dy = __fadd2_rn(ty, hi(a0)), dz = __fadd2_rn(tz, lo(a1));
+    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
+    const float2 ri = make_float2(rsd::inv_sqrt<kNormal>(r2.x), rsd::inv_sqrt<kNormal>(r2.y));
+    const float4 a4 = W.st[4][k], a5 = W.st[5][k], a6 = W.st[6][k], a7 = W.st[7][k];
+    const float2 ri2 = __fmul2_rn(ri, ri);
+    const float2 qx = __ffma2_rn(lo(a6), dz, __ffma2_rn(hi(a5), dy, __fmul2_rn(lo(a4), dx)));
+    const float2 qy = __ffma2_rn(hi(a6), dz, __fmul2_rn(hi(a4), dy));
+    const float2 dqd = __ffma2_rn(qx, dx, __ffma2_rn(qy, dy, __fmul2_rn(__fmul2_rn(lo(a5), dz), dz)));
+    const float2 pd = __ffma2_rn(hi(a2), dx, __ffma2_rn(lo(a3), dy, __ffma2_rn(hi(a3), dz, lo(a7))));
+    const float2 quad = __ffma2_rn(dqd, ri2, pd);
+    blk = __ffma2_rn(lo(a2), ri, blk);
+    blk = __ffma2_rn(__fmul2_rn(ri2, ri), quad, blk);
+    const float2 f = __ffma2_rn(__fmul2_rn(hi(a1), ri), kc, one);
+    R.B = __ffma2_rn(__fmul2_rn(hi(a7), __fmul2_rn(ri2, ri2)), f, R.B);
+  }
+  R.add(__fadd_rn(blk.x, blk.y));
+}
+
+// Direct sums over `cnt` leaves, two members per packed float32x2 step; slots past a leaf's count
+// hold +inf, whose term is exactly 0; the target's own term rsqrt(eps^2) is taken out once (or,
+// without a normal eps^2, skipped per pair).
+template <bool kNormal, int kSlices>
+__device__ __forceinline__ void walk_leaves(const float4* __restrict__ nx, const uint32_t* leaves, int cnt, uint32_t g,
+                                            float4 t, uint32_t self_rel, float eps2, int lane, WalkShared& W,
+                                            WalkSum& R, uint32_t& n_dir) {
+  const float inf = __int_as_float(0x7f800000);
+  auto load = [&](int k) {
+    const uint32_t i = (leaves[k] << kLeafBits) + lane;
+    return i < g ? nx[i] : make_float4(inf, inf, inf, 0.f);
+  };
+  float4 next = load(0);
+  for (int l = 0; l < cnt; ++l) {
+    const uint32_t j = leaves[l], c0 = j << kLeafBits;
+    const int n = int(min(32u, g - c0));
+    __syncwarp();
+    W.leaf[0][lane] = next.x;
+    W.leaf[1][lane] = next.y;
+    W.leaf[2][lane] = next.z;
+    __syncwarp();
+    if (l + 1 < cnt) next = load(l + 1);
+    float blk;
+    if (kNormal) {
+      const float2 ntx = make_float2(-t.x, -t.x), nty = make_float2(-t.y, -t.y), ntz = make_float2(-t.z, -t.z),
+                   e2 = make_float2(eps2, eps2);
+      float2 acc2 = make_float2(0.f, 0.f);
+      const int slice = lane / (32 / kSlices);
+#pragma unroll 8
+      for (int i = 0; i < 32 / kSlices; i += 2) {
+        const int k = 2 * slice + kSlices * i;
+        const float2 ex = __fadd2_rn(*reinterpret_cast<const float2*>(&W.leaf[0][k]), ntx);
+        const float2 ey = __fadd2_rn(*reinterpret_cast<const float2*>(&W.leaf[1][k]), nty);
+        const float2 ez = __fadd2_rn(*reinterpret_cast<const float2*>(&W.leaf[2][k]), ntz);
+        const float2 r2 = __ffma2_rn(ex, ex, __ffma2_rn(ey, ey, __ffma2_rn(ez, ez, e2)));
+        acc2 = __fadd2_rn(acc2, make_float2(rsd::inv_sqrt<true>(r2.x), rsd::inv_sqrt<true>(r2.y)));
+      }
+      blk = __fadd_rn(acc2.x, acc2.y);
+      if (self_rel >> kLeafBits == j && ((self_rel & 31u) >> 1) % kSlices == uint32_t(slice))
+        blk = __fsub_rn(blk, rsd::inv_sqrt<true>(eps2));
+    } else {
+      blk = 0.f;
+      for (int k = lane / (32 / kSlices); k < n; k += kSlices) {
+        const float ex = __fsub_rn(W.leaf[0][k], t.x), ey = __fsub_rn(W.leaf[1][k], t.y),
+                    ez = __fsub_rn(W.leaf[2][k], t.z);
+        const float wv = rsqrtf(__fmaf_rn(ex, ex, __fmaf_rn(ey, ey, __fmaf_rn(ez, ez, eps2))));
+        blk = __fadd_rn(blk, c0 + uint32_t(k) == self_rel ? 0.f : wv);
+      }
+    }
+    R.add(blk);
+    n_dir += uint32_t(n);
+  }
+}
+
+// One warp per 32 wanted targets of one node: the certified walk, then the decision. A step opens up
+// to four pending cells and tests their children side by side (lane = child) against the box of the
+// warp's targets; accepted cells and leaves to sum are listed and evaluated 32 at a time with lane =
+// target. Bound by the special-function unit in the leaves (one rsqrt a pair) and by the float32 pipe
+// in the expansions; testing one cell a step with every lane spent most of the walk on loads and
+// stack traffic. On the 2^27 snapshot (4.9e7 members) the walk went from 295 to 58 ms: 2.5 times fewer
+// interactions from the exact a and b at theta = 0.7, the rest from the form of the walk.
+// Indices inside the walk are 32-bit and relative to the node (its members are [tb, tb + g) of the
+// sorted arrays, its cells [cb, cb + cells) of the cell array).
+template <bool kNormal, int kSlices>
+__global__ void __launch_bounds__(kT, 4)
+k_tree_walk(WalkArgs A) {
+  constexpr int kTargets = 32 / kSlices;
+  __shared__ WalkShared sh[kT / 32];
+  const int lane = threadIdx.x & 31;
+  WalkShared& W = sh[threadIdx.x >> 5];
+  const int64_t items = A.item_off[A.nt], warps = int64_t(gridDim.x) * (kT / 32);
+  for (int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; w < items; w += warps) {
+    const int64_t r = rsd::upper_bound_i64(A.item_off, A.nt, w) - 1;
+    const int64_t b = A.worder[r];
+    const int64_t i0 = kTargets * (w - A.item_off[r]);
+    const bool valid = i0 + lane % kTargets < A.wcnt[r];
+    // lane 0's entry is always valid
+    const uint32_t s_self = A.wl[A.wlo[r] + i0 + (valid ? lane % kTargets : 0)];
+    const float4 t = A.TX[s_self];
+    const int64_t g = A.tg[b], tb = A.ttoff[b], cb = A.tcoff[b];
+    const int nlev = levels_of(g);
+    // per-level cell offsets inside the node, lane l holds level l's
+    const uint32_t my_lvoff = lane < nlev ? uint32_t(level_off(g, lane)) : 0u;
+    const uint32_t g32 = uint32_t(g), self_rel = s_self - uint32_t(tb);
+    // the warp's targets as a range of node-relative positions (a cell holds one of them iff its
+    // index at its level lies in [lo_rel >> sh, hi_rel >> sh]) and their box
+    uint32_t lo_rel = self_rel, hi_rel = self_rel;
+    float bl[3] = {t.x, t.y, t.z}, bh[3] = {t.x, t.y, t.z};
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+      lo_rel = min(lo_rel, __shfl_xor_sync(0xffffffffu, lo_rel, off));
+      hi_rel = max(hi_rel, __shfl_xor_sync(0xffffffffu, hi_rel, off));
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        bl[d] = fminf(bl[d], __shfl_xor_sync(0xffffffffu, bl[d], off));
+        bh[d] = fmaxf(bh[d], __shfl_xor_sync(0xffffffffu, bh[d], off));
+      }
+    }
+    const Cell* __restrict__ ncell = A.cells + cb;
+    const float4* __restrict__ nx = A.TX + tb;
+    const unsigned below = (1u << lane) - 1u;
+    WalkSum R;
+    uint32_t n_exp = 0, n_dir = 0;
+    int sp = 0, na = 0, nd = 0;
+    if (nlev == 1) {
+      nd = 1;
+      if (lane == 0) W.dir[0] = 0u;
+    } else {
+      sp = 1;
+      if (lane == 0) W.stack[0] = uint32_t(nlev - 1) << 28;
+    }
+    __syncwarp();
+    while (sp > 0) {
+      const int np = min(sp, 4);
+      const int p = lane >> 3;
+      const uint32_t e = p < np ? W.stack[sp - np + p] : 0u;
+      sp -= np;
+      const int lc = max(int(e >> 28) - 1, 0);  // the children's level
+      const uint32_t jc = ((e & 0x0fffffffu) << kBrBits) + uint32_t(lane & 7);
+      const int sh_c = kLeafBits + kBrBits * lc;
+      const uint32_t nchild = uint32_t((uint64_t(g32) + (1ull << sh_c) - 1) >> sh_c);
+      const uint32_t idx = __shfl_sync(0xffffffffu, my_lvoff, lc) + jc;
+      bool acc = false, opn = false;
+      if (p < np && jc < nchild) {
+        const float4 ca = ncell[idx].ca;
+        const float dx = fmaxf(fmaxf(bl[0] - ca.x, ca.x - bh[0]), 0.f), dy = fmaxf(fmaxf(bl[1] - ca.y, ca.y - bh[1]), 0.f),
+                    dz = fmaxf(fmaxf(bl[2] - ca.z, ca.z - bh[2]), 0.f);
+        const float r2 = __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmaf_rn(dz, dz, A.eps2)));
+        const bool overlap = jc >= (lo_rel >> sh_c) && jc <= (hi_rel >> sh_c);
+        const bool some = ca.w >= 0.f;  // a member is left in the cell (iterative unbinding)
+        acc = some && !overlap && ca.w * ca.w <= A.theta2 * r2;
+        opn = some && !acc;
+      }
+      const unsigned ba = __ballot_sync(0xffffffffu, acc), bd = __ballot_sync(0xffffffffu, opn && lc == 0),
+                     bs = __ballot_sync(0xffffffffu, opn && lc > 0);
+      if (acc) W.acc[na + __popc(ba & below)] = idx;
+      if (opn && lc == 0) W.dir[nd + __popc(bd & below)] = jc;
+      if (opn && lc > 0) W.stack[sp + __popc(bs & below)] = (uint32_t(lc) << 28) | jc;
+      na += __popc(ba);
+      nd += __popc(bd);
+      sp += __popc(bs);
+      __syncwarp();
+      if (na >= 32) {
+        na -= 32;
+        n_exp += 32;
+        walk_cells<kNormal, kSlices>(ncell, W.acc + na, 32, t, A.eps2, A.chord, lane, W, R);
+      }
+      if (nd >= 32) {
+        walk_leaves<kNormal, kSlices>(nx, W.dir, nd, g32, t, self_rel, A.eps2, lane, W, R, n_dir);
+        nd = 0;
+        __syncwarp();
+      }
+    }
+    if (na > 0) {
+      n_exp += uint32_t(na);
+      walk_cells<kNormal, kSlices>(ncell, W.acc, na, t, A.eps2, A.chord, lane, W, R);
+    }
+    if (nd > 0) walk_leaves<kNormal, kSlices>(nx, W.dir, nd, g32, t, self_rel, A.eps2, lane, W, R, n_dir);
+    float S = R.S, Bt = __fadd_rn(R.B.x, R.B.y);
+#pragma unroll
+    for (int off = kTargets; off < 32; off <<= 1) {  // the slices of a target
+      S = __fadd_rn(S, __shfl_xor_sync(0xffffffffu, S, off));
+      Bt = __fadd_rn(Bt, __shfl_xor_sync(0xffffffffu, Bt, off));
+    }
+    const bool mine = valid && lane < kTargets;
+    bool decided = false;
+    if (mine) {
+      const uint32_t p = A.tpos[s_self];
+      const int64_t q = A.tnode[b];
+      const double Sd = double(S), Bd = kBoundWiden * double(Bt);
+      const double slo = Sd * (1.0 - kSlack) - Bd, shi = Sd * (1.0 + kSlack) + Bd;
+      const double ke = kinetic(A.V[p], A.vbulk + 3 * q);
+      const double tol = 1e-12 * A.Gm * fabs(shi);
+      const double e_hi = ke - A.Gm * slo, e_lo = ke - A.Gm * shi;
+      if (slo > 0.0 && e_hi < -tol) {
+        A.bound[p] = 1;
+        decided = true;
+      } else if (e_lo > tol) {
+        A.bound[p] = 0;
+        decided = true;
+      } else {
+        A.und[s_self] = 1;
+      }
+      if (A.rec_lo) {
+        A.rec_lo[p] = slo;
+        A.rec_hi[p] = shi;
+      }
+    }
+    const unsigned dec = __ballot_sync(0xffffffffu, mine && decided);
+    const unsigned und = __ballot_sync(0xffffffffu, mine && !decided);
+    if (lane == 0) {
+      if (dec) atomicAdd(A.counters + 0, (unsigned long long)__popc(dec));
+      if (und && A.last) atomicAdd(A.counters + 1, (unsigned long long)__popc(und));
+      atomicAdd(A.counters + 2, (unsigned long long)n_exp * kTargets);
+      atomicAdd(A.counters + 3, (unsigned long long)n_dir * kTargets);
+    }
+    __syncwarp();
   }
 }
 
@@ -551,7 +747,7 @@ __global__ void k_tree_lranges(int64_t nt, const int64_t* __restrict__ ttoff, co
   const int64_t a = uf[ttoff[b]], e = uf[ttoff[b] + tg[b]];
   lofs[b] = a;
   lend[b] = e;
-  tiles[b] = (e - a + tile - 1) / tile;
+  tiles[b] = list_items(e - a, tg[b], tile);
   if (e > a) atomicAdd(list_pairs, (unsigned long long)((e - a) * tg[b]));
 }
 
@@ -622,12 +818,15 @@ int rs::tree_build(rs_ctx* ctx, cudaStream_t st) {
   RS_LAUNCHED(ctx, "k_tree_gather");
   {
     ProfScope prof_(ctx, "k_tree_build", st);
-    k_tree_leaves<<<grid_for(C * 32, kT), kT, 0, st>>>(C, nt, tcoff, tg, ttoff, TX, cells);
+    k_tree_leaves<<<grid_for(C, kLeafCells), kT, 0, st>>>(C, nt, tcoff, tg, ttoff, TX, cells);
     RS_LAUNCHED(ctx, "k_tree_leaves");
-    for (int lev = 1; lev < kMaxLevels; ++lev) {
+    const int levels = levels_of(T);  // no node is larger than all of them together
+    for (int lev = 1; lev < levels; ++lev) {
       k_tree_up<<<grid_for(C, kT), kT, 0, st>>>(C, lev, nt, tcoff, tg, cells);
       RS_LAUNCHED(ctx, "k_tree_up");
     }
+    k_tree_radius<<<grid_for(C, 32), kT, 0, st>>>(C, nt, tcoff, tg, ttoff, TX, cells);
+    RS_LAUNCHED(ctx, "k_tree_radius");
   }
   // walk order of the nodes (largest first)
   {
@@ -651,7 +850,7 @@ int rs::tree_build(rs_ctx* ctx, cudaStream_t st) {
 
 // Decide the flags of the wanted members of the tree nodes (want[p] != 0 when `want` is given,
 // else the members of the nodes with only[q] != 0 when `only` is given, else every member):
-// certified interval walk, then the exact list path (blocked float32 list sums with their
+// certified interval walks, then the exact list path (blocked float32 list sums with their
 // certified bound, float64 canonical-order potential) for the undecided ones.
 // counters: [16] float64 queue of this call, [7] float64 total of the direct sums,
 // [12..15] decided by the bound, listed for the exact path, expansions, direct pairs,
@@ -673,19 +872,15 @@ int rs::tree_decide(rs_ctx* ctx, const int* only, const uint8_t* want, const dou
   int64_t* uf = scratch_t<int64_t>(ctx, S_T_UF, size_t(T) + 1);
   uint32_t* ulist = scratch_t<uint32_t>(ctx, S_T_LIST, size_t(T));
   int64_t* lr = scratch_t<int64_t>(ctx, S_T_LR, size_t(nt) * 3 + 3);
-  float* Sx = scratch_t<float>(ctx, S_T_SX, size_t(T));
+  double* Sd = scratch_t<double>(ctx, S_T_SX, size_t(T));
   uint32_t* ambig = scratch_t<uint32_t>(ctx, S_U_AMBIG, size_t(ctx->n_members) + 1);
-  if (!wf || !wl || !wr || !uf || !ulist || !lr || !Sx || !ambig) return RS_ERR_OOM;
+  if (!wf || !wl || !wr || !uf || !ulist || !lr || !Sd || !ambig) return RS_ERR_OOM;
   int64_t *wlo = wr, *wcnt = wr + nt, *items = wr + 2 * nt;
   k_tree_want<<<grid_for(T, kT), kT, 0, st>>>(T, tpos, h.mnode, only, want, wf);
   RS_LAUNCHED(ctx, "k_tree_want");
   RS_TRY(exclusive_scan_i64(ctx, T, wf, wf + T, st));
   k_tree_wlist<<<grid_for(T, kT), kT, 0, st>>>(T, wf, wl);
   RS_LAUNCHED(ctx, "k_tree_wlist");
-  k_tree_items<<<grid_for(nt, kT), kT, 0, st>>>(nt, worder, ttoff, tg, wf, wlo, wcnt, items);
-  RS_LAUNCHED(ctx, "k_tree_items");
-  RS_TRY(exclusive_scan_i64(ctx, nt, items, items + nt, st));
-  RS_CUDA(ctx, cudaMemsetAsync(uf, 0, sizeof(int64_t) * (size_t(T) + 1), st));
   // an upper bound of the warps (items): T / 32 + nt
   const int64_t warps_ub = T / 32 + nt + 1;
   WalkArgs A;
@@ -694,7 +889,6 @@ int rs::tree_decide(rs_ctx* ctx, const int* only, const uint8_t* want, const dou
   A.worder = worder;
   A.wlo = wlo;
   A.wcnt = wcnt;
-  A.wl = wl;
   A.TX = TX;
   A.tpos = tpos;
   A.ttoff = ttoff;
@@ -705,39 +899,60 @@ int rs::tree_decide(rs_ctx* ctx, const int* only, const uint8_t* want, const dou
   A.V = h.V;
   A.vbulk = vbulk;
   A.eps2 = ctx->cfg.softening * ctx->cfg.softening;
-  A.theta2 = ctx->tree_theta * ctx->tree_theta;
   A.Gm = ctx->cfg.G * ctx->cfg.particle_mass;
   A.bound = bound;
-  A.und = uf;
   A.rec_lo = ctx->tree_record ? static_cast<double*>(ctx->buf[S_T_REC].ptr) : nullptr;
   A.rec_hi = A.rec_lo ? A.rec_lo + ctx->n_members : nullptr;
   A.counters = counters + 12;
-  {
-    ProfScope prof_(ctx, "k_tree_walk", st);
-    k_tree_walk<<<grid_for(warps_ub * 32, kT), kT, 0, st>>>(A);
-  }
-  RS_LAUNCHED(ctx, "k_tree_walk");
-  // exact path for the undecided members
-  RS_TRY(exclusive_scan_i64(ctx, T, uf, uf + T, st));
+  // the wanted members at the opening angle, then the undecided ones at a smaller one
   unsigned long long* ucount = counters + 17;
-  k_tree_ulist<<<grid_for(T, kT), kT, 0, st>>>(T, uf, ulist, ucount);
-  RS_LAUNCHED(ctx, "k_tree_ulist");
-  const int R = ctx->tune_list_r ? ctx->tune_list_r : 4;
+  for (const bool last : {false, true}) {
+    const float theta = last ? kRefine * ctx->tree_theta : ctx->tree_theta;
+    const int targets = last ? 32 / kRefineSlices : 32;
+    k_tree_items<<<grid_for(nt, kT), kT, 0, st>>>(nt, worder, ttoff, tg, wf, targets, wlo, wcnt, items);
+    RS_LAUNCHED(ctx, "k_tree_items");
+    RS_TRY(exclusive_scan_i64(ctx, nt, items, items + nt, st));
+    RS_CUDA(ctx, cudaMemsetAsync(uf, 0, sizeof(int64_t) * (size_t(T) + 1), st));
+    A.theta2 = theta * theta;
+    A.chord = 1.0f / (1.0f - theta);
+    A.last = last;
+    A.wl = wl;
+    A.und = uf;
+    {
+      ProfScope prof_(ctx, "k_tree_walk", st);
+      const bool normal = normal_eps2(A.eps2);
+      if (last) {  // few warps: a grid of one wave strides over them
+        auto* kernel = normal ? k_tree_walk<true, kRefineSlices> : k_tree_walk<false, kRefineSlices>;
+        kernel<<<std::min(grid_for(warps_ub * kRefineSlices * 32, kT), 152u * 4u), kT, 0, st>>>(A);
+      } else {
+        auto* kernel = normal ? k_tree_walk<true, 1> : k_tree_walk<false, 1>;
+        kernel<<<grid_for(warps_ub * 32, kT), kT, 0, st>>>(A);
+      }
+    }
+    RS_LAUNCHED(ctx, "k_tree_walk");
+    RS_TRY(exclusive_scan_i64(ctx, T, uf, uf + T, st));
+    k_tree_ulist<<<grid_for(T, kT), kT, 0, st>>>(T, uf, ulist, ucount);
+    RS_LAUNCHED(ctx, "k_tree_ulist");
+    std::swap(wf, uf);  // the undecided members are the next walk's targets, then the exact list
+    std::swap(wl, ulist);
+  }
+  std::swap(wf, uf);
+  std::swap(wl, ulist);
+  // exact path for the undecided members
+  constexpr int R = 2;  // the lists are short: few lanes of a tile are filled
   int64_t *lofs = lr, *lend = lr + nt, *ltiles = lr + 2 * nt;
   k_tree_lranges<<<grid_for(nt, kT), kT, 0, st>>>(nt, ttoff, tg, uf, kListThreads * R, lofs, lend, ltiles,
                                                   counters + 18);
   RS_LAUNCHED(ctx, "k_tree_lranges");
   RS_TRY(exclusive_scan_i64(ctx, nt, ltiles, ltiles + nt, st));
   const float eps2 = ctx->cfg.softening * ctx->cfg.softening;
-  const unsigned grid = grid_for(T / (kListThreads * R) + nt + 1, 1);
   {
     ProfScope prof_(ctx, "k_potential_list", st);
-    launch_potential_list(R, eps2, grid, st, nt, ltiles, tnode, lofs, lend, ulist, tpos, h.node_off, h.node_size,
-                          h.U, eps2, Sx);
+    RS_TRY(launch_potential_list(ctx, R, eps2, int64_t(1) << 30, T, Sd, st, nt, ltiles, tnode, lofs, lend, ulist, tpos,
+                                 h.node_off, h.node_size, h.U));
   }
-  RS_LAUNCHED(ctx, "k_potential_list");
   const double Gm = ctx->cfg.G * ctx->cfg.particle_mass;
-  k_flags_list<<<grid_for(T, kT), kT, 0, st>>>(ucount, ulist, tpos, h.mnode, h.V, vbulk, eps2, Gm, Sx, bound,
+  k_flags_list<<<grid_for(T, kT), kT, 0, st>>>(ucount, ulist, tpos, h.mnode, h.V, vbulk, eps2, Gm, Sd, bound,
                                               ambig, counters + 16);
   RS_LAUNCHED(ctx, "k_flags_list");
   RS_TRY(unbind_fallback(ctx, counters + 16, ambig, vbulk, bound, st));
