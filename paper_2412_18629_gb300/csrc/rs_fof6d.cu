@@ -344,8 +344,8 @@ k_nn6d(int64_t nb, int64_t nn, const int64_t* __restrict__ tile_off, const int64
   if (valid) nn2[base + i - mb] = best;
 }
 
-// Exact k-th smallest nn2 of each node, k = ceil(f_num g / f_den) - 1: 4 passes of 8-bit radix
-// select on the (non-negative) float bit patterns. Nodes up to kSelectWarpMax members take one
+// Exact k-th smallest nn2 of each node, k = ceil(f_num g / f_den) - 1: radix select on the
+// (non-negative) float bit patterns. Nodes up to kSelectWarpMax members take one
 // warp each (k_select_l2_warp), larger ones a block (k_select_l2).
 constexpr int64_t kSelectWarpMax = 4096;
 constexpr int64_t kPrunedMinMembers = 4096;
@@ -410,45 +410,62 @@ k_select_l2_warp(int64_t nb, int64_t nn, const int64_t* __restrict__ node_off,
   if (lane == 0) inv[q].z = __uint_as_float(prefix);
 }
 
+// Blocks of 1024 threads stride over the level's nodes and select in the large ones, 11 bits a pass
+// (31 value bits: three passes). Bound by the latency of one block's loads: 256 threads and four
+// passes took 20.3 ms per 2^27 pass (33 launches, nodes up to 1.5e6 members), this form 3.1 ms.
 // only (if given): int [nn], the nodes to select for (the others keep their l2).
-__global__ void __launch_bounds__(kT)
-k_select_l2(int64_t nb, const int64_t* __restrict__ node_off, const int64_t* __restrict__ node_size,
+constexpr int kSelThreads = 1024;
+constexpr int kSelBits = 11;
+
+__global__ void __launch_bounds__(kSelThreads)
+k_select_l2(int64_t nb, int64_t nn, const int64_t* __restrict__ node_off, const int64_t* __restrict__ node_size,
             const float* __restrict__ nn2, int64_t mb, int f_num, int f_den, float4* __restrict__ inv,
             const int* __restrict__ only) {
-  __shared__ uint32_t hist[256];
-  __shared__ uint32_t s_prefix, s_k;
-  const int64_t q = nb + blockIdx.x;
-  const int64_t base = node_off[q] - mb, g = node_size[q];
-  if (g <= kSelectWarpMax || (only && !only[blockIdx.x])) return;
-  if (threadIdx.x == 0) {
-    s_prefix = 0;
-    s_k = uint32_t((int64_t(f_num) * g + f_den - 1) / f_den - 1);
-  }
-  uint32_t mask = 0;
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = 24 - 8 * pass;
-    for (int d = threadIdx.x; d < 256; d += blockDim.x) hist[d] = 0;
-    __syncthreads();
-    const uint32_t prefix = s_prefix;
-    for (int64_t a = threadIdx.x; a < g; a += blockDim.x) {
-      const uint32_t bits = __float_as_uint(nn2[base + a]);
-      if ((bits & mask) == prefix) atomicAdd(&hist[(bits >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t kk = s_k, cum = 0;
-      int d = 0;
-      for (; d < 256; ++d) {
-        if (cum + hist[d] > kk) break;
-        cum += hist[d];
+  __shared__ uint32_t hist[1 << kSelBits];
+  __shared__ uint32_t wsum[kSelThreads / 32];
+  __shared__ uint32_t s_digit, s_k;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int64_t k = blockIdx.x; k < nn; k += gridDim.x) {
+    const int64_t q = nb + k, g = node_size[q];
+    if (g <= kSelectWarpMax || (only && !only[k])) continue;
+    const float* __restrict__ v = nn2 + (node_off[q] - mb);
+    uint32_t rank = uint32_t((int64_t(f_num) * g + f_den - 1) / f_den - 1), prefix = 0, mask = 0;
+#pragma unroll
+    for (int shift = 31 - kSelBits; shift >= 0; shift = shift == 0 ? -1 : max(shift - kSelBits, 0)) {
+      const int bits = shift == 0 ? 31 - 2 * kSelBits : kSelBits;
+      hist[2 * threadIdx.x] = 0;
+      hist[2 * threadIdx.x + 1] = 0;
+      __syncthreads();
+#pragma unroll 8
+      for (int64_t a = threadIdx.x; a < g; a += kSelThreads) {
+        const uint32_t b = __float_as_uint(v[a]);
+        if ((b & mask) == prefix) atomicAdd(&hist[(b >> shift) & ((1u << bits) - 1u)], 1u);
       }
-      s_k = kk - cum;
-      s_prefix = prefix | (uint32_t(d) << shift);
+      __syncthreads();
+      const uint32_t h0 = hist[2 * threadIdx.x], h1 = hist[2 * threadIdx.x + 1];
+      uint32_t incl = h0 + h1;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += t;
+      }
+      if (lane == 31) wsum[warp] = incl;
+      __syncthreads();
+      uint32_t before = incl - h0 - h1;
+      for (int w = 0; w < warp; ++w) before += wsum[w];
+      if (before <= rank && rank < before + h0 + h1) {
+        const bool second = rank >= before + h0;
+        s_digit = 2 * threadIdx.x + second;
+        s_k = rank - before - (second ? h0 : 0u);
+      }
+      __syncthreads();
+      rank = s_k;
+      prefix |= s_digit << shift;
+      mask |= ((1u << bits) - 1u) << shift;
+      __syncthreads();
     }
-    mask |= 255u << shift;
-    __syncthreads();
+    if (threadIdx.x == 0) inv[q].z = __uint_as_float(prefix);
   }
-  if (threadIdx.x == 0) inv[q].z = __uint_as_float(s_prefix);
 }
 
 __global__ void k_iota_u32(int64_t n, uint32_t* __restrict__ a) {
@@ -872,8 +889,11 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       k_select_l2_warp<<<grid_for(nn, kT / 32), kT, 0, st>>>(nb, nn, hs.node_off, hs.node_size, nn2, mb, f_num,
                                                             f_den, hs.inv, only);
       RS_LAUNCHED(ctx, "k_select_l2_warp");
-      k_select_l2<<<unsigned(nn), kT, 0, st>>>(nb, hs.node_off, hs.node_size, nn2, mb, f_num, f_den, hs.inv, only);
-      RS_LAUNCHED(ctx, "k_select_l2");
+      if (m > kSelectWarpMax) {  // a larger node is possible
+        k_select_l2<<<unsigned(std::min<int64_t>(nn, 152 * 2)), kSelThreads, 0, st>>>(
+            nb, nn, hs.node_off, hs.node_size, nn2, mb, f_num, f_den, hs.inv, only);
+        RS_LAUNCHED(ctx, "k_select_l2");
+      }
       return RS_OK;
     };
     if (batched) {
