@@ -254,10 +254,13 @@ __device__ __forceinline__ void test_roots(const LinkArgs& A, uint32_t a, uint32
   if (rsd::uf_find(A.C.parent, a) != rsd::uf_find(A.C.parent, b)) test_cells(A, a, b);
 }
 
-// Tests queued pairs while more than `keep` are left; every lane of the warp takes part.
+// Tests queued pairs while more than `keep` are left. Every lane of the warp takes part, with the
+// length that one lane read: no lane goes on to queue its next row's pairs before all know it.
 __device__ __forceinline__ void flush_pairs(const LinkArgs& A, PairQueue& Q, int keep, int lane) {
   __syncwarp();
-  int n = min(Q.n, 64);  // pairs beyond the queue were tested where they were found
+  const int queued = __shfl_sync(0xffffffffu, min(Q.n, 64), 0);  // the pairs beyond were tested at once
+  if (queued <= keep) return;
+  int n = queued;
   while (n > keep) {
     const int k = max(n - 32, 0);
     if (k + lane < n) test_roots(A, Q.a[k + lane], Q.b[k + lane]);
@@ -334,8 +337,7 @@ __global__ void __launch_bounds__(kThreads) k_link_cells(LinkArgs A) {
         if (xa < 0) scan_cells<kFar>(A, c, pc, r, xa + ns, ns - 1, near_row, kx, Q);
         if (xb >= ns) scan_cells<kFar>(A, c, pc, r, max(xa - ns, 0), xb - ns, near_row, kx, Q);
       }
-      __syncwarp();
-      if (Q.n >= 32) flush_pairs(A, Q, 31, lane);
+      flush_pairs(A, Q, 31, lane);
     }
   flush_pairs(A, Q, 0, lane);
 }
