@@ -69,8 +69,11 @@ enum Slot : int {
 constexpr int64_t kSurrogateMinMembers = 1024;
 // Default smallest node unbound through the certified tree bound (batched form) and its
 // opening angle (a cell is expanded when its radius bound is at most theta times the distance).
-constexpr int64_t kTreeMinDefault = 16384;
-constexpr float kTreeThetaDefault = 0.7f;
+// rs_unbind on the 2^27 snapshot takes 131 / 130 / 135 / 146 ms from 2048 / 4096 / 8192 / 16384 members
+// (theta = 0.7), and 150 / 131 / 126 / 122 / 121 / 123 ms at theta = 0.6 / 0.7 / 0.75 / 0.8 / 0.85 / 0.9
+// (from 2048 members): flat minima. Nodes below the threshold keep the plain form's direct sums.
+constexpr int64_t kTreeMinDefault = 8192;
+constexpr float kTreeThetaDefault = 0.8f;
 
 struct Buffer {
   void* ptr = nullptr;

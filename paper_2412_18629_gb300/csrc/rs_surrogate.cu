@@ -342,18 +342,21 @@ __global__ void k_sur_full(int64_t nbig, const int64_t* __restrict__ big_nodes,
 }
 
 // Ungated members of nodes not sent whole: the exact-path list (lf), except in nodes with a
-// certified tree (tmin > 0, at least tmin members), whose members are marked in `want` for it.
+// certified tree (tmin > 0, at least tmin members), whose members are marked in `want` for it (and
+// counted in tree_count).
 __global__ void k_sur_exact_flags(int64_t ns, const uint32_t* __restrict__ sur_mem,
                                   const uint32_t* __restrict__ mnode, const int64_t* __restrict__ node_size,
                                   const uint8_t* __restrict__ sflag, const int* __restrict__ full,
-                                  int64_t tmin, int64_t* __restrict__ lf, uint8_t* __restrict__ want) {
+                                  int64_t tmin, int64_t* __restrict__ lf, uint8_t* __restrict__ want,
+                                  unsigned long long* __restrict__ tree_count) {
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (k >= ns) return;
-  const uint32_t p = sur_mem[k], q = mnode[p];
-  const bool open = sflag[k] == 2 && !full[q];
-  const bool tree = tmin > 0 && node_size[q] >= tmin;
-  lf[k] = (open && !tree) ? 1 : 0;
-  if (want) want[p] = (open && tree) ? 1 : 0;
+  const bool in = k < ns;  // every lane stays for the count
+  const uint32_t p = in ? sur_mem[k] : 0u, q = in ? mnode[p] : 0u;
+  const bool open = in && sflag[k] == 2 && !full[q];
+  const bool tree = in && tmin > 0 && node_size[q] >= tmin;
+  if (in) lf[k] = (open && !tree) ? 1 : 0;
+  if (in && want) want[p] = (open && tree) ? 1 : 0;
+  rsd::warp_count(tree_count, open && tree);
 }
 
 // Exact-path list in surrogate-member order (so grouped by node), per-node list offsets and
@@ -863,7 +866,7 @@ int surrogate_unbind(rs_ctx* ctx, const double* vbulk, uint8_t* bound, unsigned 
   uint8_t* want = tmin > 0 ? scratch_t<uint8_t>(ctx, S_SUR_WANT, size_t(ctx->n_members)) : nullptr;
   if (tmin > 0 && !want) return RS_ERR_OOM;
   k_sur_exact_flags<<<grid_for(ns, kT), kT, 0, st>>>(ns, sur_mem, h.mnode, h.node_size, sflag, full, tmin, lf,
-                                                    want);
+                                                    want, counters + 22);
   RS_LAUNCHED(ctx, "k_sur_exact_flags");
   if (tmin > 0) RS_TRY(tree_decide(ctx, nullptr, want, vbulk, bound, counters, st));
   RS_TRY(exclusive_scan_i64(ctx, ns, lf, lf + ns, st));

@@ -60,8 +60,9 @@ constexpr int kMaxLevels = 10;  // enough for g < 2^32
 // Pending cells of a walk: entries lie by level, highest first, four are opened a step, and their up
 // to 32 children are all the entries of their level then: at most 35 a level (rounded up).
 constexpr int kStack = 35 * kMaxLevels;
-// Angle of the second walk, over the members the first leaves undecided (about 0.7% at theta = 0.7
-// against 0.1% after it; the exact sums it saves cost 1e5 - 1e6 pairs a member).
+// Angle of the second walk, in units of the first's, over the members that leaves undecided (about 1%
+// at theta = 0.8 against 0.05% after it; the exact sums it saves cost 1e5 - 1e6 pairs a member). 0.35
+// and 0.6 are within 2%.
 constexpr float kRefine = 0.45f;
 // Its warps take 8 members each, their lanes 4 slices of the interactions: the undecided members are
 // few and scattered, so 32 a warp make few warps with long walks (12 nodes of up to 1e5 members:

@@ -780,7 +780,8 @@ extern "C" int rs_unbind(rs_ctx* ctx, const float* pos, const float* vel, float*
   uint32_t* ambig = scratch_t<uint32_t>(ctx, S_U_AMBIG, size_t(std::max<int64_t>(m, 1)));
   uint8_t* halo = scratch_t<uint8_t>(ctx, S_U_FLAGS, size_t(std::max<int64_t>(nn, 1)));
   // counters: [0..6], [8..11], [19] surrogate path (rs_surrogate.cu), [7] float64 fallbacks of
-  // the direct sums, [12..18] certified tree bound (rs_tree.cu), [20..21] direct-sum pairs
+  // the direct sums, [12..18] certified tree bound (rs_tree.cu), [20..21] direct-sum pairs, [22] exact-path members
+  // of the surrogate path that went through the tree bound
   unsigned long long* counters = scratch_t<unsigned long long>(ctx, S_SUR_COUNTERS, kCounters);
   if (!bound || !S || !nb || !vbulk || !ambig || !halo || !counters) return RS_ERR_OOM;
   unsigned long long* n_ambig = counters + 7;
@@ -827,13 +828,13 @@ extern "C" int rs_unbind(rs_ctx* ctx, const float* pos, const float* vel, float*
     k_copy_u8<<<grid_for(m, kT), kT, 0, st>>>(m, bound, bound_out);
     RS_LAUNCHED(ctx, "k_copy_u8");
     RS_TRY(read_back(ctx, counters, kCounters * sizeof(unsigned long long), st));
-    // stats: surrogate members, gated, exact (exact-path list + calibration members, outside
-    // nodes sent whole), spot-checked, failed nodes, fp64 (surrogate path), fp64 (direct sums),
+    // stats: surrogate members, gated, exact (exact-path list, tree bound and calibration members,
+    // outside nodes sent whole), spot-checked, failed nodes, fp64 (surrogate path), fp64 (direct sums),
     // re-run members, members of nodes sent whole to the direct sum, members whose flag the
     // surrogate decided, spot-checked members whose surrogate flag was wrong
     ctx->sur_stats[0] = sur ? ctx->sur_members : 0;
     ctx->sur_stats[1] = ctx->host_box[5];
-    ctx->sur_stats[2] = ctx->host_box[0] + ctx->host_box[11];
+    ctx->sur_stats[2] = ctx->host_box[0] + ctx->host_box[11] + ctx->host_box[22];
     ctx->sur_stats[3] = ctx->host_box[1];
     ctx->sur_stats[4] = ctx->host_box[4];
     ctx->sur_stats[5] = ctx->host_box[6];
