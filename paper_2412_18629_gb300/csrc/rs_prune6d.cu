@@ -33,7 +33,7 @@
 // (about 0.3 a member instead of 17).
 //
 // Measured on the 2^27-particle snapshot (12 levels, 1.2e8 members), before and after this form:
-// nearest-neighbour kernels 382 -> 99 ms, link kernels 266 -> 100 ms (3D Hilbert buckets with
+// nearest-neighbour kernels 382 -> 99 ms, link kernels 266 -> 89 ms (3D Hilbert buckets with
 // sub-boxes, lane = query). Both are bound by issue slots (box tests and distance evaluations from
 // L1 and L2).
 #include "rs_cro.cuh"
@@ -248,6 +248,29 @@ __device__ __forceinline__ void warp_box(const float (&a)[6], bool valid, float 
 __device__ __forceinline__ Box make_box(const float (&lo)[6], const float (&hi)[6]) {
   return Box{make_float4(lo[0], lo[3], lo[1], lo[4]), make_float4(-hi[0], -hi[3], -hi[1], -hi[4]),
              make_float2(lo[2], lo[5]), make_float2(-hi[2], -hi[5])};
+}
+
+__device__ __forceinline__ Box query_box(const float (&c)[6], bool open) {
+  float lo[6], hi[6];
+  warp_box(c, open, lo, hi);
+  return make_box(lo, hi);
+}
+
+// The warp's query box again once half of the queries it was made for are closed.
+__device__ __forceinline__ void refresh_box(Box& QB, int& boxed, const float (&c)[6], bool open) {
+  const int n = __popc(__ballot_sync(kFull, open));
+  if (n == 0 || 2 * n > boxed) return;
+  QB = query_box(c, open);
+  boxed = n;
+}
+
+// Takes the set bit of a non-empty mask nearest to position `own`: near stretches of the curve first.
+__device__ __forceinline__ int next_outward(unsigned& mask, int own) {
+  const unsigned up = mask & ~((1u << own) - 1u), dn = mask & ((1u << own) - 1u);
+  const int iu = up ? __ffs(up) - 1 : 64, id = dn ? 31 - __clz(dn) : -64;
+  const int i = iu - own <= own - id ? iu : id;
+  mask &= ~(1u << i);
+  return i;
 }
 
 // One warp per bucket (padding warps write a queue key that sorts last): bucket table entry, box,
@@ -557,11 +580,9 @@ k_nn_near(SearchArgs A, float* __restrict__ nn2, uint32_t* __restrict__ friend_o
       const float lim = __uint_as_float(__reduce_max_sync(kFull, valid ? best : 0u));
       unsigned mask = stage_boxes<kCount>(A, b_lo, b_hi, A.box[a], lim, s, lane, W, T);
       const int own = int(a - b_lo);
-      unsigned up = mask & ~((2u << own) - 1u), dn = mask & ((1u << own) - 1u);
-      while (up | dn) {  // outward from the query bucket: near buckets lower the limit first
-        const int iu = up ? __ffs(up) - 1 : 64, id = dn ? 31 - __clz(dn) : -64;
-        const int i = iu - own <= own - id ? iu : id;
-        if (i > own) up &= up - 1u; else dn &= ~(1u << i);
+      mask &= ~(1u << own);
+      while (mask) {  // outward from the query bucket: near buckets lower the limit first
+        const int i = next_outward(mask, own);
         const bool need = valid && lb_point_box(Q, W.box[i], s) <= __uint_as_float(best);
         if (kCount) T.box += valid;
         const unsigned nm = __ballot_sync(kFull, need);
@@ -642,9 +663,7 @@ k_nn_far(SearchArgs A, FarArgs F, float* __restrict__ nn2, uint32_t* __restrict_
     W.nz[lane] = Q.nc;
     __syncwarp();
     const float c[6] = {xy.x, xy.z, z.x, xy.y, xy.w, z.y};
-    float lo[6], hi[6];
-    warp_box(c, open, lo, hi);
-    const Box QB = make_box(lo, hi);
+    const Box QB = query_box(c, open);
     float lim = open ? fminf(__uint_as_float(best), bd.y) : -1.f;
     int wl = __reduce_max_sync(kFull, __float_as_int(lim));  // signed: a closed lane's -1 is below all
     const int64_t own = own_rel >> 5, nsb = Aq.sbcount;
@@ -690,14 +709,15 @@ k_nn_far(SearchArgs A, FarArgs F, float* __restrict__ nn2, uint32_t* __restrict_
 // ---- Links ------------------------------------------------------------------------------------
 
 // Unite the queries in `need` with the members of one bucket that lie within l2 and do not share
-// their root yet. rj: this lane's target's root. kSelf: the bucket is the query bucket itself
+// their root yet (returns whether there were any). rj: this lane's target's root. kSelf: the bucket is the query bucket itself
 // (pairs j > l only).
 template <bool kCount, bool kSelf>
-__device__ __forceinline__ void link_eval(const SearchArgs& A, uint32_t* uf, uint32_t start, int cnt, unsigned need,
+__device__ __forceinline__ bool link_eval(const SearchArgs& A, uint32_t* uf, uint32_t start, int cnt, unsigned need,
                                           float2 s, float l2, uint32_t rj, int lane, WarpShared& W, Tally& T) {
   float4 xy;
   float2 z;
   load_targets(A.XY, A.Z, start, cnt, lane, xy, z);
+  bool united = false;
   while (need) {
     const int l = __ffs(need) - 1;
     need &= need - 1u;
@@ -707,6 +727,7 @@ __device__ __forceinline__ void link_eval(const SearchArgs& A, uint32_t* uf, uin
     if (kCount) T.d6 += cand;
     const bool hit = cand && d6_pair(xy, z, W.nxy[l], W.nz[l], s) <= l2;
     if (!__any_sync(kFull, hit)) continue;
+    united = true;
     if (hit) rsd::uf_unite(uf, rq, rj);
     __syncwarp();
     const uint32_t r = rsd::uf_find(uf, rq);
@@ -715,6 +736,7 @@ __device__ __forceinline__ void link_eval(const SearchArgs& A, uint32_t* uf, uin
     if (kSelf && hit) W.root[lane] = r;
     __syncwarp();
   }
+  return united;
 }
 
 // Links inside every superbucket (bucket pairs b >= a).
@@ -795,7 +817,10 @@ k_link_uniform(int64_t nb, const int64_t* __restrict__ nbk, const Bucket* __rest
     atomicMax(big + (int64_t(B.node) - nb), ((unsigned long long)cnt[r] << 32) | r);
 }
 
-// Links between superbuckets, for the members outside their node's largest component.
+// Links between superbuckets, for the members outside their node's largest component; members that
+// have joined it meanwhile are done too (from the near stretches of the curve on, and with the query
+// box made again as they go: 69 -> 58 ms on the 2^27 snapshot. The nearest-neighbour search gains
+// nothing from that order: its limit is known from the start).
 template <bool kCount>
 __global__ void __launch_bounds__(kT, 4)
 k_link_far(SearchArgs A, const uint32_t* __restrict__ uni, const unsigned long long* __restrict__ big,
@@ -818,7 +843,7 @@ k_link_far(SearchArgs A, const uint32_t* __restrict__ uni, const unsigned long l
     const bool valid = lane < int(Aq.count);
     const uint32_t si = Aq.start + (valid ? lane : 0);
     const uint32_t rl = rsd::uf_find(uf, si);
-    const bool open = valid && rl != uint32_t(big[int64_t(Aq.node) - A.nb]);
+    bool open = valid && rl != uint32_t(big[int64_t(Aq.node) - A.nb]);
     if (!__any_sync(kFull, open)) continue;
     const float4 xy = A.XY[si];
     const float2 z = A.Z[si];
@@ -829,25 +854,27 @@ k_link_far(SearchArgs A, const uint32_t* __restrict__ uni, const unsigned long l
     W.root[lane] = rl;
     __syncwarp();
     const float c[6] = {xy.x, xy.z, z.x, xy.y, xy.w, z.y};
-    float lo[6], hi[6];
-    warp_box(c, open, lo, hi);
-    const Box QB = make_box(lo, hi);
+    Box QB = query_box(c, open);
+    unsigned left = __ballot_sync(kFull, open);
+    int boxed = __popc(left);
     const int64_t own = (a - int64_t(Aq.first)) >> 5, nsb = Aq.sbcount;
-    for (int64_t s0 = 0; s0 < nsb; s0 += 32) {
+    const int64_t nchunk = (nsb + 31) >> 5, chunk0 = own >> 5;
+    for (int64_t k = 0; k < nchunk && left; ++k) {  // from the query's own stretch of the curve on
+      const int64_t s0 = 32 * (chunk0 + k < nchunk ? chunk0 + k : chunk0 + k - nchunk);
       bool near = false;
       if (s0 + lane < nsb && s0 + lane != own) {
         near = lb_box_box(QB, A.sbox[Aq.sbfirst + s0 + lane], s) <= l2;
         if (kCount) T.box += 1;
       }
       unsigned sm = __ballot_sync(kFull, near);
-      while (sm) {
-        const int64_t sb = s0 + __ffs(sm) - 1;
-        sm &= sm - 1u;
+      while (sm && left) {
+        const int64_t sb = s0 + next_outward(sm, k == 0 ? int(own & 31) : 0);
         const int64_t b_lo = int64_t(Aq.first) + 32 * sb;
         const int64_t b_hi = rsd::min64(b_lo + 32, int64_t(Aq.last) + 1);
         unsigned mask = stage_boxes<kCount>(A, b_lo, b_hi, QB, l2, s, lane, W, T);
         if (b_lo + lane < b_hi) W.uni[lane] = uni[b_lo + lane];
         __syncwarp();
+        bool united = false;
         while (mask) {
           const int i = __ffs(mask) - 1;
           mask &= mask - 1u;
@@ -859,7 +886,13 @@ k_link_far(SearchArgs A, const uint32_t* __restrict__ uni, const unsigned long l
           const int cnt = b == int64_t(Aq.last) ? int(A.bk[b].count) : 32;
           const uint32_t start = uint32_t(int64_t(Aq.start) + 32 * (b - a));
           const uint32_t rj = lane < cnt ? rsd::uf_find(uf, start + lane) : 0u;
-          link_eval<kCount, false>(A, uf, start, cnt, nm, s, l2, rj, lane, W, T);
+          united |= link_eval<kCount, false>(A, uf, start, cnt, nm, s, l2, rj, lane, W, T);
+        }
+        if (united) {  // members that have joined the largest component are done, like its others
+          const uint32_t rb = rsd::uf_find(uf, uint32_t(big[int64_t(Aq.node) - A.nb]));
+          if (open) open = rsd::uf_find(uf, W.root[lane]) != rb;
+          left = __ballot_sync(kFull, open);
+          refresh_box(QB, boxed, c, open);
         }
       }
     }
