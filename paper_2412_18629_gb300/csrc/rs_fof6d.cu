@@ -63,6 +63,21 @@ k_max_id(int64_t n, const int64_t* __restrict__ ids, const int64_t* __restrict__
   }
 }
 
+// Sizes of a level's nodes for the choice of its searches: stat[0] += sum of g^2, stat[1] = max g (one
+// atomic each per warp that holds a node; every lane of the warp calls this).
+__device__ __forceinline__ void level_stat(unsigned long long* __restrict__ stat, bool node, int64_t g) {
+  if (!__any_sync(0xffffffffu, node)) return;
+  unsigned long long sq = node ? (unsigned long long)(g * g) : 0ull;
+  unsigned mx = node ? unsigned(g) : 0u;
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(stat, sq);
+    atomicMax(stat + 1, (unsigned long long)mx);
+  }
+}
+
 // ---- level 0 over a dense label range (max label < 2 n + 4096): per-label member counts, the
 // kept labels' node indices and member offsets from two scans over the label range, then one
 // sort of the kept particles only, by (node, id).
@@ -73,10 +88,12 @@ __global__ void k_label_count(int64_t n, const int64_t* __restrict__ lab, uint32
 }
 
 __global__ void k_label_keep(int64_t nl, const uint32_t* __restrict__ cnt, int min_size,
-                             int64_t* __restrict__ knode, int64_t* __restrict__ ksize) {
+                             int64_t* __restrict__ knode, int64_t* __restrict__ ksize,
+                             unsigned long long* __restrict__ stat) {
   const int64_t l = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const bool keep = l < nl && cnt[l] >= uint32_t(min_size);
+  level_stat(stat, keep, keep ? int64_t(cnt[l]) : 0);
   if (l >= nl) return;
-  const bool keep = cnt[l] >= uint32_t(min_size);
   knode[l] = keep ? 1 : 0;
   ksize[l] = keep ? int64_t(cnt[l]) : 0;
 }
@@ -154,11 +171,13 @@ __global__ void k_run_starts(int64_t n, const uint64_t* __restrict__ keys, int b
 }
 
 __global__ void k_run_keep(int64_t nruns, int64_t n, const int64_t* __restrict__ run_start,
-                           int min_size, int64_t* __restrict__ keep, int64_t* __restrict__ size) {
+                           int min_size, int64_t* __restrict__ keep, int64_t* __restrict__ size,
+                           unsigned long long* __restrict__ stat) {
   const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (r >= nruns) return;
-  const int64_t e = (r + 1 < nruns) ? run_start[r + 1] : n;
-  const int64_t s = e - run_start[r];
+  const bool in = r < nruns;
+  const int64_t s = in ? (r + 1 < nruns ? run_start[r + 1] : n) - run_start[r] : 0;
+  level_stat(stat, in && s >= min_size, s);
+  if (!in) return;
   size[r] = s;
   keep[r] = s >= min_size ? 1 : 0;
 }
@@ -303,52 +322,76 @@ __device__ __forceinline__ float d6(float4 ui, float4 vi, float4 uj, float4 vj, 
   return __fadd_rn(__fmul_rn(rx, isx), __fmul_rn(rv, isv));
 }
 
-__global__ void k_tile_counts(int64_t nb, int64_t nn, const int64_t* __restrict__ node_size, int tile,
-                              int64_t* __restrict__ out) {
-  const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (k < nn) out[k] = (node_size[nb + k] + tile - 1) / tile;
+// All-pairs kernels: a block per (tile of kTile6 members, chunk of kChunk6 targets) of a node, so that a
+// single large node of a small level still spreads over the GPU (one block per tile over all targets
+// took as long as the largest node has members).
+constexpr int kChunk6 = 1024;
+
+__host__ __device__ __forceinline__ int64_t pair_items(int64_t g) {
+  return ((g + kTile6 - 1) / kTile6) * ((g + kChunk6 - 1) / kChunk6);
 }
 
-// Nearest-neighbour d6 per member: block = (node, i-tile of 128), j-tiles staged in shared memory.
+__global__ void k_pair_items(int64_t nb, int64_t nn, const int64_t* __restrict__ node_size,
+                             int64_t* __restrict__ out) {
+  const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (k < nn) out[k] = pair_items(node_size[nb + k]);
+}
+
+// Nearest-neighbour d6 per member (nn2 starts at +inf): the chunk's j-tiles staged in shared memory;
+// the chunks of a member combine by an atomic minimum of the float bits (distances are not negative).
 __global__ void __launch_bounds__(kTile6)
-k_nn6d(int64_t nb, int64_t nn, const int64_t* __restrict__ tile_off, const int64_t* __restrict__ node_off,
+k_nn6d(int64_t nb, int64_t nn, const int64_t* __restrict__ item_off, const int64_t* __restrict__ node_off,
        const int64_t* __restrict__ node_size, const float4* __restrict__ inv,
        const float4* __restrict__ U, const float4* __restrict__ V, float* __restrict__ nn2, int64_t mb) {
   __shared__ float4 su[kTile6], sv[kTile6];
   const int64_t b = blockIdx.x;
-  if (b >= tile_off[nn]) return;
-  const int64_t k = rsd::upper_bound_i64(tile_off, nn, b) - 1;
-  const int64_t t = b - tile_off[k];
+  if (b >= item_off[nn]) return;
+  const int64_t k = rsd::upper_bound_i64(item_off, nn, b) - 1;
   const int64_t q = nb + k;
   const int64_t base = node_off[q], g = node_size[q];
+  const int64_t chunks = (g + kChunk6 - 1) / kChunk6, t = (b - item_off[k]) / chunks,
+                c = (b - item_off[k]) - t * chunks;
   const float isx = inv[q].x, isv = inv[q].y;
-  const int64_t i = t * kTile6 + threadIdx.x;
+  const int64_t i = t * kTile6 + threadIdx.x, j_end = rsd::min64(g, (c + 1) * kChunk6);
   const bool valid = i < g;
   const float4 ui = valid ? U[base + i] : make_float4(0, 0, 0, 0);
   const float4 vi = valid ? V[base + i] : make_float4(0, 0, 0, 0);
   float best = __int_as_float(0x7f800000);
-  for (int64_t j0 = 0; j0 < g; j0 += kTile6) {
+  for (int64_t j0 = c * kChunk6; j0 < j_end; j0 += kTile6) {
     const int64_t j = j0 + threadIdx.x;
-    if (j < g) {
+    if (j < j_end) {
       su[threadIdx.x] = U[base + j];
       sv[threadIdx.x] = V[base + j];
     }
     __syncthreads();
-    const int jn = int(rsd::min64(kTile6, g - j0));
-    for (int jj = 0; jj < jn; ++jj) {
-      if (j0 + jj == i) continue;
-      best = fminf(best, d6(ui, vi, su[jj], sv[jj], isx, isv));
+    const int jn = int(rsd::min64(kTile6, j_end - j0));
+    if (j0 != t * kTile6) {
+#pragma unroll 4
+      for (int jj = 0; jj < jn; ++jj) best = fminf(best, d6(ui, vi, su[jj], sv[jj], isx, isv));
+    } else {  // the members' own tile
+      for (int jj = 0; jj < jn; ++jj) {
+        if (jj == int(threadIdx.x)) continue;
+        best = fminf(best, d6(ui, vi, su[jj], sv[jj], isx, isv));
+      }
     }
     __syncthreads();
   }
-  if (valid) nn2[base + i - mb] = best;
+  if (!valid) return;
+  if (chunks == 1)
+    nn2[base + i - mb] = best;
+  else
+    atomicMin(reinterpret_cast<unsigned int*>(nn2 + (base + i - mb)), __float_as_uint(best));
 }
 
 // Exact k-th smallest nn2 of each node, k = ceil(f_num g / f_den) - 1: radix select on the
 // (non-negative) float bit patterns. Nodes up to kSelectWarpMax members take one
 // warp each (k_select_l2_warp), larger ones a block (k_select_l2).
 constexpr int64_t kSelectWarpMax = 4096;
-constexpr int64_t kPrunedMinMembers = 4096;
+// Levels of more ordered pairs (sum of g^2) take the pruned searches of the batched form; below, the
+// all-pairs kernels cost less than their set-up (about 40 launches; 4e7 pairs are 0.05 ms of work on the
+// whole GPU). A 2^18-particle pass takes 600 device operations and 4.7 ms of device time with this line,
+// 794 and 5.7 ms when every level above 4096 members was pruned.
+constexpr unsigned long long kPrunedMinPairs = 40000000ull;
 
 // only (if given): int [nn], the nodes to select for (the others keep their l2).
 __global__ void __launch_bounds__(kT)
@@ -468,25 +511,38 @@ k_select_l2(int64_t nb, int64_t nn, const int64_t* __restrict__ node_off, const 
   }
 }
 
-__global__ void k_iota_u32(int64_t n, uint32_t* __restrict__ a) {
+// Start of a level: every member its own root, no neighbour yet, no child counted.
+__global__ void k_level_init(int64_t m, uint32_t* __restrict__ uf, float* __restrict__ nn2,
+                             unsigned long long* __restrict__ stat) {
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < n) a[i] = uint32_t(i);
+  if (i < 2) stat[i] = 0;
+  if (i >= m) return;
+  uf[i] = uint32_t(i);
+  nn2[i] = __int_as_float(0x7f800000);
 }
 
-// Union-find over pairs with d6 <= l2: block = (node, i-tile); j-tiles from the i-tile on.
+// Union-find over pairs with d6 <= l2: block = (node, i-tile, chunk of targets), pairs j > i. Targets
+// carry the root they had when their tile was staged: those that share the member's root already are
+// skipped, so most of the dense middle's links (dozens a member) cost no union. Roots that were equal
+// once stay in one component.
+constexpr uint32_t kNoRoot = 0xffffffffu;
+
 __global__ void __launch_bounds__(kTile6)
-k_link6d(int64_t nb, int64_t nn, const int64_t* __restrict__ tile_off, const int64_t* __restrict__ node_off,
+k_link6d(int64_t nb, int64_t nn, const int64_t* __restrict__ item_off, const int64_t* __restrict__ node_off,
          const int64_t* __restrict__ node_size, const float4* __restrict__ inv,
          const float4* __restrict__ U, const float4* __restrict__ V, const float* __restrict__ nn2,
          uint32_t* __restrict__ uf, int64_t mb) {
   __shared__ float4 su[kTile6], sv[kTile6];
-  __shared__ float snn[kTile6];
+  __shared__ uint32_t sroot[kTile6];  // kNoRoot: no friend at all
   const int64_t b = blockIdx.x;
-  if (b >= tile_off[nn]) return;
-  const int64_t k = rsd::upper_bound_i64(tile_off, nn, b) - 1;
-  const int64_t t = b - tile_off[k];
+  if (b >= item_off[nn]) return;
+  const int64_t k = rsd::upper_bound_i64(item_off, nn, b) - 1;
   const int64_t q = nb + k;
   const int64_t base = node_off[q], g = node_size[q];
+  const int64_t chunks = (g + kChunk6 - 1) / kChunk6, t = (b - item_off[k]) / chunks,
+                c = (b - item_off[k]) - t * chunks;
+  const int64_t j_end = rsd::min64(g, (c + 1) * kChunk6), j_begin = max(c * int64_t(kChunk6), t * int64_t(kTile6));
+  if (j_begin >= j_end) return;  // below the diagonal
   const float4 iv = inv[q];
   const float isx = iv.x, isv = iv.y, l2 = iv.z;
   const int64_t i = t * kTile6 + threadIdx.x;
@@ -494,21 +550,34 @@ k_link6d(int64_t nb, int64_t nn, const int64_t* __restrict__ tile_off, const int
   const float4 ui = valid ? U[base + i] : make_float4(0, 0, 0, 0);
   const float4 vi = valid ? V[base + i] : make_float4(0, 0, 0, 0);
   const bool active = valid && nn2[base + i - mb] <= l2;  // others have no friend at all
-  const uint32_t li = uint32_t(base + i - mb);
-  for (int64_t j0 = t * kTile6; j0 < g; j0 += kTile6) {
+  uint32_t root = active ? rsd::uf_find(uf, uint32_t(base + i - mb)) : kNoRoot;
+  for (int64_t j0 = j_begin; j0 < j_end; j0 += kTile6) {
     const int64_t j = j0 + threadIdx.x;
-    if (j < g) {
+    if (j < j_end) {
       su[threadIdx.x] = U[base + j];
       sv[threadIdx.x] = V[base + j];
-      snn[threadIdx.x] = nn2[base + j - mb];
+      sroot[threadIdx.x] = nn2[base + j - mb] <= l2 ? rsd::uf_find(uf, uint32_t(base + j - mb)) : kNoRoot;
     }
     __syncthreads();
-    const int jn = int(rsd::min64(kTile6, g - j0));
-    if (active) {
-      for (int jj = 0; jj < jn; ++jj) {
-        if (j0 + jj <= i || snn[jj] > l2) continue;
-        if (d6(ui, vi, su[jj], sv[jj], isx, isv) <= l2)
-          rsd::uf_unite(uf, li, uint32_t(base + j0 + jj - mb));
+    const int jn = int(rsd::min64(kTile6, j_end - j0));
+    const int first = j0 == t * kTile6 ? int(threadIdx.x) + 1 : 0;  // its own tile: j > i
+    for (int jb = 0; jb < jn; jb += 32) {
+      unsigned hits = 0;
+      if (active) {
+        for (int jj = max(jb, first); jj < min(jb + 32, jn); ++jj) {
+          const uint32_t rj = sroot[jj];
+          if (rj != root && rj != kNoRoot && d6(ui, vi, su[jj], sv[jj], isx, isv) <= l2) hits |= 1u << (jj - jb);
+        }
+      }
+      while (__any_sync(0xffffffffu, hits)) {  // one union a lane and round, the lanes side by side
+        if (hits) {
+          const uint32_t rj = sroot[jb + __ffs(hits) - 1];
+          hits &= hits - 1u;
+          if (rj != root) {
+            rsd::uf_unite(uf, root, rj);
+            root = rsd::uf_find(uf, root);
+          }
+        }
       }
     }
     __syncthreads();
@@ -529,15 +598,18 @@ __global__ void k_comp_count(int64_t m, uint32_t* __restrict__ uf, uint32_t* __r
 __global__ void k_child_flags(int64_t m, int64_t mb, const uint32_t* __restrict__ uf,
                               const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ mnode,
                               const int64_t* __restrict__ node_size, int min_size,
-                              int64_t* __restrict__ flag) {
+                              int64_t* __restrict__ flag, int64_t* __restrict__ flag2,
+                              unsigned long long* __restrict__ stat) {
   const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (p >= m) return;
-  int64_t f = 0;
-  if (uf[p] == uint32_t(p)) {
-    const int64_t c = cnt[p];
+  int64_t f = 0, c = 0;
+  if (p < m && uf[p] == uint32_t(p)) {
+    c = cnt[p];
     f = (c >= min_size && c < node_size[mnode[mb + p]]) ? 1 : 0;
   }
+  level_stat(stat, f != 0, c);
+  if (p >= m) return;
   flag[p] = f;
+  flag2[p] = f;  // the copy that is scanned into child indices
 }
 
 // member flag: 1 if the member's root is a child root.
@@ -726,6 +798,8 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
   uint32_t* deep_pos = scratch_t<uint32_t>(ctx, S_H_DEEPPOS, size_t(std::max<int64_t>(n, 1)));
   if (!deep) return RS_ERR_OOM;
   int64_t nodes = 0, members = 0;
+  uint64_t level_pairs = 0;  // sum of g^2 over the level's nodes
+  int64_t level_max = 0;     // its largest node
   if (n == 0) {
     RS_TRY(ensure_nodes(ctx, 0, 1, st));
     RS_TRY(ensure_members(ctx, 0, 1, st));
@@ -737,7 +811,8 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
     if (!deep_pos) return RS_ERR_OOM;
     unsigned long long* mx = scratch_t<unsigned long long>(ctx, S_COUNTER, 16);
     if (!mx) return RS_ERR_OOM;
-    RS_CUDA(ctx, cudaMemsetAsync(mx, 0, 16, st));
+    unsigned long long* stat = mx + 4;  // sum of g^2 and largest node of the level being built
+    RS_CUDA(ctx, cudaMemsetAsync(mx, 0, 48, st));
     k_max_id<<<std::min(grid_for(n, kT), 152u * 8u), kT, 0, st>>>(n, ids, fof_label, mx);
     RS_LAUNCHED(ctx, "k_max_id");
     RS_TRY(read_back(ctx, mx, 16, st));
@@ -756,15 +831,18 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       RS_CUDA(ctx, cudaMemsetAsync(cntl, 0, sizeof(uint32_t) * nl, st));
       k_label_count<<<grid_for(n, kT), kT, 0, st>>>(n, fof_label, cntl);
       RS_LAUNCHED(ctx, "k_label_count");
-      k_label_keep<<<grid_for(nl, kT), kT, 0, st>>>(nl, cntl, min_size, knode, koff);
+      k_label_keep<<<grid_for(nl, kT), kT, 0, st>>>(nl, cntl, min_size, knode, koff, stat);
       RS_LAUNCHED(ctx, "k_label_keep");
       RS_TRY(exclusive_scan_i64(ctx, nl, knode, knode + nl, st));
       RS_TRY(exclusive_scan_i64(ctx, nl, koff, koff + nl, st));
       RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box, knode + nl, 8, cudaMemcpyDeviceToHost, st));
       RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 1, koff + nl, 8, cudaMemcpyDeviceToHost, st));
+      RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 2, stat, 16, cudaMemcpyDeviceToHost, st));
       RS_CUDA(ctx, cudaStreamSynchronize(st));
       nodes = ctx->host_box[0];
       members = ctx->host_box[1];
+      level_pairs = uint64_t(ctx->host_box[2]);
+      level_max = ctx->host_box[3];
       RS_TRY(ensure_nodes(ctx, 0, std::max<int64_t>(nodes, 1) * 2, st));
       RS_TRY(ensure_members(ctx, 0, std::max<int64_t>(members, 1) * 2, st));
       Hier h = hier_of(ctx);
@@ -822,7 +900,7 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       const int64_t nruns = ctx->host_box[0];
       k_run_starts<<<grid_for(n, kT), kT, 0, st>>>(n, keys, b, head, run_start);
       RS_LAUNCHED(ctx, "k_run_starts");
-      k_run_keep<<<grid_for(nruns, kT), kT, 0, st>>>(nruns, n, run_start, min_size, keep, rsize);
+      k_run_keep<<<grid_for(nruns, kT), kT, 0, st>>>(nruns, n, run_start, min_size, keep, rsize, stat);
       RS_LAUNCHED(ctx, "k_run_keep");
       RS_CUDA(ctx, cudaMemcpyAsync(node_of_run, keep, sizeof(int64_t) * nruns,
                                    cudaMemcpyDeviceToDevice, st));
@@ -832,9 +910,12 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       RS_TRY(exclusive_scan_i64(ctx, nruns, mem_off, mem_off + nruns, st));
       RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box, node_of_run + nruns, 8, cudaMemcpyDeviceToHost, st));
       RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 1, mem_off + nruns, 8, cudaMemcpyDeviceToHost, st));
+      RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 2, stat, 16, cudaMemcpyDeviceToHost, st));
       RS_CUDA(ctx, cudaStreamSynchronize(st));
       nodes = ctx->host_box[0];
       members = ctx->host_box[1];
+      level_pairs = uint64_t(ctx->host_box[2]);
+      level_max = ctx->host_box[3];
       RS_TRY(ensure_nodes(ctx, 0, std::max<int64_t>(nodes, 1) * 2, st));
       RS_TRY(ensure_members(ctx, 0, std::max<int64_t>(members, 1) * 2, st));
       Hier h = hier_of(ctx);
@@ -868,19 +949,24 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
                                           MomentTerm{h.U, h.V}, sums, st)));
     k_node_inv<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.node_size, sums, h.inv, h.mom);
     RS_LAUNCHED(ctx, "k_node_inv");
-    // tiles of 128 members
-    int64_t* tile_off = scratch_t<int64_t>(ctx, S_SELECT, size_t(nn) + 1);
+    int64_t* item_off = scratch_t<int64_t>(ctx, S_SELECT, size_t(nn) + 1);
     float* nn2 = scratch_t<float>(ctx, S_NN2, size_t(m));
     uint32_t* uf = scratch_t<uint32_t>(ctx, S_UF, size_t(m));
     uint32_t* cnt = scratch_t<uint32_t>(ctx, S_ROOT_CNT, size_t(m));
     int64_t* cflag = scratch_t<int64_t>(ctx, S_FLAGS, size_t(m) + 1);
     int64_t* cidx = scratch_t<int64_t>(ctx, S_CHILD_IDX, size_t(m) + 1);
     int64_t* mpos = scratch_t<int64_t>(ctx, S_GKEY_A, size_t(m) + 1);
-    if (!tile_off || !nn2 || !uf || !cnt || !cflag || !cidx || !mpos) return RS_ERR_OOM;
-    // batched form: pruned searches, except on levels of at most kPrunedMinMembers members,
-    // where the brute-force pair kernels (identical results) cost less than the bucket set-up
-    const bool batched = ctx->cfg.batched != 0 && m > kPrunedMinMembers;
-    const int64_t tiles_ub = nn + m / kTile6 + 1;
+    unsigned long long* stat = scratch_t<unsigned long long>(ctx, S_COUNTER, 16);
+    if (!item_off || !nn2 || !uf || !cnt || !cflag || !cidx || !mpos || !stat) return RS_ERR_OOM;
+    stat += 4;
+    // batched form: pruned searches, except on levels of few pairs (unless a smallest node for the
+    // bounded searches was asked for and the level has one)
+    const bool batched = ctx->cfg.batched != 0 && (level_pairs > kPrunedMinPairs ||
+                                                   (ctx->nn_bound_min > 0 && level_max >= ctx->nn_bound_min));
+    // at most (g / 128 + 1) (g / 1024 + 1) items a node
+    const int64_t items_ub = int64_t(level_pairs / (uint64_t(kTile6) * kChunk6)) + m / kTile6 + m / kChunk6 + nn + 1;
+    k_level_init<<<grid_for(m, kT), kT, 0, st>>>(m, uf, nn2, stat);
+    RS_LAUNCHED(ctx, "k_level_init");
     // k-th smallest nn2 of the level's nodes (of those with only[k] != 0 when `only` is given); the
     // batched form's nn2 is in its sorted order, in which every node keeps its range
     auto select = [&](const int* only) -> int {
@@ -903,12 +989,12 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       RS_TRY(prune6d_far(ctx, nb, nn, mb, m, nn2, st));
       h = hier_of(ctx);
     } else {
-      k_tile_counts<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.node_size, kTile6, tile_off);
-      RS_LAUNCHED(ctx, "k_tile_counts");
-      RS_TRY(exclusive_scan_i64(ctx, nn, tile_off, tile_off + nn, st));
+      k_pair_items<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.node_size, item_off);
+      RS_LAUNCHED(ctx, "k_pair_items");
+      RS_TRY(exclusive_scan_i64(ctx, nn, item_off, item_off + nn, st));
       {
         ProfScope prof_(ctx, "k_nn6d", st);
-        k_nn6d<<<grid_for(tiles_ub, 1), kTile6, 0, st>>>(nb, nn, tile_off, h.node_off, h.node_size, h.inv,
+        k_nn6d<<<grid_for(items_ub, 1), kTile6, 0, st>>>(nb, nn, item_off, h.node_off, h.node_size, h.inv,
                                                         h.U, h.V, nn2, mb);
       }
       RS_LAUNCHED(ctx, "k_nn6d");
@@ -920,14 +1006,12 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       if (failed) RS_TRY(select(failed));
       h = hier_of(ctx);
     }
-    k_iota_u32<<<grid_for(m, kT), kT, 0, st>>>(m, uf);
-    RS_LAUNCHED(ctx, "k_iota_u32");
     if (batched) {
       RS_TRY(prune6d_link(ctx, nb, nn, mb, m, nn2, uf, st));
     } else {
       {
         ProfScope prof_(ctx, "k_link6d", st);
-        k_link6d<<<grid_for(tiles_ub, 1), kTile6, 0, st>>>(nb, nn, tile_off, h.node_off, h.node_size,
+        k_link6d<<<grid_for(items_ub, 1), kTile6, 0, st>>>(nb, nn, item_off, h.node_off, h.node_size,
                                                           h.inv, h.U, h.V, nn2, uf, mb);
       }
       RS_LAUNCHED(ctx, "k_link6d");
@@ -935,9 +1019,8 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
     RS_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * m, st));
     k_comp_count<<<grid_for(m, kT), kT, 0, st>>>(m, uf, cnt);
     RS_LAUNCHED(ctx, "k_comp_count");
-    k_child_flags<<<grid_for(m, kT), kT, 0, st>>>(m, mb, uf, cnt, h.mnode, h.node_size, min_size, cflag);
+    k_child_flags<<<grid_for(m, kT), kT, 0, st>>>(m, mb, uf, cnt, h.mnode, h.node_size, min_size, cflag, cidx, stat);
     RS_LAUNCHED(ctx, "k_child_flags");
-    RS_CUDA(ctx, cudaMemcpyAsync(cidx, cflag, sizeof(int64_t) * m, cudaMemcpyDeviceToDevice, st));
     RS_TRY(exclusive_scan_i64(ctx, m, cidx, cidx + m, st));
     k_member_flags<<<grid_for(m, kT), kT, 0, st>>>(m, uf, cflag, mpos);
     RS_LAUNCHED(ctx, "k_member_flags");
@@ -946,7 +1029,10 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
     RS_LAUNCHED(ctx, "k_deepest");
     RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box, cidx + m, 8, cudaMemcpyDeviceToHost, st));
     RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 1, mpos + m, 8, cudaMemcpyDeviceToHost, st));
+    RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 2, stat, 16, cudaMemcpyDeviceToHost, st));
     RS_CUDA(ctx, cudaStreamSynchronize(st));
+    level_pairs = uint64_t(ctx->host_box[2]);
+    level_max = ctx->host_box[3];
     const int64_t nchild = ctx->host_box[0], mchild = ctx->host_box[1];
     ++levels;
     if (nchild == 0) {
