@@ -151,9 +151,11 @@ extern "C" int rs_use_graphs(rs_ctx* ctx, int enable) {
 namespace {
 struct ArrayTerm {
   const double* a;
+  using Value = double;
+  __device__ __forceinline__ Value load(int64_t p) const { return a[p]; }
   template <bool kFirst>
-  __device__ __forceinline__ void add(int64_t, int64_t p, int64_t, double* acc) const {
-    rsd::cro_add<kFirst>(acc[0], a[p]);
+  __device__ __forceinline__ void add(int64_t, Value v, double* acc) const {
+    rsd::cro_add<kFirst>(acc[0], v);
   }
 };
 

@@ -431,12 +431,10 @@ __device__ __forceinline__ void warp_count(unsigned long long* ctr, bool pred) {
 
 // Canonical-order combination of the 32 lane partial sums of a warp: halving tree
 // s[l] += s[l + off], off = 16 .. 1, realised as an xor butterfly (IEEE + commutes, so lane
-// 0 ends with exactly the halving-tree value). When only lanes below 2 off0 hold terms (the
-// others hold 0.0 and no lane sum is -0.0), the steps above off0 add 0.0 to every sum they
-// touch, so starting at off0 gives lane 0 the same value.
-__device__ __forceinline__ double warp_cro_combine(double s, int off0 = 16) {
+// 0 ends with exactly the halving-tree value).
+__device__ __forceinline__ double warp_cro_combine(double s) {
 #pragma unroll
-  for (int off = off0; off >= 1; off >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, off));
+  for (int off = 16; off >= 1; off >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, off));
   return s;
 }
 

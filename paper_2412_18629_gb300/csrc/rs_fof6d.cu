@@ -270,9 +270,13 @@ __global__ void k_node_ref(int64_t nb, int64_t ne, const uint32_t* __restrict__ 
 struct MomentTerm {
   const float4* U;
   const float4* V;
+  struct Value {
+    float4 u, v;
+  };
+  __device__ __forceinline__ Value load(int64_t p) const { return {U[p], V[p]}; }
   template <bool kFirst>
-  __device__ __forceinline__ void add(int64_t, int64_t p, int64_t, double* acc) const {
-    const float4 u = U[p], v = V[p];
+  __device__ __forceinline__ void add(int64_t, const Value& t, double* acc) const {
+    const float4 u = t.u, v = t.v;
     const double a[3] = {rsd::f2d(u.x), rsd::f2d(u.y), rsd::f2d(u.z)};
     const double b[3] = {rsd::f2d(v.x), rsd::f2d(v.y), rsd::f2d(v.z)};
     const float uc[3] = {u.x, u.y, u.z}, vc[3] = {v.x, v.y, v.z};

@@ -76,9 +76,13 @@ __global__ void k_seed_segments(int64_t nn, const int* __restrict__ nkids, const
 struct SeedTerm {  // u^s and v of a member of seed s
   const float4* U;
   const float4* V;
+  struct Value {
+    float4 u, v;
+  };
+  __device__ __forceinline__ Value load(int64_t p) const { return {U[p], V[p]}; }
   template <bool kFirst>
-  __device__ __forceinline__ void add(int64_t, int64_t p, int64_t, double* acc) const {
-    const float4 u = U[p], v = V[p];
+  __device__ __forceinline__ void add(int64_t, const Value& t, double* acc) const {
+    const float4 u = t.u, v = t.v;
     rsd::cro_add<kFirst>(acc[0], rsd::f2d(u.x));
     rsd::cro_add<kFirst>(acc[1], rsd::f2d(u.y));
     rsd::cro_add<kFirst>(acc[2], rsd::f2d(u.z));

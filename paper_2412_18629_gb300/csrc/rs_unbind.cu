@@ -298,9 +298,10 @@ k_potential_blocked(int64_t nn, const int64_t* __restrict__ tile_off, const uint
 
 struct VelTerm {
   const float4* V;
+  using Value = float4;
+  __device__ __forceinline__ Value load(int64_t p) const { return V[p]; }
   template <bool kFirst>
-  __device__ __forceinline__ void add(int64_t, int64_t p, int64_t, double* acc) const {
-    const float4 v = V[p];
+  __device__ __forceinline__ void add(int64_t, Value v, double* acc) const {
     rsd::cro_add<kFirst>(acc[0], rsd::f2d(v.x));
     rsd::cro_add<kFirst>(acc[1], rsd::f2d(v.y));
     rsd::cro_add<kFirst>(acc[2], rsd::f2d(v.z));
@@ -311,13 +312,17 @@ struct VelTerm {
 struct VelTermMasked {
   const float4* V;
   const uint8_t* in;
+  struct Value {
+    float4 v;
+    bool keep;
+  };
+  __device__ __forceinline__ Value load(int64_t p) const { return {V[p], in[p] != 0}; }
   template <bool kFirst>
-  __device__ __forceinline__ void add(int64_t, int64_t p, int64_t, double* acc) const {
-    const float4 v = V[p];
-    const bool keep = in[p] != 0;
-    rsd::cro_add<kFirst>(acc[0], keep ? rsd::f2d(v.x) : 0.0);
-    rsd::cro_add<kFirst>(acc[1], keep ? rsd::f2d(v.y) : 0.0);
-    rsd::cro_add<kFirst>(acc[2], keep ? rsd::f2d(v.z) : 0.0);
+  __device__ __forceinline__ void add(int64_t, const Value& t, double* acc) const {
+    if (!t.keep) return;  // adding 0.0 leaves a lane sum as it is (never -0.0; the first is 0.0)
+    rsd::cro_add<kFirst>(acc[0], rsd::f2d(t.v.x));
+    rsd::cro_add<kFirst>(acc[1], rsd::f2d(t.v.y));
+    rsd::cro_add<kFirst>(acc[2], rsd::f2d(t.v.z));
   }
 };
 
@@ -474,14 +479,15 @@ struct PropTerm1 {  // bound-masked u, u^2, v, v^2
   const float4* U;
   const float4* V;
   const uint8_t* bound;
+  struct Value {
+    float4 u, v;
+    bool bound;
+  };
+  __device__ __forceinline__ Value load(int64_t p) const { return {U[p], V[p], bound[p] != 0}; }
   template <bool kFirst>
-  __device__ __forceinline__ void add(int64_t, int64_t p, int64_t, double* acc) const {
-    if (!bound[p]) {
-#pragma unroll
-      for (int s = 0; s < 12; ++s) rsd::cro_add<kFirst>(acc[s], 0.0);
-      return;
-    }
-    const float4 u = U[p], v = V[p];
+  __device__ __forceinline__ void add(int64_t, const Value& t, double* acc) const {
+    if (!t.bound) return;  // adding 0.0 leaves a lane sum as it is (never -0.0; the first is 0.0)
+    const float4 u = t.u, v = t.v;
     const double a[3] = {rsd::f2d(u.x), rsd::f2d(u.y), rsd::f2d(u.z)};
     const double b[3] = {rsd::f2d(v.x), rsd::f2d(v.y), rsd::f2d(v.z)};
     const float uc[3] = {u.x, u.y, u.z}, vc[3] = {v.x, v.y, v.z};
@@ -499,14 +505,15 @@ struct PropTerm2 {  // bound-masked second moments about the bound mean
   const float4* U;
   const uint8_t* bound;
   const double* mean;  // [node][3]
+  struct Value {
+    float4 u;
+    bool bound;
+  };
+  __device__ __forceinline__ Value load(int64_t p) const { return {U[p], bound[p] != 0}; }
   template <bool kFirst>
-  __device__ __forceinline__ void add(int64_t q, int64_t p, int64_t, double* acc) const {
-    if (!bound[p]) {
-#pragma unroll
-      for (int s = 0; s < 6; ++s) rsd::cro_add<kFirst>(acc[s], 0.0);
-      return;
-    }
-    const float4 u = U[p];
+  __device__ __forceinline__ void add(int64_t q, const Value& t, double* acc) const {
+    if (!t.bound) return;  // adding 0.0 leaves a lane sum as it is (never -0.0; the first is 0.0)
+    const float4 u = t.u;
     const double* mu = mean + 3 * q;
     const double d[3] = {__dsub_rn(rsd::f2d(u.x), mu[0]), __dsub_rn(rsd::f2d(u.y), mu[1]),
                          __dsub_rn(rsd::f2d(u.z), mu[2])};
