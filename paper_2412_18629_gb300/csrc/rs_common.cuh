@@ -26,7 +26,7 @@ enum Slot : int {
   S_KEY_A, S_KEY_B, S_VAL_A, S_VAL_B, S_SORT_HIST, S_POS_SORTED, S_ROW_CELL, S_CELL_OF,
   S_CELL_TILES, S_CELL_START, S_CELL_ROW, S_CELL_X, S_CELL_PAIRS, S_PARENT, S_MINID, S_COUNTER,
   // rs_fof6d (level work)
-  S_GKEY_A, S_GKEY_B, S_GVAL_A, S_GVAL_B, S_NN2, S_UF, S_ROOT_CNT, S_CHILD_IDX, S_FLAGS,
+  S_GKEY_A, S_GKEY_B, S_GVAL_A, S_GVAL_B, S_NN2, S_UF, S_ROOT_CNT, S_CHILD_IDX,
   S_SCAN_TMP, S_CHUNK_OFF, S_CHUNK_SUM, S_NODE_TMP, S_SELECT,
   // hierarchy state (persists until the next rs_fof6d)
   S_H_MEM, S_H_MNODE, S_H_U, S_H_V, S_H_NODE_OFF, S_H_NODE_SIZE, S_H_NODE_PARENT,
@@ -210,7 +210,26 @@ int radix_sort_u64(rs_ctx* ctx, int64_t n, int nbits, uint64_t* keys_a, uint32_t
                    uint64_t* keys_b, uint32_t* vals_b, uint64_t** keys_out,
                    uint32_t** vals_out, cudaStream_t st);
 
-// Exclusive prefix sum of int64 values in place; returns the total via *total_dev (device).
+// Whether that sort's output is in the B buffers (one pass per 8 bits, each from one side to the other).
+inline bool sort_ends_in_b(int64_t n, int nbits) { return n > 1 && nbits > 0 && ((nbits + 7) / 8) % 2 == 1; }
+
+// One exclusive prefix sum of int64 values: out[i] = first + the sum of the elements before i of `in`
+// (which may be `out`), *total (device, may be null) = first + their sum. An element counts as its
+// value, or with tile > 0 as the number of 2^tile rows it fills, times with chunk > 0 the number of
+// 2^chunk columns. A ScanJobs is up to three scans of one length in the same launches (out = null ends it).
+struct ScanJob {
+  const int64_t* in;
+  int64_t* out;
+  int64_t* total;
+  int tile, chunk;
+  int64_t first;
+};
+struct ScanJobs {
+  ScanJob job[3];
+};
+int exclusive_scans(rs_ctx* ctx, int64_t n, const ScanJobs& jobs, cudaStream_t st);
+
+// Exclusive prefix sum in place; returns the total via *total_dev (device).
 int exclusive_scan_i64(rs_ctx* ctx, int64_t n, int64_t* data, int64_t* total_dev,
                        cudaStream_t st);
 

@@ -213,16 +213,16 @@ namespace rs {
 // Segmented CRO driver: segment q covers global positions [seg_off[q], seg_off[q] + seg_size[q]);
 // `total` = sum of the sizes (bounds the chunk count without a host round trip).
 // Writes seg_sums[q * NS + s]. Uses the S_CHUNK_OFF / S_CHUNK_SUM scratch slots.
-// chunk_off[q] = sum over earlier segments of ceil(size / 1024); chunk_off[nseg] = total chunks.
-int cro_prepare(rs_ctx* ctx, int64_t nseg, const int64_t* seg_size, int64_t** chunk_off,
-                cudaStream_t st);
-
+// `also` is an independent scan over the segments (`out` null: none) that shares the launches of the
+// chunk offsets' scan: chunk_off[q] = sum over earlier segments of ceil(size / 1024), chunk_off[nseg] =
+// total chunks.
 template <int NS, class Term>
 int cro_segmented(rs_ctx* ctx, int64_t nseg, const int64_t* seg_off, const int64_t* seg_size,
-                  int64_t total, Term term, double* seg_sums, cudaStream_t st) {
+                  int64_t total, Term term, double* seg_sums, cudaStream_t st, ScanJob also = {}) {
   if (nseg <= 0) return RS_OK;
-  int64_t* chunk_off;
-  RS_TRY(cro_prepare(ctx, nseg, seg_size, &chunk_off, st));
+  int64_t* chunk_off = scratch_t<int64_t>(ctx, S_CHUNK_OFF, size_t(nseg) + 1);
+  if (!chunk_off) return RS_ERR_OOM;
+  RS_TRY(exclusive_scans(ctx, nseg, ScanJobs{{{seg_size, chunk_off, chunk_off + nseg, 10, 0, 0}, also}}, st));
   const int64_t nchunks_ub = nseg + total / 1024 + 1;
   double* chunk_sums = scratch_t<double>(ctx, S_CHUNK_SUM, size_t(nchunks_ub) * NS);
   if (!chunk_sums) return RS_ERR_OOM;

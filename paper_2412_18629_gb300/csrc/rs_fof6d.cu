@@ -4,13 +4,13 @@
 //
 // Level-synchronous: level 0 = FoF groups with >= min members (sorted by (label, id)); each
 // level runs, over all of its nodes at once,
-//   k_member_node   owning node of every member position
-//   k_gather_uv     u = wrapped offset from the node's smallest-id member, v, as float4
+//   k_level_members owning node of every member position; u = wrapped offset from the node's
+//                   smallest-id member, v, as float4
 //   CRO moments     12 float64 sums per node -> inv_sx2, inv_sv2 (k_node_inv)
 //   k_nn6d          brute-force nearest-neighbour d6 per member, j-tiles in shared memory
 //   k_select_l2     exact k-th smallest nn2 per node (radix select on the float bit patterns)
 //   k_link6d        union-find over pairs with d6 <= l2 (upper triangle of each node)
-//   k_comp_count    roots and component sizes; k_child_flags marks children
+//   k_comp_count    roots and component sizes; k_child_flags marks children; k_children
 //   compaction + stable radix sort by child index -> next level's member list (ascending id
 //   inside each child because member positions ascend with id)
 // Every float32 operation of d6 is rounded separately (no FMA), so the result equals the
@@ -20,20 +20,22 @@
 namespace {
 
 constexpr int kT = 256;
-constexpr int kTile6 = 128;
+constexpr int kTile6Bits = 7, kTile6 = 1 << kTile6Bits;
 
 // ---------------------------------------------------------------------------------------------
 // Level 0 from FoF labels.
 
-// out[0] = max id, out[1] = max label (~0 in both when any id or label is negative).
+// out[0] = max id, out[1] = max label (~0 in both when any id or label is negative); no particle has
+// a deepest node yet.
 __global__ void __launch_bounds__(256)
 k_max_id(int64_t n, const int64_t* __restrict__ ids, const int64_t* __restrict__ lab,
-         unsigned long long* __restrict__ out) {
+         unsigned long long* __restrict__ out, int64_t* __restrict__ deepest) {
   __shared__ unsigned long long wmax[2][8];
   unsigned long long mi = 0, ml = 0;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x) {
     const int64_t a = ids[i], b = lab[i];
+    deepest[i] = -1;
     if (a < 0 || b < 0) {
       mi = ml = ~0ull;
     } else {
@@ -98,11 +100,12 @@ __global__ void k_label_keep(int64_t nl, const uint32_t* __restrict__ cnt, int m
   ksize[l] = keep ? int64_t(cnt[l]) : 0;
 }
 
-__global__ void k_label_nodes(int64_t nl, const uint32_t* __restrict__ cnt, int min_size,
+__global__ void k_label_nodes(int64_t nl, int64_t nodes, int64_t members, const uint32_t* __restrict__ cnt, int min_size,
                               const int64_t* __restrict__ knode, const int64_t* __restrict__ koff,
                               int64_t* __restrict__ node_off, int64_t* __restrict__ node_size,
                               int64_t* __restrict__ node_parent, int32_t* __restrict__ node_level) {
   const int64_t l = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (l == 0) node_off[nodes] = members;
   if (l >= nl || cnt[l] < uint32_t(min_size)) return;
   const int64_t q = knode[l];
   node_off[q] = koff[l];
@@ -129,13 +132,6 @@ __global__ void k_label_keys(int64_t n, const int64_t* __restrict__ ids, const i
   const unsigned long long pos = base + __popc(b & ((1u << lane) - 1u));
   keys[pos] = (uint64_t(knode[l]) << bid) | uint64_t(ids[i]);
   vals[pos] = uint32_t(i);
-}
-
-__global__ void k_level0_minid(int64_t nodes, const int64_t* __restrict__ node_off,
-                               const uint32_t* __restrict__ mem, const int64_t* __restrict__ ids,
-                               int64_t* __restrict__ node_minid) {
-  const int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (q < nodes) node_minid[q] = ids[mem[node_off[q]]];  // members ascend by id
 }
 
 // Sparse labels: all particles ordered by (label, id) with two stable radix sorts, first by id
@@ -183,22 +179,20 @@ __global__ void k_run_keep(int64_t nruns, int64_t n, const int64_t* __restrict__
 }
 
 // Level-0 node table and member list (particle indices), from kept runs.
-__global__ void k_level0_nodes(int64_t nruns, const int64_t* __restrict__ run_start,
+__global__ void k_level0_nodes(int64_t nruns, int64_t nodes, int64_t members,
                                const int64_t* __restrict__ size, const int64_t* __restrict__ keep,
                                const int64_t* __restrict__ node_of_run /*scan of keep*/,
                                const int64_t* __restrict__ mem_off /*scan of kept sizes*/,
-                               const uint32_t* __restrict__ vals, const int64_t* __restrict__ ids,
                                int64_t* __restrict__ node_off, int64_t* __restrict__ node_size,
-                               int64_t* __restrict__ node_parent, int32_t* __restrict__ node_level,
-                               int64_t* __restrict__ node_minid) {
+                               int64_t* __restrict__ node_parent, int32_t* __restrict__ node_level) {
   const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (r == 0) node_off[nodes] = members;
   if (r >= nruns || !keep[r]) return;
   const int64_t q = node_of_run[r];
   node_off[q] = mem_off[r];
   node_size[q] = size[r];
   node_parent[q] = -1;
   node_level[q] = 0;
-  node_minid[q] = ids[vals[run_start[r]]];
 }
 
 // run_heads holds the exclusive scan of the head flags: a run start sees its own run index,
@@ -221,10 +215,7 @@ __global__ void k_level0_members(int64_t n, const uint64_t* __restrict__ keys, i
   mem[mem_off[r] + (i - run_start[r])] = vals[i];
 }
 
-__global__ void k_fill_i64(int64_t n, int64_t* __restrict__ a, int64_t v) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < n) a[i] = v;
-}
+__global__ void k_fill_i64(int64_t* __restrict__ a, int64_t v) { *a = v; }
 
 __global__ void k_size_mask(int64_t n, const int64_t* __restrict__ keep, const int64_t* __restrict__ size,
                             int64_t* __restrict__ out) {
@@ -236,11 +227,43 @@ __global__ void k_size_mask(int64_t n, const int64_t* __restrict__ keep, const i
 // Per-level kernels. Member positions p are global (into the hierarchy's member list);
 // level-local position = p - mb.
 
-__global__ void k_member_node(int64_t mb, int64_t me, int64_t nb, int64_t nn,
-                              const int64_t* __restrict__ node_off, uint32_t* __restrict__ mnode) {
-  const int64_t p = mb + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+// U, V of the member at position p, relative to its node's first member r (the smallest id).
+__device__ __forceinline__ void member_uv(int64_t p, int64_t i, int64_t r, const float* __restrict__ pos,
+                                          const float* __restrict__ vel, float L, float4* __restrict__ U,
+                                          float4* __restrict__ V) {
+  const float hL = 0.5f * L;
+  U[p] = make_float4(rsd::wrap_diff(pos[3 * r], pos[3 * i], L, hL),
+                     rsd::wrap_diff(pos[3 * r + 1], pos[3 * i + 1], L, hL),
+                     rsd::wrap_diff(pos[3 * r + 2], pos[3 * i + 2], L, hL), 0.f);
+  V[p] = make_float4(vel[3 * i], vel[3 * i + 1], vel[3 * i + 2], 0.f);
+}
+
+// Start of a level, one thread a member: its node, U and V; itself as its root, no neighbour yet, no
+// component member counted. The thread of a node's first member also writes the node's reference
+// position and smallest id (members ascend by id). One launch: on a level of a few thousand members a
+// launch takes longer than the whole pass.
+__global__ void k_level_members(int64_t mb, int64_t me, int64_t nb, int64_t nn,
+                                const uint32_t* __restrict__ mem, const int64_t* __restrict__ node_off,
+                                const int64_t* __restrict__ ids, const float* __restrict__ pos,
+                                const float* __restrict__ vel, float L, uint32_t* __restrict__ mnode,
+                                float4* __restrict__ U, float4* __restrict__ V, float4* __restrict__ ref,
+                                int64_t* __restrict__ node_minid, uint32_t* __restrict__ uf,
+                                float* __restrict__ nn2, uint32_t* __restrict__ cnt,
+                                unsigned long long* __restrict__ stat) {
+  const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x, p = mb + k;
+  if (k < 2) stat[k] = 0;
   if (p >= me) return;
-  mnode[p] = uint32_t(nb + rsd::upper_bound_i64(node_off + nb, nn, p) - 1);
+  const int64_t q = nb + rsd::upper_bound_i64(node_off + nb, nn, p) - 1, first = node_off[q];
+  const int64_t i = mem[p], r = mem[first];
+  mnode[p] = uint32_t(q);
+  member_uv(p, i, r, pos, vel, L, U, V);
+  uf[k] = uint32_t(k);
+  nn2[k] = __int_as_float(0x7f800000);
+  cnt[k] = 0;
+  if (p == first) {
+    ref[q] = make_float4(pos[3 * r], pos[3 * r + 1], pos[3 * r + 2], 0.f);
+    node_minid[q] = ids[r];
+  }
 }
 
 __global__ void k_gather_uv(int64_t mb, int64_t me, const uint32_t* __restrict__ mem,
@@ -249,13 +272,7 @@ __global__ void k_gather_uv(int64_t mb, int64_t me, const uint32_t* __restrict__
                             float4* __restrict__ U, float4* __restrict__ V) {
   const int64_t p = mb + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (p >= me) return;
-  const int64_t i = mem[p];
-  const int64_t r = mem[node_off[mnode[p]]];
-  const float hL = 0.5f * L;
-  U[p] = make_float4(rsd::wrap_diff(pos[3 * r], pos[3 * i], L, hL),
-                     rsd::wrap_diff(pos[3 * r + 1], pos[3 * i + 1], L, hL),
-                     rsd::wrap_diff(pos[3 * r + 2], pos[3 * i + 2], L, hL), 0.f);
-  V[p] = make_float4(vel[3 * i], vel[3 * i + 1], vel[3 * i + 2], 0.f);
+  member_uv(p, mem[p], mem[node_off[mnode[p]]], pos, vel, L, U, V);
 }
 
 __global__ void k_node_ref(int64_t nb, int64_t ne, const uint32_t* __restrict__ mem,
@@ -329,17 +346,7 @@ __device__ __forceinline__ float d6(float4 ui, float4 vi, float4 uj, float4 vj, 
 // All-pairs kernels: a block per (tile of kTile6 members, chunk of kChunk6 targets) of a node, so that a
 // single large node of a small level still spreads over the GPU (one block per tile over all targets
 // took as long as the largest node has members).
-constexpr int kChunk6 = 1024;
-
-__host__ __device__ __forceinline__ int64_t pair_items(int64_t g) {
-  return ((g + kTile6 - 1) / kTile6) * ((g + kChunk6 - 1) / kChunk6);
-}
-
-__global__ void k_pair_items(int64_t nb, int64_t nn, const int64_t* __restrict__ node_size,
-                             int64_t* __restrict__ out) {
-  const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (k < nn) out[k] = pair_items(node_size[nb + k]);
-}
+constexpr int kChunk6Bits = 10, kChunk6 = 1 << kChunk6Bits;
 
 // Nearest-neighbour d6 per member (nn2 starts at +inf): the chunk's j-tiles staged in shared memory;
 // the chunks of a member combine by an atomic minimum of the float bits (distances are not negative).
@@ -515,16 +522,6 @@ k_select_l2(int64_t nb, int64_t nn, const int64_t* __restrict__ node_off, const 
   }
 }
 
-// Start of a level: every member its own root, no neighbour yet, no child counted.
-__global__ void k_level_init(int64_t m, uint32_t* __restrict__ uf, float* __restrict__ nn2,
-                             unsigned long long* __restrict__ stat) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < 2) stat[i] = 0;
-  if (i >= m) return;
-  uf[i] = uint32_t(i);
-  nn2[i] = __int_as_float(0x7f800000);
-}
-
 // Union-find over pairs with d6 <= l2: block = (node, i-tile, chunk of targets), pairs j > i. Targets
 // carry the root they had when their tile was staged: those that share the member's root already are
 // skipped, so most of the dense middle's links (dozens a member) cost no union. Roots that were equal
@@ -598,85 +595,57 @@ __global__ void k_comp_count(int64_t m, uint32_t* __restrict__ uf, uint32_t* __r
   if (valid && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(cnt + r, uint32_t(__popc(peers)));
 }
 
-// child flag at each root that forms a child (>= min and < its node's size).
+// Does the component of root r (c members) of node q go on as a child?
+__device__ __forceinline__ bool is_child(int64_t c, int min_size, int64_t g) { return c >= min_size && c < g; }
+
+// Per member: cidx = 1 at each root that forms a child, mpos = 1 for the members of children (the two
+// are scanned into child indices and member positions). A member that goes on into no child has its
+// deepest node here: node and position are written once.
 __global__ void k_child_flags(int64_t m, int64_t mb, const uint32_t* __restrict__ uf,
-                              const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ mnode,
-                              const int64_t* __restrict__ node_size, int min_size,
-                              int64_t* __restrict__ flag, int64_t* __restrict__ flag2,
+                              const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ mem,
+                              const uint32_t* __restrict__ mnode, const int64_t* __restrict__ node_size,
+                              int min_size, int64_t* __restrict__ cidx, int64_t* __restrict__ mpos,
+                              int64_t* __restrict__ deepest, uint32_t* __restrict__ deepest_pos,
                               unsigned long long* __restrict__ stat) {
   const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  int64_t f = 0, c = 0;
-  if (p < m && uf[p] == uint32_t(p)) {
-    c = cnt[p];
-    f = (c >= min_size && c < node_size[mnode[mb + p]]) ? 1 : 0;
+  int64_t c = 0;
+  bool child = false, root = false;
+  if (p < m) {
+    const uint32_t r = uf[p], q = mnode[mb + p];
+    c = cnt[r];
+    child = is_child(c, min_size, node_size[q]);
+    root = child && r == uint32_t(p);
+    cidx[p] = root ? 1 : 0;
+    mpos[p] = child ? 1 : 0;
+    if (!child) {
+      const uint32_t i = mem[mb + p];
+      deepest[i] = q;
+      deepest_pos[i] = uint32_t(mb + p);
+    }
   }
-  level_stat(stat, f != 0, c);
-  if (p >= m) return;
-  flag[p] = f;
-  flag2[p] = f;  // the copy that is scanned into child indices
+  level_stat(stat, root, c);
 }
 
-// member flag: 1 if the member's root is a child root.
-__global__ void k_member_flags(int64_t m, const uint32_t* __restrict__ uf, const int64_t* __restrict__ cflag,
-                               int64_t* __restrict__ mflag) {
+// (child index, particle index) of the children's members in compacted order, and the children's node
+// table entries (global node index ne + child index) from their roots.
+__global__ void k_children(int64_t m, int64_t mb, int64_t ne, const uint32_t* __restrict__ uf,
+                           const uint32_t* __restrict__ cnt, const int64_t* __restrict__ cidx,
+                           const int64_t* __restrict__ mpos, const uint32_t* __restrict__ mem,
+                           const uint32_t* __restrict__ mnode, int min_size, uint64_t* __restrict__ keys,
+                           uint32_t* __restrict__ vals, int64_t* node_size,
+                           int64_t* __restrict__ node_parent, int32_t* node_level) {
   const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (p >= m) return;
-  mflag[p] = cflag[uf[p]];
-}
-
-// Scatter (child index, particle index) of child members into compacted order.
-__global__ void k_child_members(int64_t m, int64_t mb, const uint32_t* __restrict__ uf,
-                                const int64_t* __restrict__ cidx, const int64_t* __restrict__ cflag,
-                                const int64_t* __restrict__ mpos, const uint32_t* __restrict__ mem,
-                                uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-  const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (p >= m) return;
-  const uint32_t r = uf[p];
-  if (!cflag[r]) return;
-  keys[mpos[p]] = uint64_t(cidx[r]);
-  vals[mpos[p]] = mem[mb + p];
-}
-
-// Child node table entries (global node index ne + child index).
-__global__ void k_child_nodes(int64_t m, int64_t mb, int64_t ne, const uint32_t* __restrict__ uf,
-                              const uint32_t* __restrict__ cnt, const int64_t* __restrict__ cflag,
-                              const int64_t* __restrict__ cidx, const uint32_t* __restrict__ mnode,
-                              const uint32_t* __restrict__ mem, const int64_t* __restrict__ ids,
-                              int64_t* __restrict__ node_size, int64_t* __restrict__ node_parent,
-                              int32_t* node_level, int64_t* __restrict__ node_minid) {
-  const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (p >= m || uf[p] != uint32_t(p) || !cflag[p]) return;
-  const int64_t q = ne + cidx[p];
-  const uint32_t par = mnode[mb + p];
-  node_size[q] = cnt[p];
-  node_parent[q] = par;
-  node_level[q] = node_level[par] + 1;
-  node_minid[q] = ids[mem[mb + p]];
-}
-
-__global__ void k_copy_u32(int64_t n, const uint32_t* __restrict__ src, uint32_t* __restrict__ dst) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = src[i];
-}
-
-__global__ void k_offsets_add(int64_t n, const int64_t* __restrict__ src, int64_t add,
-                              int64_t* __restrict__ dst) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = src[i] + add;
-}
-
-// Deepest node per particle and the particle's member position in that node.
-// Deepest node per particle and the particle's member position in that node, written once:
-// at the level where the member does not go on into a child (its root is not a child root).
-__global__ void k_deepest(int64_t mb, int64_t me, const uint32_t* __restrict__ mem,
-                          const uint32_t* __restrict__ mnode, const uint32_t* __restrict__ uf,
-                          const int64_t* __restrict__ cflag, int64_t* __restrict__ deepest,
-                          uint32_t* __restrict__ deepest_pos) {
-  const int64_t p = mb + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (p < me && !cflag[uf[p - mb]]) {
-    deepest[mem[p]] = mnode[p];
-    deepest_pos[mem[p]] = uint32_t(p);
-  }
+  const uint32_t r = uf[p], q = mnode[mb + p];
+  const int64_t c = cnt[r];
+  if (!is_child(c, min_size, node_size[q])) return;
+  const int64_t ci = cidx[r], at = mpos[p];
+  keys[at] = uint64_t(ci);
+  vals[at] = mem[mb + p];
+  if (r != uint32_t(p)) return;
+  node_size[ne + ci] = c;
+  node_parent[ne + ci] = q;
+  node_level[ne + ci] = node_level[q] + 1;
 }
 
 // Grow a persistent hierarchy buffer, keeping its first `used` bytes.
@@ -807,17 +776,15 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
   if (n == 0) {
     RS_TRY(ensure_nodes(ctx, 0, 1, st));
     RS_TRY(ensure_members(ctx, 0, 1, st));
-    k_fill_i64<<<1, 1, 0, st>>>(1, hier_of(ctx).node_off, 0);
-    RS_LAUNCHED(ctx, "k_fill_i64");
   } else {
-    k_fill_i64<<<grid_for(n, kT), kT, 0, st>>>(n, deep, -1);
-    RS_LAUNCHED(ctx, "k_fill_i64");
     if (!deep_pos) return RS_ERR_OOM;
     unsigned long long* mx = scratch_t<unsigned long long>(ctx, S_COUNTER, 16);
     if (!mx) return RS_ERR_OOM;
-    unsigned long long* stat = mx + 4;  // sum of g^2 and largest node of the level being built
-    RS_CUDA(ctx, cudaMemsetAsync(mx, 0, 48, st));
-    k_max_id<<<std::min(grid_for(n, kT), 152u * 8u), kT, 0, st>>>(n, ids, fof_label, mx);
+    // sum of g^2 and largest node of the level being built, then its nodes and members
+    unsigned long long* stat = mx + 4;
+    int64_t* totals = reinterpret_cast<int64_t*>(stat + 2);
+    RS_CUDA(ctx, cudaMemsetAsync(mx, 0, 128, st));
+    k_max_id<<<std::min(grid_for(n, kT), 152u * 8u), kT, 0, st>>>(n, ids, fof_label, mx, deep);
     RS_LAUNCHED(ctx, "k_max_id");
     RS_TRY(read_back(ctx, mx, 16, st));
     const uint64_t max_id = uint64_t(ctx->host_box[0]), max_lab = uint64_t(ctx->host_box[1]);
@@ -837,16 +804,12 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       RS_LAUNCHED(ctx, "k_label_count");
       k_label_keep<<<grid_for(nl, kT), kT, 0, st>>>(nl, cntl, min_size, knode, koff, stat);
       RS_LAUNCHED(ctx, "k_label_keep");
-      RS_TRY(exclusive_scan_i64(ctx, nl, knode, knode + nl, st));
-      RS_TRY(exclusive_scan_i64(ctx, nl, koff, koff + nl, st));
-      RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box, knode + nl, 8, cudaMemcpyDeviceToHost, st));
-      RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 1, koff + nl, 8, cudaMemcpyDeviceToHost, st));
-      RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 2, stat, 16, cudaMemcpyDeviceToHost, st));
-      RS_CUDA(ctx, cudaStreamSynchronize(st));
-      nodes = ctx->host_box[0];
-      members = ctx->host_box[1];
-      level_pairs = uint64_t(ctx->host_box[2]);
-      level_max = ctx->host_box[3];
+      RS_TRY(exclusive_scans(ctx, nl, ScanJobs{{{knode, knode, totals}, {koff, koff, totals + 1}}}, st));
+      RS_TRY(read_back(ctx, stat, 32, st));
+      level_pairs = uint64_t(ctx->host_box[0]);
+      level_max = ctx->host_box[1];
+      nodes = ctx->host_box[2];
+      members = ctx->host_box[3];
       RS_TRY(ensure_nodes(ctx, 0, std::max<int64_t>(nodes, 1) * 2, st));
       RS_TRY(ensure_members(ctx, 0, std::max<int64_t>(members, 1) * 2, st));
       Hier h = hier_of(ctx);
@@ -856,21 +819,17 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
         uint32_t* va = scratch_t<uint32_t>(ctx, S_VAL_A, size_t(members));
         uint32_t* vb = scratch_t<uint32_t>(ctx, S_VAL_B, size_t(members));
         if (!ka || !kb || !va || !vb) return RS_ERR_OOM;
-        k_label_nodes<<<grid_for(nl, kT), kT, 0, st>>>(nl, cntl, min_size, knode, koff, h.node_off,
+        k_label_nodes<<<grid_for(nl, kT), kT, 0, st>>>(nl, nodes, members, cntl, min_size, knode, koff, h.node_off,
                                                       h.node_size, h.node_parent, h.node_level);
         RS_LAUNCHED(ctx, "k_label_nodes");
-        RS_CUDA(ctx, cudaMemsetAsync(mx, 0, 8, st));
+        const int bits = bits_for(uint64_t(std::max<int64_t>(nodes - 1, 1))) + bid;
+        (sort_ends_in_b(members, bits) ? vb : va) = h.mem;
         k_label_keys<<<grid_for(n, kT), kT, 0, st>>>(n, ids, fof_label, cntl, min_size, knode, bid,
-                                                    mx, ka, va);
+                                                    mx + 8, ka, va);
         RS_LAUNCHED(ctx, "k_label_keys");
         uint64_t* keys;
         uint32_t* vals;
-        RS_TRY(radix_sort_u64(ctx, members, bits_for(uint64_t(std::max<int64_t>(nodes - 1, 1))) + bid,
-                              ka, va, kb, vb, &keys, &vals, st));
-        k_copy_u32<<<grid_for(members, kT), kT, 0, st>>>(members, vals, h.mem);
-        RS_LAUNCHED(ctx, "k_copy_u32");
-        k_level0_minid<<<grid_for(nodes, kT), kT, 0, st>>>(nodes, h.node_off, h.mem, ids, h.node_minid);
-        RS_LAUNCHED(ctx, "k_level0_minid");
+        RS_TRY(radix_sort_u64(ctx, members, bits, ka, va, kb, vb, &keys, &vals, st));  // vals == h.mem
       }
     } else {
       uint64_t* ka = scratch_t<uint64_t>(ctx, S_KEY_A, n);
@@ -906,35 +865,30 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       RS_LAUNCHED(ctx, "k_run_starts");
       k_run_keep<<<grid_for(nruns, kT), kT, 0, st>>>(nruns, n, run_start, min_size, keep, rsize, stat);
       RS_LAUNCHED(ctx, "k_run_keep");
-      RS_CUDA(ctx, cudaMemcpyAsync(node_of_run, keep, sizeof(int64_t) * nruns,
-                                   cudaMemcpyDeviceToDevice, st));
-      RS_TRY(exclusive_scan_i64(ctx, nruns, node_of_run, node_of_run + nruns, st));
       k_size_mask<<<grid_for(nruns, kT), kT, 0, st>>>(nruns, keep, rsize, mem_off);
       RS_LAUNCHED(ctx, "k_size_mask");
-      RS_TRY(exclusive_scan_i64(ctx, nruns, mem_off, mem_off + nruns, st));
-      RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box, node_of_run + nruns, 8, cudaMemcpyDeviceToHost, st));
-      RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 1, mem_off + nruns, 8, cudaMemcpyDeviceToHost, st));
-      RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 2, stat, 16, cudaMemcpyDeviceToHost, st));
-      RS_CUDA(ctx, cudaStreamSynchronize(st));
-      nodes = ctx->host_box[0];
-      members = ctx->host_box[1];
-      level_pairs = uint64_t(ctx->host_box[2]);
-      level_max = ctx->host_box[3];
+      RS_TRY(exclusive_scans(ctx, nruns, ScanJobs{{{keep, node_of_run, totals}, {mem_off, mem_off, totals + 1}}}, st));
+      RS_TRY(read_back(ctx, stat, 32, st));
+      level_pairs = uint64_t(ctx->host_box[0]);
+      level_max = ctx->host_box[1];
+      nodes = ctx->host_box[2];
+      members = ctx->host_box[3];
       RS_TRY(ensure_nodes(ctx, 0, std::max<int64_t>(nodes, 1) * 2, st));
       RS_TRY(ensure_members(ctx, 0, std::max<int64_t>(members, 1) * 2, st));
       Hier h = hier_of(ctx);
       if (nruns > 0) {
-        k_level0_nodes<<<grid_for(nruns, kT), kT, 0, st>>>(nruns, run_start, rsize, keep, node_of_run,
-                                                         mem_off, vals, ids, h.node_off, h.node_size,
-                                                         h.node_parent, h.node_level, h.node_minid);
+        k_level0_nodes<<<grid_for(nruns, kT), kT, 0, st>>>(nruns, nodes, members, rsize, keep, node_of_run,
+                                                         mem_off, h.node_off, h.node_size, h.node_parent,
+                                                         h.node_level);
         RS_LAUNCHED(ctx, "k_level0_nodes");
         k_level0_members<<<grid_for(n, kT), kT, 0, st>>>(n, keys, b, head, run_start, keep, mem_off,
                                                          vals, h.mem);
         RS_LAUNCHED(ctx, "k_level0_members");
       }
     }
-    Hier h = hier_of(ctx);
-    k_fill_i64<<<1, 1, 0, st>>>(1, h.node_off + nodes, members);
+  }
+  if (members == 0) {
+    k_fill_i64<<<1, 1, 0, st>>>(hier_of(ctx).node_off, 0);
     RS_LAUNCHED(ctx, "k_fill_i64");
   }
   // ---------------- levels
@@ -944,33 +898,33 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
   while (ne > nb) {
     const int64_t nn = ne - nb, m = me - mb;
     Hier h = hier_of(ctx);
-    k_member_node<<<grid_for(m, kT), kT, 0, st>>>(mb, me, nb, nn, h.node_off, h.mnode);
-    RS_LAUNCHED(ctx, "k_member_node");
-    RS_TRY(gather_members(ctx, mb, me, nb, ne, pos, vel, st));
     double* sums = scratch_t<double>(ctx, S_NODE_TMP, size_t(nn) * 12);
-    if (!sums) return RS_ERR_OOM;
-    RS_TRY((cro_segmented<12, MomentTerm>(ctx, nn, h.node_off + nb, h.node_size + nb, m,
-                                          MomentTerm{h.U, h.V}, sums, st)));
-    k_node_inv<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.node_size, sums, h.inv, h.mom);
-    RS_LAUNCHED(ctx, "k_node_inv");
     int64_t* item_off = scratch_t<int64_t>(ctx, S_SELECT, size_t(nn) + 1);
     float* nn2 = scratch_t<float>(ctx, S_NN2, size_t(m));
     uint32_t* uf = scratch_t<uint32_t>(ctx, S_UF, size_t(m));
     uint32_t* cnt = scratch_t<uint32_t>(ctx, S_ROOT_CNT, size_t(m));
-    int64_t* cflag = scratch_t<int64_t>(ctx, S_FLAGS, size_t(m) + 1);
-    int64_t* cidx = scratch_t<int64_t>(ctx, S_CHILD_IDX, size_t(m) + 1);
-    int64_t* mpos = scratch_t<int64_t>(ctx, S_GKEY_A, size_t(m) + 1);
+    int64_t* cidx = scratch_t<int64_t>(ctx, S_CHILD_IDX, size_t(m));
+    int64_t* mpos = scratch_t<int64_t>(ctx, S_GKEY_A, size_t(m));
+    // of the children: sum of g^2, largest g, number, members
     unsigned long long* stat = scratch_t<unsigned long long>(ctx, S_COUNTER, 16);
-    if (!item_off || !nn2 || !uf || !cnt || !cflag || !cidx || !mpos || !stat) return RS_ERR_OOM;
+    if (!sums || !item_off || !nn2 || !uf || !cnt || !cidx || !mpos || !stat) return RS_ERR_OOM;
     stat += 4;
+    int64_t* totals = reinterpret_cast<int64_t*>(stat + 2);
+    k_level_members<<<grid_for(m, kT), kT, 0, st>>>(mb, me, nb, nn, h.mem, h.node_off, ids, pos, vel, L, h.mnode,
+                                                   h.U, h.V, h.ref, h.node_minid, uf, nn2, cnt, stat);
+    RS_LAUNCHED(ctx, "k_level_members");
     // batched form: pruned searches, except on levels of few pairs (unless a smallest node for the
     // bounded searches was asked for and the level has one)
     const bool batched = ctx->cfg.batched != 0 && (level_pairs > kPrunedMinPairs ||
                                                    (ctx->nn_bound_min > 0 && level_max >= ctx->nn_bound_min));
-    // at most (g / 128 + 1) (g / 1024 + 1) items a node
+    // all pairs: ceil(g / kTile6) ceil(g / kChunk6) items a node, at most (g / 128 + 1) (g / 1024 + 1)
+    const ScanJob items = batched ? ScanJob{}
+                                  : ScanJob{h.node_size + nb, item_off, item_off + nn, kTile6Bits, kChunk6Bits, 0};
     const int64_t items_ub = int64_t(level_pairs / (uint64_t(kTile6) * kChunk6)) + m / kTile6 + m / kChunk6 + nn + 1;
-    k_level_init<<<grid_for(m, kT), kT, 0, st>>>(m, uf, nn2, stat);
-    RS_LAUNCHED(ctx, "k_level_init");
+    RS_TRY((cro_segmented<12, MomentTerm>(ctx, nn, h.node_off + nb, h.node_size + nb, m,
+                                          MomentTerm{h.U, h.V}, sums, st, items)));
+    k_node_inv<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.node_size, sums, h.inv, h.mom);
+    RS_LAUNCHED(ctx, "k_node_inv");
     // k-th smallest nn2 of the level's nodes (of those with only[k] != 0 when `only` is given); the
     // batched form's nn2 is in its sorted order, in which every node keeps its range
     auto select = [&](const int* only) -> int {
@@ -979,7 +933,7 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       k_select_l2_warp<<<grid_for(nn, kT / 32), kT, 0, st>>>(nb, nn, hs.node_off, hs.node_size, nn2, mb, f_num,
                                                             f_den, hs.inv, only);
       RS_LAUNCHED(ctx, "k_select_l2_warp");
-      if (m > kSelectWarpMax) {  // a larger node is possible
+      if (level_max > kSelectWarpMax) {
         k_select_l2<<<unsigned(std::min<int64_t>(nn, 152 * 2)), kSelThreads, 0, st>>>(
             nb, nn, hs.node_off, hs.node_size, nn2, mb, f_num, f_den, hs.inv, only);
         RS_LAUNCHED(ctx, "k_select_l2");
@@ -993,9 +947,6 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       RS_TRY(prune6d_far(ctx, nb, nn, mb, m, nn2, st));
       h = hier_of(ctx);
     } else {
-      k_pair_items<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.node_size, item_off);
-      RS_LAUNCHED(ctx, "k_pair_items");
-      RS_TRY(exclusive_scan_i64(ctx, nn, item_off, item_off + nn, st));
       {
         ProfScope prof_(ctx, "k_nn6d", st);
         k_nn6d<<<grid_for(items_ub, 1), kTile6, 0, st>>>(nb, nn, item_off, h.node_off, h.node_size, h.inv,
@@ -1020,24 +971,16 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       }
       RS_LAUNCHED(ctx, "k_link6d");
     }
-    RS_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * m, st));
     k_comp_count<<<grid_for(m, kT), kT, 0, st>>>(m, uf, cnt);
     RS_LAUNCHED(ctx, "k_comp_count");
-    k_child_flags<<<grid_for(m, kT), kT, 0, st>>>(m, mb, uf, cnt, h.mnode, h.node_size, min_size, cflag, cidx, stat);
+    k_child_flags<<<grid_for(m, kT), kT, 0, st>>>(m, mb, uf, cnt, h.mem, h.mnode, h.node_size, min_size, cidx,
+                                                 mpos, deep, deep_pos, stat);
     RS_LAUNCHED(ctx, "k_child_flags");
-    RS_TRY(exclusive_scan_i64(ctx, m, cidx, cidx + m, st));
-    k_member_flags<<<grid_for(m, kT), kT, 0, st>>>(m, uf, cflag, mpos);
-    RS_LAUNCHED(ctx, "k_member_flags");
-    RS_TRY(exclusive_scan_i64(ctx, m, mpos, mpos + m, st));
-    k_deepest<<<grid_for(m, kT), kT, 0, st>>>(mb, me, h.mem, h.mnode, uf, cflag, deep, deep_pos);
-    RS_LAUNCHED(ctx, "k_deepest");
-    RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box, cidx + m, 8, cudaMemcpyDeviceToHost, st));
-    RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 1, mpos + m, 8, cudaMemcpyDeviceToHost, st));
-    RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 2, stat, 16, cudaMemcpyDeviceToHost, st));
-    RS_CUDA(ctx, cudaStreamSynchronize(st));
-    level_pairs = uint64_t(ctx->host_box[2]);
-    level_max = ctx->host_box[3];
-    const int64_t nchild = ctx->host_box[0], mchild = ctx->host_box[1];
+    RS_TRY(exclusive_scans(ctx, m, ScanJobs{{{cidx, cidx, totals}, {mpos, mpos, totals + 1}}}, st));
+    RS_TRY(read_back(ctx, stat, 32, st));
+    level_pairs = uint64_t(ctx->host_box[0]);
+    level_max = ctx->host_box[1];
+    const int64_t nchild = ctx->host_box[2], mchild = ctx->host_box[3];
     ++levels;
     if (nchild == 0) {
       nb = ne;
@@ -1050,24 +993,17 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
     uint64_t* kb = scratch_t<uint64_t>(ctx, S_KEY_B, size_t(mchild));
     uint32_t* va = scratch_t<uint32_t>(ctx, S_VAL_A, size_t(mchild));
     uint32_t* vb = scratch_t<uint32_t>(ctx, S_VAL_B, size_t(mchild));
-    int64_t* csize = scratch_t<int64_t>(ctx, S_GVAL_A, size_t(nchild) + 1);
-    if (!ka || !kb || !va || !vb || !csize) return RS_ERR_OOM;
-    k_child_members<<<grid_for(m, kT), kT, 0, st>>>(m, mb, uf, cidx, cflag, mpos, h.mem, ka, va);
-    RS_LAUNCHED(ctx, "k_child_members");
+    if (!ka || !kb || !va || !vb) return RS_ERR_OOM;
+    const int bits = bits_for(uint64_t(nchild));
+    (sort_ends_in_b(mchild, bits) ? vb : va) = h.mem + me;  // the sorted members are the level's list
+    k_children<<<grid_for(m, kT), kT, 0, st>>>(m, mb, ne, uf, cnt, cidx, mpos, h.mem, h.mnode, min_size, ka, va,
+                                              h.node_size, h.node_parent, h.node_level);
+    RS_LAUNCHED(ctx, "k_children");
     uint64_t* skeys;
     uint32_t* svals;
-    RS_TRY(radix_sort_u64(ctx, mchild, bits_for(uint64_t(nchild)), ka, va, kb, vb, &skeys, &svals, st));
-    k_copy_u32<<<grid_for(mchild, kT), kT, 0, st>>>(mchild, svals, h.mem + me);
-    RS_LAUNCHED(ctx, "k_copy_u32");
-    k_child_nodes<<<grid_for(m, kT), kT, 0, st>>>(m, mb, ne, uf, cnt, cflag, cidx, h.mnode, h.mem, ids,
-                                                 h.node_size, h.node_parent, h.node_level,
-                                                 h.node_minid);
-    RS_LAUNCHED(ctx, "k_child_nodes");
-    RS_CUDA(ctx, cudaMemcpyAsync(csize, h.node_size + ne, sizeof(int64_t) * nchild,
-                                 cudaMemcpyDeviceToDevice, st));
-    RS_TRY(exclusive_scan_i64(ctx, nchild, csize, csize + nchild, st));
-    k_offsets_add<<<grid_for(nchild + 1, kT), kT, 0, st>>>(nchild + 1, csize, me, h.node_off + ne);
-    RS_LAUNCHED(ctx, "k_offsets_add");
+    RS_TRY(radix_sort_u64(ctx, mchild, bits, ka, va, kb, vb, &skeys, &svals, st));  // svals == h.mem + me
+    RS_TRY(exclusive_scans(ctx, nchild, ScanJobs{{{h.node_size + ne, h.node_off + ne, h.node_off + ne + nchild,
+                                                   0, 0, me}}}, st));
     nb = ne;
     ne += nchild;
     mb = me;

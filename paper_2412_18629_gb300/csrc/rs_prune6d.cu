@@ -964,8 +964,7 @@ int build_buckets(rs_ctx* ctx, int64_t nb, int64_t nn, int64_t m, const int64_t*
   if (!boff || !sboff || !bk || !box || !sbox || !qk || !qk2 || !qv || !qv2 || !qorder) return RS_ERR_OOM;
   k_bucket_counts<<<grid_for(nn, kT), kT, 0, st>>>(nn, cnt, boff, sboff);
   RS_LAUNCHED(ctx, "k_bucket_counts");
-  RS_TRY(exclusive_scan_i64(ctx, nn, boff, boff + nn, st));
-  RS_TRY(exclusive_scan_i64(ctx, nn, sboff, sboff + nn, st));
+  RS_TRY(exclusive_scans(ctx, nn, ScanJobs{{{boff, boff, boff + nn}, {sboff, sboff, sboff + nn}}}, st));
   k_buckets<<<grid_for(nbk_ub * 32, kT), kT, 0, st>>>(nb, nn, nbk_ub, boff, sboff, start, cnt, XY, Z, bk, box, qk,
                                                      qv);
   RS_LAUNCHED(ctx, "k_buckets");

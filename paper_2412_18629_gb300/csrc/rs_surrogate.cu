@@ -697,8 +697,7 @@ static int sur_prepare(rs_ctx* ctx, const double* vbulk, int64_t* ns_out, cudaSt
   if (!sur_off || !rank || !stt) return RS_ERR_OOM;
   k_sur_node_flags<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_size, sur_off, rank);
   RS_LAUNCHED(ctx, "k_sur_node_flags");
-  RS_TRY(exclusive_scan_i64(ctx, nn, sur_off, sur_off + nn, st));
-  RS_TRY(exclusive_scan_i64(ctx, nn, rank, rank + nn, st));
+  RS_TRY(exclusive_scans(ctx, nn, ScanJobs{{{sur_off, sur_off, sur_off + nn}, {rank, rank, rank + nn}}}, st));
   RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box, sur_off + nn, 8, cudaMemcpyDeviceToHost, st));
   RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 1, rank + nn, 8, cudaMemcpyDeviceToHost, st));
   RS_CUDA(ctx, cudaStreamSynchronize(st));

@@ -782,9 +782,8 @@ int rs::tree_build(rs_ctx* ctx, cudaStream_t st) {
   if (!tsz || !trank || !tcells) return RS_ERR_OOM;
   k_tree_sel<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_size, tmin, tsz, trank, tcells);
   RS_LAUNCHED(ctx, "k_tree_sel");
-  RS_TRY(exclusive_scan_i64(ctx, nn, tsz, tsz + nn, st));
-  RS_TRY(exclusive_scan_i64(ctx, nn, trank, trank + nn, st));
-  RS_TRY(exclusive_scan_i64(ctx, nn, tcells, tcells + nn, st));
+  RS_TRY(exclusive_scans(ctx, nn, ScanJobs{{{tsz, tsz, tsz + nn}, {trank, trank, trank + nn},
+                                            {tcells, tcells, tcells + nn}}}, st));
   RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box, tsz + nn, 8, cudaMemcpyDeviceToHost, st));
   RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 1, trank + nn, 8, cudaMemcpyDeviceToHost, st));
   RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 2, tcells + nn, 8, cudaMemcpyDeviceToHost, st));

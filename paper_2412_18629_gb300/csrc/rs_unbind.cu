@@ -604,8 +604,8 @@ int potential_tiles(rs_ctx* ctx, int64_t sur_min, const int* only, int64_t max_g
   RS_TRY(radix_sort_u64(ctx, nn, 8, ka, va, kb, vb, &ko, perm, st));
   k_perm_tiles<<<grid_for(nn, kT), kT, 0, st>>>(nn, *perm, tile_big, tile_perm);
   RS_LAUNCHED(ctx, "k_perm_tiles");
-  RS_TRY(exclusive_scan_i64(ctx, nn, tile_small, tile_small + nn, st));
-  RS_TRY(exclusive_scan_i64(ctx, nn, tile_perm, tile_perm + nn, st));
+  RS_TRY(exclusive_scans(ctx, nn, ScanJobs{{{tile_small, tile_small, tile_small + nn},
+                                            {tile_perm, tile_perm, tile_perm + nn}}}, st));
   return RS_OK;
 }
 
