@@ -33,29 +33,24 @@ __global__ void k_seed_kids(int64_t nn, const int64_t* __restrict__ parent, int*
   if (q < nn && parent[q] >= 0) atomicAdd(nkids + parent[q], 1);
 }
 
-__global__ void k_seed_total(int64_t nn, const int* __restrict__ nkids, unsigned long long* __restrict__ n_seeds) {
+// Per node the walk up its parents (as many steps as its level): its level-0 ancestor, and for a seed a
+// count at each node of the walk and at itself. Also the segments of the seeds for the canonical-order
+// sums (size 0 otherwise) and the number of seeds. The walk replaced seven pointer-jumping launches.
+__global__ void k_seed_roots(int64_t nn, const int64_t* __restrict__ parent, const int* __restrict__ nkids,
+                             const int64_t* __restrict__ node_size, int64_t* __restrict__ root,
+                             unsigned long long* __restrict__ cnt, int64_t* __restrict__ seg_size,
+                             unsigned long long* __restrict__ n_seeds) {
   const int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  rsd::warp_count(n_seeds, q < nn && nkids[q] == 0);
-}
-
-// Pointer jumping towards the level-0 ancestor: out[q] = in[in[q]] (level-0 nodes point at
-// themselves).
-__global__ void k_seed_jump(int64_t nn, const int64_t* __restrict__ in, int64_t* __restrict__ out) {
-  const int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (q < nn) out[q] = in[in[q]];
-}
-
-__global__ void k_seed_root_init(int64_t nn, const int64_t* __restrict__ parent, int64_t* __restrict__ r) {
-  const int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (q < nn) r[q] = parent[q] < 0 ? q : parent[q];
-}
-
-// Per seed: add 1 to every ancestor's (and its own) count of seeds under it.
-__global__ void k_seed_under_count(int64_t nn, const int64_t* __restrict__ parent, const int* __restrict__ nkids,
-                                   unsigned long long* __restrict__ cnt) {
-  const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (s >= nn || nkids[s] != 0) return;
-  for (int64_t q = s; q >= 0; q = parent[q]) atomicAdd(cnt + q, 1ull);
+  const bool seed = q < nn && nkids[q] == 0;
+  rsd::warp_count(n_seeds, seed);
+  if (q >= nn) return;
+  seg_size[q] = seed ? node_size[q] : 0;
+  int64_t r = q;
+  for (int64_t p = q; p >= 0; p = parent[p]) {
+    r = p;
+    if (seed) atomicAdd(cnt + p, 1ull);
+  }
+  root[q] = r;
 }
 
 __global__ void k_seed_under_fill(int64_t nn, const int64_t* __restrict__ parent, const int* __restrict__ nkids,
@@ -64,13 +59,6 @@ __global__ void k_seed_under_fill(int64_t nn, const int64_t* __restrict__ parent
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (s >= nn || nkids[s] != 0) return;
   for (int64_t q = s; q >= 0; q = parent[q]) list[off[q] + int64_t(atomicAdd(fill + q, 1ull))] = s;
-}
-
-// Segments of the seeds for the canonical-order sums (node offset and size; size 0 otherwise).
-__global__ void k_seed_segments(int64_t nn, const int* __restrict__ nkids, const int64_t* __restrict__ node_size,
-                                int64_t* __restrict__ seg_size) {
-  const int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (q < nn) seg_size[q] = nkids[q] == 0 ? node_size[q] : 0;
 }
 
 struct SeedTerm {  // u^s and v of a member of seed s
@@ -131,14 +119,9 @@ __global__ void k_seed_assign(int64_t n, const int64_t* __restrict__ deepest, co
                               const float4* __restrict__ bulk, const float4* __restrict__ inv,
                               int64_t* __restrict__ seed, unsigned long long* __restrict__ count) {
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int64_t dq = deepest[i];
-  if (dq < 0) {
-    seed[i] = -1;
-    return;
-  }
+  const int64_t dq = i < n ? deepest[i] : -1;
   int64_t arg = dq;
-  if (nkids[dq] != 0) {
+  if (dq >= 0 && nkids[dq] != 0) {
     const int64_t r0 = mem[node_off[root[dq]]];
     const float hL = 0.5f * L;
     const float ux = rsd::wrap_diff(pos[3 * r0], pos[3 * i], L, hL);
@@ -157,8 +140,10 @@ __global__ void k_seed_assign(int64_t n, const int64_t* __restrict__ deepest, co
       }
     }
   }
-  seed[i] = arg;
-  atomicAdd(count + arg, 1ull);
+  if (i < n) seed[i] = arg;
+  // one addition per seed and warp
+  const unsigned peers = __match_any_sync(0xffffffffu, arg);
+  if (arg >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(count + arg, (unsigned long long)__popc(peers));
 }
 
 // One thread per seed: its host among the seeds of its level-0 node ranking above it.
@@ -220,46 +205,35 @@ extern "C" int rs_assign_seeds(rs_ctx* ctx, const float* pos, const float* vel, 
   }
   Hier h = hier_of(ctx);
   int* nkids = scratch_t<int>(ctx, S_SEED_KIDS, size_t(nn));
-  int64_t* ra = scratch_t<int64_t>(ctx, S_SEED_ROOT, 2 * size_t(nn));
+  int64_t* root = scratch_t<int64_t>(ctx, S_SEED_ROOT, size_t(nn));
   unsigned long long* ucnt = scratch_t<unsigned long long>(ctx, S_SEED_UCNT, 2 * size_t(nn) + 2);
   int64_t* uoff = scratch_t<int64_t>(ctx, S_SEED_UOFF, size_t(nn) + 1);
   float4* cen = scratch_t<float4>(ctx, S_SEED_CEN, 2 * size_t(nn));
   double* sums = scratch_t<double>(ctx, S_SEED_SUMS, 6 * size_t(nn));
   int64_t* segsz = scratch_t<int64_t>(ctx, S_SEED_SEG, size_t(nn));
   unsigned long long* count = scratch_t<unsigned long long>(ctx, S_SEED_COUNT, size_t(nn));
-  if (!nkids || !ra || !ucnt || !uoff || !cen || !sums || !segsz || !count) return RS_ERR_OOM;
+  if (!nkids || !root || !ucnt || !uoff || !cen || !sums || !segsz || !count) return RS_ERR_OOM;
   float4* bulk = cen + nn;
   unsigned long long* fill = ucnt + nn + 1;
   RS_CUDA(ctx, cudaMemsetAsync(nkids, 0, 4 * size_t(nn), st));
   k_seed_kids<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids);
   RS_LAUNCHED(ctx, "k_seed_kids");
-  // level-0 ancestor of every node: pointer jumping (2^7 > any depth of the hierarchy)
-  int64_t* rin = ra;
-  int64_t* rout = ra + nn;
-  k_seed_root_init<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, rin);
-  RS_LAUNCHED(ctx, "k_seed_root_init");
-  for (int it = 0; it < 7; ++it) {
-    k_seed_jump<<<grid_for(nn, kT), kT, 0, st>>>(nn, rin, rout);
-    RS_LAUNCHED(ctx, "k_seed_jump");
-    std::swap(rin, rout);
-  }
-  const int64_t* root = rin;
-  // the seeds under every node: counts, offsets, lists
+  // level-0 ancestor of every node and the seeds under it: counts, offsets, lists
   RS_CUDA(ctx, cudaMemsetAsync(ucnt, 0, 8 * (2 * size_t(nn) + 2), st));
-  k_seed_under_count<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids, ucnt);
-  RS_LAUNCHED(ctx, "k_seed_under_count");
+  unsigned long long* n_seeds = fill + nn;  // the spare last counter slot
+  k_seed_roots<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids, h.node_size, root, ucnt, segsz, n_seeds);
+  RS_LAUNCHED(ctx, "k_seed_roots");
   static_assert(sizeof(unsigned long long) == sizeof(int64_t), "counts scanned as int64");
-  RS_CUDA(ctx, cudaMemcpyAsync(uoff, ucnt, 8 * size_t(nn), cudaMemcpyDeviceToDevice, st));
-  RS_TRY(exclusive_scan_i64(ctx, nn, uoff, uoff + nn, st));
+  RS_TRY(exclusive_scans(ctx, nn, ScanJobs{{{reinterpret_cast<int64_t*>(ucnt), uoff, uoff + nn}}}, st));
+  RS_CUDA(ctx, cudaMemcpyAsync(ctx->host_box + 1, n_seeds, 8, cudaMemcpyDeviceToHost, st));
   RS_TRY(read_back(ctx, uoff + nn, 8, st));
+  const int64_t seeds = ctx->host_box[1];
   const int64_t total = ctx->host_box[0];
   int64_t* ulist = scratch_t<int64_t>(ctx, S_SEED_LIST, size_t(std::max<int64_t>(total, 1)));
   if (!ulist) return RS_ERR_OOM;
   k_seed_under_fill<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids, uoff, fill, ulist);
   RS_LAUNCHED(ctx, "k_seed_under_fill");
   // seed centres and bulk velocities (canonical-order sums over the seeds' members)
-  k_seed_segments<<<grid_for(nn, kT), kT, 0, st>>>(nn, nkids, h.node_size, segsz);
-  RS_LAUNCHED(ctx, "k_seed_segments");
   RS_TRY((cro_segmented<6, SeedTerm>(ctx, nn, h.node_off, segsz, m, SeedTerm{h.U, h.V}, sums, st)));
   k_seed_stats<<<grid_for(nn, kT), kT, 0, st>>>(nn, nkids, root, h.node_off, h.node_size, h.mem, pos,
                                                ctx->cfg.box_L, sums, cen, bulk);
@@ -276,12 +250,8 @@ extern "C" int rs_assign_seeds(rs_ctx* ctx, const float* pos, const float* vel, 
                                               node_host, node_count);
   RS_LAUNCHED(ctx, "k_seed_host");
   if (n_seeds_out) {
-    unsigned long long* ns = fill + nn;  // the spare last counter slot
-    RS_CUDA(ctx, cudaMemsetAsync(ns, 0, 8, st));
-    k_seed_total<<<grid_for(nn, kT), kT, 0, st>>>(nn, nkids, ns);
-    RS_LAUNCHED(ctx, "k_seed_total");
-    RS_TRY(read_back(ctx, ns, 8, st));
-    *n_seeds_out = ctx->host_box[0];
+    *n_seeds_out = seeds;
+    RS_CUDA(ctx, cudaStreamSynchronize(st));
   }
   return RS_OK;
 }
