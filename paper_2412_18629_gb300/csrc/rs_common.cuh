@@ -53,7 +53,7 @@ enum Slot : int {
   S_T_CELL, S_T_ORDER, S_T_WF, S_T_WL, S_T_WR, S_T_UF, S_T_LIST, S_T_LR, S_T_SX, S_T_REC,
   S_T_WANT, S_SUR_SD,
   // seed halos (rs_seeds.cu)
-  S_SEED_KIDS, S_SEED_ROOT, S_SEED_UCNT, S_SEED_UOFF, S_SEED_CEN, S_SEED_SUMS, S_SEED_SEG,
+  S_SEED_KIDS, S_SEED_ROOT, S_SEED_UCNT, S_SEED_UOFF, S_SEED_CEN, S_SEED_REC, S_SEED_SUMS, S_SEED_SEG,
   S_SEED_COUNT, S_SEED_LIST,
   // temporal tracking (rs_track.cu)
   S_TRK_HEAD, S_TRK_RSTART, S_TRK_RKEY, S_TRK_KA, S_TRK_KB, S_TRK_VA, S_TRK_VB, S_TRK_H1,
@@ -95,6 +95,7 @@ struct rs_ctx {
   int64_t n_particles = 0;
   int64_t n_nodes = 0;
   int64_t n_members = 0;
+  int64_t n_level0 = 0;  // members of the level-0 nodes (the first positions)
   int32_t n_levels = 0;
   bool have_unbind = false;
   bool have_mlp = false;        // surrogate weights loaded or trained

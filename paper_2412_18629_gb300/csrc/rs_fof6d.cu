@@ -307,34 +307,31 @@ struct MomentTerm {
   }
 };
 
-// Total variance ((Q0/g - m0^2) + (Q1/g - m1^2)) + (Q2/g - m2^2), m_d = S_d / g.
-__device__ __forceinline__ double total_var(const double* S, const double* Q, double g) {
-  double var = 0.0;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const double m = __ddiv_rn(S[d], g);
-    const double t = __dsub_rn(__ddiv_rn(Q[d], g), __dmul_rn(m, m));
-    var = (d == 0) ? t : __dadd_rn(var, t);
-  }
-  return var;
-}
-
 // Metric scales of the node's split, and (mean u, sigma_v,1D) in float32 for the surrogate's
-// features.
+// features. Total variance ((Q0/g - m0^2) + (Q1/g - m1^2)) + (Q2/g - m2^2), m_d = S_d / g.
+// Sixteen lanes a node, one division each: a thread of its own did the 12 divisions one after the other,
+// 9 us however few the nodes.
 __global__ void k_node_inv(int64_t nb, int64_t nn, const int64_t* __restrict__ node_size,
                            const double* __restrict__ sums, float4* __restrict__ inv,
                            float4* __restrict__ mom) {
-  const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (k >= nn) return;
-  const double g = double(node_size[nb + k]);
-  const double* S = sums + 12 * k;
-  const double vx = total_var(S, S + 3, g);
-  const double vv = total_var(S + 6, S + 9, g);
-  const float ix = vx > 0.0 ? __double2float_rn(__ddiv_rn(1.0, vx)) : 0.f;
-  const float iv = vv > 0.0 ? __double2float_rn(__ddiv_rn(1.0, vv)) : 0.f;
-  inv[nb + k] = make_float4(ix, iv, 0.f, 0.f);
-  mom[nb + k] = make_float4(float(__ddiv_rn(S[0], g)), float(__ddiv_rn(S[1], g)), float(__ddiv_rn(S[2], g)),
-                            float(sqrt(fmax(vv, 0.0) / 3.0)));
+  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x, k = t >> 4;
+  const int l = int(t & 15);
+  const bool in = k < nn && l < 12;  // every lane stays for the shuffles
+  const double g = in ? double(node_size[nb + k]) : 1.0;
+  const double x = __ddiv_rn(in ? sums[12 * k + l] : 0.0, g);  // m (0-2, 6-8) and Q / g (3-5, 9-11)
+  const double y = __shfl_down_sync(0xffffffffu, x, 3, 16);
+  const double v0 = __dsub_rn(y, __dmul_rn(x, x));
+  const double v1 = __shfl_down_sync(0xffffffffu, v0, 1, 16), v2 = __shfl_down_sync(0xffffffffu, v0, 2, 16);
+  const double var = __dadd_rn(__dadd_rn(v0, v1), v2);  // lane 0: of u, lane 6: of v
+  const bool whole = in && (l == 0 || l == 6);
+  const float scale = whole && var > 0.0 ? __double2float_rn(__ddiv_rn(1.0, var)) : 0.f;
+  const float sig = whole ? float(sqrt(fmax(var, 0.0) / 3.0)) : 0.f;
+  const float iv = __shfl_sync(0xffffffffu, scale, 6, 16), s1 = __shfl_sync(0xffffffffu, sig, 6, 16);
+  const float mx = float(x), my = __shfl_sync(0xffffffffu, mx, 1, 16), mz = __shfl_sync(0xffffffffu, mx, 2, 16);
+  if (in && l == 0) {
+    inv[nb + k] = make_float4(scale, iv, 0.f, 0.f);
+    mom[nb + k] = make_float4(mx, my, mz, s1);
+  }
 }
 
 __device__ __forceinline__ float d6(float4 ui, float4 vi, float4 uj, float4 vj, float isx, float isv) {
@@ -923,7 +920,7 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
     const int64_t items_ub = int64_t(level_pairs / (uint64_t(kTile6) * kChunk6)) + m / kTile6 + m / kChunk6 + nn + 1;
     RS_TRY((cro_segmented<12, MomentTerm>(ctx, nn, h.node_off + nb, h.node_size + nb, m,
                                           MomentTerm{h.U, h.V}, sums, st, items)));
-    k_node_inv<<<grid_for(nn, kT), kT, 0, st>>>(nb, nn, h.node_size, sums, h.inv, h.mom);
+    k_node_inv<<<grid_for(nn * 16, kT), kT, 0, st>>>(nb, nn, h.node_size, sums, h.inv, h.mom);
     RS_LAUNCHED(ctx, "k_node_inv");
     // k-th smallest nn2 of the level's nodes (of those with only[k] != 0 when `only` is given); the
     // batched form's nn2 is in its sorted order, in which every node keeps its range
@@ -1015,6 +1012,7 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
   ctx->n_particles = n;
   ctx->n_nodes = ne;
   ctx->n_members = me;
+  ctx->n_level0 = members;
   ctx->n_levels = levels;
   if (n_nodes_out) *n_nodes_out = ne;
   if (n_members_out) *n_members_out = me;

@@ -534,29 +534,40 @@ __global__ void k_prop_means(int64_t nn, const unsigned long long* __restrict__ 
   for (int d = 0; d < 3; ++d) mean[3 * q + d] = nb[q] ? __ddiv_rn(s1[12 * q + d], c) : 0.0;
 }
 
+// Sixteen lanes a node, one of its 16 divisions each (one thread for all of them took 21 us however few
+// the nodes); the first puts the record together.
 __global__ void k_prop_final(int64_t nn, const int64_t* __restrict__ node_size,
                              const unsigned long long* __restrict__ nb, const uint8_t* __restrict__ is_halo,
                              const double* __restrict__ s1, const double* __restrict__ s2,
                              const double* __restrict__ mean, const float4* __restrict__ ref,
                              float L, double m, double rho_bar, rs_halo_props_t* __restrict__ out) {
-  const int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (q >= nn) return;
+  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x, q = t >> 4;
+  const int l = int(t & 15);
+  const bool in = q < nn && nb[q] > 0;  // every lane stays for the shuffles
+  const double c = in ? double(nb[q]) : 1.0, m_bound = __dmul_rn(c, m);
+  const double pi = 3.14159265358979323846;
+  const double num = !in ? 0.0 : l < 9 ? s1[12 * q + 3 + l] : l < 15 ? s2[6 * q + l - 9] : __dmul_rn(3.0, m_bound);
+  const double den = l < 15 ? c : __dmul_rn(__dmul_rn(__dmul_rn(4.0, pi), 200.0), rho_bar);
+  const double x = __ddiv_rn(num, den);
+  double y[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) y[k] = __shfl_sync(0xffffffffu, x, k, 16);
+  if (q >= nn || l != 0) return;
   rs_halo_props_t P;
   memset(&P, 0, sizeof(P));
   P.n = node_size[q];
   P.n_bound = int64_t(nb[q]);
   P.is_halo = is_halo[q];
   P.m_bound = __dmul_rn(double(nb[q]), m);
-  if (nb[q] > 0) {
-    const double c = double(nb[q]);
-    const double* S = s1 + 12 * q;
+  if (in) {
     double varx = 0.0, varv = 0.0;
     const float rp[3] = {ref[q].x, ref[q].y, ref[q].z};
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
       const double mu = mean[3 * q + d];
-      const double mv = __ddiv_rn(S[6 + d], c);
-      const double tx = __dsub_rn(__ddiv_rn(S[3 + d], c), __dmul_rn(mu, mu));
-      const double tv = __dsub_rn(__ddiv_rn(S[9 + d], c), __dmul_rn(mv, mv));
+      const double mv = y[3 + d];
+      const double tx = __dsub_rn(y[d], __dmul_rn(mu, mu));
+      const double tv = __dsub_rn(y[6 + d], __dmul_rn(mv, mv));
       varx = (d == 0) ? tx : __dadd_rn(varx, tx);
       varv = (d == 0) ? tv : __dadd_rn(varv, tv);
       double cen = __dadd_rn(double(rp[d]), mu);
@@ -567,10 +578,9 @@ __global__ void k_prop_final(int64_t nn, const int64_t* __restrict__ node_size,
     }
     P.sigma_x = __dsqrt_rn(varx > 0.0 ? varx : 0.0);
     P.sigma_v = __dsqrt_rn(varv > 0.0 ? varv : 0.0);
-    const double pi = 3.14159265358979323846;
-    P.r_vir = cbrt(__ddiv_rn(__dmul_rn(3.0, P.m_bound),
-                             __dmul_rn(__dmul_rn(__dmul_rn(4.0, pi), 200.0), rho_bar)));
-    for (int k = 0; k < 6; ++k) P.inertia[k] = __ddiv_rn(s2[6 * q + k], c);
+    P.r_vir = cbrt(y[15]);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) P.inertia[k] = y[9 + k];
   }
   out[q] = P;
 }
@@ -954,7 +964,7 @@ extern "C" int rs_halo_props(rs_ctx* ctx, rs_halo_props_t* props_out, void* stre
                                       s2, st)));
   const double L = ctx->cfg.box_L;
   const double rho_bar = double(ctx->n_particles) * ctx->cfg.particle_mass / (L * L * L);
-  k_prop_final<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_size, nb, halo, s1, s2, mean, h.ref,
+  k_prop_final<<<grid_for(nn * 16, kT), kT, 0, st>>>(nn, h.node_size, nb, halo, s1, s2, mean, h.ref,
                                                ctx->cfg.box_L, ctx->cfg.particle_mass, rho_bar,
                                                props_out);
   RS_LAUNCHED(ctx, "k_prop_final");
