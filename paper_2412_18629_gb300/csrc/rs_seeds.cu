@@ -53,14 +53,6 @@ __global__ void k_seed_roots(int64_t nn, const int64_t* __restrict__ parent, con
   root[q] = r;
 }
 
-__global__ void k_seed_under_fill(int64_t nn, const int64_t* __restrict__ parent, const int* __restrict__ nkids,
-                                  const int64_t* __restrict__ off, unsigned long long* __restrict__ fill,
-                                  int64_t* __restrict__ list) {
-  const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (s >= nn || nkids[s] != 0) return;
-  for (int64_t q = s; q >= 0; q = parent[q]) list[off[q] + int64_t(atomicAdd(fill + q, 1ull))] = s;
-}
-
 struct SeedTerm {  // u^s and v of a member of seed s
   const float4* U;
   const float4* V;
@@ -80,12 +72,19 @@ struct SeedTerm {  // u^s and v of a member of seed s
   }
 };
 
+// A seed as the searches read it, beside the others under the same node: centre and position scale, bulk
+// velocity and velocity scale, its index. Read through a list of indices into four tables, the loads of
+// one seed waited for the index; the records of a node are one run of memory.
+struct SeedRec {
+  float4 c, w;
+};
+
 // Seed centres (level-0 frame) and bulk velocities from the canonical-order sums.
 __global__ void k_seed_stats(int64_t nn, const int* __restrict__ nkids, const int64_t* __restrict__ root,
                              const int64_t* __restrict__ node_off, const int64_t* __restrict__ node_size,
                              const uint32_t* __restrict__ mem, const float* __restrict__ pos, float L,
-                             const double* __restrict__ sums, float4* __restrict__ cen,
-                             float4* __restrict__ bulk) {
+                             const double* __restrict__ sums, const float4* __restrict__ inv,
+                             SeedRec* __restrict__ rec) {
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (s >= nn || nkids[s] != 0) return;
   const int64_t rs_ = mem[node_off[s]], r0 = mem[node_off[root[s]]];
@@ -99,48 +98,62 @@ __global__ void k_seed_stats(int64_t nn, const int* __restrict__ nkids, const in
     c[d] = __double2float_rn(__dadd_rn(double(o), __ddiv_rn(S[d], g)));
     w[d] = __double2float_rn(__ddiv_rn(S[3 + d], g));
   }
-  cen[s] = make_float4(c[0], c[1], c[2], 0.f);
-  bulk[s] = make_float4(w[0], w[1], w[2], 0.f);
+  const float4 iv = inv[s];
+  rec[s] = {make_float4(c[0], c[1], c[2], iv.x), make_float4(w[0], w[1], w[2], iv.y)};
 }
 
-__device__ __forceinline__ float seed_metric(float ax, float ay, float az, float4 c, float vx, float vy,
-                                             float vz, float4 w, float isx, float isv) {
-  const float rx = rsd::sq3(__fsub_rn(ax, c.x), __fsub_rn(ay, c.y), __fsub_rn(az, c.z));
-  const float rv = rsd::sq3(__fsub_rn(vx, w.x), __fsub_rn(vy, w.y), __fsub_rn(vz, w.z));
-  return __fadd_rn(__fmul_rn(rx, isx), __fmul_rn(rv, isv));
+__device__ __forceinline__ float seed_metric(float ax, float ay, float az, float vx, float vy, float vz,
+                                             const SeedRec& s) {
+  const float rx = rsd::sq3(__fsub_rn(ax, s.c.x), __fsub_rn(ay, s.c.y), __fsub_rn(az, s.c.z));
+  const float rv = rsd::sq3(__fsub_rn(vx, s.w.x), __fsub_rn(vy, s.w.y), __fsub_rn(vz, s.w.z));
+  return __fadd_rn(__fmul_rn(rx, s.c.w), __fmul_rn(rv, s.w.w));
 }
 
-// One thread per particle: its seed (argmin over the seeds under its deepest node).
-__global__ void k_seed_assign(int64_t n, const int64_t* __restrict__ deepest, const int* __restrict__ nkids,
-                              const int64_t* __restrict__ root, const int64_t* __restrict__ node_off,
-                              const uint32_t* __restrict__ mem, const float* __restrict__ pos,
-                              const float* __restrict__ vel, float L, const int64_t* __restrict__ uoff,
-                              const int64_t* __restrict__ ulist, const float4* __restrict__ cen,
-                              const float4* __restrict__ bulk, const float4* __restrict__ inv,
+// Every seed into the lists of its own node and of the nodes above it.
+__global__ void k_seed_under_fill(int64_t nn, const int64_t* __restrict__ parent, const int* __restrict__ nkids,
+                                  const int64_t* __restrict__ off, const SeedRec* __restrict__ rec,
+                                  unsigned long long* __restrict__ fill, int64_t* __restrict__ list,
+                                  SeedRec* __restrict__ lrec) {
+  const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (s >= nn || nkids[s] != 0) return;
+  const SeedRec t = rec[s];
+  for (int64_t q = s; q >= 0; q = parent[q]) {
+    const int64_t at = off[q] + int64_t(atomicAdd(fill + q, 1ull));
+    list[at] = s;
+    lrec[at] = t;
+  }
+}
+
+// One thread per member of a level-0 node, in the member list's order: its seed (argmin over the seeds
+// under its deepest node). Neighbours share their group's list of seeds, and u in the level-0 frame and v
+// are the member's own U and V; in the order of the particles every lane walked another list (101 us for
+// 2^21 particles in groups of up to 3e4 members, 27 us in this order).
+__global__ void k_seed_assign(int64_t m0, const uint32_t* __restrict__ mem, const int64_t* __restrict__ deepest,
+                              const int* __restrict__ nkids, const float4* __restrict__ U,
+                              const float4* __restrict__ V, const int64_t* __restrict__ uoff,
+                              const int64_t* __restrict__ ulist, const SeedRec* __restrict__ lrec,
                               int64_t* __restrict__ seed, unsigned long long* __restrict__ count) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t dq = i < n ? deepest[i] : -1;
+  const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const bool in = p < m0;  // every lane stays for the match
+  const int64_t i = in ? mem[p] : 0, dq = in ? deepest[i] : -1;
   int64_t arg = dq;
-  if (dq >= 0 && nkids[dq] != 0) {
-    const int64_t r0 = mem[node_off[root[dq]]];
-    const float hL = 0.5f * L;
-    const float ux = rsd::wrap_diff(pos[3 * r0], pos[3 * i], L, hL);
-    const float uy = rsd::wrap_diff(pos[3 * r0 + 1], pos[3 * i + 1], L, hL);
-    const float uz = rsd::wrap_diff(pos[3 * r0 + 2], pos[3 * i + 2], L, hL);
-    const float vx = vel[3 * i], vy = vel[3 * i + 1], vz = vel[3 * i + 2];
+  if (in && nkids[dq] != 0) {
+    const float4 u = U[p], v = V[p];
     float best = 0.f;
     arg = -1;
-    for (int64_t k = uoff[dq]; k < uoff[dq + 1]; ++k) {
+    const int64_t k1 = uoff[dq + 1];
+#pragma unroll 4
+    for (int64_t k = uoff[dq]; k < k1; ++k) {
+      const SeedRec t = lrec[k];
       const int64_t s = ulist[k];
-      const float4 sc = inv[s];
-      const float d = seed_metric(ux, uy, uz, cen[s], vx, vy, vz, bulk[s], sc.x, sc.y);
+      const float d = seed_metric(u.x, u.y, u.z, v.x, v.y, v.z, t);
       if (arg < 0 || d < best || (d == best && s < arg)) {
         best = d;
         arg = s;
       }
     }
   }
-  if (i < n) seed[i] = arg;
+  if (in) seed[i] = arg;
   // one addition per seed and warp
   const unsigned peers = __match_any_sync(0xffffffffu, arg);
   if (arg >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(count + arg, (unsigned long long)__popc(peers));
@@ -149,8 +162,8 @@ __global__ void k_seed_assign(int64_t n, const int64_t* __restrict__ deepest, co
 // One thread per seed: its host among the seeds of its level-0 node ranking above it.
 __global__ void k_seed_host(int64_t nn, const int* __restrict__ nkids, const int64_t* __restrict__ root,
                             const int64_t* __restrict__ uoff, const int64_t* __restrict__ ulist,
-                            const float4* __restrict__ cen, const float4* __restrict__ bulk,
-                            const float4* __restrict__ inv, const unsigned long long* __restrict__ count,
+                            const SeedRec* __restrict__ rec, const SeedRec* __restrict__ lrec,
+                            const unsigned long long* __restrict__ count,
                             int64_t* __restrict__ host, int64_t* __restrict__ count_out) {
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (s >= nn) return;
@@ -160,17 +173,17 @@ __global__ void k_seed_host(int64_t nn, const int* __restrict__ nkids, const int
     return;
   }
   const unsigned long long ns = count[s];
-  const float4 c = cen[s], w = bulk[s];
-  const int64_t r = root[s];
+  const float4 c = rec[s].c, w = rec[s].w;
+  const int64_t r = root[s], k1 = uoff[r + 1];
   float best = 0.f;
   int64_t arg = -1;
-  for (int64_t k = uoff[r]; k < uoff[r + 1]; ++k) {
+#pragma unroll 4
+  for (int64_t k = uoff[r]; k < k1; ++k) {
     const int64_t h = ulist[k];
-    if (h == s) continue;
     const unsigned long long nh = count[h];
-    if (!(nh > ns || (nh == ns && h < s))) continue;
-    const float4 sc = inv[h];
-    const float d = seed_metric(c.x, c.y, c.z, cen[h], w.x, w.y, w.z, bulk[h], sc.x, sc.y);
+    const SeedRec t = lrec[k];
+    if (h == s || !(nh > ns || (nh == ns && h < s))) continue;
+    const float d = seed_metric(c.x, c.y, c.z, w.x, w.y, w.z, t);
     if (arg < 0 || d < best || (d == best && h < arg)) {
       best = d;
       arg = h;
@@ -208,12 +221,11 @@ extern "C" int rs_assign_seeds(rs_ctx* ctx, const float* pos, const float* vel, 
   int64_t* root = scratch_t<int64_t>(ctx, S_SEED_ROOT, size_t(nn));
   unsigned long long* ucnt = scratch_t<unsigned long long>(ctx, S_SEED_UCNT, 2 * size_t(nn) + 2);
   int64_t* uoff = scratch_t<int64_t>(ctx, S_SEED_UOFF, size_t(nn) + 1);
-  float4* cen = scratch_t<float4>(ctx, S_SEED_CEN, 2 * size_t(nn));
+  SeedRec* rec = scratch_t<SeedRec>(ctx, S_SEED_CEN, size_t(nn));
   double* sums = scratch_t<double>(ctx, S_SEED_SUMS, 6 * size_t(nn));
   int64_t* segsz = scratch_t<int64_t>(ctx, S_SEED_SEG, size_t(nn));
   unsigned long long* count = scratch_t<unsigned long long>(ctx, S_SEED_COUNT, size_t(nn));
-  if (!nkids || !root || !ucnt || !uoff || !cen || !sums || !segsz || !count) return RS_ERR_OOM;
-  float4* bulk = cen + nn;
+  if (!nkids || !root || !ucnt || !uoff || !rec || !sums || !segsz || !count) return RS_ERR_OOM;
   unsigned long long* fill = ucnt + nn + 1;
   RS_CUDA(ctx, cudaMemsetAsync(nkids, 0, 4 * size_t(nn), st));
   k_seed_kids<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids);
@@ -230,23 +242,24 @@ extern "C" int rs_assign_seeds(rs_ctx* ctx, const float* pos, const float* vel, 
   const int64_t seeds = ctx->host_box[1];
   const int64_t total = ctx->host_box[0];
   int64_t* ulist = scratch_t<int64_t>(ctx, S_SEED_LIST, size_t(std::max<int64_t>(total, 1)));
-  if (!ulist) return RS_ERR_OOM;
-  k_seed_under_fill<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids, uoff, fill, ulist);
-  RS_LAUNCHED(ctx, "k_seed_under_fill");
+  SeedRec* lrec = scratch_t<SeedRec>(ctx, S_SEED_REC, size_t(std::max<int64_t>(total, 1)));
+  if (!ulist || !lrec) return RS_ERR_OOM;
   // seed centres and bulk velocities (canonical-order sums over the seeds' members)
   RS_TRY((cro_segmented<6, SeedTerm>(ctx, nn, h.node_off, segsz, m, SeedTerm{h.U, h.V}, sums, st)));
   k_seed_stats<<<grid_for(nn, kT), kT, 0, st>>>(nn, nkids, root, h.node_off, h.node_size, h.mem, pos,
-                                               ctx->cfg.box_L, sums, cen, bulk);
+                                               ctx->cfg.box_L, sums, h.inv, rec);
   RS_LAUNCHED(ctx, "k_seed_stats");
+  k_seed_under_fill<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids, uoff, rec, fill, ulist, lrec);
+  RS_LAUNCHED(ctx, "k_seed_under_fill");
   RS_CUDA(ctx, cudaMemsetAsync(count, 0, 8 * size_t(nn), st));
+  RS_CUDA(ctx, cudaMemsetAsync(particle_seed, 0xff, 8 * size_t(n), st));  // -1: in no group
   {
     ProfScope prof_(ctx, "k_seed_assign", st);
-    k_seed_assign<<<grid_for(n, kT), kT, 0, st>>>(n, h.deepest, nkids, root, h.node_off, h.mem, pos, vel,
-                                                 ctx->cfg.box_L, uoff, ulist, cen, bulk, h.inv,
-                                                 particle_seed, count);
+    k_seed_assign<<<grid_for(ctx->n_level0, kT), kT, 0, st>>>(ctx->n_level0, h.mem, h.deepest, nkids, h.U, h.V, uoff,
+                                                             ulist, lrec, particle_seed, count);
   }
   RS_LAUNCHED(ctx, "k_seed_assign");
-  k_seed_host<<<grid_for(nn, kT), kT, 0, st>>>(nn, nkids, root, uoff, ulist, cen, bulk, h.inv, count,
+  k_seed_host<<<grid_for(nn, kT), kT, 0, st>>>(nn, nkids, root, uoff, ulist, rec, lrec, count,
                                               node_host, node_count);
   RS_LAUNCHED(ctx, "k_seed_host");
   if (n_seeds_out) {
