@@ -83,10 +83,52 @@ __device__ __forceinline__ void level_stat(unsigned long long* __restrict__ stat
 // ---- level 0 over a dense label range (max label < 2 n + 4096): per-label member counts, the
 // kept labels' node indices and member offsets from two scans over the label range, then one
 // sort of the kept particles only, by (node, id).
-__global__ void k_label_count(int64_t n, const int64_t* __restrict__ lab, uint32_t* __restrict__ cnt) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const bool valid = i < n;  // every lane stays for the warp-aggregated atomics
-  rsd::warp_run_add<uint32_t>(cnt, valid ? uint32_t(lab[i]) : 0u, valid, 1u);
+// Particles of one large group are all over the input, and additions to one counter queue (about 1 ns
+// each). So a block first counts in a table of its own in shared memory: a label takes a free slot, and
+// where another label holds the slot the addition goes to its counter (equal neighbours at once). A group
+// of a fraction f of the particles gets its slot with a probability near f / (f + 1 / kCountSlots), and
+// blocks mix the labels differently. 2^27 particles: 12.1 -> 4.4 ms.
+constexpr int kCountThreads = 512, kCountPer = 4, kCountBits = 11, kCountSlots = 1 << kCountBits;
+
+__global__ void __launch_bounds__(kCountThreads)
+k_label_count(int64_t n, const int64_t* __restrict__ lab, uint32_t* __restrict__ cnt) {
+  constexpr uint32_t kFree = 0xffffffffu;  // labels are below 2^31
+  __shared__ uint32_t skey[kCountSlots], scnt[kCountSlots];
+  for (int t = threadIdx.x; t < kCountSlots; t += kCountThreads) {
+    skey[t] = kFree;
+    scnt[t] = 0;
+  }
+  __syncthreads();
+  const uint32_t salt = blockIdx.x * 0x85ebca6bu;
+  const int64_t step = int64_t(gridDim.x) * kCountThreads * kCountPer;
+  for (int64_t i0 = int64_t(blockIdx.x) * kCountThreads * kCountPer; i0 < n; i0 += step) {
+    uint32_t l[kCountPer];
+#pragma unroll
+    for (int k = 0; k < kCountPer; ++k) {
+      const int64_t i = i0 + k * kCountThreads + threadIdx.x;
+      l[k] = i < n ? uint32_t(lab[i]) : kFree;
+    }
+#pragma unroll
+    for (int k = 0; k < kCountPer; ++k) {
+      bool miss = l[k] != kFree;
+      if (miss) {
+        const uint32_t slot = ((l[k] ^ salt) * 0x9e3779b1u) >> (32 - kCountBits);
+        uint32_t key = skey[slot];
+        if (key == kFree) {
+          key = atomicCAS(skey + slot, kFree, l[k]);
+          if (key == kFree) key = l[k];
+        }
+        if (key == l[k]) {
+          atomicAdd(scnt + slot, 1u);
+          miss = false;
+        }
+      }
+      rsd::warp_run_add<uint32_t>(cnt, l[k], miss, 1u);  // every lane
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < kCountSlots; t += kCountThreads)
+    if (scnt[t]) atomicAdd(cnt + skey[t], scnt[t]);
 }
 
 __global__ void k_label_keep(int64_t nl, const uint32_t* __restrict__ cnt, int min_size,
@@ -114,24 +156,58 @@ __global__ void k_label_nodes(int64_t nl, int64_t nodes, int64_t members, const 
   node_level[q] = 0;
 }
 
-// Keys (node << bid | id) of the particles of kept groups, appended with one atomic per warp.
-__global__ void k_label_keys(int64_t n, const int64_t* __restrict__ ids, const int64_t* __restrict__ lab,
-                             const uint32_t* __restrict__ cnt, int min_size,
-                             const int64_t* __restrict__ knode, int bid,
-                             unsigned long long* __restrict__ ctr, uint64_t* __restrict__ keys,
-                             uint32_t* __restrict__ vals) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const int64_t l = i < n ? lab[i] : 0;
-  const bool keep = i < n && cnt[l] >= uint32_t(min_size);
-  const unsigned b = __ballot_sync(0xffffffffu, keep);
-  unsigned long long base = 0;
-  if (lane == 0 && b) base = atomicAdd(ctr, (unsigned long long)__popc(b));
-  base = __shfl_sync(0xffffffffu, base, 0);
-  if (!keep) return;
-  const unsigned long long pos = base + __popc(b & ((1u << lane) - 1u));
-  keys[pos] = (uint64_t(knode[l]) << bid) | uint64_t(ids[i]);
-  vals[pos] = uint32_t(i);
+// Keys (node << bid | id) of the particles of kept groups, appended with one addition to the counter a
+// block (one a warp queued at it: 2^27 particles 6.9 -> 2.1 ms). A kept label is one whose node index the
+// scan raised, so both come from the same 32 bytes.
+constexpr int kKeysPer = 8;
+
+__global__ void __launch_bounds__(kT)
+k_label_keys(int64_t n, const int64_t* __restrict__ ids, const int64_t* __restrict__ lab, int64_t nl,
+             int64_t nodes, const int64_t* __restrict__ knode, int bid, unsigned long long* __restrict__ ctr,
+             uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+  __shared__ unsigned wsum[kT / 32];
+  __shared__ unsigned long long sbase;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i0 = int64_t(blockIdx.x) * (kT * kKeysPer) + threadIdx.x;
+  int64_t node[kKeysPer];
+  unsigned votes[kKeysPer], total = 0;
+#pragma unroll
+  for (int k = 0; k < kKeysPer; ++k) {
+    const int64_t i = i0 + k * kT;
+    node[k] = -1;
+    if (i < n) {
+      const int64_t l = lab[i], q = knode[l];
+      if ((l + 1 < nl ? knode[l + 1] : nodes) != q) node[k] = q;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < kKeysPer; ++k) {
+    votes[k] = __ballot_sync(0xffffffffu, node[k] >= 0);
+    total += __popc(votes[k]);
+  }
+  if (lane == 0) wsum[warp] = total;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned all = 0;
+    for (int w = 0; w < kT / 32; ++w) {
+      const unsigned c = wsum[w];
+      wsum[w] = all;
+      all += c;
+    }
+    sbase = all ? atomicAdd(ctr, (unsigned long long)all) : 0ull;
+  }
+  __syncthreads();
+  unsigned long long pos = sbase + wsum[warp];
+#pragma unroll
+  for (int k = 0; k < kKeysPer; ++k) {
+    if (node[k] >= 0) {
+      const int64_t i = i0 + k * kT;
+      const unsigned long long at = pos + __popc(votes[k] & ((1u << lane) - 1u));
+      keys[at] = (uint64_t(node[k]) << bid) | uint64_t(ids[i]);
+      vals[at] = uint32_t(i);
+    }
+    pos += __popc(votes[k]);
+  }
 }
 
 // Sparse labels: all particles ordered by (label, id) with two stable radix sorts, first by id
@@ -797,7 +873,7 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
       int64_t* koff = scratch_t<int64_t>(ctx, S_GKEY_B, size_t(nl) + 1);
       if (!cntl || !knode || !koff) return RS_ERR_OOM;
       RS_CUDA(ctx, cudaMemsetAsync(cntl, 0, sizeof(uint32_t) * nl, st));
-      k_label_count<<<grid_for(n, kT), kT, 0, st>>>(n, fof_label, cntl);
+      k_label_count<<<std::min(grid_for(n, kCountThreads * kCountPer), 152u * 4u), kCountThreads, 0, st>>>(n, fof_label, cntl);
       RS_LAUNCHED(ctx, "k_label_count");
       k_label_keep<<<grid_for(nl, kT), kT, 0, st>>>(nl, cntl, min_size, knode, koff, stat);
       RS_LAUNCHED(ctx, "k_label_keep");
@@ -821,8 +897,7 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
         RS_LAUNCHED(ctx, "k_label_nodes");
         const int bits = bits_for(uint64_t(std::max<int64_t>(nodes - 1, 1))) + bid;
         (sort_ends_in_b(members, bits) ? vb : va) = h.mem;
-        k_label_keys<<<grid_for(n, kT), kT, 0, st>>>(n, ids, fof_label, cntl, min_size, knode, bid,
-                                                    mx + 8, ka, va);
+        k_label_keys<<<grid_for(n, kT * kKeysPer), kT, 0, st>>>(n, ids, fof_label, nl, nodes, knode, bid, mx + 8, ka, va);
         RS_LAUNCHED(ctx, "k_label_keys");
         uint64_t* keys;
         uint32_t* vals;
