@@ -211,7 +211,7 @@ NODE_BYTES_PER_MEMBER = 40.0    # 6D level: u 12 + v 12 + id 8 + label 8 per mem
 OPS_D6 = 20.0                   # 6D distance: 6 sub, 6 mul, 4 add, 2 scale mul, 1 add, 1 compare
 OPS_PAIR = 7.0                  # potential pair: 3 sub, 3 FMA, 1 add (+ 1 MUFU rsqrt)
 OPS_EXPANSION = 50.0            # tree walk: one quadrupole expansion with its bound and test
-TREE_MIN_DEFAULT = 16384        # the library's default smallest node of the tree bound
+TREE_MIN_DEFAULT = 8192         # the library's default smallest node of the tree bound
 
 
 def _measured_peaks():
