@@ -469,8 +469,10 @@ k_nn6d(int64_t nb, int64_t nn, const int64_t* __restrict__ item_off, const int64
 
 // Exact k-th smallest nn2 of each node, k = ceil(f_num g / f_den) - 1: radix select on the
 // (non-negative) float bit patterns. Nodes up to kSelectWarpMax members take one
-// warp each (k_select_l2_warp), larger ones a block (k_select_l2).
-constexpr int64_t kSelectWarpMax = 4096;
+// warp each (k_select_l2_warp), larger ones a block (k_select_l2): on a level of few nodes the largest
+// node's warp is all there is to wait for. 2^18 particles, both kernels: 170 us with the line at 4096
+// members, 117 us at 1024; the pass over 2^27 particles takes the same within 0.1%.
+constexpr int64_t kSelectWarpMax = 1024;
 // Levels of more ordered pairs (sum of g^2) take the pruned searches of the batched form; below, the
 // all-pairs kernels cost less than their set-up (about 40 launches; 4e7 pairs are 0.05 ms of work on the
 // whole GPU). A 2^18-particle pass takes 600 device operations and 4.7 ms of device time with this line,
