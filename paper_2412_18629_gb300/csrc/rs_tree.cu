@@ -27,8 +27,7 @@
 //           of the warp's targets, a leaf is summed directly (self excluded), otherwise its children
 //           are visited;
 //   slack   float32 evaluation and summation (per direct term <= ~8u, 32-term leaf blocks
-//           summed as two packed halves <= 31u, the target's own term rsqrt(eps^2) taken out of
-//           its leaf once <= u of the leaf sum, expansions with FMAs <= ~20u of n/R' in 32-cell
+//           summed as two packed halves <= 31u, the target's own term left out, expansions with FMAs <= ~20u of n/R' in 32-cell
 //           blocks <= 31u, Kahan across blocks <= 2u) stay below 1e-5 relative; the truncation
 //           terms are summed in float32 and widened by 0.1%:
 //           S_lo = S~ (1 - 1e-5) - 1.001 B, S_hi = S~ (1 + 1e-5) + 1.001 B;
@@ -532,8 +531,9 @@ __device__ __forceinline__ void walk_cells(const Cell* __restrict__ ncell, const
 }
 
 // Direct sums over `cnt` leaves, two members per packed float32x2 step; slots past a leaf's count
-// hold +inf, whose term is exactly 0; the target's own term rsqrt(eps^2) is taken out once (or,
-// without a normal eps^2, skipped per pair).
+// hold +inf, whose term is exactly 0. The target's own term 1 / eps never enters: it would leave its
+// rounding behind, which no multiple of the other terms bounds. The leaves that hold a target of the
+// warp (one or a few of hundreds) test for it per pair.
 template <bool kNormal, int kSlices>
 __device__ __forceinline__ void walk_leaves(const float4* __restrict__ nx, const uint32_t* leaves, int cnt, uint32_t g,
                                             float4 t, uint32_t self_rel, float eps2, int lane, WalkShared& W,
@@ -559,18 +559,27 @@ __device__ __forceinline__ void walk_leaves(const float4* __restrict__ nx, const
                    e2 = make_float2(eps2, eps2);
       float2 acc2 = make_float2(0.f, 0.f);
       const int slice = lane / (32 / kSlices);
-#pragma unroll 8
-      for (int i = 0; i < 32 / kSlices; i += 2) {
-        const int k = 2 * slice + kSlices * i;
+      auto pair = [&](int k) {
         const float2 ex = __fadd2_rn(*reinterpret_cast<const float2*>(&W.leaf[0][k]), ntx);
         const float2 ey = __fadd2_rn(*reinterpret_cast<const float2*>(&W.leaf[1][k]), nty);
         const float2 ez = __fadd2_rn(*reinterpret_cast<const float2*>(&W.leaf[2][k]), ntz);
         const float2 r2 = __ffma2_rn(ex, ex, __ffma2_rn(ey, ey, __ffma2_rn(ez, ez, e2)));
-        acc2 = __fadd2_rn(acc2, make_float2(rsd::inv_sqrt<true>(r2.x), rsd::inv_sqrt<true>(r2.y)));
+        return make_float2(rsd::inv_sqrt<true>(r2.x), rsd::inv_sqrt<true>(r2.y));
+      };
+      const bool own = self_rel >> kLeafBits == j;
+      if (__any_sync(0xffffffffu, own)) {
+        const int self = own ? int(self_rel & 31u) : -1;
+#pragma unroll 8
+        for (int i = 0; i < 32 / kSlices; i += 2) {
+          const int k = 2 * slice + kSlices * i;
+          const float2 w = pair(k);
+          acc2 = __fadd2_rn(acc2, make_float2(k == self ? 0.f : w.x, k + 1 == self ? 0.f : w.y));
+        }
+      } else {
+#pragma unroll 8
+        for (int i = 0; i < 32 / kSlices; i += 2) acc2 = __fadd2_rn(acc2, pair(2 * slice + kSlices * i));
       }
       blk = __fadd_rn(acc2.x, acc2.y);
-      if (self_rel >> kLeafBits == j && ((self_rel & 31u) >> 1) % kSlices == uint32_t(slice))
-        blk = __fsub_rn(blk, rsd::inv_sqrt<true>(eps2));
     } else {
       blk = 0.f;
       for (int k = lane / (32 / kSlices); k < n; k += kSlices) {
