@@ -418,8 +418,10 @@ __device__ __forceinline__ float d6(float4 ui, float4 vi, float4 uj, float4 vj, 
 
 // All-pairs kernels: a block per (tile of kTile6 members, chunk of kChunk6 targets) of a node, so that a
 // single large node of a small level still spreads over the GPU (one block per tile over all targets
-// took as long as the largest node has members).
+// took as long as the largest node has members). The blocks stride over these items: a node of 2^24 members
+// has 2^31 of them, one more than a grid can have blocks.
 constexpr int kChunk6Bits = 10, kChunk6 = 1 << kChunk6Bits;
+constexpr int64_t kMaxBlocks6 = 1 << 16;
 
 // Nearest-neighbour d6 per member (nn2 starts at +inf): the chunk's j-tiles staged in shared memory;
 // the chunks of a member combine by an atomic minimum of the float bits (distances are not negative).
@@ -428,43 +430,43 @@ k_nn6d(int64_t nb, int64_t nn, const int64_t* __restrict__ item_off, const int64
        const int64_t* __restrict__ node_size, const float4* __restrict__ inv,
        const float4* __restrict__ U, const float4* __restrict__ V, float* __restrict__ nn2, int64_t mb) {
   __shared__ float4 su[kTile6], sv[kTile6];
-  const int64_t b = blockIdx.x;
-  if (b >= item_off[nn]) return;
-  const int64_t k = rsd::upper_bound_i64(item_off, nn, b) - 1;
-  const int64_t q = nb + k;
-  const int64_t base = node_off[q], g = node_size[q];
-  const int64_t chunks = (g + kChunk6 - 1) / kChunk6, t = (b - item_off[k]) / chunks,
-                c = (b - item_off[k]) - t * chunks;
-  const float isx = inv[q].x, isv = inv[q].y;
-  const int64_t i = t * kTile6 + threadIdx.x, j_end = rsd::min64(g, (c + 1) * kChunk6);
-  const bool valid = i < g;
-  const float4 ui = valid ? U[base + i] : make_float4(0, 0, 0, 0);
-  const float4 vi = valid ? V[base + i] : make_float4(0, 0, 0, 0);
-  float best = __int_as_float(0x7f800000);
-  for (int64_t j0 = c * kChunk6; j0 < j_end; j0 += kTile6) {
-    const int64_t j = j0 + threadIdx.x;
-    if (j < j_end) {
-      su[threadIdx.x] = U[base + j];
-      sv[threadIdx.x] = V[base + j];
-    }
-    __syncthreads();
-    const int jn = int(rsd::min64(kTile6, j_end - j0));
-    if (j0 != t * kTile6) {
-#pragma unroll 4
-      for (int jj = 0; jj < jn; ++jj) best = fminf(best, d6(ui, vi, su[jj], sv[jj], isx, isv));
-    } else {  // the members' own tile
-      for (int jj = 0; jj < jn; ++jj) {
-        if (jj == int(threadIdx.x)) continue;
-        best = fminf(best, d6(ui, vi, su[jj], sv[jj], isx, isv));
+  for (int64_t b = blockIdx.x, items = item_off[nn]; b < items; b += gridDim.x) {
+    const int64_t k = rsd::upper_bound_i64(item_off, nn, b) - 1;
+    const int64_t q = nb + k;
+    const int64_t base = node_off[q], g = node_size[q];
+    const int64_t chunks = (g + kChunk6 - 1) / kChunk6, t = (b - item_off[k]) / chunks,
+                  c = (b - item_off[k]) - t * chunks;
+    const float isx = inv[q].x, isv = inv[q].y;
+    const int64_t i = t * kTile6 + threadIdx.x, j_end = rsd::min64(g, (c + 1) * kChunk6);
+    const bool valid = i < g;
+    const float4 ui = valid ? U[base + i] : make_float4(0, 0, 0, 0);
+    const float4 vi = valid ? V[base + i] : make_float4(0, 0, 0, 0);
+    float best = __int_as_float(0x7f800000);
+    for (int64_t j0 = c * kChunk6; j0 < j_end; j0 += kTile6) {
+      const int64_t j = j0 + threadIdx.x;
+      if (j < j_end) {
+        su[threadIdx.x] = U[base + j];
+        sv[threadIdx.x] = V[base + j];
       }
+      __syncthreads();
+      const int jn = int(rsd::min64(kTile6, j_end - j0));
+      if (j0 != t * kTile6) {
+#pragma unroll 4
+        for (int jj = 0; jj < jn; ++jj) best = fminf(best, d6(ui, vi, su[jj], sv[jj], isx, isv));
+      } else {  // the members' own tile
+        for (int jj = 0; jj < jn; ++jj) {
+          if (jj == int(threadIdx.x)) continue;
+          best = fminf(best, d6(ui, vi, su[jj], sv[jj], isx, isv));
+        }
+      }
+      __syncthreads();
     }
-    __syncthreads();
+    if (!valid) continue;
+    if (chunks == 1)
+      nn2[base + i - mb] = best;
+    else
+      atomicMin(reinterpret_cast<unsigned int*>(nn2 + (base + i - mb)), __float_as_uint(best));
   }
-  if (!valid) return;
-  if (chunks == 1)
-    nn2[base + i - mb] = best;
-  else
-    atomicMin(reinterpret_cast<unsigned int*>(nn2 + (base + i - mb)), __float_as_uint(best));
 }
 
 // Exact k-th smallest nn2 of each node, k = ceil(f_num g / f_den) - 1: radix select on the
@@ -610,53 +612,54 @@ k_link6d(int64_t nb, int64_t nn, const int64_t* __restrict__ item_off, const int
          uint32_t* __restrict__ uf, int64_t mb) {
   __shared__ float4 su[kTile6], sv[kTile6];
   __shared__ uint32_t sroot[kTile6];  // kNoRoot: no friend at all
-  const int64_t b = blockIdx.x;
-  if (b >= item_off[nn]) return;
-  const int64_t k = rsd::upper_bound_i64(item_off, nn, b) - 1;
-  const int64_t q = nb + k;
-  const int64_t base = node_off[q], g = node_size[q];
-  const int64_t chunks = (g + kChunk6 - 1) / kChunk6, t = (b - item_off[k]) / chunks,
-                c = (b - item_off[k]) - t * chunks;
-  const int64_t j_end = rsd::min64(g, (c + 1) * kChunk6), j_begin = max(c * int64_t(kChunk6), t * int64_t(kTile6));
-  if (j_begin >= j_end) return;  // below the diagonal
-  const float4 iv = inv[q];
-  const float isx = iv.x, isv = iv.y, l2 = iv.z;
-  const int64_t i = t * kTile6 + threadIdx.x;
-  const bool valid = i < g;
-  const float4 ui = valid ? U[base + i] : make_float4(0, 0, 0, 0);
-  const float4 vi = valid ? V[base + i] : make_float4(0, 0, 0, 0);
-  const bool active = valid && nn2[base + i - mb] <= l2;  // others have no friend at all
-  uint32_t root = active ? rsd::uf_find(uf, uint32_t(base + i - mb)) : kNoRoot;
-  for (int64_t j0 = j_begin; j0 < j_end; j0 += kTile6) {
-    const int64_t j = j0 + threadIdx.x;
-    if (j < j_end) {
-      su[threadIdx.x] = U[base + j];
-      sv[threadIdx.x] = V[base + j];
-      sroot[threadIdx.x] = nn2[base + j - mb] <= l2 ? rsd::uf_find(uf, uint32_t(base + j - mb)) : kNoRoot;
-    }
-    __syncthreads();
-    const int jn = int(rsd::min64(kTile6, j_end - j0));
-    const int first = j0 == t * kTile6 ? int(threadIdx.x) + 1 : 0;  // its own tile: j > i
-    for (int jb = 0; jb < jn; jb += 32) {
-      unsigned hits = 0;
-      if (active) {
-        for (int jj = max(jb, first); jj < min(jb + 32, jn); ++jj) {
-          const uint32_t rj = sroot[jj];
-          if (rj != root && rj != kNoRoot && d6(ui, vi, su[jj], sv[jj], isx, isv) <= l2) hits |= 1u << (jj - jb);
-        }
+  for (int64_t b = blockIdx.x, items = item_off[nn]; b < items; b += gridDim.x) {
+    const int64_t k = rsd::upper_bound_i64(item_off, nn, b) - 1;
+    const int64_t q = nb + k;
+    const int64_t base = node_off[q], g = node_size[q];
+    const int64_t chunks = (g + kChunk6 - 1) / kChunk6, t = (b - item_off[k]) / chunks,
+                  c = (b - item_off[k]) - t * chunks;
+    const int64_t j_end = rsd::min64(g, (c + 1) * kChunk6),
+                  j_begin = max(c * int64_t(kChunk6), t * int64_t(kTile6));
+    if (j_begin >= j_end) continue;  // below the diagonal
+    const float4 iv = inv[q];
+    const float isx = iv.x, isv = iv.y, l2 = iv.z;
+    const int64_t i = t * kTile6 + threadIdx.x;
+    const bool valid = i < g;
+    const float4 ui = valid ? U[base + i] : make_float4(0, 0, 0, 0);
+    const float4 vi = valid ? V[base + i] : make_float4(0, 0, 0, 0);
+    const bool active = valid && nn2[base + i - mb] <= l2;  // others have no friend at all
+    uint32_t root = active ? rsd::uf_find(uf, uint32_t(base + i - mb)) : kNoRoot;
+    for (int64_t j0 = j_begin; j0 < j_end; j0 += kTile6) {
+      const int64_t j = j0 + threadIdx.x;
+      if (j < j_end) {
+        su[threadIdx.x] = U[base + j];
+        sv[threadIdx.x] = V[base + j];
+        sroot[threadIdx.x] = nn2[base + j - mb] <= l2 ? rsd::uf_find(uf, uint32_t(base + j - mb)) : kNoRoot;
       }
-      while (__any_sync(0xffffffffu, hits)) {  // one union a lane and round, the lanes side by side
-        if (hits) {
-          const uint32_t rj = sroot[jb + __ffs(hits) - 1];
-          hits &= hits - 1u;
-          if (rj != root) {
-            rsd::uf_unite(uf, root, rj);
-            root = rsd::uf_find(uf, root);
+      __syncthreads();
+      const int jn = int(rsd::min64(kTile6, j_end - j0));
+      const int first = j0 == t * kTile6 ? int(threadIdx.x) + 1 : 0;  // its own tile: j > i
+      for (int jb = 0; jb < jn; jb += 32) {
+        unsigned hits = 0;
+        if (active) {
+          for (int jj = max(jb, first); jj < min(jb + 32, jn); ++jj) {
+            const uint32_t rj = sroot[jj];
+            if (rj != root && rj != kNoRoot && d6(ui, vi, su[jj], sv[jj], isx, isv) <= l2) hits |= 1u << (jj - jb);
+          }
+        }
+        while (__any_sync(0xffffffffu, hits)) {  // one union a lane and round, the lanes side by side
+          if (hits) {
+            const uint32_t rj = sroot[jb + __ffs(hits) - 1];
+            hits &= hits - 1u;
+            if (rj != root) {
+              rsd::uf_unite(uf, root, rj);
+              root = rsd::uf_find(uf, root);
+            }
           }
         }
       }
+      __syncthreads();
     }
-    __syncthreads();
   }
 }
 
@@ -995,6 +998,7 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
     const ScanJob items = batched ? ScanJob{}
                                   : ScanJob{h.node_size + nb, item_off, item_off + nn, kTile6Bits, kChunk6Bits, 0};
     const int64_t items_ub = int64_t(level_pairs / (uint64_t(kTile6) * kChunk6)) + m / kTile6 + m / kChunk6 + nn + 1;
+    const unsigned blocks6 = unsigned(rsd::min64(items_ub, kMaxBlocks6));
     RS_TRY((cro_segmented<12, MomentTerm>(ctx, nn, h.node_off + nb, h.node_size + nb, m,
                                           MomentTerm{h.U, h.V}, sums, st, items)));
     k_node_inv<<<grid_for(nn * 16, kT), kT, 0, st>>>(nb, nn, h.node_size, sums, h.inv, h.mom);
@@ -1023,7 +1027,7 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
     } else {
       {
         ProfScope prof_(ctx, "k_nn6d", st);
-        k_nn6d<<<grid_for(items_ub, 1), kTile6, 0, st>>>(nb, nn, item_off, h.node_off, h.node_size, h.inv,
+        k_nn6d<<<blocks6, kTile6, 0, st>>>(nb, nn, item_off, h.node_off, h.node_size, h.inv,
                                                         h.U, h.V, nn2, mb);
       }
       RS_LAUNCHED(ctx, "k_nn6d");
@@ -1040,7 +1044,7 @@ extern "C" int rs_fof6d(rs_ctx* ctx, int64_t n, const float* pos, const float* v
     } else {
       {
         ProfScope prof_(ctx, "k_link6d", st);
-        k_link6d<<<grid_for(items_ub, 1), kTile6, 0, st>>>(nb, nn, item_off, h.node_off, h.node_size,
+        k_link6d<<<blocks6, kTile6, 0, st>>>(nb, nn, item_off, h.node_off, h.node_size,
                                                           h.inv, h.U, h.V, nn2, uf, mb);
       }
       RS_LAUNCHED(ctx, "k_link6d");
