@@ -218,7 +218,8 @@ int rs_potential_pairs(rs_ctx* ctx, int64_t* pairs_out);
  *   host of seed s: among the other seeds of s's level-0 node ranking above s (more assigned
  *     particles; equal counts: smaller node index), the nearest by the candidate's metric at
  *     (c_s, w_s); -1 when none ranks above.
- * pos, vel: the arrays given to rs_fof6d (others are re-gathered).
+ * pos, vel: positions and velocities of rs_fof6d's particles; the call reads them anew, so they may have
+ * moved since.
  * particle_seed: int64 [n] device: node index of the particle's seed, -1 outside every node.
  * node_host, node_count: int64 [n_nodes] device or NULL: host seed (-2 for nodes that are not
  * seeds), particles assigned (0 for nodes that are not seeds).

@@ -54,7 +54,7 @@ enum Slot : int {
   S_T_WANT, S_SUR_SD,
   // seed halos (rs_seeds.cu)
   S_SEED_KIDS, S_SEED_ROOT, S_SEED_UCNT, S_SEED_UOFF, S_SEED_CEN, S_SEED_REC, S_SEED_SUMS, S_SEED_SEG,
-  S_SEED_COUNT, S_SEED_LIST,
+  S_SEED_COUNT, S_SEED_LIST, S_SEED_REF,
   // temporal tracking (rs_track.cu)
   S_TRK_HEAD, S_TRK_RSTART, S_TRK_RKEY, S_TRK_KA, S_TRK_KB, S_TRK_VA, S_TRK_VB, S_TRK_H1,
   S_TRK_FLAG,

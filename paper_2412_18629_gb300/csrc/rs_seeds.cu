@@ -5,7 +5,7 @@
 //   seeds   the nodes without children (each level-0 node has at least one under it);
 //   frame   u = wrapped offset from the level-0 node's reference member r0 (smallest id);
 //   seed s  centre c_s = float(double(wrap(x_{r_s} - x_{r0})) + CRO(u^s) / g_s), u^s the
-//           offsets from s's own reference member r_s (the hierarchy's U), bulk velocity
+//           offsets from s's own reference member r_s, bulk velocity
 //           w_s = float(CRO(v) / g_s), and the metric scales (inv_sx2, inv_sv2) of s's split;
 //   metric  fl(|u - c_s|^2 inv_sx2_s) + fl(|v - w_s|^2 inv_sv2_s), float32 in d6's order;
 //   particle  the seed holding it when its deepest node is a seed, otherwise the nearest seed
@@ -15,12 +15,9 @@
 //           candidate's metric at (c_s, w_s); -1 if none.
 // Every comparison uses the same float32 operations as the CPU oracle, so the results are
 // identical to it.
+// Positions and velocities are read from the call's own arrays throughout: the hierarchy's U and V hold
+// the contents that rs_fof6d or rs_unbind saw, and an address does not tell whether they still are.
 #include "rs_cro.cuh"
-
-namespace rs {
-int gather_members(rs_ctx* ctx, int64_t mb, int64_t me, int64_t nb, int64_t ne, const float* pos,
-                   const float* vel, cudaStream_t st);
-}  // namespace rs
 
 using namespace rs;
 
@@ -34,17 +31,22 @@ __global__ void k_seed_kids(int64_t nn, const int64_t* __restrict__ parent, int*
 }
 
 // Per node the walk up its parents (as many steps as its level): its level-0 ancestor, and for a seed a
-// count at each node of the walk and at itself. Also the segments of the seeds for the canonical-order
-// sums (size 0 otherwise) and the number of seeds. The walk replaced seven pointer-jumping launches.
+// count at each node of the walk and at itself. Also the position of its reference member, the segments of
+// the seeds for the canonical-order sums (size 0 otherwise) and the number of seeds. The walk replaced
+// seven pointer-jumping launches.
 __global__ void k_seed_roots(int64_t nn, const int64_t* __restrict__ parent, const int* __restrict__ nkids,
                              const int64_t* __restrict__ node_size, int64_t* __restrict__ root,
                              unsigned long long* __restrict__ cnt, int64_t* __restrict__ seg_size,
-                             unsigned long long* __restrict__ n_seeds) {
+                             unsigned long long* __restrict__ n_seeds, const int64_t* __restrict__ node_off,
+                             const uint32_t* __restrict__ mem, const float* __restrict__ pos,
+                             float4* __restrict__ ref) {
   const int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const bool seed = q < nn && nkids[q] == 0;
   rsd::warp_count(n_seeds, seed);
   if (q >= nn) return;
   seg_size[q] = seed ? node_size[q] : 0;
+  const int64_t i = mem[node_off[q]];
+  ref[q] = make_float4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], 0.f);
   int64_t r = q;
   for (int64_t p = q; p >= 0; p = parent[p]) {
     r = p;
@@ -53,16 +55,30 @@ __global__ void k_seed_roots(int64_t nn, const int64_t* __restrict__ parent, con
   root[q] = r;
 }
 
+struct Particle {
+  float3 x, v;
+};
+
+__device__ __forceinline__ Particle load_particle(const float* __restrict__ pos, const float* __restrict__ vel, int64_t i) {
+  return {make_float3(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2]), make_float3(vel[3 * i], vel[3 * i + 1], vel[3 * i + 2])};
+}
+
+// Wrapped offset of x from the reference position r.
+__device__ __forceinline__ float3 offset_from(float4 r, float3 x, float L) {
+  const float hL = 0.5f * L;
+  return make_float3(rsd::wrap_diff(r.x, x.x, L, hL), rsd::wrap_diff(r.y, x.y, L, hL), rsd::wrap_diff(r.z, x.z, L, hL));
+}
+
 struct SeedTerm {  // u^s and v of a member of seed s
-  const float4* U;
-  const float4* V;
-  struct Value {
-    float4 u, v;
-  };
-  __device__ __forceinline__ Value load(int64_t p) const { return {U[p], V[p]}; }
+  const uint32_t* mem;
+  const float4* ref;
+  const float *pos, *vel;
+  float L;
+  using Value = Particle;
+  __device__ __forceinline__ Value load(int64_t p) const { return load_particle(pos, vel, mem[p]); }
   template <bool kFirst>
-  __device__ __forceinline__ void add(int64_t, const Value& t, double* acc) const {
-    const float4 u = t.u, v = t.v;
+  __device__ __forceinline__ void add(int64_t q, const Value& t, double* acc) const {
+    const float3 u = offset_from(ref[q], t.x, L), v = t.v;
     rsd::cro_add<kFirst>(acc[0], rsd::f2d(u.x));
     rsd::cro_add<kFirst>(acc[1], rsd::f2d(u.y));
     rsd::cro_add<kFirst>(acc[2], rsd::f2d(u.z));
@@ -81,21 +97,20 @@ struct SeedRec {
 
 // Seed centres (level-0 frame) and bulk velocities from the canonical-order sums.
 __global__ void k_seed_stats(int64_t nn, const int* __restrict__ nkids, const int64_t* __restrict__ root,
-                             const int64_t* __restrict__ node_off, const int64_t* __restrict__ node_size,
-                             const uint32_t* __restrict__ mem, const float* __restrict__ pos, float L,
+                             const int64_t* __restrict__ node_size, const float4* __restrict__ ref, float L,
                              const double* __restrict__ sums, const float4* __restrict__ inv,
                              SeedRec* __restrict__ rec) {
   const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (s >= nn || nkids[s] != 0) return;
-  const int64_t rs_ = mem[node_off[s]], r0 = mem[node_off[root[s]]];
+  const float4 rs_ = ref[s];
+  const float3 u = offset_from(ref[root[s]], make_float3(rs_.x, rs_.y, rs_.z), L);
   const double g = double(node_size[s]);
   const double* S = sums + 6 * s;
-  const float hL = 0.5f * L;
+  const float o[3] = {u.x, u.y, u.z};
   float c[3], w[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const float o = rsd::wrap_diff(pos[3 * r0 + d], pos[3 * rs_ + d], L, hL);
-    c[d] = __double2float_rn(__dadd_rn(double(o), __ddiv_rn(S[d], g)));
+    c[d] = __double2float_rn(__dadd_rn(double(o[d]), __ddiv_rn(S[d], g)));
     w[d] = __double2float_rn(__ddiv_rn(S[3 + d], g));
   }
   const float4 iv = inv[s];
@@ -125,20 +140,22 @@ __global__ void k_seed_under_fill(int64_t nn, const int64_t* __restrict__ parent
 }
 
 // One thread per member of a level-0 node, in the member list's order: its seed (argmin over the seeds
-// under its deepest node). Neighbours share their group's list of seeds, and u in the level-0 frame and v
-// are the member's own U and V; in the order of the particles every lane walked another list (101 us for
-// 2^21 particles in groups of up to 3e4 members, 27 us in this order).
-__global__ void k_seed_assign(int64_t m0, const uint32_t* __restrict__ mem, const int64_t* __restrict__ deepest,
-                              const int* __restrict__ nkids, const float4* __restrict__ U,
-                              const float4* __restrict__ V, const int64_t* __restrict__ uoff,
+// under its deepest node). Neighbours share their group's list of seeds; in the order of the particles every
+// lane walked another list (101 us for 2^21 particles in groups of up to 3e4 members, 36 us in this order;
+// from the hierarchy's streamed U and V, which may be of another time, 27 us).
+__global__ void k_seed_assign(int64_t m0, const uint32_t* __restrict__ mem, const uint32_t* __restrict__ mnode,
+                              const float4* __restrict__ ref, const int64_t* __restrict__ deepest,
+                              const int* __restrict__ nkids, const float* __restrict__ pos,
+                              const float* __restrict__ vel, float L, const int64_t* __restrict__ uoff,
                               const int64_t* __restrict__ ulist, const SeedRec* __restrict__ lrec,
                               int64_t* __restrict__ seed, unsigned long long* __restrict__ count) {
   const int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const bool in = p < m0;  // every lane stays for the match
   const int64_t i = in ? mem[p] : 0, dq = in ? deepest[i] : -1;
+  const Particle own = load_particle(pos, vel, i);  // beside the chain of loads to the node's list
   int64_t arg = dq;
   if (in && nkids[dq] != 0) {
-    const float4 u = U[p], v = V[p];
+    const float3 u = offset_from(ref[mnode[p]], own.x, L), v = own.v;
     float best = 0.f;
     arg = -1;
     const int64_t k1 = uoff[dq + 1];
@@ -211,11 +228,6 @@ extern "C" int rs_assign_seeds(rs_ctx* ctx, const float* pos, const float* vel, 
     if (n > 0) RS_CUDA(ctx, cudaMemsetAsync(particle_seed, 0xff, 8 * size_t(n), st));  // -1
     return RS_OK;
   }
-  if (pos != ctx->h_pos || vel != ctx->h_vel) {  // other arrays than rs_fof6d's: re-gather
-    RS_TRY(gather_members(ctx, 0, m, 0, nn, pos, vel, st));
-    ctx->h_pos = pos;
-    ctx->h_vel = vel;
-  }
   Hier h = hier_of(ctx);
   int* nkids = scratch_t<int>(ctx, S_SEED_KIDS, size_t(nn));
   int64_t* root = scratch_t<int64_t>(ctx, S_SEED_ROOT, size_t(nn));
@@ -225,7 +237,8 @@ extern "C" int rs_assign_seeds(rs_ctx* ctx, const float* pos, const float* vel, 
   double* sums = scratch_t<double>(ctx, S_SEED_SUMS, 6 * size_t(nn));
   int64_t* segsz = scratch_t<int64_t>(ctx, S_SEED_SEG, size_t(nn));
   unsigned long long* count = scratch_t<unsigned long long>(ctx, S_SEED_COUNT, size_t(nn));
-  if (!nkids || !root || !ucnt || !uoff || !rec || !sums || !segsz || !count) return RS_ERR_OOM;
+  float4* ref = scratch_t<float4>(ctx, S_SEED_REF, size_t(nn));
+  if (!nkids || !root || !ucnt || !uoff || !rec || !sums || !segsz || !count || !ref) return RS_ERR_OOM;
   unsigned long long* fill = ucnt + nn + 1;
   RS_CUDA(ctx, cudaMemsetAsync(nkids, 0, 4 * size_t(nn), st));
   k_seed_kids<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids);
@@ -233,7 +246,8 @@ extern "C" int rs_assign_seeds(rs_ctx* ctx, const float* pos, const float* vel, 
   // level-0 ancestor of every node and the seeds under it: counts, offsets, lists
   RS_CUDA(ctx, cudaMemsetAsync(ucnt, 0, 8 * (2 * size_t(nn) + 2), st));
   unsigned long long* n_seeds = fill + nn;  // the spare last counter slot
-  k_seed_roots<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids, h.node_size, root, ucnt, segsz, n_seeds);
+  k_seed_roots<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids, h.node_size, root, ucnt, segsz, n_seeds,
+                                              h.node_off, h.mem, pos, ref);
   RS_LAUNCHED(ctx, "k_seed_roots");
   static_assert(sizeof(unsigned long long) == sizeof(int64_t), "counts scanned as int64");
   RS_TRY(exclusive_scans(ctx, nn, ScanJobs{{{reinterpret_cast<int64_t*>(ucnt), uoff, uoff + nn}}}, st));
@@ -245,9 +259,9 @@ extern "C" int rs_assign_seeds(rs_ctx* ctx, const float* pos, const float* vel, 
   SeedRec* lrec = scratch_t<SeedRec>(ctx, S_SEED_REC, size_t(std::max<int64_t>(total, 1)));
   if (!ulist || !lrec) return RS_ERR_OOM;
   // seed centres and bulk velocities (canonical-order sums over the seeds' members)
-  RS_TRY((cro_segmented<6, SeedTerm>(ctx, nn, h.node_off, segsz, m, SeedTerm{h.U, h.V}, sums, st)));
-  k_seed_stats<<<grid_for(nn, kT), kT, 0, st>>>(nn, nkids, root, h.node_off, h.node_size, h.mem, pos,
-                                               ctx->cfg.box_L, sums, h.inv, rec);
+  RS_TRY((cro_segmented<6, SeedTerm>(ctx, nn, h.node_off, segsz, m, SeedTerm{h.mem, ref, pos, vel, ctx->cfg.box_L},
+                                     sums, st)));
+  k_seed_stats<<<grid_for(nn, kT), kT, 0, st>>>(nn, nkids, root, h.node_size, ref, ctx->cfg.box_L, sums, h.inv, rec);
   RS_LAUNCHED(ctx, "k_seed_stats");
   k_seed_under_fill<<<grid_for(nn, kT), kT, 0, st>>>(nn, h.node_parent, nkids, uoff, rec, fill, ulist, lrec);
   RS_LAUNCHED(ctx, "k_seed_under_fill");
@@ -255,8 +269,9 @@ extern "C" int rs_assign_seeds(rs_ctx* ctx, const float* pos, const float* vel, 
   RS_CUDA(ctx, cudaMemsetAsync(particle_seed, 0xff, 8 * size_t(n), st));  // -1: in no group
   {
     ProfScope prof_(ctx, "k_seed_assign", st);
-    k_seed_assign<<<grid_for(ctx->n_level0, kT), kT, 0, st>>>(ctx->n_level0, h.mem, h.deepest, nkids, h.U, h.V, uoff,
-                                                             ulist, lrec, particle_seed, count);
+    k_seed_assign<<<grid_for(ctx->n_level0, kT), kT, 0, st>>>(ctx->n_level0, h.mem, h.mnode, ref, h.deepest,
+                                                             nkids, pos, vel, ctx->cfg.box_L, uoff, ulist, lrec,
+                                                             particle_seed, count);
   }
   RS_LAUNCHED(ctx, "k_seed_assign");
   k_seed_host<<<grid_for(nn, kT), kT, 0, st>>>(nn, nkids, root, uoff, ulist, rec, lrec, count,
