@@ -191,13 +191,29 @@ struct PairItem {
 };
 constexpr uint32_t kPairChunk = 1024;
 
+// Pairs whose larger cell holds at most kSmallPair particles share the first `cap` items; when those are
+// full a thread tests the pair by itself. The other pairs have items of their own after them, enough for
+// all there can be (pair_items), so that no thread is left with the pairs of two large cells: 1e8 pairs of
+// particles took one thread 22 s.
+constexpr uint32_t kSmallPair = 512;
+
+// Most items of pairs with a cell above kSmallPair. A pair takes ceil(s / kPairChunk) items, s its larger
+// cell's particles; a cell has at most `reach` others in its stencil, and all pairs of a few cells are few.
+int64_t pair_items(int64_t n, int ns, int R) {
+  const int64_t cells = rsd::min64(n, int64_t(ns) * ns * ns), d = rsd::min64(2 * int64_t(R) + 1, ns);
+  const int64_t reach = d * d * d - 1;
+  const double per_cell = double(reach) * double(n) * (1.0 / kPairChunk + 1.0 / kSmallPair);
+  const double all_pairs = double(cells) * (double(n) / kPairChunk + 0.5 * double(cells));
+  return int64_t(std::min(per_cell, all_pairs)) + 1;
+}
+
 struct LinkArgs {
   Cells C;
   int ns, R;
   bool full;
   float L, hL, ll2;
   PairItem* items;
-  unsigned long long* n_items;
+  unsigned long long* n_items;  // [0] of small pairs, [1] of the others
   unsigned long long cap;
 };
 
@@ -208,8 +224,7 @@ __device__ __forceinline__ bool linked(const LinkArgs& A, float4 p, float4 q) {
 
 // Cells a and b with different roots: unite them if one pair of their particles is linked. All pairs
 // when there are at most kInline of them; otherwise a 4 x 4 sample first (two dense adjacent cells are
-// linked by almost any pair), and the pair of cells is listed when the sample has no link (and tested
-// here after all when the list is full).
+// linked by almost any pair), and the pair of cells is listed when the sample has no link.
 constexpr uint32_t kInline = 64;
 
 __device__ __forceinline__ void test_cells(const LinkArgs& A, uint32_t a, uint32_t b) {
@@ -225,13 +240,18 @@ __device__ __forceinline__ void test_cells(const LinkArgs& A, uint32_t a, uint32
       }
   }
   if (small) return;
-  const uint32_t chunks = (na + kPairChunk - 1) / kPairChunk;
-  const unsigned long long k = atomicAdd(A.n_items, (unsigned long long)chunks);
-  if (k + chunks <= A.cap) {
-    for (uint32_t c = 0; c < chunks; ++c) A.items[k + c] = PairItem{a, b, c};
+  const uint32_t larger = max(na, nb);
+  if (larger > kSmallPair) {
+    const uint32_t chunks = (larger + kPairChunk - 1) / kPairChunk;
+    const unsigned long long k = A.cap + atomicAdd(A.n_items + 1, (unsigned long long)chunks);
+    for (uint32_t c = 0; c < chunks; ++c) A.items[k + c] = na < nb ? PairItem{b, a, c} : PairItem{a, b, c};
     return;
   }
-  for (unsigned long long i = k; i < A.cap; ++i) A.items[i] = PairItem{a, a, 0};  // unused slots: no-ops
+  const unsigned long long k = atomicAdd(A.n_items, 1ull);
+  if (k < A.cap) {
+    A.items[k] = na < nb ? PairItem{b, a, 0} : PairItem{a, b, 0};
+    return;
+  }
   for (uint32_t i = 0; i < na; ++i) {
     const float4 p = A.C.pos[a0 + i];
     for (uint32_t j = 0; j < nb; ++j)
@@ -346,9 +366,9 @@ __global__ void __launch_bounds__(kThreads) k_link_cells(LinkArgs A) {
 __global__ void __launch_bounds__(kThreads) k_link_pairs(LinkArgs A) {
   __shared__ float4 tile[kThreads];
   __shared__ int skip;
-  const unsigned long long total = min(*A.n_items, A.cap);
+  const unsigned long long few = min(A.n_items[0], A.cap), total = few + A.n_items[1];
   for (unsigned long long w = blockIdx.x; w < total; w += gridDim.x) {
-    const PairItem it = A.items[w];
+    const PairItem it = A.items[w < few ? w : A.cap + (w - few)];
     __syncthreads();
     if (threadIdx.x == 0) skip = rsd::uf_find(A.C.parent, it.a) == rsd::uf_find(A.C.parent, it.b);
     __syncthreads();
@@ -509,7 +529,7 @@ extern "C" int rs_fof3d(rs_ctx* ctx, int64_t n, const float* pos, const int64_t*
   unsigned long long* minid = scratch_t<unsigned long long>(ctx, S_MINID, n);
   unsigned long long* counter = scratch_t<unsigned long long>(ctx, S_COUNTER, 8);
   const int64_t cap = n / 8 + 4096;
-  PairItem* items = scratch_t<PairItem>(ctx, S_CELL_PAIRS, size_t(cap));
+  PairItem* items = scratch_t<PairItem>(ctx, S_CELL_PAIRS, size_t(cap + pair_items(n, g.ns, g.R)));
   Cells C;
   C.count = tile_off + tiles;
   C.start = scratch_t<uint32_t>(ctx, S_CELL_START, size_t(n) + 1);
@@ -537,14 +557,14 @@ extern "C" int rs_fof3d(rs_ctx* ctx, int64_t n, const float* pos, const int64_t*
   RS_LAUNCHED(ctx, "k_cells");
   k_row_cells<<<grid_for(rows + 1, kThreads), kThreads, 0, st>>>(C, rows, row_cell);
   RS_LAUNCHED(ctx, "k_row_cells");
-  RS_CUDA(ctx, cudaMemsetAsync(counter, 0, 3 * sizeof(unsigned long long), st));
+  RS_CUDA(ctx, cudaMemsetAsync(counter, 0, 5 * sizeof(unsigned long long), st));
   RS_CUDA(ctx, cudaMemsetAsync(minid, 0xff, sizeof(unsigned long long) * size_t(n), st));
-  // counter[0]: groups, [1] and [2]: listed pairs of the two link passes (every launch below covers n
+  // counter[0]: groups, [1, 2] and [3, 4]: items of the two link passes (every launch below covers n
   // cells, the most there can be)
   for (const bool far : {false, true}) {
     if (far && g.full) break;
     const LinkArgs A{C, g.ns, g.R, g.full, ctx->cfg.box_L, 0.5f * ctx->cfg.box_L, ctx->cfg.link_len * ctx->cfg.link_len,
-                     items, counter + (far ? 2 : 1), (unsigned long long)cap};
+                     items, counter + (far ? 3 : 1), (unsigned long long)cap};
     {
       ProfScope prof_(ctx, "k_fof_link", st);
       (far ? k_link_cells<true> : k_link_cells<false>)<<<grid, kThreads, 0, st>>>(A);
