@@ -524,22 +524,17 @@ extern "C" int rs_fof3d(rs_ctx* ctx, int64_t n, const float* pos, const int64_t*
   float4* posS = scratch_t<float4>(ctx, S_POS_SORTED, n);
   const int64_t rows = int64_t(g.ns) * g.ns, tiles = (n + kHeadTile - 1) / kHeadTile;
   uint32_t* row_cell = scratch_t<uint32_t>(ctx, S_ROW_CELL, size_t(rows) + 1);
-  uint32_t* cell_of = scratch_t<uint32_t>(ctx, S_CELL_OF, n);
   int64_t* tile_off = scratch_t<int64_t>(ctx, S_CELL_TILES, size_t(tiles) + 1);
-  unsigned long long* minid = scratch_t<unsigned long long>(ctx, S_MINID, n);
   unsigned long long* counter = scratch_t<unsigned long long>(ctx, S_COUNTER, 8);
   const int64_t cap = n / 8 + 4096;
   PairItem* items = scratch_t<PairItem>(ctx, S_CELL_PAIRS, size_t(cap + pair_items(n, g.ns, g.R)));
   Cells C;
   C.count = tile_off + tiles;
   C.start = scratch_t<uint32_t>(ctx, S_CELL_START, size_t(n) + 1);
-  C.row = scratch_t<uint32_t>(ctx, S_CELL_ROW, n);
   C.x = scratch_t<uint16_t>(ctx, S_CELL_X, n);
-  C.parent = scratch_t<uint32_t>(ctx, S_PARENT, n);
   C.row_cell = row_cell;
   C.pos = posS;
-  if (!ka || !kb || !va || !vb || !posS || !row_cell || !cell_of || !tile_off || !minid || !counter || !items ||
-      !C.start || !C.row || !C.x || !C.parent)
+  if (!ka || !kb || !va || !vb || !posS || !row_cell || !tile_off || !counter || !items || !C.start || !C.x)
     return RS_ERR_OOM;
   const unsigned grid = grid_for(n, kThreads);
   k_cell_keys<<<grid, kThreads, 0, st>>>(n, pos, g.inv_sc, g.ns, ka, va);
@@ -550,6 +545,10 @@ extern "C" int rs_fof3d(rs_ctx* ctx, int64_t n, const float* pos, const int64_t*
   int kbits = 1;
   while (kbits < 64 && ((ns3 - 1) >> kbits) != 0) ++kbits;
   RS_TRY(radix_sort_u64(ctx, n, kbits, ka, va, kb, vb, &keys, &idx, st));
+  // the sort's other buffers: 51 bytes a particle in all instead of 67
+  uint32_t* cell_of = idx == va ? vb : va;
+  C.row = reinterpret_cast<uint32_t*>(keys == ka ? kb : ka);
+  C.parent = C.row + n;
   k_cell_heads<<<unsigned(tiles), kThreads, 0, st>>>(n, keys, tile_off);
   RS_LAUNCHED(ctx, "k_cell_heads");
   RS_TRY(exclusive_scan_i64(ctx, tiles, tile_off, tile_off + tiles, st));
@@ -558,6 +557,7 @@ extern "C" int rs_fof3d(rs_ctx* ctx, int64_t n, const float* pos, const int64_t*
   k_row_cells<<<grid_for(rows + 1, kThreads), kThreads, 0, st>>>(C, rows, row_cell);
   RS_LAUNCHED(ctx, "k_row_cells");
   RS_CUDA(ctx, cudaMemsetAsync(counter, 0, 5 * sizeof(unsigned long long), st));
+  unsigned long long* minid = reinterpret_cast<unsigned long long*>(keys);  // the cells hold what the keys told
   RS_CUDA(ctx, cudaMemsetAsync(minid, 0xff, sizeof(unsigned long long) * size_t(n), st));
   // counter[0]: groups, [1, 2] and [3, 4]: items of the two link passes (every launch below covers n
   // cells, the most there can be)
