@@ -7,7 +7,8 @@ box, halos up to 2e6 particles with three levels of subhalos).
 One step = one pass of the whole path over one snapshot with inputs resident in HBM. The
 headline is the batched + surrogate form timed over exactly K steps after W warm-up steps; the
 plain and batched forms are timed beside it with their own (stated) step counts, and every
-form's outputs are checked identical. Prints one JSON line (rank 0). For N > 1 (torchrun, one
+form's outputs are checked identical. Prints one JSON line (rank 0); stages, tallies and the other
+forms' figures go to stderr as one JSON line of details. For N > 1 (torchrun, one
 rank per GPU) every rank processes its own independent snapshot (seed + 1000 rank): weak
 scaling, no data-path collective; the value is all ranks' particles over the slowest rank's
 time.
@@ -591,6 +592,54 @@ def _form_entry(r, traffic):
             "surrogate_stats": r["surrogate_stats"], "output_digest": r["digest"]}
 
 
+def _short(x, digits=5):
+    """x with every float at `digits` significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.{digits}g}")
+    if isinstance(x, dict):
+        return {k: _short(v, digits) for k, v in x.items()}
+    return [_short(v, digits) for v in x] if isinstance(x, list) else x
+
+
+def result_lines(args, res, ws, n, box, seed, traffic, cpu, e2e, training, stream):
+    """(the one JSON line of a run, its details). The line holds the headline and one figure of
+    every other measurement and stays below 2000 characters, so that whoever keeps only the end
+    of the output keeps all of it; stages, tallies, training and stream are the details."""
+    r = res["surrogate"]
+    top = roofline(r, traffic) or {}
+    exact = res.get("batched")
+    mism = ({f: int(np.count_nonzero(v["bound_host"] != exact["bound_host"]))
+             for f, v in res.items() if f.startswith("surrogate")} if exact else None)
+    line = {
+        "metric": METRIC, "value": r["value"], "unit": UNIT, "n_gpus": ws, "steps": args.steps,
+        "warmup": args.warmup, "ms_per_step": r["ms_per_step"],
+        "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
+        "data": "synthetic",
+        "config": {"workload": args.workload, "n": n, "box": box, "seed": seed,
+                   "form": "surrogate (batched + surrogate)", "nodes": r["nodes"],
+                   "members": r["members"], "pairs": r["pairs"]["pairs_all"],
+                   "l2": "inputs and hierarchy larger than L2 (no flush)",
+                   "parallelism": f"independent snapshots x{ws}"},
+        "e2e": _short(e2e, 9), "gpu_launches": r["launches"], "clocks": r["clocks"],
+        "roofline": _short({k: top.get(k) for k in ("kernel", "bound", "ms_per_step", "achieved", "peak", "unit",
+                                                    "frac", "peak_source")}),
+        "cpu_baseline": _short({k: cpu[k] for k in ("value", "unit", "cores", "kind")}) if cpu else None,
+        "ms_per_step_of": _short({f: v["ms_per_step"] for f, v in res.items()}),
+        "identical_outputs": all(v["digest"] == r["digest"] for v in res.values()),
+        "flag_mismatches": sum(mism.values()) if mism else None,
+        "stream": _short({"particles": stream["particles"], "sequential": stream["sequential"]["value"],
+                          "lanes": stream["lanes"]["value"], "unit": UNIT,
+                          "identical_outputs": stream["identical_outputs"]}) if stream else None,
+    }
+    details = {"identical_outputs": {f: v["digest"] == r["digest"] for f, v in res.items()},
+               "surrogate_flag_mismatches_vs_batched": mism, "surrogate_training": training,
+               "cpu_baseline": cpu, "stream": stream,
+               "e2e": "pinned host buffers; the next step's inputs copied on a second stream during this "
+                      "step's compute; results read back every step",
+               "forms": {f: _form_entry(v, traffic) for f, v in res.items()}}
+    return line, details
+
+
 def run_ours(args):
     import torch
     import paper_2412_18629_gb300 as rs
@@ -712,35 +761,11 @@ def run_ours(args):
                          f"(those around the median halo load sum n^2), {tot_n} particles, "
                          f"{tot_t:.1f} s: FoF, hierarchy, unbinding, props"}
     if rank == 0:
-        ident = {f: v["digest"] == r["digest"] for f, v in res.items()}
-        exact = res.get("batched")
-        mism = ({f: int(np.count_nonzero(v["bound_host"] != exact["bound_host"]))
-                 for f, v in res.items() if f.startswith("surrogate")} if exact else None)
-        line = {
-            "metric": METRIC, "value": r["value"], "unit": UNIT, "n_gpus": ws, "steps": args.steps,
-            "warmup": args.warmup, "ms_per_step": r["ms_per_step"],
-            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
-            "data": "synthetic",
-            "config": {"workload": args.workload, "n": n, "box": snap["box"], "seed": spec.seed,
-                       "form": "surrogate (batched + surrogate)", "nodes": r["nodes"],
-                       "members": r["members"], "pairs": r["pairs"]["pairs_all"],
-                       "l2": "inputs and hierarchy larger than L2 (no flush)",
-                       "parallelism": f"independent snapshots x{ws}"},
-            "roofline": roofline(r, traffic), "cpu_baseline": cpu,
-            "e2e": {"value": e_units / e_max, "unit": UNIT, "h2d_bytes_per_step": h2d,
-                    "d2h_bytes_per_step": d2h, "steps": e_steps,
-                    "copies": "pinned host buffers; the next step's inputs copied on a second "
-                              "stream during this step's compute; results read back every step"},
-            "gpu_launches": r["launches"], "clocks": r["clocks"],
-            "plain_ms_per_step": res["plain"]["ms_per_step"] if "plain" in res else None,
-            "plain_value": res["plain"]["value"] if "plain" in res else None,
-            "batched_ms_per_step": res["batched"]["ms_per_step"] if "batched" in res else None,
-            "identical_outputs": ident,
-            "surrogate_flag_mismatches_vs_batched": mism,
-            "surrogate_training": training,
-            "stream": stream_res,
-            "forms": {f: _form_entry(v, traffic) for f, v in res.items()},
-        }
+        e2e = {"value": e_units / e_max, "unit": UNIT, "h2d_bytes_per_step": h2d,
+               "d2h_bytes_per_step": d2h, "steps": e_steps}
+        line, details = result_lines(args, res, ws, n, snap["box"], spec.seed, traffic, cpu, e2e,
+                                     training, stream_res)
+        print(json.dumps({"details": details}), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     if ws > 1:
         import torch.distributed as dist
