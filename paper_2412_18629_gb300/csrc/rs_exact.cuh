@@ -150,7 +150,9 @@ int launch_potential_list(rs_ctx* ctx, int R, float eps2, int64_t items_ub, int6
 // Flags of the exact-path list from S_all: S = S_all - w0. With B = 41u the bound of the blocked
 // sums relative to S_all = S + w0, |S - S_true| <= B (S + w0), so the member's relative bound is
 // Bi = B (1 + w0 / S) (plus slack, which covers the float64 additions); the flag is certain when
-// |KE + phi~| > 2 Bi |phi~|, otherwise the member is queued for the float64 potential.
+// |KE + phi~| > 2 Bi |phi~|, otherwise the member is queued for the float64 potential. w0 is the value that
+// the sums of the same kNormal hold.
+template <bool kNormal>
 __global__ void k_flags_list(const unsigned long long* __restrict__ count, const uint32_t* __restrict__ list,
                              const uint32_t* __restrict__ mem_of, const uint32_t* __restrict__ mnode,
                              const float4* __restrict__ V, const double* __restrict__ vbulk,
@@ -160,7 +162,7 @@ __global__ void k_flags_list(const unsigned long long* __restrict__ count, const
   if (w >= int64_t(*count)) return;
   const uint32_t k = list[w];
   const uint32_t p = mem_of[k], q = mnode[p];
-  const double w0 = double(rsqrtf(eps2));
+  const double w0 = double(rsd::inv_sqrt<kNormal>(eps2));
   const double S = Sd[w] - w0;
   const double ph = -__dmul_rn(Gm, S);
   const double e = __dadd_rn(kinetic(V[p], vbulk + 3 * int64_t(q)), ph);

@@ -916,8 +916,9 @@ int surrogate_unbind(rs_ctx* ctx, const double* vbulk, uint8_t* bound, unsigned 
       cudaEventDestroy(e1);
     }
   }
-  k_flags_list<<<grid_for(ns, kT), kT, 0, st>>>(counters + 0, exact_list, sur_mem, h.mnode, h.V, vbulk,
-                                               eps * eps, Gm, Sd, bound, ambig, counters + 2);
+  auto* flags = normal_eps2(eps * eps) ? k_flags_list<true> : k_flags_list<false>;
+  flags<<<grid_for(ns, kT), kT, 0, st>>>(counters + 0, exact_list, sur_mem, h.mnode, h.V, vbulk, eps * eps, Gm, Sd,
+                                        bound, ambig, counters + 2);
   RS_LAUNCHED(ctx, "k_flags_list");
   RS_TRY(unbind_fallback(ctx, counters + 2, ambig, vbulk, bound, st));
   k_acc_counter<<<1, 1, 0, st>>>(counters, 2, 6);

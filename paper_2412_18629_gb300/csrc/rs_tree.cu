@@ -961,8 +961,9 @@ int rs::tree_decide(rs_ctx* ctx, const int* only, const uint8_t* want, const dou
                                  h.node_off, h.node_size, h.U));
   }
   const double Gm = ctx->cfg.G * ctx->cfg.particle_mass;
-  k_flags_list<<<grid_for(T, kT), kT, 0, st>>>(ucount, ulist, tpos, h.mnode, h.V, vbulk, eps2, Gm, Sd, bound,
-                                              ambig, counters + 16);
+  auto* flags = normal_eps2(eps2) ? k_flags_list<true> : k_flags_list<false>;
+  flags<<<grid_for(T, kT), kT, 0, st>>>(ucount, ulist, tpos, h.mnode, h.V, vbulk, eps2, Gm, Sd, bound, ambig,
+                                       counters + 16);
   RS_LAUNCHED(ctx, "k_flags_list");
   RS_TRY(unbind_fallback(ctx, counters + 16, ambig, vbulk, bound, st));
   k_tree_acc<<<1, 1, 0, st>>>(counters, 16, 7);
