@@ -26,10 +26,18 @@
 //           expansion when a <= theta R' for the distance to the warp's target box and it holds none
 //           of the warp's targets, a leaf is summed directly (self excluded), otherwise its children
 //           are visited;
-//   slack   float32 evaluation and summation (per direct term <= ~8u, 32-term leaf blocks
-//           summed as two packed halves <= 31u, the target's own term left out, expansions with FMAs <= ~20u of n/R' in 32-cell
-//           blocks <= 31u, Kahan across blocks <= 2u) stay below 1e-5 relative; the truncation
-//           terms are summed in float32 and widened by 0.1%:
+//   slack   u = 2^-24, A = n/R', q^2 = tr(Q)/(n R'^2) <= h^2. A cell's R'^2 is within 6u (differences, three
+//           FMAs, eps^2), 1/R' within 5.2u (rsqrt.approx 2^-22.9), so n/R' is within 5.2u A and the
+//           quadrupole part, at most q^2 A, within 72u q^2 A (sum of the absolute values of its terms
+//           <= 2 q^2 A, its R'^-5 the most part); 32-cell blocks add at most 32 terms in each packed half, Kahan
+//           across blocks and the slices' sums 4u: at most 42u A + 109u q^2 A a cell. A <= (1 + q) S_cell
+//           (every member's kernel is at least (1/R')/(1 + h_j)), so the first part is below 80u of the
+//           cell's sum for theta <= 0.9. Direct terms: 8u each, 31u in a block, 2u Kahan; the target's own
+//           term is left out. All of it is below 81u < 5e-6 relative, half of the slack of 1e-5. The
+//           quadrupole part is covered by widening the truncation bound by 0.1%: that is at least
+//           0.001 q^3 A (power means: b >= n (tr(Q)/n)^(3/2)), half of which exceeds 109u q^2 A from
+//           q = 0.013 on, and below that it is under 0.02u A. The other half covers the bound's own
+//           rounding, 30u a cell and 18u for its sums (16 adds a half of a block, Kahan across blocks):
 //           S_lo = S~ (1 - 1e-5) - 1.001 B, S_hi = S~ (1 + 1e-5) + 1.001 B;
 //           the float64 sum differs from the exact one by < g 2^-53 relative.
 //   decide  bound iff KE - G m S_lo < -tol, unbound iff KE - G m S_hi > tol (tol = 1e-12 G m
@@ -472,16 +480,18 @@ struct __align__(16) WalkShared {
   uint32_t dir[64];
 };
 
-// Sum and truncation bound of one target over the tree, for the warp's lanes.
+// Sum and truncation bound of one target over the tree, for the warp's lanes: Kahan sums over blocks.
 struct WalkSum {
-  float S = 0.f, C = 0.f;  // Kahan sum over blocks
-  float2 B = {0.f, 0.f};   // truncation bound (two halves)
-  __device__ __forceinline__ void add(float blk) {
-    const float y = __fsub_rn(blk, C);
-    const float t = __fadd_rn(S, y);
-    C = __fsub_rn(__fsub_rn(t, S), y);
-    S = t;
+  float S = 0.f, C = 0.f;
+  float B = 0.f, D = 0.f;
+  static __device__ __forceinline__ void add(float& sum, float& carry, float blk) {
+    const float y = __fsub_rn(blk, carry);
+    const float t = __fadd_rn(sum, y);
+    carry = __fsub_rn(__fsub_rn(t, sum), y);
+    sum = t;
   }
+  __device__ __forceinline__ void add(float blk) { add(S, C, blk); }
+  __device__ __forceinline__ void add_bound(float blk) { add(B, D, blk); }
 };
 
 // Quadrupole expansions of `cnt` (1..32) accepted cells: lane = cell while they are staged (as pairs,
@@ -507,7 +517,7 @@ __device__ __forceinline__ void walk_cells(const Cell* __restrict__ ncell, const
   __syncwarp();
   const float2 tx = make_float2(t.x, t.x), ty = make_float2(t.y, t.y), tz = make_float2(t.z, t.z);
   const float2 e2 = make_float2(eps2, eps2), kc = make_float2(chord, chord), one = make_float2(1.f, 1.f);
-  float2 blk = make_float2(0.f, 0.f);
+  float2 blk = make_float2(0.f, 0.f), bnd = make_float2(0.f, 0.f);
   auto lo = [](float4 a) { return make_float2(a.x, a.y); };
   auto hi = [](float4 a) { return make_float2(a.z, a.w); };
   for (int k = lane / (32 / kSlices); 2 * k < cnt; k += kSlices) {
@@ -525,9 +535,10 @@ __device__ __forceinline__ void walk_cells(const Cell* __restrict__ ncell, const
     blk = __ffma2_rn(lo(a2), ri, blk);
     blk = __ffma2_rn(__fmul2_rn(ri2, ri), quad, blk);
     const float2 f = __ffma2_rn(__fmul2_rn(hi(a1), ri), kc, one);
-    R.B = __ffma2_rn(__fmul2_rn(hi(a7), __fmul2_rn(ri2, ri2)), f, R.B);
+    bnd = __ffma2_rn(__fmul2_rn(hi(a7), __fmul2_rn(ri2, ri2)), f, bnd);
   }
   R.add(__fadd_rn(blk.x, blk.y));
+  R.add_bound(__fadd_rn(bnd.x, bnd.y));
 }
 
 // Direct sums over `cnt` leaves, two members per packed float32x2 step; slots past a leaf's count
@@ -698,7 +709,7 @@ k_tree_walk(WalkArgs A) {
       walk_cells<kNormal, kSlices>(ncell, W.acc, na, t, A.eps2, A.chord, lane, W, R);
     }
     if (nd > 0) walk_leaves<kNormal, kSlices>(nx, W.dir, nd, g32, t, self_rel, A.eps2, lane, W, R, n_dir);
-    float S = R.S, Bt = __fadd_rn(R.B.x, R.B.y);
+    float S = R.S, Bt = R.B;
 #pragma unroll
     for (int off = kTargets; off < 32; off <<= 1) {  // the slices of a target
       S = __fadd_rn(S, __shfl_xor_sync(0xffffffffu, S, off));
