@@ -30,8 +30,7 @@ enum Slot : int {
   S_SCAN_TMP, S_CHUNK_OFF, S_CHUNK_SUM, S_NODE_TMP, S_SELECT,
   // hierarchy state (persists until the next rs_fof6d)
   S_H_MEM, S_H_MNODE, S_H_U, S_H_V, S_H_NODE_OFF, S_H_NODE_SIZE, S_H_NODE_PARENT,
-  S_H_NODE_LEVEL, S_H_NODE_MINID, S_H_NODE_REF, S_H_NODE_INV, S_H_DEEPEST, S_H_DEEPPOS, S_H_WORK,
-  S_H_NODE_MOM,
+  S_H_NODE_LEVEL, S_H_NODE_MINID, S_H_NODE_REF, S_H_NODE_INV, S_H_DEEPEST, S_H_DEEPPOS, S_H_NODE_MOM,
   // rs_unbind / rs_halo_props state
   S_U_PHI, S_U_BOUND, S_U_NB, S_U_VBULK, S_U_AMBIG, S_U_FLAGS, S_U_TILEBIG,
   S_U_TILEPERM, S_U_OKEY_A, S_U_OKEY_B, S_U_OVAL_A, S_U_OVAL_B, S_U_FBMAX, S_U_FBCHUNK,
@@ -51,7 +50,7 @@ enum Slot : int {
   // certified tree bound of the potential (rs_tree.cu)
   S_T_OFF, S_T_RANK, S_T_COFF, S_T_NODES, S_T_BOX, S_T_KA, S_T_KB, S_T_VA, S_T_VB, S_T_X, S_T_POS,
   S_T_CELL, S_T_ORDER, S_T_WF, S_T_WL, S_T_WR, S_T_UF, S_T_LIST, S_T_LR, S_T_SX, S_T_REC,
-  S_T_WANT, S_SUR_SD,
+  S_SUR_SD,
   // seed halos (rs_seeds.cu)
   S_SEED_KIDS, S_SEED_ROOT, S_SEED_UCNT, S_SEED_UOFF, S_SEED_CEN, S_SEED_REC, S_SEED_SUMS, S_SEED_SEG,
   S_SEED_COUNT, S_SEED_LIST, S_SEED_REF,

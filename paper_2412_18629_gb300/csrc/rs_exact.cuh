@@ -127,13 +127,12 @@ k_potential_list(int64_t nbig, const int64_t* __restrict__ item_off, const int64
 }
 
 // The sums of a list of at most `len_ub` members with R members per thread (2, 4 or 8); Sd is zeroed
-// first. items_ub bounds the item count (the launch is persistent).
+// first. Eight blocks an SM stride over the items, whose number only the device knows.
 template <class... Args>
-int launch_potential_list(rs_ctx* ctx, int R, float eps2, int64_t items_ub, int64_t len_ub, double* Sd,
+int launch_potential_list(rs_ctx* ctx, int R, float eps2, int64_t len_ub, double* Sd,
                           cudaStream_t st, Args... args) {
   RS_CUDA(ctx, cudaMemsetAsync(Sd, 0, sizeof(double) * size_t(len_ub), st));
-  const unsigned grid = unsigned(std::max<int64_t>(1, std::min<int64_t>(items_ub, 152 * 8)));
-  auto launch = [&](auto kernel) { kernel<<<grid, kListThreads, 0, st>>>(args..., eps2, Sd); };
+  auto launch = [&](auto kernel) { kernel<<<152 * 8, kListThreads, 0, st>>>(args..., eps2, Sd); };
   if (rs::normal_eps2(eps2)) {
     if (R == 2) launch(k_potential_list<2, true>);
     else if (R == 8) launch(k_potential_list<8, true>);

@@ -895,7 +895,7 @@ int surrogate_unbind(rs_ctx* ctx, const double* vbulk, uint8_t* bound, unsigned 
       if (c < 3) RS_CUDA(ctx, cudaEventRecord(e0, st));
       {
         ProfScope prof_(ctx, c < 3 ? "k_potential_list_tune" : "k_potential_list", st);
-        RS_TRY(launch_potential_list(ctx, R, eps * eps, int64_t(1) << 30, ns, Sd, st, nbig, ltiles, big_nodes, lofs,
+        RS_TRY(launch_potential_list(ctx, R, eps * eps, ns, Sd, st, nbig, ltiles, big_nodes, lofs,
                                      lend, exact_list, sur_mem, h.node_off, h.node_size, h.U));
       }
       if (c < 3) {

@@ -968,7 +968,7 @@ int rs::tree_decide(rs_ctx* ctx, const int* only, const uint8_t* want, const dou
   const float eps2 = ctx->cfg.softening * ctx->cfg.softening;
   {
     ProfScope prof_(ctx, "k_potential_list", st);
-    RS_TRY(launch_potential_list(ctx, R, eps2, int64_t(1) << 30, T, Sd, st, nt, ltiles, tnode, lofs, lend, ulist, tpos,
+    RS_TRY(launch_potential_list(ctx, R, eps2, T, Sd, st, nt, ltiles, tnode, lofs, lend, ulist, tpos,
                                  h.node_off, h.node_size, h.U));
   }
   const double Gm = ctx->cfg.G * ctx->cfg.particle_mass;
