@@ -171,7 +171,8 @@ int rs_fof6d_copy(rs_ctx* ctx, int64_t* node_parent, int32_t* node_level, int64_
  * its adaptive squared link length. Errors: RS_ERR_STATE, RS_ERR_CUDA. */
 int rs_fof6d_node_params(rs_ctx* ctx, float* params_out, void* stream);
 
-/* Unbinding of every node of the last rs_fof6d hierarchy (pos, vel: the same arrays).
+/* Unbinding of every node of the last rs_fof6d hierarchy (pos, vel: the same arrays, with the contents that
+ * rs_fof6d saw, which the context keeps; arrays at other addresses are gathered anew).
  * phi_i = -G m sum_{j != i} 1 / sqrt(|u_j - u_i|^2 + eps^2) over the node's members;
  * KE_i = 0.5 |v_i - v_bulk|^2 (float64, v_bulk = mean member velocity); bound iff
  * KE_i + phi_i < 0 with phi the float64 canonical-order sum; halo iff
@@ -312,7 +313,8 @@ int rs_run_batched(rs_ctx* ctx, int32_t n_snap, const rs_snapshot* snaps, int32_
  * terms evaluated by the walk, pair terms of the exact list sums (tree and surrogate paths), 0.
  * rs_tree_record(ctx, 1): later rs_unbind calls also record every bounded member's interval;
  * rs_tree_bounds then copies them out: lo_out, hi_out float64 [n_members] device (member CSR
- * order), NaN for members whose flag did not come from the bound walk. Errors: RS_ERR_STATE when
+ * order), NaN for members whose flag did not come from the bound walk. An interval holds the member's sum;
+ * its width depends on tree_theta and the walk and is no part of the contract. Errors: RS_ERR_STATE when
  * the last rs_unbind recorded nothing. Instrumentation for tests, not part of the method. */
 int rs_tree_stats(rs_ctx* ctx, int64_t* stats_out);
 int rs_tree_record(rs_ctx* ctx, int enable);
@@ -439,9 +441,9 @@ int rs_profile(rs_ctx* ctx, int enable);
 
 /* Work counting of the batched form's pruned 6D kernels (instrumentation, not part of the
  * method): while enabled, k_nn6d_pruned and k_link6d_pruned run a variant that tallies, per
- * query lane, the d6 evaluations it performs and the box lower bounds it computes (bucket,
- * sub-bucket and superbucket tests; box-box tests counted once per warp); the results are
- * unchanged. rs_count_work(ctx, 1, NULL) clears the tallies and enables counting;
+ * query lane, the d6 evaluations it performs and the box lower bounds it computes (bucket and
+ * superbucket tests, each box-box test counted once); the results are unchanged. Levels of few pairs
+ * (sum of g^2 at most 4e7) run the all-pairs kernels, which are not tallied. rs_count_work(ctx, 1, NULL) clears the tallies and enables counting;
  * rs_count_work(ctx, 0, counts) disables it. counts_out (host int64 [6], may be NULL) receives,
  * after a device synchronisation: NN d6 evaluations, NN box tests, link d6 evaluations, link
  * box tests, nodes whose nearest-neighbour search ran with sampled bounds, and those of them

@@ -70,7 +70,10 @@ constexpr int64_t kSurrogateMinMembers = 1024;
 // opening angle (a cell is expanded when its radius bound is at most theta times the distance).
 // rs_unbind on the 2^27 snapshot takes 131 / 130 / 135 / 146 ms from 2048 / 4096 / 8192 / 16384 members
 // (theta = 0.7), and 150 / 131 / 126 / 122 / 121 / 123 ms at theta = 0.6 / 0.7 / 0.75 / 0.8 / 0.85 / 0.9
-// (from 2048 members): flat minima. Nodes below the threshold keep the plain form's direct sums.
+// (from 2048 members): flat minima. From 4096 / 8192 / 16384 members at theta = 0.8, and from 8192 at 0.6 /
+// 0.7 / 0.9: 2^25 particles 24.5 / 25.9 / 29.8, 30.0 / 27.4 / 25.7 ms; 2^24 9.5 / 10.2 / 12.6, 11.6 / 10.8 /
+// 9.9 ms; 2^22 2.65 / 2.84 / 3.41, 3.01 / 2.93 / 2.78 ms; 2^20 1.59 / 1.78 / 1.93, 2.00 / 1.90 / 1.72 ms; 2^18
+// 1.08 / 1.18 / 1.22, 1.15 / 1.17 / 1.16 ms. Nodes below the threshold keep the plain form's direct sums.
 constexpr int64_t kTreeMinDefault = 8192;
 constexpr float kTreeThetaDefault = 0.8f;
 
@@ -304,8 +307,7 @@ __device__ __forceinline__ float sq3(float dx, float dy, float dz) {
   return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
 }
 
-// 1 / sqrt(x) for the float32 potentials, which are bound by issue slots and the special-function unit. The
-// PTX instruction with .ftz takes subnormal arguments as zero; with a normal squared softening every
+// 1 / sqrt(x) for the float32 potentials, one a pair. The PTX instruction with .ftz takes subnormal arguments as zero; with a normal squared softening every
 // argument is at least eps^2, so kNormal takes that form: direct sums of the 2^27 snapshot 56.3 -> 41.8 ms
 // (nodes below 16384 members), list sums 110 -> 82 ms. Both forms give the same value for every normal
 // argument and infinity (compared over all of them by a test).

@@ -85,7 +85,7 @@ __device__ __forceinline__ double warp_cro_combine_all(const double (&acc)[NS], 
 // position), Term::add<first>(q, value, acc) adds its NS terms (first: the lane's first term, added to
 // 0.0 by rsd::cro_add<true>). Elements are loaded kCroAhead at a time before they are added in order.
 // The totals of a segment of one chunk are its sums. Bound by the float64 pipe (two lanes a clock and
-// SM): consecutive chunks go to different blocks, so that the chunks of a large node do not queue at
+// SM; busy 77% of the cycles for the 12 moments of 2^24 particles' groups): consecutive chunks go to different blocks, so that the chunks of a large node do not queue at
 // one SM's pipe (2^18 particles: 312 -> 225 us over eight
 // levels; 2^27: 8.3 -> 6.0 ms, properties 16.5 -> 10.6 ms).
 // chunk_off has nseg + 1 entries (the last one is the total number of chunks).

@@ -19,9 +19,10 @@
 //
 // A thread per particle searching the stencil repeated each search for all particles of a dense cell,
 // with two root searches per visited cell. Measured on 2^24 particles in L = 256 Mpc/h: link kernels
-// 6.4 -> 2.0 ms, the whole call 8.8 -> 4.2 ms; 2^27 particles in L = 512: 51 -> 15 ms. Bound by issue
-// slots in the row searches (searching the rows of one z side by side, to overlap their loads, was
-// slower: 20 ms).
+// 6.4 -> 2.0 ms, the whole call 8.8 -> 4.2 ms; 2^27 particles in L = 512: 51 -> 15 ms. In the 2^24 case (ncu) the
+// far pass has its issue slots busy 75% of the cycles (row searches); the near pass 52%, its warps waiting 14
+// cycles an instruction for gathers. Searching the rows of one z side by side, to overlap their loads, was
+// slower: 20 ms.
 #include <cmath>
 
 #include "rs_common.cuh"

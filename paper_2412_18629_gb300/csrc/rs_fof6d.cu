@@ -477,8 +477,10 @@ k_nn6d(int64_t nb, int64_t nn, const int64_t* __restrict__ item_off, const int64
 constexpr int64_t kSelectWarpMax = 1024;
 // Levels of more ordered pairs (sum of g^2) take the pruned searches of the batched form; below, the
 // all-pairs kernels cost less than their set-up (about 40 launches; 4e7 pairs are 0.05 ms of work on the
-// whole GPU). A 2^18-particle pass takes 600 device operations and 4.7 ms of device time with this line,
-// 794 and 5.7 ms when every level above 4096 members was pruned.
+// whole GPU). rs_fof6d with the line at 0 / 1e7 / 4e7 / 1.6e8 pairs: 2^16 particles 2.98 / 1.72 / 1.36 /
+// 1.35 ms, 2^18 5.35 / 4.53 / 4.14 / 3.64 ms, 2^20 6.32 / 5.25 / 4.85 / 4.33 ms (groups of up to 1e5 members
+// 6.63 / 5.58 / 5.17 / 5.18 ms), 2^22 9.67 / 8.60 / 8.28 / 7.83 ms. The tests of the pruned searches' tallies
+// hold it below 4.6e7.
 constexpr unsigned long long kPrunedMinPairs = 40000000ull;
 
 // only (if given): int [nn], the nodes to select for (the others keep their l2).
@@ -541,8 +543,8 @@ k_select_l2_warp(int64_t nb, int64_t nn, const int64_t* __restrict__ node_off,
   if (lane == 0) inv[q].z = __uint_as_float(prefix);
 }
 
-// Blocks of 1024 threads stride over the level's nodes and select in the large ones, 11 bits a pass
-// (31 value bits: three passes). Bound by the latency of one block's loads: 256 threads and four
+// Blocks of 1024 threads stride over the level's nodes and select in the large ones, 11, 11 and 9 bits a
+// pass (31 value bits). Bound by the latency of one block's loads: 256 threads and four
 // passes took 20.3 ms per 2^27 pass (33 launches, nodes up to 1.5e6 members), this form 3.1 ms.
 // only (if given): int [nn], the nodes to select for (the others keep their l2).
 constexpr int kSelThreads = 1024;

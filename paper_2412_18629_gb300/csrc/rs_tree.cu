@@ -608,9 +608,10 @@ __device__ __forceinline__ void walk_leaves(const float4* __restrict__ nx, const
 // One warp per 32 wanted targets of one node: the certified walk, then the decision. A step opens up
 // to four pending cells and tests their children side by side (lane = child) against the box of the
 // warp's targets; accepted cells and leaves to sum are listed and evaluated 32 at a time with lane =
-// target. Bound by the special-function unit in the leaves (one rsqrt a pair) and by the float32 pipe
-// in the expansions; testing one cell a step with every lane spent most of the walk on loads and
-// stack traffic. On the 2^27 snapshot (4.9e7 members) the walk went from 295 to 58 ms: 2.5 times fewer
+// target. In a 2^24-particle pass (ncu) the issue slots are busy 64% of the cycles, the float32 pipe 35%, the
+// special-function unit 24%; warps wait for shared memory and for the units' queues (2.6 and 1.5 cycles
+// an instruction). Testing one cell a step with every lane spent most of the walk on loads and stack
+// traffic. On the 2^27 snapshot (4.9e7 members) the walk went from 295 to 58 ms: 2.5 times fewer
 // interactions from the exact a and b at theta = 0.7, the rest from the form of the walk.
 // Indices inside the walk are 32-bit and relative to the node (its members are [tb, tb + g) of the
 // sorted arrays, its cells [cb, cb + cells) of the cell array).

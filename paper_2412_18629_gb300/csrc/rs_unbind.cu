@@ -93,10 +93,11 @@ k_potential(int64_t m, const uint32_t* __restrict__ mnode, const int64_t* __rest
 // are formed as u_j + (-u_i), which equals fl(u_j - u_i). The per-member summation is
 // unchanged (32-term sequential blocks, Kahan across blocks), so the certified bound kCertB
 // holds as is. The self pair is tested only on the diagonal j-tiles. Blocks are ordered by
-// the node's size class, largest first, so the longest blocks start first. Bound by issue slots
-// and the special-function unit (one rsqrt a pair); the flush-to-zero rsqrt (rsd::inv_sqrt) took
-// this kernel from 56.3 to 41.8 ms on the nodes below 16384 members of the 2^27 snapshot and the
-// list form of rs_exact.cuh from 110 to 82 ms.
+// the node's size class, largest first, so the longest blocks start first. Its issue
+// slots are busy 72% of the cycles, the special-function unit (one rsqrt a pair) 43%, the float32 pipe 39% (ncu,
+// 2^24 particles, two members a thread). The flush-to-zero rsqrt (rsd::inv_sqrt) took this kernel from
+// 56.3 to 41.8 ms on the nodes below 16384 members of the 2^27 snapshot and the list form of rs_exact.cuh
+// from 110 to 82 ms.
 constexpr int kBlkThreads = 128;
 // Members per thread (kBlkR) is a template parameter chosen per context by the autotuner among
 // 2, 4 and 8 (tiles of 256, 512 or 1024 members); every choice gives bit-identical sums.
