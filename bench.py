@@ -341,10 +341,10 @@ def roofline(r, traffic=None):
 
 
 def _traffic_table():
-    """DRAM bytes (read + write) per launch of the profiled kernels, from one ncu capture of the
-    bench command (profiles/dram_traffic.json, written from that capture; the summary beside it
-    gives the command): {workload: {kernel: bytes per launch}}. A kernel changed since its
-    capture has no entry."""
+    """DRAM bytes (read + write) per launch of the profiled kernels, from one ncu capture
+    (profiles/dram_traffic.json, written from that capture; the summary beside it gives the
+    command): {workload: {kernel: bytes per launch}}. A kernel changed since its capture has no
+    entry, and a workload without a capture of the present kernels has none."""
     path = os.path.join(ROOT, "profiles", "dram_traffic.json")
     try:
         with open(path) as f:
