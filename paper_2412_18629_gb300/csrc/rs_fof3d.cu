@@ -194,8 +194,8 @@ constexpr uint32_t kPairChunk = 1024;
 
 // Pairs whose larger cell holds at most kSmallPair particles share the first `cap` items; when those are
 // full a thread tests the pair by itself. The other pairs have items of their own after them, enough for
-// all there can be (pair_items), so that no thread is left with the pairs of two large cells: 1e8 pairs of
-// particles took one thread 22 s.
+// all there can be (pair_items), so that no thread is left with the pairs of two large cells: a call with
+// 1e8 pairs of particles beside a full list took 22 s on one thread, 7 ms in this form.
 constexpr uint32_t kSmallPair = 512;
 
 // Most items of pairs with a cell above kSmallPair. A pair takes ceil(s / kPairChunk) items, s its larger
